@@ -40,7 +40,7 @@ struct hsd_ctx {
   bool pdl;           // kernels are launched with programmatic stream serialization
   int force_bn, force_splits;   // hsd_debug_set_gemm_tile
   int pair;                     // GEMMs may run as CTA pairs
-  int attn_target_items, attn_min_chunk;   // attention plan: items aimed at per launch, fewest 128-key KV tiles per slice
+  int attn_target_items, attn_min_chunk;   // attention plan: items aimed at per launch, fewest 64-key KV blocks per slice
   int tap_layer, tap_which;                // hsd_debug_tap: armed for the next forward (tap_layer < 0: none)
   void* tap_dst;
   size_t tap_bytes;
@@ -89,8 +89,8 @@ struct Ws {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// CTAs of an attention launch: as many as are resident at once (two per SM with head_dim 64, one with 128)
-inline int attn_grid(const hsd_ctx* c) { return (c->md.D == 128 ? 1 : 2) * c->n_sms; }
+// CTAs of an attention launch: as many as are resident at once
+inline int attn_grid(const hsd_ctx* c) { return 2 * c->n_sms; }
 
 inline int attn_max_tiles(const ModelDims& md, int T, int S) { return T / (128 / md.group) + S; }
 // Split-KV partial results: per (q-tile, kv head, slice) 128 rows of an fp32 accumulator row plus (max, sum).
@@ -146,7 +146,7 @@ Ws carve(const hsd_ctx* c, void* base, int T, int S) {
     w.plan.items_unsorted = static_cast<int4*>(take(sizeof(int4) * 2 * (size_t)mt * kAttnMaxSplits));
     w.plan.tile_seq = static_cast<int*>(take(sizeof(int) * mt));
     w.plan.tile_nkv = static_cast<int*>(take(sizeof(int) * mt));
-    w.plan.counters = static_cast<int*>(take(sizeof(int) * (size_t)mt * md.Hkv));
+    w.plan.counters = static_cast<int*>(take(sizeof(int) * (size_t)mt * md.Hkv * 4));
     w.plan.first = static_cast<int4*>(take(sizeof(int4) * 3 * 2 * (size_t)c->n_sms));
     w.plan.n_items = w.status ? w.status + 5 : nullptr;
     w.plan.n_kv_heads = md.Hkv;
@@ -281,7 +281,7 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
   CUtensorMap tm_h, tm_attn, tm_act, tm_q, tm_k, tm_v, tm_x_add, tm_q_st, tm_act_st;
   if (!c->attn_simt) {
     Scope s(c, st, KC_SETUP);
-    // items per launch: a few per CTA slot (two CTAs per SM), at least attn_min_chunk KV tiles each
+    // items per launch: about one per CTA slot (two CTAs per SM), at least attn_min_chunk KV blocks each
     // (a context with a fixed summation order never cuts a KV range: where the cuts fall depends on the batch)
     launch_attn_plan(st, w.rm, w.plan, kv, a.n_seqs, tokens_per_tile, max(1, c->attn_target_items / md.Hkv),
                      c->max_splits == 1 ? (1 << 20) : c->attn_min_chunk,
@@ -570,7 +570,7 @@ int hsd_create(const hsd_model_config* cfg, const hsd_weights* w, hsd_ctx** out)
   c->hg_exec = nullptr;
   c->hg_launches = 0;
   c->attn_target_items = attn_grid(c);   // one item per CTA slot: slicing costs a partial hand-over per slice
-  c->attn_min_chunk = 4;
+  c->attn_min_chunk = 8;
   c->tap_layer = -1; c->tap_which = 0; c->tap_dst = nullptr; c->tap_bytes = 0;
   c->last_cuda_error = 0;
   c->launches = 0;
@@ -1134,7 +1134,7 @@ int hsd_debug_set_gemm_tile(hsd_ctx* c, int tile_n, int k_slices) {
 int hsd_debug_set_attn_plan(hsd_ctx* c, int target_items, int min_kv_tiles) {
   if (!c || target_items < 0 || min_kv_tiles < 0) return HSD_ERR_INVALID_ARG;
   c->attn_target_items = target_items ? target_items : attn_grid(c);
-  c->attn_min_chunk = min_kv_tiles ? min_kv_tiles : 4;
+  c->attn_min_chunk = 2 * (min_kv_tiles ? min_kv_tiles : 4);
   return HSD_OK;
 }
 

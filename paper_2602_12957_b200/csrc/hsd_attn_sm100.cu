@@ -4,60 +4,63 @@
 // (the chain case of the paper's tree-ancestry mask, Sec. 3.2 / Fig. 2(c)).
 //
 // Work item = (q-tile, kv slice, kv head).  A q-tile is 128 MMA rows: 128/group consecutive tokens of one
-// sequence x the `group` query heads that share the kv head (GQA packing, so K/V tiles are read once per
+// sequence x the `group` query heads that share the kv head (GQA packing, so K/V blocks are read once per
 // group).  The KV range a q-tile can see is cut into up to kAttnMaxSplits slices so that a launch has about one item
 // per CTA slot whatever the mix of context lengths (one page chunk over a long context, or many short regions); the
 // plan is made once per step on the device (attn_plan_kernel) and reused by every layer.  Slices leave (unnormalised
 // O, exponent reference, sum) partials in the workspace and the last slice to finish combines them in slice order, so
 // the result does not depend on which CTA ran what.
 //
-// A KV tile is 128 keys = two paged blocks [64 keys][head_dim] per kv head, fetched by TMA through the block table,
-// 64 dims at a time, into adjacent halves of a stage; K is the K-major B operand of S = Q K^T (one 128 x 128 x
-// head_dim product per tile), V the MN-major B operand of O += P V (128 x head_dim x 128).  Persistent CTAs walk the
-// item list: two per SM with head_dim 64, one with 128 (tensor-memory columns).  Warp roles:
-// warp 0 = TMA producers (lane 0: Q and the K ring, lane 1: the V ring; K is free as soon as S has been formed, V
-// only after the second product, so the two rings run at their own pace and two stages each suffice), warp 1 = MMA
-// issuer + TMEM owner, warps 2..9 = softmax: warp w works on TMEM lane quarter w mod 4 (the hardware's rule), warps
-// 2..5 on keys 0..63 of the tile and warps 6..9 on keys 64..127, one thread per (row, half).
-// Per tile: S (TMEM, 128 fp32 columns) -> softmax in registers -> P (bf16, back into TMEM: 64 columns, the A operand
-// of the second product, so P never passes through shared memory) -> O += P V accumulated in tensor memory.
-// What the measurements behind this shape said (64-key tiles, four softmax warps, P through shared memory, per tile
-// and CTA): the softmax warps' own instruction stream ~1,950 cycles, half of it the 64 exponentials of a row queueing
-// with the other CTA's on the SM's 16 exp lanes per clock; the issuing thread ~1,300 (140-220 cycles for every probe
-// of an already completed barrier, 70-90 per MMA or commit).  Twice the keys per barrier round and MMA group, twice
-// the warps on the exponentials, and no shared-memory round trip for P attack both.
-// The exponent reference of a row is not its running maximum but a value that is raised only when the maximum has
-// grown by more than kRescaleBits binary orders since it was set (P stays below 2^kRescaleBits, far inside bf16 and
-// fp32 range): then, and only then, the row's accumulator is read, scaled and written back; after the first tiles of
-// a row that is rare.  The two threads of a row swap their halves' maxima through shared memory once per tile, so they
-// take the same decisions.  Every wait is a bounded mbarrier wait, so one that gives up takes the whole CTA to the
-// common exit.
+// The KV range is walked in paged blocks of 64 keys [64 keys][head_dim] per kv head, fetched by TMA through the block
+// table; K is the K-major B operand of S = Q K^T (128 x 64 x head_dim), V the MN-major B operand of O += P V (128 x
+// head_dim x 64).  Persistent CTAs, two per SM, walk the item list.  Warp roles:
+//   warp 0      TMA producer: Q, the K ring and the V ring
+//   warp 1      MMA issuer + TMEM owner
+//   warps 2..5  softmax: warp w works on TMEM lane quarter w mod 4 (the hardware's rule), one thread per q row
+// Per block: S (TMEM, 64 fp32 columns) -> softmax in registers -> P (bf16) over the same columns, the A operand of the
+// second product, so P never passes through shared memory -> O += P V accumulated in tensor memory.  NBUF score
+// buffers rotate: while the softmax warps work on block t, S(t + 1) .. S(t + NBUF - 1) are formed already, and the
+// buffer of block t is taken by S(t + NBUF) once the product that reads P(t) has completed.  Nothing in the softmax
+// warps' loop waits for a product of the same block.
+//
+// What bounds it: the exp unit, 16 results per clock and SM, i.e. 512 cycles for the 128 x 64 scores of a block, and
+// the softmax warps' own dependent chain around it.  One thread owns a row, so a row's threads have nothing to agree
+// on, and the exponent reference does not wait for a maximum: it is the maximum of the first 64 keys the row saw, later
+// exponentials start as soon as their scores are in registers, and the row sum, which is needed anyway, shows whether a
+// score has outgrown the reference (P and the sums are scale-free in bf16 / fp32 as long as they stay in range).  Where
+// a sum of 64 exceeds kRescaleSum the 64 are taken again under a new reference and the accumulator row is rescaled.
+// Measured, one launch of a 2,048-row chunk over 16,384 committed rows, 16 / 8 heads of 64: 294 us with eight softmax
+// warps, two threads a row swapping maxima through shared memory ahead of the exponentials, on 128-key tiles with one
+// score buffer; 274 us with one thread a row and the reference checked by the sum; 245 us with 64-key blocks, rotating
+// score buffers and elected issue.  8 heads of 128: 233 us (one CTA per SM) to 145 us.  A block takes the two CTAs of an
+// SM 1,340 cycles for their two (the exp unit would need 1,024); of a softmax warp's own ~1,100 cycles 700 are the 64
+// exponentials of its rows.  Fetching the next block's scores before the P store is waited for was slower (register
+// moves), and so was a barrier probe without the suspend-time hint.
+// Every wait is a bounded mbarrier wait, so one that gives up takes the whole CTA to the common exit.
 #include "hsd_kernels.h"
 
 namespace hsd {
 
-constexpr int kSoftmaxWarps = 8;
+constexpr int kSoftmaxWarps = 4;
 constexpr int kAttnThreads = 32 * (2 + kSoftmaxWarps);
-constexpr int KV_STAGES = 2;                       // per ring
-constexpr int SUB_BYTES = 128 * 128;               // one K-major operand sub-tile: 128 rows (q rows / keys) x 64 dims
+constexpr int SUB_BYTES = 128 * 128;               // one K-major operand sub-tile of Q: 128 rows x 64 dims
 constexpr int KV_BLOCK_BYTES = 64 * 128;           // one paged block of K or of V for one kv head, 64 dims of it
 constexpr int ATTN_BAR_BYTES = 256;
-constexpr int ATTN_XCH_BYTES = 2 * 128 * 2 + 2 * 128 * 4;   // per (half, row): the tile's half-row maximum (bf16); the item's half-row sum (fp32)
-constexpr float kRescaleBits = 8.f;
+constexpr float kRescaleSum = 1099511627776.f;     // 2^40: a row's 64 exponentials that sum to more ask for a new reference
 // Head dimension HD = 64 or 128.  An operand tile is HD / 64 sub-tiles of 64 dims each (a 128-byte-swizzled row is 64
-// bf16): Q [sub][128 rows][64], a K or V stage [sub][block 0, block 1][64 keys][64].  The accumulator has HD columns.
-// No alignment slack: with HD = 64 two CTAs of this size plus the per-CTA reserve share an SM, so the kernel relies
-// on the 1024-byte alignment it declares for its dynamic shared memory (the swizzled tiles need it) and checks it.
+// bf16): Q [sub][128 rows][64], a K or V stage [sub][64 keys][64].  The accumulator has HD columns and NBUF score
+// buffers of 64 share the 256 columns with it, so two CTAs fit the 512 columns of an SM at either head size.
+// No alignment slack: two CTAs of this size plus the per-CTA reserve share an SM, so the kernel relies on the 1024-byte
+// alignment it declares for its dynamic shared memory (the swizzled tiles need it) and checks it.
 template <int HD>
 struct AttnCfg {
   static constexpr int NSUB = HD / 64;
   static constexpr int Q_BYTES = NSUB * SUB_BYTES;
-  static constexpr int KV_TILE_BYTES = NSUB * SUB_BYTES;           // 128 keys
-  static constexpr int SMEM = Q_BYTES + 2 * KV_STAGES * KV_TILE_BYTES + ATTN_XCH_BYTES + ATTN_BAR_BYTES;
-  static constexpr int COL_O = 128, COL_P = 128 + HD;              // S: 128 fp32 columns, O: HD, P: 64 (two keys per column)
-  static constexpr int TMEM_COLS = HD == 64 ? 256 : 512;           // allocations are powers of two
-  static constexpr int CTAS_PER_SM = HD == 64 ? 2 : 1;             // tensor memory has 512 columns
-  static constexpr int OWN = HD / 2;                               // accumulator columns of one softmax thread
+  static constexpr int KV_BYTES = NSUB * KV_BLOCK_BYTES;           // one stage of a ring: 64 keys
+  static constexpr int STAGES = HD == 64 ? 4 : 2;                  // per ring
+  static constexpr int SMEM = Q_BYTES + 2 * STAGES * KV_BYTES + ATTN_BAR_BYTES;
+  static constexpr int TMEM_COLS = 256;
+  static constexpr int COL_O = TMEM_COLS - HD, NBUF = COL_O / 64;  // score buffers at columns 64 b
 };
 
 struct AttnParams {
@@ -65,7 +68,7 @@ struct AttnParams {
   const int* block_table;
   int max_blocks, n_blocks, Hq, Hkv, group, layer;
   bf16* out;            // [T, Hq*HD]
-  float* split_ws;      // partials of sliced items: [q-tile][kv head][slice][2 + HD][128 rows]
+  float* split_ws;      // partials of sliced items: [q-tile][kv head][quarter][slice][2 + HD][32 rows]
   const uint4* anc;     // [T] ancestry masks of candidate-tree rows, or nullptr: plain causal order within the call
   int* status;
 };
@@ -75,25 +78,30 @@ __device__ __forceinline__ float ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// packed pairs: one instruction for two fp32 operations
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+      "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+      "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float y;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
   return y;
 }
-__device__ __forceinline__ void named_bar_sync(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-// Barrier among whole warps on an mbarrier whose count is the number of warps: every lane's earlier shared-memory
-// writes are visible to every participant afterwards.  `phase` counts this thread's uses of `bar`.
-__device__ __forceinline__ bool warps_sync(uint64_t* bar, uint32_t& phase, int lane, volatile int* abort_flag,
-                                           int* status, int where) {
-  __syncwarp();
-  if (lane == 0) mbar_arrive(bar);
-  const bool ok = mbar_wait(bar, phase & 1u, abort_flag, status, where);
-  ++phase;
-  return __all_sync(0xffffffffu, ok);
-}
-
 // The item x kv-head index that CTA `bx` of a grid of `G` takes in round r of its walk (-1: none).  Round r: CTA i
 // takes index r G + i in even rounds and r G + (G - 1 - i) in odd ones (the list is sorted longest first, so the CTA
 // that drew a long item in one round draws a short one in the next).  A launch with fewer items than CTAs leaves
@@ -113,7 +121,7 @@ __device__ __forceinline__ int attn_item_at(int r, int total, int bx, int G) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// Plan: one CTA.  For every q-tile the KV tiles it can see and into how many slices that range is cut, then
+// Plan: one CTA.  For every q-tile the KV blocks it can see and into how many slices that range is cut, then
 // the flat list of (q-tile, slice) items with everything a CTA needs to run one.
 __global__ void attn_plan_kernel(RowMeta rm, AttnPlan pl, KvView kv, int n_seqs, int tokens_per_tile, int target_items,
                                  int min_chunk, const int* tile_count, const int* status) {
@@ -134,7 +142,7 @@ __global__ void attn_plan_kernel(RowMeta rm, AttnPlan pl, KvView kv, int n_seqs,
     const int L = rm.seq_len[s], n = rm.seq_n[s];
     for (int t = t0; t < t1; ++t) {
       const int tok_end = min(n, (t - t0 + 1) * tokens_per_tile);
-      const int n_kv = (L + tok_end + 127) >> 7;         // 128-key tiles (two paged blocks): the unit slices are cut in
+      const int n_kv = (L + tok_end + 63) >> 6;          // 64-key blocks: the unit slices are cut in
       pl.tile_seq[t] = s;
       pl.tile_nkv[t] = n_kv;
       my += n_kv;
@@ -142,7 +150,7 @@ __global__ void attn_plan_kernel(RowMeta rm, AttnPlan pl, KvView kv, int n_seqs,
   }
   atomicAdd(&s_total, my);
   __syncthreads();
-  // KV tiles per slice: start from an even share.  Rounding up the slice count of every q-tile can leave the
+  // KV blocks per slice: start from an even share.  Rounding up the slice count of every q-tile can leave the
   // launch with somewhat more items than CTA slots, and then the few CTAs that draw a second item double its
   // length: in that band (1 to 1.6 items per slot) the share is grown until every slot has at most one item.
   // Well beyond it a second round is about full and the sorted walk balances it, so the share is kept.
@@ -172,15 +180,13 @@ __global__ void attn_plan_kernel(RowMeta rm, AttnPlan pl, KvView kv, int n_seqs,
       const int s = pl.tile_seq[t];
       const int tok0 = (t - rm.seq_tile0[s]) * tokens_per_tile;
       const int n_tok = min(tokens_per_tile, rm.seq_n[s] - tok0);
-      const int blocks = (rm.seq_len[s] + tok0 + n_tok + 63) >> 6;    // 64-key blocks the q-tile can see
       const int ns = max(1, min(kAttnMaxSplits, (n_kv + chunk - 1) / chunk));
       const int base = n_kv / ns, rem = n_kv % ns;
       int lo = 0;
       for (int k = 0; k < ns; ++k) {
         const int len = base + (k < rem ? 1 : 0);
-        // the item's range in 64-key blocks: only the last slice of a q-tile can end on half a tile
         pl.items_unsorted[2 * n] = make_int4(rm.seq_q0[s] + tok0, rm.seq_len[s] + tok0, n_tok, rm.seq_slot[s]);
-        pl.items_unsorted[2 * n + 1] = make_int4((2 * lo) | (min(blocks, 2 * (lo + len)) << 16), k | (ns << 8) | (tok0 << 16), t, len);
+        pl.items_unsorted[2 * n + 1] = make_int4(lo | ((lo + len) << 16), k | (ns << 8) | (tok0 << 16), t, len);
         ++n;
         lo += len;
       }
@@ -190,7 +196,7 @@ __global__ void attn_plan_kernel(RowMeta rm, AttnPlan pl, KvView kv, int n_seqs,
   }
   __syncthreads();
   // longest first (rank sort, ties by creation order): the attention CTAs walk the list in boustrophedon order, so
-  // every CTA's share of KV tiles comes out about equal
+  // every CTA's share of KV blocks comes out about equal
   const int n = s_n;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const int len = pl.items_unsorted[2 * i + 1].w;
@@ -202,10 +208,10 @@ __global__ void attn_plan_kernel(RowMeta rm, AttnPlan pl, KvView kv, int n_seqs,
     pl.items[2 * rank] = pl.items_unsorted[2 * i];
     pl.items[2 * rank + 1] = pl.items_unsorted[2 * i + 1];
   }
-  // slice-arrival counters of every (q-tile, kv head): zero at the start of a step, reset by the combiner
-  for (int i = threadIdx.x; i < n_tiles * pl.n_kv_heads; i += blockDim.x) pl.counters[i] = 0;
+  // slice-arrival counters of every (q-tile, kv head, quarter): zero at the start of a step, reset by the combiner
+  for (int i = threadIdx.x; i < n_tiles * pl.n_kv_heads * 4; i += blockDim.x) pl.counters[i] = 0;
   // what every CTA of the attention grid starts with, in one record: its first item and the physical blocks of that
-  // item's first KV tile, so that a CTA's first loads do not wait for a chain of dependent reads (item -> block table)
+  // item's first two KV blocks, so that a CTA's first loads do not wait for a chain of dependent reads (item -> block table)
   __syncthreads();
   const int total = n * pl.n_kv_heads;
   for (int b = threadIdx.x; b < pl.grid; b += blockDim.x) {
@@ -237,33 +243,28 @@ void launch_attn_plan(cudaStream_t st, const RowMeta& rm, const AttnPlan& pl, co
 
 // ------------------------------------------------------------------------------------------------
 template <int HD>
-__global__ void __launch_bounds__(kAttnThreads, AttnCfg<HD>::CTAS_PER_SM)
+__global__ void __launch_bounds__(kAttnThreads, 2)
 attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                   const __grid_constant__ CUtensorMap tmV, AttnParams p) {
   using C = AttnCfg<HD>;
-  constexpr int Q_BYTES = C::Q_BYTES, KV_TILE_BYTES = C::KV_TILE_BYTES, NSUB = C::NSUB;
-  constexpr int TMEM_COL_O = C::COL_O, TMEM_COL_P = C::COL_P, OWN = C::OWN;
+  constexpr int NSUB = C::NSUB, STAGES = C::STAGES, NBUF = C::NBUF;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* sQ = smem;
-  uint8_t* sK = sQ + Q_BYTES;                          // ring stage s: sK + s * KV_TILE_BYTES, per sub-tile block 0 then block 1
-  uint8_t* sV = sK + KV_STAGES * KV_TILE_BYTES;
-  __nv_bfloat16* xch = reinterpret_cast<__nv_bfloat16*>(sV + KV_STAGES * KV_TILE_BYTES);   // [half][row] maxima
-  float* lx = reinterpret_cast<float*>(xch + 2 * 128);                                         // [half][row] sums
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sV + KV_STAGES * KV_TILE_BYTES + ATTN_XCH_BYTES);
+  uint8_t* sK = sQ + C::Q_BYTES;                       // ring stage s: sK + s * C::KV_BYTES, per sub-tile 64 keys
+  uint8_t* sV = sK + STAGES * C::KV_BYTES;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sV + STAGES * C::KV_BYTES);
   uint64_t* q_full = bars;                 // Q tile landed                       (one phase per item)
   uint64_t* q_empty = bars + 1;            // every S MMA of the item has read Q   (one phase per item)
   uint64_t* k_full = bars + 2;             // [stage]
-  uint64_t* k_empty = k_full + KV_STAGES;  // [stage] S of the tile has been formed
-  uint64_t* v_full = k_empty + KV_STAGES;
-  uint64_t* v_empty = v_full + KV_STAGES;  // [stage] O += P V of the tile has completed
-  uint64_t* s_full = v_empty + KV_STAGES;  // S(t) is in tensor memory
-  uint64_t* s_empty = s_full + 1;          // the softmax warps hold S(t) in registers
-  uint64_t* p_full = s_empty + 1;          // P(t) is in tensor memory (and the accumulator rescaled, if it had to be)
-  uint64_t* o_full = p_full + 1;           // O += P(t) V(t) has completed
-  uint64_t* group_bar = o_full + 1;        // the eight softmax warps (slice hand-over)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(group_bar + 1);
+  uint64_t* k_empty = k_full + STAGES;     // [stage] S of the block has been formed
+  uint64_t* v_full = k_empty + STAGES;
+  uint64_t* v_empty = v_full + STAGES;     // [stage] O += P V of the block has completed
+  uint64_t* s_full = v_empty + STAGES;     // [buffer] S(t) is in tensor memory
+  uint64_t* p_full = s_full + NBUF;        // [buffer] P(t) is in tensor memory (and the accumulator rescaled, if it had to be)
+  uint64_t* o_full = p_full + NBUF;        // [buffer] O += P(t) V(t) has completed.  (One barrier for all blocks would not do:
+                                           // a wait for block t passes on the parity of t - 2 where t - 1 is still running.)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_full + NBUF);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* s_flag = abort_flag + 1;   // combine: "this CTA ran the last slice to finish"
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (smem_u32(smem) & 1023u) {            // uniform over the CTA: nothing has been set up yet
@@ -273,17 +274,17 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
     mbar_init(q_empty, 1);
-    for (int s = 0; s < KV_STAGES; ++s) {
+    for (int s = 0; s < STAGES; ++s) {
       mbar_init(k_full + s, 1);
       mbar_init(k_empty + s, 1);
       mbar_init(v_full + s, 1);
       mbar_init(v_empty + s, 1);
     }
-    mbar_init(s_full, 1);
-    mbar_init(s_empty, kSoftmaxWarps);
-    mbar_init(p_full, kSoftmaxWarps);
-    mbar_init(o_full, 1);
-    mbar_init(group_bar, kSoftmaxWarps);
+    for (int b = 0; b < NBUF; ++b) {
+      mbar_init(s_full + b, 1);
+      mbar_init(p_full + b, kSoftmaxWarps);
+      mbar_init(o_full + b, 1);
+    }
     *abort_flag = 0;
     fence_mbar_init();
     tma_prefetch_desc(&tmQ);
@@ -299,12 +300,13 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  pdl_wait();               // q, the K/V rows of this step, the row metadata and the plan come from earlier kernels
-  pdl_launch_dependents();
-
-  // The plan's record of this CTA's first item (the item and the physical blocks of its first KV tile) for the two
-  // warps that start the pipeline: read together with the status word and the item count, before any of them is
-  // used, so that the first TMA loads are one round trip away instead of four (status -> count -> item -> block table).
+  // The plan's record of this CTA's first item (the item and the physical blocks of its first keys) for the two warps
+  // that start the pipeline: read together with the status word and the item count, before any of them is used, so that
+  // the first TMA loads are one round trip away instead of four (status -> count -> item -> block table).
+  // All of it, like the block table and the K/V rows committed before this step, was written before the kernel that
+  // precedes this one in the step: that kernel waited for ITS predecessor before it let this one start, so these reads
+  // need no wait of their own, and the first K/V blocks load while the predecessor (which writes q and this step's own
+  // K/V rows) is still running.
   int4 rec_a = make_int4(0, 0, 0, 0), rec_b = rec_a, rec_c = rec_a;
   if (warp < 2) {
     const int4* rec = p.plan.first + 3 * (size_t)blockIdx.x;
@@ -317,125 +319,152 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   const int n_rounds = (total + (int)gridDim.x - 1) / (int)gridDim.x;
   auto item_of_round = [&](int r) -> int { return attn_item_at(r, total, (int)blockIdx.x, (int)gridDim.x); };
 
-  // Tile counter t (all 128-key tiles of all items of this CTA): ring stage = t % KV_STAGES, and every barrier's
-  // parity follows from how often t has used it; n counts items (Q hand-over barriers).
+  // Block counter t (all 64-key blocks of all items of this CTA): ring stage = t % STAGES, score buffer = t % NBUF, and
+  // every barrier's parity follows from how often t has used it; n counts items (Q hand-over barriers).
+  //
+  // The producer and the MMA warp run their loops as whole warps and elect one lane for the instructions that one thread
+  // issues: with warp-uniform control flow descriptors and coordinates live in uniform registers, where those
+  // instructions want them (run by lane 0 alone, an MMA took ~90 cycles to issue; elected, ~25).
   if (warp == 0) {
-    if (lane < 2) {
-      // lane 0: Q and the K ring; lane 1: the V ring
-      const bool is_k = lane == 0;
-      uint64_t* full = is_k ? k_full : v_full;
-      uint64_t* empty = is_k ? k_empty : v_empty;
-      uint8_t* ring = is_k ? sK : sV;
-      const CUtensorMap* tm = is_k ? &tmK : &tmV;
-      uint32_t t = 0;
-      int n = 0;
-      for (int r = 0; r < n_rounds; ++r) {
-        const int w = r == 0 ? (total > 0 ? rec_c.x : -1) : item_of_round(r);
-        if (w < 0) continue;
-        int4 ia = rec_a, ib = rec_b;
-        int kvh = rec_c.y;
-        if (r != 0) {
-          ia = p.plan.items[2 * (w / p.Hkv)];
-          ib = p.plan.items[2 * (w / p.Hkv) + 1];
-          kvh = w % p.Hkv;
-        }
-        const int kt_lo = ib.x & 0xffff, kt_hi = ib.x >> 16;
-        const int* bt = p.block_table + (size_t)ia.w * p.max_blocks;
-        if (is_k) {
-          if (!mbar_wait(q_empty, (n & 1) ^ 1u, abort_flag, p.status, 400)) goto done;
-          mbar_expect_tx(q_full, Q_BYTES);
+    uint32_t t = 0;                                      // the K blocks of t + 1 go out before the V block of t
+    int n = 0;
+    auto load = [&](const CUtensorMap* tm, uint8_t* ring, uint64_t* full, uint64_t* empty, uint32_t at, int phys, int kvh) -> bool {
+      const int st = at % STAGES;
+      if (!mbar_wait(empty + st, ((at / STAGES) & 1) ^ 1u, abort_flag, p.status, 401)) return false;
+      const int row = (((p.layer * p.n_blocks) + phys) * p.Hkv + kvh) * 64;
+      if (elect_one()) {
+        mbar_expect_tx(full + st, C::KV_BYTES);
 #pragma unroll
-          for (int h = 0; h < NSUB; ++h) tma_load_3d(sQ + h * SUB_BYTES, &tmQ, q_full, 64 * h, kvh * p.group, ia.x);
-        }
-        for (int kt = kt_lo; kt < kt_hi; kt += 2, ++t) {
-          // the tile's two blocks; a slice of odd length ends with half a tile: the last block is staged twice and
-          // the softmax warps mask its second copy
-          int phys0 = rec_c.z, phys1 = rec_c.w;
-          if (r != 0 || kt != kt_lo) {
-            phys0 = bt[kt];
-            phys1 = bt[kt + 1 < kt_hi ? kt + 1 : kt];
-          }
-          const int st = t % KV_STAGES;
-          if (!mbar_wait(empty + st, ((t / KV_STAGES) & 1) ^ 1u, abort_flag, p.status, 401)) goto done;
-          const int row0 = (((p.layer * p.n_blocks) + phys0) * p.Hkv + kvh) * 64;
-          const int row1 = (((p.layer * p.n_blocks) + phys1) * p.Hkv + kvh) * 64;
-          uint8_t* dst = ring + st * KV_TILE_BYTES;
-          mbar_expect_tx(full + st, KV_TILE_BYTES);
-#pragma unroll
-          for (int h = 0; h < NSUB; ++h) {
-            tma_load_2d(dst + h * SUB_BYTES, tm, full + st, 64 * h, row0);
-            tma_load_2d(dst + h * SUB_BYTES + KV_BLOCK_BYTES, tm, full + st, 64 * h, row1);
-          }
-        }
-        ++n;
+        for (int h = 0; h < NSUB; ++h) tma_load_2d(ring + st * C::KV_BYTES + h * KV_BLOCK_BYTES, tm, full + st, 64 * h, row);
       }
+      __syncwarp();
+      return true;
+    };
+    for (int r = 0; r < n_rounds; ++r) {
+      const int w = r == 0 ? (total > 0 ? rec_c.x : -1) : item_of_round(r);
+      if (w < 0) continue;
+      int4 ia = rec_a, ib = rec_b;
+      int kvh = rec_c.y;
+      if (r != 0) {
+        ia = p.plan.items[2 * (w / p.Hkv)];
+        ib = p.plan.items[2 * (w / p.Hkv) + 1];
+        kvh = w % p.Hkv;
+      }
+      const int kt_lo = ib.x & 0xffff, kt_hi = ib.x >> 16;
+      const int* bt = p.block_table + (size_t)ia.w * p.max_blocks;
+      auto phys_of = [&](int kt) -> int { return r == 0 && kt < kt_lo + 2 ? (kt == kt_lo ? rec_c.z : rec_c.w) : bt[kt]; };
+      int early = kt_lo;                                 // K and V of [kt_lo, early) are on their way
+      if (r == 0) {
+        // blocks that hold committed rows only, as many as the rings take, ahead of the grid dependency
+        const int committed = min(kt_hi, (ia.y - (ib.y >> 16)) >> 6);
+        for (; early < committed && early - kt_lo < STAGES; ++early) {
+          const int phys = phys_of(early);
+          if (!load(&tmK, sK, k_full, k_empty, t + (early - kt_lo), phys, kvh)) goto done;
+          if (!load(&tmV, sV, v_full, v_empty, t + (early - kt_lo), phys, kvh)) goto done;
+        }
+        pdl_wait();
+      }
+      if (!mbar_wait(q_empty, (n & 1) ^ 1u, abort_flag, p.status, 400)) goto done;
+      if (elect_one()) {
+        mbar_expect_tx(q_full, C::Q_BYTES);
+#pragma unroll
+        for (int h = 0; h < NSUB; ++h) tma_load_3d(sQ + h * SUB_BYTES, &tmQ, q_full, 64 * h, kvh * p.group, ia.x);
+      }
+      __syncwarp();
+      int phys_v = early < kt_hi ? phys_of(early) : 0;
+      if (early < kt_hi && !load(&tmK, sK, k_full, k_empty, t + (early - kt_lo), phys_v, kvh)) goto done;
+      for (int kt = early; kt < kt_hi; ++kt) {
+        int phys_k = 0;
+        if (kt + 1 < kt_hi) {
+          phys_k = phys_of(kt + 1);
+          if (!load(&tmK, sK, k_full, k_empty, t + (kt + 1 - kt_lo), phys_k, kvh)) goto done;
+        }
+        if (!load(&tmV, sV, v_full, v_empty, t + (kt - kt_lo), phys_v, kvh)) goto done;
+        phys_v = phys_k;
+      }
+      t += kt_hi - kt_lo;
+      ++n;
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc_s = umma_idesc_bf16(128);
-      constexpr uint32_t idesc_pv = umma_idesc_bf16(64, true);
-      const uint32_t q_addr = smem_u32(sQ);
-      uint32_t t = 0;
-      int n = 0;
-      for (int r = 0; r < n_rounds; ++r) {
-        const int w = r == 0 ? (total > 0 ? rec_c.x : -1) : item_of_round(r);
-        if (w < 0) continue;
-        const int4 ib = r == 0 ? rec_b : p.plan.items[2 * (w / p.Hkv) + 1];
-        const int n_it = ((ib.x >> 16) - (ib.x & 0xffff) + 1) / 2;      // 128-key tiles of the item
-        // S(ti) = Q K(ti)^T: four K = 16 steps over every 64 dims, N = 128 keys
-        auto issue_s = [&](uint32_t ti, bool last) -> bool {
-          const int st = ti % KV_STAGES;
-          if (!mbar_wait(k_full + st, (ti / KV_STAGES) & 1, abort_flag, p.status, 410)) return false;
-          if (!mbar_wait(s_empty, (ti & 1) ^ 1u, abort_flag, p.status, 411)) return false;   // S(ti - 1) is in registers
-          tc_fence_after();
-          const uint32_t k_addr = smem_u32(sK + st * KV_TILE_BYTES);
+    pdl_wait();
+    pdl_launch_dependents();
+    constexpr uint32_t idesc_s = umma_idesc_bf16(64);
+    constexpr uint32_t idesc_pv = umma_idesc_bf16(64, true);
+    const uint64_t q_desc = umma_desc_sw128(smem_u32(sQ)), k_desc = umma_desc_sw128(smem_u32(sK)),
+                   v_desc = umma_desc_sw128(smem_u32(sV));     // a byte offset adds a sixteenth of itself
+    uint32_t t = 0;
+    int n = 0;
+    for (int r = 0; r < n_rounds; ++r) {
+      const int w = r == 0 ? (total > 0 ? rec_c.x : -1) : item_of_round(r);
+      if (w < 0) continue;
+      const int4 ib = r == 0 ? rec_b : p.plan.items[2 * (w / p.Hkv) + 1];
+      const uint32_t t_end = t + (ib.x >> 16) - (ib.x & 0xffff);
+      // S(ti) = Q K(ti)^T: four K = 16 steps over every 64 dims, N = 64 keys, into the buffer P(ti - NBUF) has left
+      auto issue_s = [&](uint32_t ti) -> bool {
+        const int st = ti % STAGES;
+        if (!mbar_wait(k_full + st, (ti / STAGES) & 1, abort_flag, p.status, 410)) return false;
+        tc_fence_after();
+        const uint64_t kd = k_desc + st * (C::KV_BYTES / 16);
+        const uint32_t buf = ti % NBUF;
+        if (elect_one()) {
 #pragma unroll
           for (int h = 0; h < NSUB; ++h)
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-              umma_bf16(tmem_base, umma_desc_sw128(q_addr + h * SUB_BYTES + k * 32),
-                        umma_desc_sw128(k_addr + h * SUB_BYTES + k * 32), idesc_s, (h | k) != 0);
-          umma_commit(s_full);
+              umma_bf16(tmem_base + 64 * buf, q_desc + (h * SUB_BYTES + k * 32) / 16, kd + (h * KV_BLOCK_BYTES + k * 32) / 16,
+                        idesc_s, (h | k) != 0);
+          umma_commit(s_full + buf);
           umma_commit(k_empty + st);              // K is free once S has been formed
-          if (last) umma_commit(q_empty);         // last S MMA of the item: Q is free once it completes
-          return true;
-        };
-        if (!mbar_wait(q_full, n & 1, abort_flag, p.status, 412)) goto done;
-        if (!issue_s(t, n_it == 1)) goto done;
-        for (int j = 0; j < n_it; ++j, ++t) {
-          if (j + 1 < n_it && !issue_s(t + 1, j + 2 == n_it)) goto done;
-          // P(t) is written, and whatever had to be done to the accumulator before this product is done
-          if (!mbar_wait(p_full, t & 1, abort_flag, p.status, 413)) goto done;
-          const int st = t % KV_STAGES;
-          if (!mbar_wait(v_full + st, (t / KV_STAGES) & 1, abort_flag, p.status, 415)) goto done;
-          tc_fence_after();
-          const uint32_t v_addr = smem_u32(sV + st * KV_TILE_BYTES);
-          const uint32_t d = tmem_base + TMEM_COL_O;   // the item's accumulator: the first product of an item overwrites it
+          if (ti + 1 == t_end) umma_commit(q_empty);   // last S MMA of the item: Q is free once it completes
+        }
+        __syncwarp();
+        return true;
+      };
+      // the last product of the item before has completed: every buffer is free
+      if (t > 0 && !mbar_wait(o_full + (t - 1) % NBUF, ((t - 1) / NBUF) & 1, abort_flag, p.status, 411)) goto done;
+      if (!mbar_wait(q_full, n & 1, abort_flag, p.status, 412)) goto done;
+      for (uint32_t ti = t; ti < t_end && ti < t + NBUF; ++ti)
+        if (!issue_s(ti)) goto done;
+      for (bool first = true; t < t_end; ++t, first = false) {
+        const int st = t % STAGES;
+        const uint32_t buf = t % NBUF;
+        if (!mbar_wait(v_full + st, (t / STAGES) & 1, abort_flag, p.status, 415)) goto done;
+        // P(t) is written, and whatever had to be done to the accumulator before this product is done
+        if (!mbar_wait(p_full + buf, (t / NBUF) & 1, abort_flag, p.status, 413)) goto done;
+        tc_fence_after();
+        const uint64_t vd = v_desc + st * (C::KV_BYTES / 16);
+        if (elect_one()) {
 #pragma unroll
           for (int h = 0; h < NSUB; ++h)   // 64 output dims per product
 #pragma unroll
-            for (int k = 0; k < 8; ++k)    // 16 keys per step: 8 columns of P in tensor memory; V [key][dim] is MN-major,
-                                           // a step of 16 keys is 16 rows of 128 bytes
-              umma_bf16_ta(d + 64 * h, tmem_base + TMEM_COL_P + k * 8, umma_desc_sw128(v_addr + h * SUB_BYTES + k * 2048),
-                           idesc_pv, (j != 0 || k != 0) ? 1u : 0u);
+            for (int k = 0; k < 4; ++k)
+              // 16 keys per step: 8 columns of P in tensor memory; V [key][dim] is MN-major, a step of 16 keys is 16
+              // rows of 128 bytes; the first product of an item overwrites the accumulator
+              umma_bf16_ta(tmem_base + C::COL_O + 64 * h, tmem_base + 64 * buf + k * 8, vd + (h * KV_BLOCK_BYTES + k * 2048) / 16,
+                           idesc_pv, (!first || k != 0) ? 1u : 0u);
+          umma_commit(o_full + buf);
           umma_commit(v_empty + st);
-          umma_commit(o_full);
         }
-        ++n;
+        __syncwarp();
+        if (t + NBUF < t_end) {
+          if (!mbar_wait(o_full + buf, (t / NBUF) & 1, abort_flag, p.status, 416)) goto done;
+          if (!issue_s(t + NBUF)) goto done;
+        }
       }
-      // every stage-release arrival must land before the CTA's shared memory can be handed on
-      if (t > 0 && !mbar_wait(o_full, (t - 1) & 1, abort_flag, p.status, 414)) goto done;
+      ++n;
     }
+    // every stage-release arrival must land before the CTA's shared memory can be handed on
+    if (t > 0 && !mbar_wait(o_full + (t - 1) % NBUF, ((t - 1) / NBUF) & 1, abort_flag, p.status, 414)) goto done;
+    if (t > 0 && !mbar_wait(v_empty + (t - 1) % STAGES, ((t - 1) / STAGES) & 1, abort_flag, p.status, 417)) goto done;
   } else {
     const int quarter = warp & 3;                      // TMEM lane quarter a warp may touch = warp id mod 4
-    const int half = (warp - 2) >> 2;                  // keys [64 half, 64 half + 64) of every tile
     const int row = quarter * 32 + lane;               // q row of the tile = TMEM lane
     const int tok = row / p.group;
     const uint32_t t_lane = tmem_base + (uint32_t(quarter * 32) << 16);
-    const uint32_t t_o = t_lane + TMEM_COL_O + half * OWN;    // this thread's OWN columns of the accumulator row
-    const uint32_t t_p = t_lane + TMEM_COL_P + half * 32;     // and of the row of P: its 64 keys, two per column
+    const uint32_t t_o = t_lane + C::COL_O;
     const float sc = (HD == 64 ? 0.125f : 0.08838834764831845f) * 1.4426950408889634f;     // 1/sqrt(HD) * log2(e)
-    uint32_t t = 0, group_ph = 0;
+    uint32_t t = 0;
+    pdl_wait();
     for (int r = 0; r < n_rounds; ++r) {
       const int w = item_of_round(r);
       if (w < 0) continue;
@@ -455,10 +484,10 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       // they keep step with the barriers but skip the loads, the exps and the P rows (which only feed their own,
       // never stored, output rows)
       const bool warp_ok = (quarter * 32) / p.group < n_tok;
-      float m_ref = -INFINITY, l = 0.f;                // exponent reference (log2 units, scaled); sum of this thread's P
+      // exponent reference (log2 units, scaled; a row that is no token asks for none); sum of the row's P
+      float m_ref = row_ok ? -INFINITY : 0.f, l = 0.f;
       // visibility of the 32 keys from `key0` on for this thread's row, as a bit mask
-      auto visible = [&](int key0, int key_end) -> uint32_t {
-        if (key0 >= key_end) return 0u;                 // the second copy of a slice's last block
+      auto visible = [&](int key0) -> uint32_t {
         if (p.anc) {
           auto word = [&](int i) -> uint32_t {
             return i < 0 ? 0xffffffffu : i == 0 ? am.x : i == 1 ? am.y : i == 2 ? am.z : i == 3 ? am.w : 0u;
@@ -472,221 +501,195 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         const int nvis = pos_row - key0 + 1;            // keys key0 .. pos_row are visible
         return nvis >= 32 ? 0xffffffffu : (nvis <= 0 ? 0u : ((1u << nvis) - 1u));
       };
+      const int first_masked = p.anc ? len0 : pos0 + 1;  // keys below it are visible to every row of the q-tile
 
-      for (int kt = kt_lo; kt < kt_hi; kt += 2, ++t) {
-        bool ok = mbar_wait(s_full, t & 1, abort_flag, p.status, 420);
+      for (int kt = kt_lo; kt < kt_hi; ++kt, ++t) {
+        const uint32_t buf = t % NBUF;
+        bool ok = mbar_wait(s_full + buf, (t / NBUF) & 1, abort_flag, p.status, 420);
         if (!__all_sync(0xffffffffu, ok)) goto done;
         tc_fence_after();
-        if (!warp_ok) {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(s_empty);
-          // S(t + 1) is issued before P(t) is consumed, so this warp could be back here for the next tile while phase
-          // t of p_full is still open, and its arrival would then be counted there: like the warps that do write P,
-          // it arrives for tile t only once the product of tile t - 1 (hence phase t - 1 of p_full) is complete
-          if (t > 0) {
-            ok = mbar_wait(o_full, (t - 1) & 1, abort_flag, p.status, 424);
-            if (!__all_sync(0xffffffffu, ok)) goto done;
-          }
-          if (lane == 0) mbar_arrive(p_full);
-          continue;
-        }
-        const int key_end = min(kt + 2, kt_hi) * 64;    // keys of this tile that belong to the slice
-        const int kb_own = kt * 64 + half * 64;
-        // does any key of the tile need masking for some row of the q-tile?  (warp-uniform)
-        const bool masked_tile = p.anc ? (kt * 64 + 127 >= len0) : (kt * 64 + 127 > pos0);
-        const bool partial_tile = key_end < kt * 64 + 128;
-        uint32_t s0[32], s1[32];
-        tmem_ld32(t_lane + half * 64, s0);
-        tmem_ld32(t_lane + half * 64 + 32, s1);
-        tmem_ld_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(s_empty);
-        if (masked_tile || partial_tile) {
-          const uint32_t v0 = visible(kb_own, key_end), v1 = visible(kb_own + 32, key_end);
+        if (warp_ok) {
+          const uint32_t t_s = t_lane + 64 * buf;
+          uint32_t a[32], b[32], pk[32];
+          tmem_ld32(t_s, a);
+          tmem_ld32(t_s + 32, b);
+          tmem_ld_wait(a);
+          tmem_ld_wait(b);
+          if (kt * 64 + 63 >= first_masked) {            // (warp-uniform)
+            const uint32_t va = visible(kt * 64), vb = visible(kt * 64 + 32);
 #pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            if (!((v0 >> e) & 1u)) s0[e] = 0xff800000u;            // -inf
-            if (!((v1 >> e) & 1u)) s1[e] = 0xff800000u;
-          }
-        }
-        float mx = -INFINITY, mx_b = -INFINITY;              // two chains
-#pragma unroll
-        for (int e = 0; e < 32; e += 2) {
-          mx = max3(mx, __uint_as_float(s0[e]), __uint_as_float(s1[e]));
-          mx_b = max3(mx_b, __uint_as_float(s0[e + 1]), __uint_as_float(s1[e + 1]));
-        }
-        mx = fmaxf(mx, mx_b);
-        // The row's maximum over all 128 keys: the two threads of a row swap their halves' maxima through shared memory.
-        // Both use the bf16-rounded values of BOTH halves, so they arrive at the same number (the reference only has to
-        // be near the maximum, and identical for the row's two threads).
-        {
-          const __nv_bfloat16 mine = __float2bfloat16_rn(mx);
-          xch[half * 128 + row] = mine;
-          named_bar_sync(1 + quarter, 64);                 // the two warps of this lane quarter
-          mx = fmaxf(__bfloat162float(mine), __bfloat162float(xch[(half ^ 1) * 128 + row]));
-          named_bar_sync(1 + quarter, 64);                 // both have read before either writes the next tile's
-        }
-        mx *= sc;
-        // The reference moves only when the maximum has outgrown it by more than kRescaleBits (or nothing has been
-        // accumulated under it yet: then moving it costs nothing).  `l` is this thread's half of the row sum; whether
-        // anything has been accumulated is a property of the row, so the test uses the reference itself.
-        float alpha = 1.f;
-        bool rescale = false;
-        if (mx > m_ref) {
-          if (m_ref == -INFINITY) {
-            m_ref = mx;                                   // nothing accumulated so far (first tile, or all keys masked)
-          } else if (mx > m_ref + kRescaleBits) {
-            alpha = ex2(m_ref - mx);
-            m_ref = mx;
-            rescale = true;
-          }
-        }
-        const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
-        float sum = 0.f, sum_b = 0.f, sum_c = 0.f, sum_d = 0.f;   // four chains
-        uint32_t pk[32];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          const float a0 = ex2(fmaf(__uint_as_float(s0[2 * e]), sc, -m_use));
-          const float a1 = ex2(fmaf(__uint_as_float(s0[2 * e + 1]), sc, -m_use));
-          if (e & 1) sum_b += a0 + a1; else sum += a0 + a1;
-          pk[e] = pack_bf16(a0, a1);
-        }
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          const float a0 = ex2(fmaf(__uint_as_float(s1[2 * e]), sc, -m_use));
-          const float a1 = ex2(fmaf(__uint_as_float(s1[2 * e + 1]), sc, -m_use));
-          if (e & 1) sum_d += a0 + a1; else sum_c += a0 + a1;
-          pk[16 + e] = pack_bf16(a0, a1);
-        }
-        l = l * alpha + ((sum + sum_b) + (sum_c + sum_d));
-        // P's columns are read by the product of tile t - 1, which also still adds into the accumulator
-        if (t > 0) {
-          ok = mbar_wait(o_full, (t - 1) & 1, abort_flag, p.status, 421);
-          if (!__all_sync(0xffffffffu, ok)) goto done;
-          tc_fence_after();
-        }
-        if (__any_sync(0xffffffffu, rescale)) {
-          // rare: scale this thread's half of the accumulator row (alpha = 1 where not needed)
-#pragma unroll 1
-          for (int c = 0; c < OWN; c += 32) {
-            uint32_t o[32];
-            tmem_ld32(t_o + c, o);
-            tmem_ld_wait();
-#pragma unroll
-            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-            tmem_st32(t_o + c, o);
-          }
-          tmem_st_wait();
-          tc_fence_before();
-        }
-        // P row -> tensor memory, where the second product reads it as its A operand (no shared-memory round trip)
-        tmem_st32(t_p, pk);
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(p_full);
-      }
-      // the item's last product (products complete in issue order, so all of them)
-      if (kt_hi > kt_lo) {
-        bool ok = mbar_wait(o_full, (t - 1) & 1, abort_flag, p.status, 422);
-        if (!__all_sync(0xffffffffu, ok)) goto done;
-        tc_fence_after();
-      }
-      // the row sum is the sum of its two threads' halves
-      float l_row = l;
-      if (warp_ok) {
-        lx[half * 128 + row] = l;
-        named_bar_sync(1 + quarter, 64);                 // the two warps of this lane quarter
-        l_row += lx[(half ^ 1) * 128 + row];
-        named_bar_sync(1 + quarter, 64);                 // both have read before either writes the next item's
-      }
-
-      // ---- item epilogue: this thread owns dims [OWN half, OWN half + OWN) of its row
-      const int head = kvh * p.group + row % p.group;
-      uint4* out_row = reinterpret_cast<uint4*>(p.out + (size_t)(q_row0 + tok) * p.Hq * HD + head * HD + half * OWN);
-      if (n_split == 1) {
-        if (warp_ok) {                                     // (a whole warp reads tensor memory together)
-          const float inv = 1.f / l_row;
-#pragma unroll 1
-          for (int c0 = 0; c0 < OWN; c0 += 32) {
-            uint32_t o[32];
-            tmem_ld32(t_o + c0, o);
-            tmem_ld_wait();
-            if (row_ok) {
-              uint4* dst = out_row + c0 / 8;
-#pragma unroll
-              for (int c = 0; c < 4; ++c)
-                dst[c] = make_uint4(
-                    pack_bf16(__uint_as_float(o[8 * c]) * inv, __uint_as_float(o[8 * c + 1]) * inv),
-                    pack_bf16(__uint_as_float(o[8 * c + 2]) * inv, __uint_as_float(o[8 * c + 3]) * inv),
-                    pack_bf16(__uint_as_float(o[8 * c + 4]) * inv, __uint_as_float(o[8 * c + 5]) * inv),
-                    pack_bf16(__uint_as_float(o[8 * c + 6]) * inv, __uint_as_float(o[8 * c + 7]) * inv));
+            for (int e = 0; e < 32; ++e) {
+              if (!((va >> e) & 1u)) a[e] = 0xff800000u;               // -inf
+              if (!((vb >> e) & 1u)) b[e] = 0xff800000u;
             }
           }
-          tc_fence_before();
-        }
-      } else {
-        // partials of this (q-tile, kv head): [slice][2 + HD][128 rows] floats, entry 0 the exponent reference (log2
-        // units), 1 the row sum under it, 2.. the HD unnormalised outputs; a warp's accesses are 128-byte lines
-        constexpr int PART = (2 + HD) * 128;
-        float* tile_part = p.split_ws + ((size_t)(ib.z * p.Hkv + kvh) * kAttnMaxSplits) * PART + row;
-        if (warp_ok) {
-          float* part = tile_part + (size_t)split * PART;
-          if (half == 0) {
-            part[0] = m_ref;
-            part[128] = l_row;
-          }
-#pragma unroll 1
-          for (int c0 = 0; c0 < OWN; c0 += 32) {
-            uint32_t o[32];
-            tmem_ld32(t_o + c0, o);
-            tmem_ld_wait();
+          bool retake = m_ref == -INFINITY;              // no reference yet: it is the maximum of these 64 scores
+          float sum;
+          for (;;) {
+            if (__any_sync(0xffffffffu, retake)) {
+              float mx = -INFINITY, mx_b = -INFINITY;    // two chains
 #pragma unroll
-            for (int e = 0; e < 32; ++e) part[(2 + half * OWN + c0 + e) * 128] = __uint_as_float(o[e]);
-          }
-          tc_fence_before();
-        }
-        __threadfence();
-        if (!warps_sync(group_bar, group_ph, lane, abort_flag, p.status, 427)) goto done;
-        if (warp == 2 && lane == 0) {
-          int* ctr = p.plan.counters + ib.z * p.Hkv + kvh;
-          const int old = atomicAdd(ctr, 1);
-          *s_flag = (old == n_split - 1);
-          if (old == n_split - 1) *ctr = 0;             // ready for the next layer
-        }
-        if (!warps_sync(group_bar, group_ph, lane, abort_flag, p.status, 428)) goto done;
-        if (*s_flag && warp_ok) {
-          __threadfence();
-          float M = -INFINITY;
-          for (int s = 0; s < n_split; ++s) M = fmaxf(M, __ldcg(tile_part + (size_t)s * PART));
+              for (int e = 0; e < 32; e += 2) {
+                mx = max3(mx, __uint_as_float(a[e]), __uint_as_float(b[e]));
+                mx_b = max3(mx_b, __uint_as_float(a[e + 1]), __uint_as_float(b[e + 1]));
+              }
+              mx = fmaxf(mx, mx_b) * sc;
+              // Rows that ask for it, and only those (a row's result does not depend on its neighbours), take the new
+              // reference and rescale what they have accumulated, once the product before has completed.
+              float alpha = 1.f;
+              if (retake) {
+                if (m_ref != -INFINITY) alpha = ex2(m_ref - mx);
+                m_ref = mx;
+                l *= alpha;
+              }
+              if (__any_sync(0xffffffffu, alpha != 1.f)) {
+                ok = mbar_wait(o_full + (t - 1) % NBUF, ((t - 1) / NBUF) & 1, abort_flag, p.status, 421);
+                if (!__all_sync(0xffffffffu, ok)) goto done;
+                tc_fence_after();
 #pragma unroll 1
-          for (int c0 = 0; c0 < OWN; c0 += 32) {
-            float Lsum = 0.f;
+                for (int c = 0; c < HD; c += 32) {
+                  tmem_ld32(t_o + c, pk);
+                  tmem_ld_wait(pk);
+#pragma unroll
+                  for (int e = 0; e < 32; ++e) pk[e] = __float_as_uint(__uint_as_float(pk[e]) * alpha);
+                  tmem_st32(t_o + c, pk);
+                  tmem_st_wait();
+                }
+              }
+            }
+            const float m_use = m_ref == -INFINITY ? 0.f : m_ref;
+            const float2 sc2 = make_float2(sc, sc), m2 = make_float2(-m_use, -m_use);
+            float2 sum0 = make_float2(0.f, 0.f), sum1 = sum0;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              float2 x = fma2(make_float2(__uint_as_float(a[2 * e]), __uint_as_float(a[2 * e + 1])), sc2, m2);
+              x = make_float2(ex2(x.x), ex2(x.y));
+              if (e & 1) sum1 = add2(sum1, x); else sum0 = add2(sum0, x);
+              pk[e] = pack_bf16(x.x, x.y);
+            }
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              float2 x = fma2(make_float2(__uint_as_float(b[2 * e]), __uint_as_float(b[2 * e + 1])), sc2, m2);
+              x = make_float2(ex2(x.x), ex2(x.y));
+              if (e & 1) sum1 = add2(sum1, x); else sum0 = add2(sum0, x);
+              pk[16 + e] = pack_bf16(x.x, x.y);
+            }
+            sum = (sum0.x + sum0.y) + (sum1.x + sum1.y);
+            retake = row_ok && sum > kRescaleSum;        // some score has outgrown the reference
+            if (!__any_sync(0xffffffffu, retake)) break;
+          }
+          l += sum;
+          // P over the scores it came from, where the second product reads it as its A operand
+          tmem_st32(t_s, pk);
+          tmem_st_wait();
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(p_full + buf);
+      }
+      if (!warp_ok) continue;
+      // the item's last product (products complete in issue order, so all of them)
+      if (kt_hi > kt_lo) {
+        bool ok = mbar_wait(o_full + (t - 1) % NBUF, ((t - 1) / NBUF) & 1, abort_flag, p.status, 423);
+        if (!__all_sync(0xffffffffu, ok)) goto done;
+        tc_fence_after();
+      }
+
+      // ---- item epilogue: one output row per thread
+      const int head = kvh * p.group + row % p.group;
+      uint4* out_row = reinterpret_cast<uint4*>(p.out + (size_t)(q_row0 + tok) * p.Hq * HD + head * HD);
+      auto store32 = [&](const float (&o)[32], float inv, uint4* dst) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          dst[c] = make_uint4(pack_bf16(o[8 * c] * inv, o[8 * c + 1] * inv), pack_bf16(o[8 * c + 2] * inv, o[8 * c + 3] * inv),
+                              pack_bf16(o[8 * c + 4] * inv, o[8 * c + 5] * inv), pack_bf16(o[8 * c + 6] * inv, o[8 * c + 7] * inv));
+      };
+      if (n_split == 1) {
+        const float inv = 1.f / l;
+#pragma unroll 1
+        for (int c0 = 0; c0 < HD; c0 += 32) {              // (a whole warp reads tensor memory together)
+          uint32_t u[32];
+          tmem_ld32(t_o + c0, u);
+          tmem_ld_wait(u);
+          if (row_ok) {
+            float o[32];
+#pragma unroll
+            for (int e = 0; e < 32; ++e) o[e] = __uint_as_float(u[e]);
+            store32(o, inv, out_row + c0 / 8);
+          }
+        }
+        tc_fence_before();
+      } else {
+        // Partials of this (q-tile, kv head, quarter): per slice the 32 rows' exponent references (log2 units), their sums
+        // under them, then the unnormalised outputs, four dims of a row together: a warp's accesses are 512 contiguous
+        // bytes.  A quarter is handed over by itself: the warp whose slice arrives last combines its 32 rows, so the
+        // CTA's warps do not wait for one another here.
+        constexpr int PART = (2 + HD) * 32;
+        const int unit = (ib.z * p.Hkv + kvh) * 4 + quarter;
+        float* base = p.split_ws + (size_t)unit * kAttnMaxSplits * PART + lane;
+        float* part = base + (size_t)split * PART;
+        part[0] = m_ref;
+        part[32] = l;
+#pragma unroll 1
+        for (int c0 = 0; c0 < HD; c0 += 32) {
+          uint32_t u[32];
+          tmem_ld32(t_o + c0, u);
+          tmem_ld_wait(u);
+          float4* dst = reinterpret_cast<float4*>(part - lane + 64) + (c0 / 4) * 32 + lane;
+#pragma unroll
+          for (int v = 0; v < 8; ++v)
+            dst[v * 32] = make_float4(__uint_as_float(u[4 * v]), __uint_as_float(u[4 * v + 1]), __uint_as_float(u[4 * v + 2]),
+                                      __uint_as_float(u[4 * v + 3]));
+        }
+        tc_fence_before();
+        __threadfence();
+        __syncwarp();
+        int arrived = 0;
+        if (lane == 0) {
+          arrived = atomicAdd(p.plan.counters + unit, 1);
+          if (arrived == n_split - 1) p.plan.counters[unit] = 0;      // ready for the next layer
+        }
+        if (__shfl_sync(0xffffffffu, arrived, 0) == n_split - 1) {
+          __threadfence();
+          // every slice's weight first (all their loads in flight together), then the outputs in slice order: the result
+          // does not depend on arrival
+          float wgt[kAttnMaxSplits], ls[kAttnMaxSplits], M = -INFINITY, L = 0.f;
+#pragma unroll
+          for (int s = 0; s < kAttnMaxSplits; ++s) {
+            wgt[s] = s < n_split ? __ldcg(base + (size_t)s * PART) : -INFINITY;
+            ls[s] = s < n_split ? __ldcg(base + (size_t)s * PART + 32) : 0.f;
+          }
+#pragma unroll
+          for (int s = 0; s < kAttnMaxSplits; ++s) M = fmaxf(M, wgt[s]);
+#pragma unroll
+          for (int s = 0; s < kAttnMaxSplits; ++s) {
+            wgt[s] = wgt[s] == -INFINITY ? 0.f : ex2(wgt[s] - M);
+            L += wgt[s] * ls[s];
+          }
+          const float inv = 1.f / L;
+#pragma unroll 1
+          for (int c0 = 0; c0 < HD; c0 += 32) {
             float o[32];
 #pragma unroll
             for (int e = 0; e < 32; ++e) o[e] = 0.f;
-            for (int s = 0; s < n_split; ++s) {           // fixed slice order: the result does not depend on arrival
-              const float* ps = tile_part + (size_t)s * PART;
-              const float mxs = __ldcg(ps);
-              const float wgt = (mxs == -INFINITY) ? 0.f : ex2(mxs - M);
-              Lsum += wgt * __ldcg(ps + 128);
 #pragma unroll
-              for (int e = 0; e < 32; ++e) o[e] += wgt * __ldcg(ps + (2 + half * OWN + c0 + e) * 128);
-            }
-            if (row_ok) {
-              const float inv = 1.f / Lsum;
-              uint4* dst = out_row + c0 / 8;
+            for (int s = 0; s < kAttnMaxSplits; ++s) {
+              if (s >= n_split) break;
+              const float4* src = reinterpret_cast<const float4*>(base - lane + (size_t)s * PART + 64) + (c0 / 4) * 32 + lane;
+              float4 x[8];
 #pragma unroll
-              for (int c = 0; c < 4; ++c)
-                dst[c] = make_uint4(pack_bf16(o[8 * c] * inv, o[8 * c + 1] * inv), pack_bf16(o[8 * c + 2] * inv, o[8 * c + 3] * inv),
-                                    pack_bf16(o[8 * c + 4] * inv, o[8 * c + 5] * inv), pack_bf16(o[8 * c + 6] * inv, o[8 * c + 7] * inv));
+              for (int v = 0; v < 8; ++v) x[v] = __ldcg(src + v * 32);
+#pragma unroll
+              for (int v = 0; v < 8; ++v) {
+                o[4 * v] += wgt[s] * x[v].x;
+                o[4 * v + 1] += wgt[s] * x[v].y;
+                o[4 * v + 2] += wgt[s] * x[v].z;
+                o[4 * v + 3] += wgt[s] * x[v].w;
+              }
             }
+            if (row_ok) store32(o, inv, out_row + c0 / 8);
           }
         }
-        // s_flag is rewritten by the next item only after all have read it
-        if (!warps_sync(group_bar, group_ph, lane, abort_flag, p.status, 429)) goto done;
       }
     }
   }

@@ -163,13 +163,13 @@ void launch_unpack_best(cudaStream_t st, const unsigned long long* row_best, int
 constexpr int kAttnMaxSplits = 8;      // most KV slices one q-tile is cut into
 struct AttnPlan {
   int4* items;      // two int4 per (q-tile, slice) item, longest first: {first packed row, position of the first
-                    // token, tokens, KV slot}, {first | (last + 1) << 16 KV tile, slice | slices << 8 | first token of the q-tile within its sequence << 16,
-                    // q-tile, KV tiles}
+                    // token, tokens, KV slot}, {first | (last + 1) << 16 KV block, slice | slices << 8 | first token of the q-tile within its sequence << 16,
+                    // q-tile, KV blocks}
   int4* items_unsorted;   // the same list in creation order (scratch of the plan kernel)
   int* n_items;
   int* tile_seq;    // [max_tiles] sequence of a q-tile
-  int* tile_nkv;    // [max_tiles] KV tiles it can see
-  int* counters;    // [max_tiles, n_kv_heads] slices that have delivered their partial
+  int* tile_nkv;    // [max_tiles] KV blocks it can see
+  int* counters;    // [max_tiles, n_kv_heads, 4] slices that have delivered their partial of a 32-row quarter
   int4* first;      // [grid CTAs][3]: the item a CTA of the attention grid starts with, ready to use: the item's two
                     // words, then {item x kv head index (-1: none), kv head, first two physical KV blocks}
   int n_kv_heads;
