@@ -40,7 +40,7 @@ struct hsd_ctx {
   bool pdl;           // kernels are launched with programmatic stream serialization
   int force_bn, force_splits;   // hsd_debug_set_gemm_tile
   int pair;                     // GEMMs may run as CTA pairs
-  int attn_target_items, attn_min_chunk;   // attention plan: items aimed at per launch, fewest 64-key KV blocks per slice
+  int attn_target_items, attn_min_chunk;   // attention plan: units (share x kv head) aimed at per launch, shortest slice in KV blocks
   int tap_layer, tap_which;                // hsd_debug_tap: armed for the next forward (tap_layer < 0: none)
   void* tap_dst;
   size_t tap_bytes;
@@ -68,7 +68,7 @@ struct hsd_ctx {
 namespace {
 
 struct Ws {
-  int* status;        // 16 ints; [4] = attention q-tile count, [5] = attention items
+  int* status;        // 16 ints; [4] = attention q-tile count, [5] = attention shares per kv head
   AttnPlan plan;
   RowMeta rm;
   int* sel_rows;
@@ -89,13 +89,21 @@ struct Ws {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// Shortest slice of a q-tile's KV range in 64-key blocks, and slices a q-tile is cut into at most: see attn_plan_kernel.
+constexpr int kAttnMinChunk = 8, kAttnMaxSlices = 12;
+
 // CTAs of an attention launch: as many as are resident at once
 inline int attn_grid(const hsd_ctx* c) { return 2 * c->n_sms; }
 
 inline int attn_max_tiles(const ModelDims& md, int T, int S) { return T / (128 / md.group) + S; }
-// Split-KV partial results: per (q-tile, kv head, slice) 128 rows of an fp32 accumulator row plus (max, sum).
-inline size_t split_ws_floats(const ModelDims& md, int T, int S) {
-  return (size_t)attn_max_tiles(md, T, S) * md.Hkv * kAttnMaxSplits * (md.D + 2) * 128;
+// Shares of a kv head in an attention launch: one per CTA slot it has.
+inline int attn_max_shares(const hsd_ctx* c) {
+  const int n = attn_grid(c) / c->md.Hkv;
+  return n < 1 ? 1 : (n > kAttnMaxShares ? kAttnMaxShares : n);
+}
+// Partial results of sliced q-tiles: two slots per share, each 128 rows of an fp32 accumulator row plus (reference, sum).
+inline size_t split_ws_floats(const hsd_ctx* c) {
+  return (size_t)2 * attn_max_shares(c) * c->md.Hkv * (c->md.D + 2) * 128;
 }
 
 Ws carve(const hsd_ctx* c, void* base, int T, int S) {
@@ -139,16 +147,16 @@ Ws carve(const hsd_ctx* c, void* base, int T, int S) {
   w.qkv_f32 = c->simt ? static_cast<float*>(take(sizeof(float) * (size_t)T * md.qkv_out)) : nullptr;
   w.row_best = static_cast<unsigned long long*>(take(sizeof(unsigned long long) * T));
   w.zdraft = static_cast<float*>(take(sizeof(float) * T));
-  w.split_ws = c->simt ? nullptr : static_cast<float*>(take(sizeof(float) * split_ws_floats(md, T, S)));
+  w.split_ws = c->simt ? nullptr : static_cast<float*>(take(sizeof(float) * split_ws_floats(c)));
   {
-    const int mt = attn_max_tiles(md, T, S);
-    w.plan.items = static_cast<int4*>(take(sizeof(int4) * 2 * (size_t)mt * kAttnMaxSplits));
-    w.plan.items_unsorted = static_cast<int4*>(take(sizeof(int4) * 2 * (size_t)mt * kAttnMaxSplits));
+    const int mt = attn_max_tiles(md, T, S), shares = attn_max_shares(c);
+    w.plan.items = static_cast<int4*>(take(sizeof(int4) * 2 * (size_t)(mt + shares)));
+    w.plan.share_start = static_cast<int*>(take(sizeof(int) * (shares + 1)));
     w.plan.tile_seq = static_cast<int*>(take(sizeof(int) * mt));
-    w.plan.tile_nkv = static_cast<int*>(take(sizeof(int) * mt));
-    w.plan.counters = static_cast<int*>(take(sizeof(int) * (size_t)mt * md.Hkv * 4));
-    w.plan.first = static_cast<int4*>(take(sizeof(int4) * 3 * 2 * (size_t)c->n_sms));
-    w.plan.n_items = w.status ? w.status + 5 : nullptr;
+    w.plan.tile_pos = static_cast<int*>(take(sizeof(int) * mt));
+    w.plan.counters = static_cast<int*>(take(sizeof(int) * 2 * (size_t)shares * md.Hkv * 4));
+    w.plan.first = static_cast<int4*>(take(sizeof(int4) * 3 * (size_t)attn_grid(c)));
+    w.plan.n_shares = w.status ? w.status + 5 : nullptr;
     w.plan.n_kv_heads = md.Hkv;
     w.plan.grid = attn_grid(c);
   }
@@ -281,11 +289,9 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
   CUtensorMap tm_h, tm_attn, tm_act, tm_q, tm_k, tm_v, tm_x_add, tm_q_st, tm_act_st;
   if (!c->attn_simt) {
     Scope s(c, st, KC_SETUP);
-    // items per launch: about one per CTA slot (two CTAs per SM), at least attn_min_chunk KV blocks each
     // (a context with a fixed summation order never cuts a KV range: where the cuts fall depends on the batch)
-    launch_attn_plan(st, w.rm, w.plan, kv, a.n_seqs, tokens_per_tile, max(1, c->attn_target_items / md.Hkv),
-                     c->max_splits == 1 ? (1 << 20) : c->attn_min_chunk,
-                     w.status + 4, w.status, c->pdl);
+    launch_attn_plan(st, w.rm, w.plan, kv, a.n_seqs, tokens_per_tile, max(1, min(attn_max_shares(c), c->attn_target_items / md.Hkv)),
+                     c->attn_min_chunk, kAttnMaxSlices, c->max_splits == 1, w.status + 4, w.status, c->pdl);
   }
   if (!c->simt) {
     if (make_tmap_2d(&tm_h, w.h, T, md.d, 128) || make_tmap_2d(&tm_attn, w.attn, T, md.Hq * md.D, 128) ||
@@ -569,8 +575,8 @@ int hsd_create(const hsd_model_config* cfg, const hsd_weights* w, hsd_ctx** out)
   c->hg_seen_valid = false;
   c->hg_exec = nullptr;
   c->hg_launches = 0;
-  c->attn_target_items = attn_grid(c);   // one item per CTA slot: slicing costs a partial hand-over per slice
-  c->attn_min_chunk = 8;
+  c->attn_target_items = attn_grid(c);
+  c->attn_min_chunk = kAttnMinChunk;
   c->tap_layer = -1; c->tap_which = 0; c->tap_dst = nullptr; c->tap_bytes = 0;
   c->last_cuda_error = 0;
   c->launches = 0;
@@ -1134,7 +1140,7 @@ int hsd_debug_set_gemm_tile(hsd_ctx* c, int tile_n, int k_slices) {
 int hsd_debug_set_attn_plan(hsd_ctx* c, int target_items, int min_kv_tiles) {
   if (!c || target_items < 0 || min_kv_tiles < 0) return HSD_ERR_INVALID_ARG;
   c->attn_target_items = target_items ? target_items : attn_grid(c);
-  c->attn_min_chunk = 2 * (min_kv_tiles ? min_kv_tiles : 4);
+  c->attn_min_chunk = min_kv_tiles ? 2 * min_kv_tiles : kAttnMinChunk;
   return HSD_OK;
 }
 

@@ -5,15 +5,15 @@
 //
 // Work item = (q-tile, kv slice, kv head).  A q-tile is 128 MMA rows: 128/group consecutive tokens of one
 // sequence x the `group` query heads that share the kv head (GQA packing, so K/V blocks are read once per
-// group).  The KV range a q-tile can see is cut into up to kAttnMaxSplits slices so that a launch has about one item
-// per CTA slot whatever the mix of context lengths (one page chunk over a long context, or many short regions); the
-// plan is made once per step on the device (attn_plan_kernel) and reused by every layer.  Slices leave (unnormalised
-// O, exponent reference, sum) partials in the workspace and the last slice to finish combines them in slice order, so
-// the result does not depend on which CTA ran what.
+// group).  A q-tile's KV range is run whole or cut into slices so that a launch has one share of work per CTA slot,
+// whatever the mix of context lengths (one page chunk over a long context, or many short regions); the plan is made
+// once per step on the device (attn_plan_kernel) and reused by every layer.  Slices leave
+// (unnormalised O, exponent reference, sum) partials in the workspace and the last slice to finish combines them in
+// slice order, so the result does not depend on which CTA ran what.
 //
 // The KV range is walked in paged blocks of 64 keys [64 keys][head_dim] per kv head, fetched by TMA through the block
 // table; K is the K-major B operand of S = Q K^T (128 x 64 x head_dim), V the MN-major B operand of O += P V (128 x
-// head_dim x 64).  Persistent CTAs, two per SM, walk the item list.  Warp roles:
+// head_dim x 64).  Persistent CTAs, two per SM, walk their shares.  Warp roles:
 //   warp 0      TMA producer: Q, the K ring and the V ring
 //   warp 1      MMA issuer + TMEM owner
 //   warps 2..5  softmax: warp w works on TMEM lane quarter w mod 4 (the hardware's rule), one thread per q row
@@ -68,7 +68,7 @@ struct AttnParams {
   const int* block_table;
   int max_blocks, n_blocks, Hq, Hkv, group, layer;
   bf16* out;            // [T, Hq*HD]
-  float* split_ws;      // partials of sliced items: [q-tile][kv head][quarter][slice][2 + HD][32 rows]
+  float* split_ws;      // partials of sliced items: [slot][kv head][quarter][2 + HD][32 rows], see slice_slot
   const uint4* anc;     // [T] ancestry masks of candidate-tree rows, or nullptr: plain causal order within the call
   int* status;
 };
@@ -102,125 +102,223 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
   return y;
 }
-// The item x kv-head index that CTA `bx` of a grid of `G` takes in round r of its walk (-1: none).  Round r: CTA i
-// takes index r G + i in even rounds and r G + (G - 1 - i) in odd ones (the list is sorted longest first, so the CTA
-// that drew a long item in one round draws a short one in the next).  A launch with fewer items than CTAs leaves
-// some SMs with one busy CTA (the grid is two CTAs per SM, and CTA b shares its SM with CTA b + G/2 under the usual
-// placement); a CTA that has its SM alone walks its tiles faster, so the longest items go to those SMs and the
-// others pair a long item with a short one.
-__device__ __forceinline__ int attn_item_at(int r, int total, int bx, int G) {
-  const int n_rounds = (total + G - 1) / G, half_grid = G / 2;
-  if (n_rounds == 1 && total > half_grid) {
-    const int n_second = total - half_grid;            // busy CTAs in the second half of the grid
-    if (bx < half_grid) return bx >= n_second ? bx - n_second : (half_grid - n_second) + bx;
-    return bx - half_grid < n_second ? total - 1 - (bx - half_grid) : -1;
-  }
-  const int i = (r & 1) ? G - 1 - bx : bx;
-  const int w = r * G + i;
-  return w < total ? w : -1;
+// The unit (share, kv head) that CTA `bx` of a grid of `G` starts with (n: none).  A launch with fewer units than CTAs
+// leaves some SMs with one busy CTA (the grid is two CTAs per SM, and CTA b shares its SM with CTA b + G/2 under the usual
+// placement); a CTA that has its SM alone walks its blocks faster, so the longest units go to those SMs and the others
+// pair a long one with a short one (shares of a one-round plan are sorted longest first).
+__device__ __forceinline__ int attn_unit_at(int bx, int n, int G) {
+  const int half = G / 2;
+  if (n <= half || n > G) return bx;
+  const int n_second = n - half;                       // busy CTAs in the second half of the grid
+  if (bx < half) return bx >= n_second ? bx - n_second : (half - n_second) + bx;
+  return bx - half < n_second ? n - 1 - (bx - half) : n;
 }
 
+// Where the partials of a sliced q-tile's slices lie.  One-round plans: every item has a slot of its own, `z` names slice
+// 0's.  Line plans: z = 2 k0 + 1 with k0 the share whose last item is slice 0; slice k > 0 is the first item of share
+// k0 + k, so two slots per share keep all slices apart.  Either way z is unique to the q-tile (its arrival counter).
+__device__ __forceinline__ int slice_slot(int z, int slice, int line) { return !line ? z + slice : slice == 0 ? z : z - 1 + 2 * slice; }
+
 // ------------------------------------------------------------------------------------------------
-// Plan: one CTA.  For every q-tile the KV blocks it can see and into how many slices that range is cut, then
-// the flat list of (q-tile, slice) items with everything a CTA needs to run one.
-__global__ void attn_plan_kernel(RowMeta rm, AttnPlan pl, KvView kv, int n_seqs, int tokens_per_tile, int target_items,
-                                 int min_chunk, const int* tile_count, const int* status) {
+// Plan: one CTA.  Work is counted in 64-key blocks.  A kv head has `max_shares` CTA slots; every kv head has the same
+// plan, so a launch runs n_shares x n_kv_heads units, unit u = share u / n_kv_heads of head u % n_kv_heads.
+//
+// One round: a q-tile is cut into equal slices of at least min_chunk blocks, each a share of its own, as fine as leaves no
+// slot with two.  A slice costs a hand-over (~3 us, four blocks' time), so nothing is cut finer than the launch needs.
+// Line: where that leaves the longest slice more than kLineGain blocks above the mean (more q-tiles than slots, or
+// q-tiles a little longer than the mean, which only halves would shorten), the q-tiles' ranges are laid end to end, each
+// with kTileCost blocks added for what an item costs beside its blocks (Q, first product, output), and the line is cut into
+// equal shares; a cut that would leave a piece of fewer than kMinPiece blocks moves to the q-tile's edge.
+// Measured, step times with equal shares of the line always against one round always: 2,048 rows over 16,384 (33
+// q-tiles of 272 blocks on 37 slots) 7.10 / 7.57 ms; 16 regions (25 q-tiles of 4 to 17 blocks) 1.78 / 1.73; 512 rows over
+// 7,936 2.07 / 2.02.
+// no_cut (contexts with a fixed summation order): q-tiles are never cut, cuts of the line move to the nearer edge.
+constexpr int kTileCost = 3, kMinPiece = 2, kLineGain = 8, kPlanThreads = 512;
+__global__ void __launch_bounds__(kPlanThreads) attn_plan_kernel(RowMeta rm, AttnPlan pl, KvView kv, int n_seqs,
+                                                                 int tokens_per_tile, int max_shares, int min_chunk,
+                                                                 int max_slices, int no_cut, const int* tile_count,
+                                                                 const int* status) {
   pdl_wait();
   pdl_launch_dependents();
-  __shared__ int s_total;
-  if (threadIdx.x == 0) s_total = 0;
-  __syncthreads();
+  // one round: creation order of the items; line: cuts (q-tile, block) and how many of them lie inside q-tiles so far
+  __shared__ int s_ct[kAttnMaxShares + 1], s_co[kAttnMaxShares + 1], s_rank[kAttnMaxShares + 1];
+  __shared__ int s_warp[kPlanThreads / 32], s_longest, s_blocks, s_count, s_slice;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (*status) {
-    if (threadIdx.x == 0) *pl.n_items = 0;
-    for (int b = threadIdx.x; b < pl.grid; b += blockDim.x) pl.first[3 * b + 2] = make_int4(-1, 0, 0, 0);
+    if (tid == 0) *pl.n_shares = 0;
+    for (int b = tid; b < pl.grid; b += kPlanThreads) pl.first[3 * b + 2] = make_int4(0, 0, 0, 0);
     return;
   }
+  if (tid == 0) s_longest = s_blocks = 0;
   const int n_tiles = *tile_count;
-  int my = 0;
-  for (int s = threadIdx.x; s < n_seqs; s += blockDim.x) {
-    const int t0 = rm.seq_tile0[s], t1 = rm.seq_tile0[s + 1];
-    const int L = rm.seq_len[s], n = rm.seq_n[s];
-    for (int t = t0; t < t1; ++t) {
-      const int tok_end = min(n, (t - t0 + 1) * tokens_per_tile);
-      const int n_kv = (L + tok_end + 63) >> 6;          // 64-key blocks: the unit slices are cut in
-      pl.tile_seq[t] = s;
-      pl.tile_nkv[t] = n_kv;
-      my += n_kv;
-    }
-  }
-  atomicAdd(&s_total, my);
+  for (int s = tid; s < n_seqs; s += kPlanThreads)
+    for (int t = rm.seq_tile0[s]; t < rm.seq_tile0[s + 1]; ++t) pl.tile_seq[t] = s;
   __syncthreads();
-  // KV blocks per slice: start from an even share.  Rounding up the slice count of every q-tile can leave the
-  // launch with somewhat more items than CTA slots, and then the few CTAs that draw a second item double its
-  // length: in that band (1 to 1.6 items per slot) the share is grown until every slot has at most one item.
-  // Well beyond it a second round is about full and the sorted walk balances it, so the share is kept.
-  __shared__ int s_n, s_count, s_longest;
-  int chunk = max(min_chunk, (s_total + target_items - 1) / max(1, target_items));
-  for (int it = 0; it < 256; ++it) {                      // every thread runs the same iterations
-    if (threadIdx.x == 0) { s_count = 0; s_longest = 0; }
-    __syncthreads();
-    int count = 0, longest = 0;
-    for (int t = threadIdx.x; t < n_tiles; t += blockDim.x) {
-      const int n_kv = pl.tile_nkv[t];
-      count += max(1, min(kAttnMaxSplits, (n_kv + chunk - 1) / chunk));
-      longest = max(longest, n_kv);
+  auto blocks_of = [&](int t) -> int {                 // 64-key blocks q-tile t can see
+    const int s = pl.tile_seq[t];
+    return (rm.seq_len[s] + min(rm.seq_n[s], (t - rm.seq_tile0[s] + 1) * tokens_per_tile) + 63) >> 6;
+  };
+  auto tile_item = [&](int t, int& tok0) -> int4 {
+    const int s = pl.tile_seq[t];
+    tok0 = (t - rm.seq_tile0[s]) * tokens_per_tile;
+    return make_int4(rm.seq_q0[s] + tok0, rm.seq_len[s] + tok0, min(tokens_per_tile, rm.seq_n[s] - tok0), rm.seq_slot[s]);
+  };
+  // exclusive sum over the CTA, in thread order; `all` = the total (every thread calls it the same number of times)
+  auto scan = [&](int v, int& all) -> int {
+    int incl = v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
     }
-    atomicAdd(&s_count, count);
-    atomicMax(&s_longest, longest);
+    if (lane == 31) s_warp[warp] = incl;
     __syncthreads();
-    const bool done = s_count <= target_items || 5 * s_count >= 8 * target_items || chunk >= s_longest;
+    int before = 0;
+    all = 0;
+    for (int w = 0; w < kPlanThreads / 32; ++w) {
+      if (w < warp) before += s_warp[w];
+      all += s_warp[w];
+    }
     __syncthreads();
-    if (done) break;
-    chunk += max(1, chunk >> 4);
+    return before + incl - v;
+  };
+  // lengths, and where every q-tile begins on the line
+  int total = 0;
+  for (int t0 = 0; t0 < n_tiles; t0 += kPlanThreads) {
+    const int t = t0 + tid;
+    const int n = t < n_tiles ? blocks_of(t) : 0;
+    int all;
+    const int pos = scan(t < n_tiles ? n + kTileCost : 0, all);
+    if (t < n_tiles) {
+      pl.tile_pos[t] = total + pos;
+      atomicMax(&s_longest, n);
+      atomicAdd(&s_blocks, n);
+    }
+    total += all;
   }
-  if (threadIdx.x == 0) {
-    int n = 0;
-    for (int t = 0; t < n_tiles; ++t) {   // serial: a few hundred tiles at most, once per step
-      const int n_kv = pl.tile_nkv[t];
-      const int s = pl.tile_seq[t];
-      const int tok0 = (t - rm.seq_tile0[s]) * tokens_per_tile;
-      const int n_tok = min(tokens_per_tile, rm.seq_n[s] - tok0);
-      const int ns = max(1, min(kAttnMaxSplits, (n_kv + chunk - 1) / chunk));
-      const int base = n_kv / ns, rem = n_kv % ns;
-      int lo = 0;
-      for (int k = 0; k < ns; ++k) {
-        const int len = base + (k < rem ? 1 : 0);
-        pl.items_unsorted[2 * n] = make_int4(rm.seq_q0[s] + tok0, rm.seq_len[s] + tok0, n_tok, rm.seq_slot[s]);
-        pl.items_unsorted[2 * n + 1] = make_int4(lo | ((lo + len) << 16), k | (ns << 8) | (tok0 << 16), t, len);
-        ++n;
-        lo += len;
+  __syncthreads();
+  const int longest = s_longest, mean = (s_blocks + max_shares - 1) / max_shares;
+  // one round: the slice length is grown until the items fit the slots
+  int chunk = max(max(min_chunk, mean), (longest + max_slices - 1) / max_slices);
+  bool line = n_tiles > max_shares;
+  if (no_cut) {
+    chunk = longest;
+  } else if (!line) {
+    for (;;) {                                            // every thread runs the same iterations
+      if (tid == 0) s_count = s_slice = 0;
+      __syncthreads();
+      for (int t = tid; t < n_tiles; t += kPlanThreads) {
+        const int n = blocks_of(t), ns = max(1, (n + chunk - 1) / chunk);
+        atomicAdd(&s_count, ns);
+        atomicMax(&s_slice, (n + ns - 1) / ns);
+      }
+      __syncthreads();
+      const int count = s_count;
+      __syncthreads();
+      if (count <= max_shares || chunk >= longest) break;
+      chunk += max(1, chunk >> 5);
+    }
+    line = s_slice > max(mean, min_chunk) + kLineGain;
+  }
+  int P;
+  if (!line) {
+    P = 0;
+    for (int t0 = 0; t0 < n_tiles; t0 += kPlanThreads) {
+      const int t = t0 + tid;
+      const int n = t < n_tiles ? blocks_of(t) : 0;
+      const int ns = t < n_tiles ? max(1, (n + chunk - 1) / chunk) : 0;
+      int all;
+      const int at = P + scan(ns, all);
+      for (int k = 0; k < ns; ++k) {                     // q-tile, slice (| slices << 16), length of item at + k
+        s_ct[at + k] = t;
+        s_co[at + k] = k | (ns << 16);
+        s_rank[at + k] = n / ns + (k < n % ns ? 1 : 0);
+      }
+      P += all;
+    }
+    __syncthreads();
+    for (int i = tid; i < P; i += kPlanThreads) {         // longest first (rank sort, ties by creation order)
+      const int len = s_rank[i], t = s_ct[i], k = s_co[i] & 0xffff, ns = s_co[i] >> 16;
+      int rank = 0;
+      for (int j = 0; j < P; ++j) rank += (s_rank[j] > len) || (s_rank[j] == len && j < i);
+      const int n = blocks_of(t), from = k * (n / ns) + min(k, n % ns);
+      int tok0;
+      pl.items[2 * rank] = tile_item(t, tok0);
+      pl.items[2 * rank + 1] = make_int4(from | ((from + len) << 16), k | (ns << 8) | (tok0 << 16), i - k, 0);
+      pl.share_start[rank] = rank;
+    }
+    if (tid == 0) pl.share_start[P] = P;
+  } else {
+    P = max(1, min(max_shares, total / max(min_chunk, (longest + max_slices - 1) / max_slices)));
+    for (int k = tid; k <= P; k += kPlanThreads) {
+      int t = n_tiles, off = 0;
+      if (k < P) {
+        const int b = (int)((long long)k * total / P);
+        int lo = 0, hi = n_tiles;                          // last q-tile that begins at or before b
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (pl.tile_pos[mid] <= b) lo = mid; else hi = mid;
+        }
+        t = lo;
+        const int n = blocks_of(t);
+        off = b - pl.tile_pos[t] - kTileCost;
+        if (off < kMinPiece || (no_cut && 2 * off < n)) {
+          off = 0;
+        } else if (no_cut || n - off < kMinPiece) {
+          ++t;
+          off = 0;
+        }
+      }
+      s_ct[k] = t;
+      s_co[k] = off;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      int sum = 0;
+      for (int k0 = 0; k0 <= P; k0 += 32) {
+        const int k = k0 + lane;
+        const unsigned in = __ballot_sync(0xffffffffu, k <= P && s_co[min(k, P)] > 0);
+        if (k <= P) s_rank[k] = sum + __popc(in & (0xffffffffu >> (31 - lane)));
+        sum += __popc(in);
       }
     }
-    *pl.n_items = n;
-    s_n = n;
-  }
-  __syncthreads();
-  // longest first (rank sort, ties by creation order): the attention CTAs walk the list in boustrophedon order, so
-  // every CTA's share of KV blocks comes out about equal
-  const int n = s_n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const int len = pl.items_unsorted[2 * i + 1].w;
-    int rank = 0;
-    for (int k = 0; k < n; ++k) {
-      const int lk = pl.items_unsorted[2 * k + 1].w;
-      rank += (lk > len) || (lk == len && k < i);
+    __syncthreads();
+    // a share begins with item (its q-tile + the cuts inside q-tiles up to it); a q-tile's slices follow one another
+    for (int k = tid; k <= P; k += kPlanThreads) pl.share_start[k] = s_ct[k] + s_rank[k];
+    for (int t = tid; t < n_tiles; t += kPlanThreads) {
+      int lo = 0, hi = P;                                  // first cut inside q-tile t or beyond it (cut P lies beyond all)
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (s_ct[mid] > t || (s_ct[mid] == t && s_co[mid] > 0)) hi = mid; else lo = mid + 1;
+      }
+      const int k0 = lo;
+      int ns = 1;
+      while (k0 + ns - 1 <= P && s_ct[k0 + ns - 1] == t) ++ns;
+      int tok0;
+      const int4 ia = tile_item(t, tok0);
+      const int n = blocks_of(t), first = t + s_rank[k0] - (s_co[k0] > 0 ? 1 : 0);
+      int from = 0;
+      for (int k = 0; k < ns; ++k) {
+        const int to = k + 1 < ns ? s_co[k0 + k] : n;
+        pl.items[2 * (first + k)] = ia;
+        pl.items[2 * (first + k) + 1] = make_int4(from | (to << 16), k | (ns << 8) | (tok0 << 16), 2 * (k0 - 1) + 1, 1);
+        from = to;
+      }
     }
-    pl.items[2 * rank] = pl.items_unsorted[2 * i];
-    pl.items[2 * rank + 1] = pl.items_unsorted[2 * i + 1];
   }
-  // slice-arrival counters of every (q-tile, kv head, quarter): zero at the start of a step, reset by the combiner
-  for (int i = threadIdx.x; i < n_tiles * pl.n_kv_heads * 4; i += blockDim.x) pl.counters[i] = 0;
+  if (tid == 0) *pl.n_shares = P;
+  // slice-arrival counters: zero at the start of a step, reset by the combiner
+  for (int i = tid; i < 2 * P * pl.n_kv_heads * 4; i += kPlanThreads) pl.counters[i] = 0;
   // what every CTA of the attention grid starts with, in one record: its first item and the physical blocks of that
   // item's first two KV blocks, so that a CTA's first loads do not wait for a chain of dependent reads (item -> block table)
   __syncthreads();
-  const int total = n * pl.n_kv_heads;
-  for (int b = threadIdx.x; b < pl.grid; b += blockDim.x) {
-    const int w = attn_item_at(0, total, b, pl.grid);
-    if (w < 0) {
-      pl.first[3 * b + 2] = make_int4(-1, 0, 0, 0);
+  for (int b = tid; b < pl.grid; b += kPlanThreads) {
+    const int share = attn_unit_at(b, P * pl.n_kv_heads, pl.grid) / pl.n_kv_heads;
+    const int i0 = share < P ? pl.share_start[share] : 0, count = share < P ? pl.share_start[share + 1] - i0 : 0;
+    if (count == 0) {
+      pl.first[3 * b + 2] = make_int4(0, 0, 0, 0);
       continue;
     }
-    const int4 ia = pl.items[2 * (w / pl.n_kv_heads)], ib = pl.items[2 * (w / pl.n_kv_heads) + 1];
+    const int4 ia = pl.items[2 * i0], ib = pl.items[2 * i0 + 1];
     const int kt_lo = ib.x & 0xffff, kt_hi = ib.x >> 16;
     int phys0 = 0, phys1 = 0;
     if (kt_hi > kt_lo && ia.w >= 0 && ia.w < kv.n_slots && kt_hi <= kv.max_blocks) {
@@ -230,15 +328,15 @@ __global__ void attn_plan_kernel(RowMeta rm, AttnPlan pl, KvView kv, int n_seqs,
     }
     pl.first[3 * b] = ia;
     pl.first[3 * b + 1] = ib;
-    pl.first[3 * b + 2] = make_int4(w, w % pl.n_kv_heads, phys0, phys1);
+    pl.first[3 * b + 2] = make_int4(i0, count, phys0, phys1);
   }
 }
 
 void launch_attn_plan(cudaStream_t st, const RowMeta& rm, const AttnPlan& pl, const KvView& kv, int n_seqs,
-                      int tokens_per_tile, int target_items, int min_chunk, const int* tile_count, const int* status,
-                      bool pdl) {
-  launch_kernel(attn_plan_kernel, dim3(1), dim3(256), 0, st, pdl, rm, pl, kv, n_seqs, tokens_per_tile, target_items,
-                min_chunk, tile_count, status);
+                      int tokens_per_tile, int max_shares, int min_chunk, int max_slices, bool no_cut, const int* tile_count,
+                      const int* status, bool pdl) {
+  launch_kernel(attn_plan_kernel, dim3(1), dim3(kPlanThreads), 0, st, pdl, rm, pl, kv, n_seqs, tokens_per_tile, max_shares,
+                min_chunk, max_slices, no_cut ? 1 : 0, tile_count, status);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -314,10 +412,9 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     rec_b = rec[1];
     rec_c = rec[2];
   }
-  const int status_now = *p.status, n_items_now = *p.plan.n_items;
-  const int total = status_now ? 0 : n_items_now * p.Hkv;
-  const int n_rounds = (total + (int)gridDim.x - 1) / (int)gridDim.x;
-  auto item_of_round = [&](int r) -> int { return attn_item_at(r, total, (int)blockIdx.x, (int)gridDim.x); };
+  const int status_now = *p.status, n_shares_now = *p.plan.n_shares;
+  const int n_units = status_now ? 0 : n_shares_now * p.Hkv;
+  const int G = (int)gridDim.x, u0 = attn_unit_at((int)blockIdx.x, n_units, G);
 
   // Block counter t (all 64-key blocks of all items of this CTA): ring stage = t % STAGES, score buffer = t % NBUF, and
   // every barrier's parity follows from how often t has used it; n counts items (Q hand-over barriers).
@@ -340,21 +437,19 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       __syncwarp();
       return true;
     };
-    for (int r = 0; r < n_rounds; ++r) {
-      const int w = r == 0 ? (total > 0 ? rec_c.x : -1) : item_of_round(r);
-      if (w < 0) continue;
-      int4 ia = rec_a, ib = rec_b;
-      int kvh = rec_c.y;
-      if (r != 0) {
-        ia = p.plan.items[2 * (w / p.Hkv)];
-        ib = p.plan.items[2 * (w / p.Hkv) + 1];
-        kvh = w % p.Hkv;
-      }
+    bool waited = false;                                 // for the kernel before this one
+    for (int u = u0; u < n_units; u += G) {
+     const int kvh = u % p.Hkv;
+     const int i0 = u == u0 ? rec_c.x : p.plan.share_start[u / p.Hkv];
+     const int i1 = u == u0 ? rec_c.x + rec_c.y : p.plan.share_start[u / p.Hkv + 1];
+     for (int i = i0; i < i1; ++i) {
+      const bool recorded = u == u0 && i == i0;
+      const int4 ia = recorded ? rec_a : p.plan.items[2 * i], ib = recorded ? rec_b : p.plan.items[2 * i + 1];
       const int kt_lo = ib.x & 0xffff, kt_hi = ib.x >> 16;
       const int* bt = p.block_table + (size_t)ia.w * p.max_blocks;
-      auto phys_of = [&](int kt) -> int { return r == 0 && kt < kt_lo + 2 ? (kt == kt_lo ? rec_c.z : rec_c.w) : bt[kt]; };
+      auto phys_of = [&](int kt) -> int { return recorded && kt < kt_lo + 2 ? (kt == kt_lo ? rec_c.z : rec_c.w) : bt[kt]; };
       int early = kt_lo;                                 // K and V of [kt_lo, early) are on their way
-      if (r == 0) {
+      if (recorded) {
         // blocks that hold committed rows only, as many as the rings take, ahead of the grid dependency
         const int committed = min(kt_hi, (ia.y - (ib.y >> 16)) >> 6);
         for (; early < committed && early - kt_lo < STAGES; ++early) {
@@ -362,7 +457,10 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           if (!load(&tmK, sK, k_full, k_empty, t + (early - kt_lo), phys, kvh)) goto done;
           if (!load(&tmV, sV, v_full, v_empty, t + (early - kt_lo), phys, kvh)) goto done;
         }
+      }
+      if (!waited) {
         pdl_wait();
+        waited = true;
       }
       if (!mbar_wait(q_empty, (n & 1) ^ 1u, abort_flag, p.status, 400)) goto done;
       if (elect_one()) {
@@ -384,6 +482,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       }
       t += kt_hi - kt_lo;
       ++n;
+     }
     }
   } else if (warp == 1) {
     pdl_wait();
@@ -394,10 +493,11 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                    v_desc = umma_desc_sw128(smem_u32(sV));     // a byte offset adds a sixteenth of itself
     uint32_t t = 0;
     int n = 0;
-    for (int r = 0; r < n_rounds; ++r) {
-      const int w = r == 0 ? (total > 0 ? rec_c.x : -1) : item_of_round(r);
-      if (w < 0) continue;
-      const int4 ib = r == 0 ? rec_b : p.plan.items[2 * (w / p.Hkv) + 1];
+    for (int u = u0; u < n_units; u += G) {
+     const int i0 = u == u0 ? rec_c.x : p.plan.share_start[u / p.Hkv];
+     const int i1 = u == u0 ? rec_c.x + rec_c.y : p.plan.share_start[u / p.Hkv + 1];
+     for (int i = i0; i < i1; ++i) {
+      const int4 ib = u == u0 && i == i0 ? rec_b : p.plan.items[2 * i + 1];
       const uint32_t t_end = t + (ib.x >> 16) - (ib.x & 0xffff);
       // S(ti) = Q K(ti)^T: four K = 16 steps over every 64 dims, N = 64 keys, into the buffer P(ti - NBUF) has left
       auto issue_s = [&](uint32_t ti) -> bool {
@@ -452,6 +552,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
       }
       ++n;
+     }
     }
     // every stage-release arrival must land before the CTA's shared memory can be handed on
     if (t > 0 && !mbar_wait(o_full + (t - 1) % NBUF, ((t - 1) / NBUF) & 1, abort_flag, p.status, 414)) goto done;
@@ -465,11 +566,11 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     const float sc = (HD == 64 ? 0.125f : 0.08838834764831845f) * 1.4426950408889634f;     // 1/sqrt(HD) * log2(e)
     uint32_t t = 0;
     pdl_wait();
-    for (int r = 0; r < n_rounds; ++r) {
-      const int w = item_of_round(r);
-      if (w < 0) continue;
-      const int4 ia = p.plan.items[2 * (w / p.Hkv)], ib = p.plan.items[2 * (w / p.Hkv) + 1];
-      const int kvh = w % p.Hkv;
+    for (int u = u0; u < n_units; u += G) {
+     const int kvh = u % p.Hkv;
+     const int i0 = p.plan.share_start[u / p.Hkv], i1 = p.plan.share_start[u / p.Hkv + 1];
+     for (int i = i0; i < i1; ++i) {
+      const int4 ia = p.plan.items[2 * i], ib = p.plan.items[2 * i + 1];
       const int q_row0 = ia.x, pos0 = ia.y, n_tok = ia.z;
       const int kt_lo = ib.x & 0xffff, kt_hi = ib.x >> 16;
       const int split = ib.y & 0xff, n_split = (ib.y >> 8) & 0xff;
@@ -625,9 +726,8 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // bytes.  A quarter is handed over by itself: the warp whose slice arrives last combines its 32 rows, so the
         // CTA's warps do not wait for one another here.
         constexpr int PART = (2 + HD) * 32;
-        const int unit = (ib.z * p.Hkv + kvh) * 4 + quarter;
-        float* base = p.split_ws + (size_t)unit * kAttnMaxSplits * PART + lane;
-        float* part = base + (size_t)split * PART;
+        auto slice = [&](int k) -> float* { return p.split_ws + (size_t)((slice_slot(ib.z, k, ib.w) * p.Hkv + kvh) * 4 + quarter) * PART; };
+        float* part = slice(split) + lane;
         part[0] = m_ref;
         part[32] = l;
 #pragma unroll 1
@@ -646,51 +746,63 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         __syncwarp();
         int arrived = 0;
         if (lane == 0) {
-          arrived = atomicAdd(p.plan.counters + unit, 1);
-          if (arrived == n_split - 1) p.plan.counters[unit] = 0;      // ready for the next layer
+          int* ctr = p.plan.counters + (ib.z * p.Hkv + kvh) * 4 + quarter;
+          arrived = atomicAdd(ctr, 1);
+          if (arrived == n_split - 1) *ctr = 0;          // ready for the next layer
         }
         if (__shfl_sync(0xffffffffu, arrived, 0) == n_split - 1) {
           __threadfence();
-          // every slice's weight first (all their loads in flight together), then the outputs in slice order: the result
-          // does not depend on arrival
-          float wgt[kAttnMaxSplits], ls[kAttnMaxSplits], M = -INFINITY, L = 0.f;
-#pragma unroll
-          for (int s = 0; s < kAttnMaxSplits; ++s) {
-            wgt[s] = s < n_split ? __ldcg(base + (size_t)s * PART) : -INFINITY;
-            ls[s] = s < n_split ? __ldcg(base + (size_t)s * PART + 32) : 0.f;
-          }
-#pragma unroll
-          for (int s = 0; s < kAttnMaxSplits; ++s) M = fmaxf(M, wgt[s]);
-#pragma unroll
-          for (int s = 0; s < kAttnMaxSplits; ++s) {
-            wgt[s] = wgt[s] == -INFINITY ? 0.f : ex2(wgt[s] - M);
-            L += wgt[s] * ls[s];
-          }
-          const float inv = 1.f / L;
+          // Slices in order, whatever the order they arrived in, under a reference that grows with them; what three slices
+          // left is in flight at once.
 #pragma unroll 1
           for (int c0 = 0; c0 < HD; c0 += 32) {
-            float o[32];
+            float o[32], L = 0.f, M = -INFINITY;
 #pragma unroll
             for (int e = 0; e < 32; ++e) o[e] = 0.f;
+#pragma unroll 1
+            for (int k = 0; k < n_split; k += 3) {
+              float m[3], ls[3];
+              float4 x[3][8];
 #pragma unroll
-            for (int s = 0; s < kAttnMaxSplits; ++s) {
-              if (s >= n_split) break;
-              const float4* src = reinterpret_cast<const float4*>(base - lane + (size_t)s * PART + 64) + (c0 / 4) * 32 + lane;
-              float4 x[8];
+              for (int j = 0; j < 3; ++j) {
+                if (k + j >= n_split) {
+                  m[j] = -INFINITY;
+                  ls[j] = 0.f;
 #pragma unroll
-              for (int v = 0; v < 8; ++v) x[v] = __ldcg(src + v * 32);
+                  for (int v = 0; v < 8; ++v) x[j][v] = make_float4(0.f, 0.f, 0.f, 0.f);
+                } else {
+                  const float* ps = slice(k + j);
+                  const float4* src = reinterpret_cast<const float4*>(ps + 64) + (c0 / 4) * 32 + lane;
+                  m[j] = __ldcg(ps + lane);
+                  ls[j] = __ldcg(ps + 32 + lane);
 #pragma unroll
-              for (int v = 0; v < 8; ++v) {
-                o[4 * v] += wgt[s] * x[v].x;
-                o[4 * v + 1] += wgt[s] * x[v].y;
-                o[4 * v + 2] += wgt[s] * x[v].z;
-                o[4 * v + 3] += wgt[s] * x[v].w;
+                  for (int v = 0; v < 8; ++v) x[j][v] = __ldcg(src + v * 32);
+                }
+              }
+              const float M_new = fmaxf(fmaxf(M, m[0]), fmaxf(m[1], m[2]));
+              const float old = M == -INFINITY ? 0.f : ex2(M - M_new);
+              M = M_new;
+              L *= old;
+#pragma unroll
+              for (int e = 0; e < 32; ++e) o[e] *= old;
+#pragma unroll
+              for (int j = 0; j < 3; ++j) {
+                const float wgt = m[j] == -INFINITY ? 0.f : ex2(m[j] - M);
+                L += wgt * ls[j];
+#pragma unroll
+                for (int v = 0; v < 8; ++v) {
+                  o[4 * v] += wgt * x[j][v].x;
+                  o[4 * v + 1] += wgt * x[j][v].y;
+                  o[4 * v + 2] += wgt * x[j][v].z;
+                  o[4 * v + 3] += wgt * x[j][v].w;
+                }
               }
             }
-            if (row_ok) store32(o, inv, out_row + c0 / 8);
+            if (row_ok) store32(o, 1.f / L, out_row + c0 / 8);
           }
         }
       }
+     }
     }
   }
 

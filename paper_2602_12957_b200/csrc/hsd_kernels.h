@@ -160,24 +160,24 @@ void launch_unpack_best(cudaStream_t st, const unsigned long long* row_best, int
                         bool pdl);
 
 // ---- attention plan (hsd_attn_sm100.cu): made once per step on the device, read by every layer's launch ----
-constexpr int kAttnMaxSplits = 8;      // most KV slices one q-tile is cut into
+constexpr int kAttnMaxShares = 1024;   // most shares the work of a kv head is cut into
 struct AttnPlan {
-  int4* items;      // two int4 per (q-tile, slice) item, longest first: {first packed row, position of the first
-                    // token, tokens, KV slot}, {first | (last + 1) << 16 KV block, slice | slices << 8 | first token of the q-tile within its sequence << 16,
-                    // q-tile, KV blocks}
-  int4* items_unsorted;   // the same list in creation order (scratch of the plan kernel)
-  int* n_items;
+  int4* items;      // two int4 per (q-tile, slice) item, share after share: {first packed row, position of the first token,
+                    // tokens, KV slot}, {first | (last + 1) << 16 KV block, slice | slices << 8 | first token of the q-tile
+                    // within its sequence << 16, slot of the q-tile's slice 0, plan form: see slice_slot}
+  int* share_start; // [shares + 1] first item of every share
+  int* n_shares;
   int* tile_seq;    // [max_tiles] sequence of a q-tile
-  int* tile_nkv;    // [max_tiles] KV blocks it can see
-  int* counters;    // [max_tiles, n_kv_heads, 4] slices that have delivered their partial of a 32-row quarter
+  int* tile_pos;    // [max_tiles] where it begins on the line the shares are cut from
+  int* counters;    // [2 shares, n_kv_heads, 4] slices that have delivered their partial of a 32-row quarter
   int4* first;      // [grid CTAs][3]: the item a CTA of the attention grid starts with, ready to use: the item's two
-                    // words, then {item x kv head index (-1: none), kv head, first two physical KV blocks}
+                    // words, then {first item of its share, items of its share, first two physical KV blocks}
   int n_kv_heads;
   int grid;         // CTAs of the attention launches this plan is made for
 };
 void launch_attn_plan(cudaStream_t st, const RowMeta& rm, const AttnPlan& pl, const KvView& kv, int n_seqs,
-                      int tokens_per_tile, int target_items, int min_chunk, const int* tile_count, const int* status,
-                      bool pdl);
+                      int tokens_per_tile, int max_shares, int min_chunk, int max_slices, bool no_cut, const int* tile_count,
+                      const int* status, bool pdl);
 int launch_attn_sm100(cudaStream_t st, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                       const AttnPlan& plan, const KvView& kv, const ModelDims& md, int layer, bf16* out, int n_sms,
                       int device, int* status, float* split_ws, const uint4* anc, bool pdl);
