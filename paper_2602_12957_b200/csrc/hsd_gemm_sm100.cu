@@ -3,13 +3,14 @@
 //
 // One persistent CTA per SM walks work units (128 x BN output tile, optionally one slice of K), M fastest so
 // CTAs running side by side share a weight tile through L2.  Warp roles:
-//   warp 0      A producer (one lane): activation tile, one 128-row TMA box per stage
-//   warp 1      MMA issuer (one lane) and TMEM owner
-//   warps 2, 3  B producers (one lane each): the two halves of the weight tile, one TMA box each per stage.
-//               A TMA instruction costs its issuing thread ~0.25 us whatever the box size, so a stage is three
-//               large boxes issued from three warps instead of many small ones from one.  Weights do not depend
-//               on the previous kernel, so these two start before the programmatic-launch wait.
-//   warps 4..7  epilogue, one TMEM lane quarter each
+//   warp 0      A producer: activation tile, one 128-row TMA box per stage
+//   warp 1      MMA issuer and TMEM owner
+//   warp 2      B producer: the two halves of the weight tile, one TMA box each per stage (a pair's CTA: its half).
+//               Weights do not depend on the previous kernel, so it starts before the programmatic-launch wait.
+//   warps 4..7  epilogue, one TMEM lane quarter each (warp w works on lane quarter w mod 4, the hardware's rule)
+// Warps 0 to 2 run their loops as whole warps and elect a lane for what one thread issues: with warp-uniform control
+// flow the coordinates, descriptors and barrier addresses live in uniform registers, where TMA and MMA instructions want
+// them.  (Run by one lane under a divergent branch, a TMA instruction cost ~0.25 us and an MMA ~90 cycles to issue.)
 // Two accumulator buffers in TMEM let the epilogue of unit i overlap the main loop of unit i+1.
 //
 // Epilogues (all fused; results leave the SM through swizzled staging buffers and TMA stores, so global
@@ -184,8 +185,8 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) {
-      // A producer + two B producers, each with its own byte count; a pair: one arrival (even CTA) for all bytes
-      mbar_init(full + s, PAIR ? 1 : 3);
+      // A producer and B producer, each with its own byte count; a pair: one arrival (even CTA) for all bytes
+      mbar_init(full + s, PAIR ? 1 : 2);
       mbar_init(empty + s, 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -219,72 +220,69 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const int total = tiles * p.splits;
   const int k_blocks = p.K / BK;
 
-  // Producer warps: lanes 0 and 1 each take every other stage (kc counts k-blocks over all units of this CTA;
-  // the stage count is even, so a lane always sees the same stages).  One thread cannot issue TMA instructions
-  // faster than about one per 0.25 us, and a barrier round trip adds to that; two lanes per operand keep the
-  // issue interval below the 128 x 256 MMA time of a k-block.
+  // kc counts k-blocks over all units of this CTA: stage = kc % STAGES, the barriers' parities follow
   if (warp == 0) {
     // ---- A producer: activations, written by the previous kernel
-    if (lane < 2) {
-      pdl_wait();
-      if (lane == 0) pdl_launch_dependents();
-      int kc = 0;
-      for (int t = cta; t < total; t += n_cta) {
-        const int tile = t % tiles, split = t / tiles;
-        const int m0 = (tile % m_tiles) * TILE_M + rank * BM;
-        const int kb0 = split * p.kb_per_split, kb1 = min(k_blocks, kb0 + p.kb_per_split);
-        for (int kb = kb0; kb < kb1; ++kb, ++kc) {
-          if ((kc & 1) != lane) continue;
-          const int s = kc % C::STAGES;
-          const uint32_t ph = (kc / C::STAGES) & 1;
-          if (!mbar_wait(empty + s, ph ^ 1u, abort_flag, p.status, 100)) goto done;
+    pdl_wait();
+    pdl_launch_dependents();
+    int s = 0;
+    uint32_t ph = 1;
+    for (int t = cta; t < total; t += n_cta) {
+      const int tile = t % tiles, split = t / tiles;
+      const int m0 = (tile % m_tiles) * TILE_M + rank * BM;
+      const int kb0 = split * p.kb_per_split, kb1 = min(k_blocks, kb0 + p.kb_per_split);
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait(empty + s, ph, abort_flag, p.status, 100)) goto done;
+        if (elect_one()) {
+          uint8_t* dst = smem + s * C::STAGE_BYTES;
           if (PAIR) {
             if (rank == 0) mbar_expect_tx(full + s, 2 * C::STAGE_BYTES);   // A and B of both CTAs land on this barrier
 #pragma unroll
-            for (int u = 0; u < KSTEPS; ++u)
-              tma_load_2d_pair(smem + s * C::STAGE_BYTES + u * A_SUB, &tmA, full + s, kb * BK + u * KSUB, m0);
+            for (int u = 0; u < KSTEPS; ++u) tma_load_2d_pair(dst + u * A_SUB, &tmA, full + s, kb * BK + u * KSUB, m0);
           } else {
             mbar_expect_tx(full + s, A_BYTES);
 #pragma unroll
-            for (int u = 0; u < KSTEPS; ++u)
-              tma_load_2d(smem + s * C::STAGE_BYTES + u * A_SUB, &tmA, full + s, kb * BK + u * KSUB, m0);
+            for (int u = 0; u < KSTEPS; ++u) tma_load_2d(dst + u * A_SUB, &tmA, full + s, kb * BK + u * KSUB, m0);
           }
         }
+        __syncwarp();
+        if (++s == C::STAGES) { s = 0; ph ^= 1u; }
       }
     }
-  } else if (warp == 2 || warp == 3) {
-    // ---- B producers: one half of the weight tile each (for SwiGLU: gate rows / up rows)
-    if (lane < 2 && !(PAIR && warp == 3)) {
-      // a pair: this CTA stages half `rank` of the tile in one box; alone: warps 2 and 3 stage one half each
-      const int half = PAIR ? rank : warp - 2;
-      int kc = 0;
-      for (int t = cta; t < total; t += n_cta) {
-        const int tile = t % tiles, split = t / tiles;
-        const int n0 = (tile / m_tiles) * OUT_N;
-        const int kb0 = split * p.kb_per_split, kb1 = min(k_blocks, kb0 + p.kb_per_split);
-        const int row = (MODE == GS_SWIGLU) ? (half ? p.n_up_off + n0 : n0) : n0 + half * (BN / 2);
-        for (int kb = kb0; kb < kb1; ++kb, ++kc) {
-          if ((kc & 1) != lane) continue;
-          const int s = kc % C::STAGES;
-          const uint32_t ph = (kc / C::STAGES) & 1;
-          if (!mbar_wait(empty + s, ph ^ 1u, abort_flag, p.status, 110 + half)) goto done;
+  } else if (warp == 2) {
+    // ---- B producer: both halves of the weight tile (for SwiGLU: gate rows / up rows); a pair's CTA stages half `rank`
+    int s = 0;
+    uint32_t ph = 1;
+    for (int t = cta; t < total; t += n_cta) {
+      const int tile = t % tiles, split = t / tiles;
+      const int n0 = (tile / m_tiles) * OUT_N;
+      const int kb0 = split * p.kb_per_split, kb1 = min(k_blocks, kb0 + p.kb_per_split);
+      const int row0 = n0, row1 = (MODE == GS_SWIGLU) ? p.n_up_off + n0 : n0 + BN / 2;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait(empty + s, ph, abort_flag, p.status, 110)) goto done;
+        if (elect_one()) {
+          uint8_t* dst = smem + s * C::STAGE_BYTES + A_BYTES;
           if (PAIR) {
 #pragma unroll
             for (int u = 0; u < KSTEPS; ++u)
-              tma_load_2d_pair(smem + s * C::STAGE_BYTES + A_BYTES + u * C::B_SUB, &tmB, full + s, kb * BK + u * KSUB, row);
+              tma_load_2d_pair(dst + u * C::B_SUB, &tmB, full + s, kb * BK + u * KSUB, rank ? row1 : row0);
           } else {
-            mbar_expect_tx(full + s, HALF_B * KSTEPS);
+            mbar_expect_tx(full + s, C::B_BYTES);
 #pragma unroll
-            for (int u = 0; u < KSTEPS; ++u)
-              tma_load_2d(smem + s * C::STAGE_BYTES + A_BYTES + u * C::B_SUB + half * HALF_B, &tmB, full + s,
-                          kb * BK + u * KSUB, row);
+            for (int u = 0; u < KSTEPS; ++u) {
+              tma_load_2d(dst + u * C::B_SUB, &tmB, full + s, kb * BK + u * KSUB, row0);
+              tma_load_2d(dst + u * C::B_SUB + HALF_B, &tmB, full + s, kb * BK + u * KSUB, row1);
+            }
           }
         }
+        __syncwarp();
+        if (++s == C::STAGES) { s = 0; ph ^= 1u; }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       constexpr uint32_t idesc = umma_idesc_bf16(BN, false, TILE_M);
+      const uint64_t desc0 = umma_desc_sw128(smem_u32(smem));      // a byte offset adds a sixteenth of itself
       int s = 0;
       uint32_t ph = 0;
       int it = 0;
@@ -299,26 +297,29 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(full + s, ph, abort_flag, p.status, 201)) goto done;
           tc_fence_after();
-          const uint32_t sa = smem_u32(smem + s * C::STAGE_BYTES);
-          const uint32_t sb = sa + A_BYTES;
+          const uint64_t da = desc0 + s * (C::STAGE_BYTES / 16), db = da + A_BYTES / 16;
+          if (elect_one()) {
 #pragma unroll
-          for (int u = 0; u < KSTEPS; ++u) {
+            for (int u = 0; u < KSTEPS; ++u) {
 #pragma unroll
-            for (int k = 0; k < KSUB / 16; ++k) {
-              const uint32_t acc = (kb != kb0 || u != 0 || k != 0) ? 1u : 0u;
-              const uint64_t da = umma_desc_sw128(sa + u * A_SUB + k * 32), db = umma_desc_sw128(sb + u * C::B_SUB + k * 32);
-              if (PAIR) umma_bf16_pair(d_tmem, da, db, idesc, acc);
-              else umma_bf16(d_tmem, da, db, idesc, acc);
+              for (int k = 0; k < KSUB / 16; ++k) {
+                const uint32_t acc = (kb != kb0 || u != 0 || k != 0) ? 1u : 0u;
+                if (PAIR) umma_bf16_pair(d_tmem, da + (u * A_SUB + k * 32) / 16, db + (u * C::B_SUB + k * 32) / 16, idesc, acc);
+                else umma_bf16(d_tmem, da + (u * A_SUB + k * 32) / 16, db + (u * C::B_SUB + k * 32) / 16, idesc, acc);
+              }
+            }
+            // smem stage reusable once these MMAs have read it (in both CTAs of a pair)
+            if (PAIR) umma_commit_pair(empty + s); else umma_commit(empty + s);
+            if (kb + 1 == kb1) {                                   // accumulator complete
+              if (PAIR) umma_commit_pair(tfull + b); else umma_commit(tfull + b);
             }
           }
-          // smem stage reusable once these MMAs have read it (in both CTAs of a pair)
-          if (PAIR) umma_commit_pair(empty + s); else umma_commit(empty + s);
+          __syncwarp();
           if (++s == C::STAGES) { s = 0; ph ^= 1u; }
         }
-        if (PAIR) umma_commit_pair(tfull + b); else umma_commit(tfull + b);   // accumulator complete
       }
     }
-  } else {
+  } else if (warp >= 4) {
     // ---- epilogue warps 4..7
     const int quarter = warp & 3;                 // TMEM lanes [32*quarter, +32) belong to this warp
     const int row_in_tile = quarter * 32 + lane;
