@@ -294,8 +294,9 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
                      c->attn_min_chunk, kAttnMaxSlices, c->max_splits == 1, w.status + 4, w.status, c->pdl);
   }
   if (!c->simt) {
-    if (make_tmap_2d(&tm_h, w.h, T, md.d, 128) || make_tmap_2d(&tm_attn, w.attn, T, md.Hq * md.D, 128) ||
-        make_tmap_2d(&tm_act, w.act, T, md.ffn, 128))
+    const uint32_t box = gemm_a_box_rows(T);
+    if (make_tmap_2d(&tm_h, w.h, T, md.d, box) || make_tmap_2d(&tm_attn, w.attn, T, md.Hq * md.D, box) ||
+        make_tmap_2d(&tm_act, w.act, T, md.ffn, box))
       return HSD_ERR_CUDA;
     // epilogue targets: residual stream (fp32 reduce-add), q and the SwiGLU activation (bf16 stores)
     if (make_tmap_2d_f32(&tm_x_add, w.x, T, md.d, 32) || make_tmap_2d(&tm_q_st, w.q, T, md.Hq * md.D, 32) ||
@@ -438,7 +439,7 @@ int run_lm_head(hsd_ctx* c, const Ws& w, int rows, const int* row_next, cudaStre
     launch_gemm_simt(st, w.h, c->lm_head, rows, md.V, md.d, GM_ARGMAX, o);
   } else {
     CUtensorMap tm_h;
-    if (make_tmap_2d(&tm_h, w.h, rows, md.d, 128)) return HSD_ERR_CUDA;
+    if (make_tmap_2d(&tm_h, w.h, rows, md.d, gemm_a_box_rows(rows))) return HSD_ERR_CUDA;
     GemmSm100Args g = {};
     g.tmA = tm_h;
     g.tmB = &c->tm_lm_head;
@@ -1078,7 +1079,7 @@ static int lm_head_argmax_impl(hsd_ctx* c, const void* h, int rows, const int* n
       launch_gemm_simt(st, static_cast<const bf16*>(h), c->lm_head, rows, md.V, md.d, GM_ARGMAX, o);
     } else {
       GemmSm100Args g = {};
-      if (make_tmap_2d(&g.tmA, h, rows, md.d, 128)) return HSD_ERR_CUDA;
+      if (make_tmap_2d(&g.tmA, h, rows, md.d, gemm_a_box_rows(rows))) return HSD_ERR_CUDA;
       g.tmB = &c->tm_lm_head;
       g.M = rows; g.n_out = md.V; g.K = md.d; g.mode = GS_ARGMAX;
       g.out = o;
@@ -1158,7 +1159,7 @@ int hsd_op_linear(hsd_ctx* c, const void* A, const void* W, void* C, int M, int 
   }
   GemmSm100Args g = {};
   WeightMaps wm;
-  if (make_tmap_2d(&g.tmA, A, M, K, 128) || make_weight_tmaps(&wm, W, n_out, K)) return HSD_ERR_CUDA;
+  if (make_tmap_2d(&g.tmA, A, M, K, gemm_a_box_rows(M)) || make_weight_tmaps(&wm, W, n_out, K)) return HSD_ERR_CUDA;
   if (mode == 1 ? make_tmap_2d_f32(&g.tmC, C, M, ldc, 32) : make_tmap_2d(&g.tmC, C, M, ldc, 32)) return HSD_ERR_CUDA;
   g.tmB = &wm;
   g.M = M; g.n_out = n_out; g.K = K; g.mode = mode;

@@ -123,6 +123,7 @@ struct Cfg {
 struct GemmDev {
   int M, n_cols, K, n_up_off;   // n_cols: output columns; n_up_off: row offset of the `up` half (SwiGLU)
   int splits, kb_per_split;     // K slices per tile (GS_ADD_F32 only) and k-blocks per slice
+  int a_box;                    // rows of an activation box (< 128 only where M is no more than that)
   GemmOut out;
   QkvEpilogue qkv;
   int* status;
@@ -240,7 +241,7 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 #pragma unroll
             for (int u = 0; u < KSTEPS; ++u) tma_load_2d_pair(dst + u * A_SUB, &tmA, full + s, kb * BK + u * KSUB, m0);
           } else {
-            mbar_expect_tx(full + s, A_BYTES);
+            mbar_expect_tx(full + s, p.a_box * (KSUB * 2) * KSTEPS);
 #pragma unroll
             for (int u = 0; u < KSTEPS; ++u) tma_load_2d(dst + u * A_SUB, &tmA, full + s, kb * BK + u * KSUB, m0);
           }
@@ -673,6 +674,7 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
   const int k_blocks = a.K / BK;
   p.splits = splits;
   p.kb_per_split = (k_blocks + splits - 1) / splits;
+  p.a_box = (int)gemm_a_box_rows(a.M);
   p.out = a.out;
   p.qkv = a.qkv;
   p.status = a.status;
@@ -706,12 +708,13 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
   return cudaLaunchKernelEx(&cfg, gemm_sm100_kernel<BN, MODE, PAIR>, a.tmA, tmB, a.tmC, p) == cudaSuccess ? 0 : -1;
 }
 
-// Tile width, CTA pairing and K slices: fewest cycles by a model calibrated on B200 (cycles per k-block of one work
-// unit, measured in steady state with every SM busy: 128 x 256 tile ~820, 128 x 128 ~700, 128 x 64 ~600, CTA pair on
-// 256 x 256 ~770 per CTA for twice the rows).  The 256-wide shapes run at the rate the whole chip's tensor pipes
-// sustain (the measured library peak corresponds to ~730 cycles for such a k-block; one SM alone would need 544); the
-// narrower ones are bound by L2 -> SM bytes.  A pair costs a cluster launch; the epilogue of the last unit of a CTA is
-// exposed.
+// Tile width, CTA pairing and K slices: fewest cycles by a model calibrated on B200.  A k-block costs the longer of its
+// MMAs (256-wide tiles run at the rate the whole chip's tensor pipes sustain: the measured library peak corresponds to
+// ~730 cycles for such a k-block, one SM alone would need 544), its fill (A box + weight tile at the ~55 B per clock an SM
+// takes from L2: measured 455 cycles for 16 + 8 KB, 560 for 16 + 16 KB) and ~250 of barrier round trip and issue.
+// Calls of at most 64 rows load activation boxes of 16, 32 or 64 rows: the rest of the MMA's 128 rows is whatever the
+// stage held (rows are independent, and rows beyond M go nowhere), where a full box would fill them with zeros at the
+// same cost as data.  A pair costs a cluster launch; the epilogue of the last unit of a CTA is exposed.
 static void pick_tile(int mode, int n_cols, int M, int K, int n_sms, int max_splits, bool allow_pair, int* bn_out,
                       int* splits_out, bool* pair_out) {
   const int k_blocks = K / BK;
@@ -720,7 +723,7 @@ static void pick_tile(int mode, int n_cols, int M, int K, int n_sms, int max_spl
   *bn_out = (mode == GS_SWIGLU || mode == GS_QKV_ROPE128) ? 128 : 64;
   *splits_out = 1;
   *pair_out = false;
-  for (int i = allow_pair ? 0 : 1; i < 4; ++i) {
+  for (int i = allow_pair && M > 64 ? 0 : 1; i < 4; ++i) {       // (a pair's tile needs whole boxes)
     const bool pair = i == 0;
     const int bn = cands[i];
     const int out_n = (mode == GS_SWIGLU) ? bn / 2 : bn;
@@ -734,7 +737,8 @@ static void pick_tile(int mode, int n_cols, int M, int K, int n_sms, int max_spl
       if (sp > 1 && (kbs < 4 || (long long)(sp - 1) * kbs >= k_blocks)) continue;
       const long long units = tiles * sp;
       const long long rounds = (units + walkers - 1) / walkers;
-      const double per_kb = pair ? 770.0 : (bn == 256 ? 820.0 : (bn == 128 ? 700.0 : 600.0));
+      const double fill = (double)(gemm_a_box_rows(M) + (pair ? bn / 2 : bn)) * (KSUB * 2) / 55.0;
+      const double per_kb = pair ? 770.0 : (fill > 250.0 ? fill : 250.0);
       const double epi = 700.0 + 10.0 * bn;
       const double cost = (double)rounds * (kbs * per_kb + 300.0) + epi + (sp > 1 ? 200.0 * sp : 0.0) + (pair ? 1500.0 : 0.0);
       if (cost < best_cost) { best_cost = cost; *bn_out = bn; *splits_out = sp; *pair_out = pair; }
@@ -755,7 +759,7 @@ static int launch_mode(cudaStream_t st, const GemmSm100Args& a) {
     if ((fbn != 64 && fbn != 128 && fbn != 256) || out_n % 64 || n_cols % out_n) return -1;
     if (MODE == GS_QKV_ROPE128 && fbn < 128) return -1;
     bn = fbn;
-    pair = a.force_bn == 512;
+    pair = a.force_bn == 512 && a.M > 64;
   }
   if (a.force_splits) {
     const int kbs = (a.K / BK + a.force_splits - 1) / a.force_splits;

@@ -220,8 +220,11 @@ struct QkvEpilogue {      // fused RoPE + paged KV write (QKV projection)
   const bf16* k_norm;
   float eps;
 };
+// Rows of the activation boxes a GEMM over M rows loads (the box height of GemmSm100Args::tmA): a call of few rows does
+// not fill the rest of its 128-row tile (see hsd_gemm_sm100.cu).
+inline uint32_t gemm_a_box_rows(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : 128; }
 struct GemmSm100Args {
-  CUtensorMap tmA;             // activations, box {64, 128}
+  CUtensorMap tmA;             // activations, box {64, gemm_a_box_rows(M)}
   const WeightMaps* tmB;       // weights
   CUtensorMap tmC;             // output through TMA: bf16 box {64, 32} (store) or fp32 box {32, 32} (reduce-add);
                                // the q buffer for GS_QKV_ROPE; unused for GS_ARGMAX
