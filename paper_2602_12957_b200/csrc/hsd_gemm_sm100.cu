@@ -87,35 +87,26 @@ int make_weight_tmaps(WeightMaps* w, const void* base, uint64_t rows, uint64_t c
 }
 
 // ------------------------------------------------------------------------------------------------
-// K extent of a pipeline stage in 64-column sub-tiles.  Two (one barrier round trip per eight MMAs instead of four)
-// measured the same cycles per k-block as one: with 256-wide tiles the main loop runs at the tensor pipes' rate.
-#ifndef HSD_GEMM_KSTEPS
-#define HSD_GEMM_KSTEPS 1
-#endif
 constexpr int BM = 128;
 constexpr int KSUB = 64;                         // one 128-byte-swizzled sub-tile spans 64 bf16 of K
-constexpr int KSTEPS = HSD_GEMM_KSTEPS;          // sub-tiles per pipeline stage
-constexpr int BK = KSUB * KSTEPS;                // K extent of one stage (one barrier round trip)
 constexpr int A_SUB = BM * KSUB * 2;             // bytes of one A sub-tile
-constexpr int A_BYTES = A_SUB * KSTEPS;
 constexpr int kGemmThreads = 256;
 constexpr int STG_BYTES = 4096;                  // one epilogue staging buffer: 32 rows x 128 bytes
 constexpr int STG_TOTAL = 4 * 2 * STG_BYTES;     // four epilogue warps, two buffers each
 
 // PAIR: two CTAs (a cluster) share one 256 x BN tile: each stages its own 128 rows of A and BN/2 rows of B.
-#ifndef HSD_GEMM_STAGES_PAIR
-#define HSD_GEMM_STAGES_PAIR (6 / KSTEPS)
-#define HSD_GEMM_STAGES_256 (4 / KSTEPS)
-#define HSD_GEMM_STAGES_128 (6 / KSTEPS)
-#define HSD_GEMM_STAGES_64 (8 / KSTEPS)
-#endif
+// KSTEPS: sub-tiles of a stage.  A stage is one barrier round trip of ~250 cycles.  The MMAs or the fill of the 128- and
+// 256-wide tiles' stages cover it (two sub-tiles: 256 wide the same, 128 wide 1 % slower steps, fewer stages being in
+// flight), those of the 64-wide tile do not: plain decode 0.965 -> 0.947 ms, short drafts 1.059 -> 1.046 with two.
 template <int BN, bool PAIR = false>
 struct Cfg {
+  static constexpr int KSTEPS = BN == 64 ? 2 : 1;
+  static constexpr int BK = KSUB * KSTEPS;                          // K extent of one stage
+  static constexpr int A_BYTES = A_SUB * KSTEPS;
   static constexpr int B_SUB = (PAIR ? BN / 2 : BN) * KSUB * 2;     // bytes of one B sub-tile this CTA stages
   static constexpr int B_BYTES = B_SUB * KSTEPS;                    // bytes of B per stage
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = PAIR ? HSD_GEMM_STAGES_PAIR
-                                     : ((BN == 256) ? HSD_GEMM_STAGES_256 : (BN == 128 ? HSD_GEMM_STAGES_128 : HSD_GEMM_STAGES_64));
+  static constexpr int STAGES = (PAIR ? 6 : BN == 256 ? 4 : BN == 128 ? 6 : 8) / KSTEPS;
   static constexpr int TMEM_COLS = 2 * BN;
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + STG_TOTAL + 1024 /*alignment slack*/ + 256 /*barriers*/;
 };
@@ -166,6 +157,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const __grid_constant__ CUtensorMap tmC, GemmDev p) {
   using C = Cfg<BN, PAIR>;
+  constexpr int KSTEPS = C::KSTEPS, BK = C::BK, A_BYTES = C::A_BYTES;
   constexpr int OUT_N = (MODE == GS_SWIGLU) ? BN / 2 : BN;   // output columns per tile
   constexpr int HALF_B = BN / 2 * KSUB * 2;                  // bytes of one weight half-tile of one sub-tile
   constexpr int TILE_M = PAIR ? 2 * BM : BM;                 // rows of one work unit (both CTAs of a pair)
@@ -219,7 +211,7 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const int n_tiles = p.n_cols / OUT_N;
   const int tiles = m_tiles * n_tiles;
   const int total = tiles * p.splits;
-  const int k_blocks = p.K / BK;
+  const int k_blocks = (p.K + BK - 1) / BK;      // (a last stage beyond K is filled with zeros)
 
   // kc counts k-blocks over all units of this CTA: stage = kc % STAGES, the barriers' parities follow
   if (warp == 0) {
@@ -671,7 +663,8 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
   p.K = a.K;
   p.n_cols = (MODE == GS_SWIGLU) ? a.n_out / 2 : a.n_out;
   p.n_up_off = a.n_out / 2;
-  const int k_blocks = a.K / BK;
+  const int k_blocks = (a.K + C::BK - 1) / C::BK;
+  while (splits > 1 && (splits - 1) * ((k_blocks + splits - 1) / splits) >= k_blocks) --splits;    // no slice is empty
   p.splits = splits;
   p.kb_per_split = (k_blocks + splits - 1) / splits;
   p.a_box = (int)gemm_a_box_rows(a.M);
@@ -717,7 +710,7 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
 // same cost as data.  A pair costs a cluster launch; the epilogue of the last unit of a CTA is exposed.
 static void pick_tile(int mode, int n_cols, int M, int K, int n_sms, int max_splits, bool allow_pair, int* bn_out,
                       int* splits_out, bool* pair_out) {
-  const int k_blocks = K / BK;
+  const int k_blocks = K / KSUB;
   const int cands[4] = {256, 256, 128, 64};     // first entry: a CTA pair on a 256 x 256 tile
   double best_cost = 1e30;
   *bn_out = (mode == GS_SWIGLU || mode == GS_QKV_ROPE128) ? 128 : 64;
@@ -762,8 +755,8 @@ static int launch_mode(cudaStream_t st, const GemmSm100Args& a) {
     pair = a.force_bn == 512 && a.M > 64;
   }
   if (a.force_splits) {
-    const int kbs = (a.K / BK + a.force_splits - 1) / a.force_splits;
-    if (MODE != GS_ADD_F32 || (a.force_splits - 1) * kbs >= a.K / BK) return -1;
+    const int kbs = (a.K / KSUB + a.force_splits - 1) / a.force_splits;
+    if (MODE != GS_ADD_F32 || (a.force_splits - 1) * kbs >= a.K / KSUB) return -1;
     splits = a.force_splits;
   }
   if (pair) return launch_one<256, MODE, true>(st, a, splits);
@@ -778,7 +771,7 @@ static int launch_mode(cudaStream_t st, const GemmSm100Args& a) {
 
 int launch_gemm_sm100(cudaStream_t st, const GemmSm100Args& a) {
   if (a.M <= 0) return 0;
-  if (a.K % BK || a.n_out % 64 || !a.tmB) return -1;
+  if (a.K % KSUB || a.n_out % 64 || !a.tmB) return -1;
   switch (a.mode) {
     case GS_STORE_BF16: return launch_mode<GS_STORE_BF16>(st, a);
     case GS_ADD_F32: return launch_mode<GS_ADD_F32>(st, a);
