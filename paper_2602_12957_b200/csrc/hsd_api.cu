@@ -72,7 +72,7 @@ struct Ws {
   AttnPlan plan;
   RowMeta rm;
   int* sel_rows;
-  int* cu_one;        // {0, n} offsets of a single-sequence call
+  int2* verdict;      // what every set-up CTA found
   int *h_tokens, *h_cu, *h_accept, *h_nemit, *h_emit;   // device staging of hsd_verify_regions_host
   size_t h_emit_ints;
   float* x;
@@ -132,7 +132,7 @@ Ws carve(const hsd_ctx* c, void* base, int T, int S) {
   w.rm.lm_src = static_cast<int*>(take(sizeof(int) * T));        // a tree call carves for 2 x its rows
   w.rm.lm_next = static_cast<int*>(take(sizeof(int) * T));
   w.sel_rows = static_cast<int*>(take(sizeof(int) * S));
-  w.cu_one = static_cast<int*>(take(sizeof(int) * 2));
+  w.verdict = static_cast<int2*>(take(sizeof(int2) * (size_t)setup_ctas(T)));
   w.h_tokens = static_cast<int*>(take(sizeof(int) * T));
   w.h_cu = static_cast<int*>(take(sizeof(int) * (S + 1)));
   w.h_accept = static_cast<int*>(take(sizeof(int) * S));
@@ -251,7 +251,6 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
   const int T = a.total_q;
   const int tokens_per_tile = 128 / md.group;
 
-  if (cudaMemsetAsync(w.status, 0, 64, st) != cudaSuccess) return check_cuda(c);
   // hsd_debug_tap: one armed tap is served by this forward, then disarmed
   const int tap_layer = c->tap_layer, tap_which = c->tap_which;
   c->tap_layer = -1;
@@ -279,19 +278,25 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
     sa.allow_embed_rows = a.prefill && a.embeds != nullptr;
     sa.rope_base = md.rope_base;
     sa.head_dim = md.D;
-    launch_setup_rows(st, sa, kv, w.rm, w.status, w.status + 4, c->pdl);
-  }
-  {
-    Scope s(c, st, KC_EMBED);
-    launch_embed(st, w.rm, c->embed, static_cast<const bf16*>(a.embeds), w.x, T, md.d, w.status, c->pdl);
+    sa.d = md.d;
+    sa.table = c->embed;
+    sa.embeds = static_cast<const bf16*>(a.embeds);
+    sa.x = w.x;
+    sa.row_best = w.row_best;
+    sa.zdraft = w.zdraft;
+    sa.verdict = w.verdict;
+    launch_setup_rows(st, sa, kv, w.rm, w.status + 4, c->pdl);
   }
 
   CUtensorMap tm_h, tm_attn, tm_act, tm_q, tm_k, tm_v, tm_x_add, tm_q_st, tm_act_st;
-  if (!c->attn_simt) {
+  if (c->attn_simt) {
+    Scope s(c, st, KC_SETUP);
+    launch_status(st, w.verdict, setup_ctas(T), w.status, c->pdl);
+  } else {
     Scope s(c, st, KC_SETUP);
     // (a context with a fixed summation order never cuts a KV range: where the cuts fall depends on the batch)
     launch_attn_plan(st, w.rm, w.plan, kv, a.n_seqs, tokens_per_tile, max(1, min(attn_max_shares(c), c->attn_target_items / md.Hkv)),
-                     c->attn_min_chunk, kAttnMaxSlices, c->max_splits == 1, w.status + 4, w.status, c->pdl);
+                     c->attn_min_chunk, kAttnMaxSlices, c->max_splits == 1, w.status + 4, w.verdict, setup_ctas(T), w.status, c->pdl);
   }
   if (!c->simt) {
     const uint32_t box = gemm_a_box_rows(T);
@@ -426,13 +431,9 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
   return check_cuda(c);
 }
 
-// Final norm + LM head + running argmax over `rows` rows of h (already selected / normalised into w.h).
+// LM head + running argmax over `rows` rows of h (already selected / normalised into w.h); the set-up kernel cleared them.
 int run_lm_head(hsd_ctx* c, const Ws& w, int rows, const int* row_next, cudaStream_t st) {
   const ModelDims& md = c->md;
-  {
-    Scope s(c, st, KC_LMHEAD);
-    launch_clear_best(st, w.row_best, w.zdraft, rows, c->pdl);
-  }
   Scope s(c, st, KC_LMHEAD);
   GemmOut o = {nullptr, 0, w.row_best, w.zdraft, row_next};
   if (c->simt) {
@@ -812,18 +813,6 @@ int hsd_kv_commit_tree(hsd_ctx* c, const hsd_kv* kv, int n_seqs, const int* seq_
   return check_cuda(c);
 }
 
-}  // extern "C"
-
-namespace {
-// cu_q = {0, n} of a single-sequence call.
-__global__ void page_cu_q_kernel(int* cu, int n) {
-  cu[0] = 0;
-  cu[1] = n;
-}
-}  // namespace
-
-extern "C" {
-
 int hsd_verify_page(hsd_ctx* c, const hsd_kv* kv, int seq_slot, const int* pending_token, const int* draft_chunk,
                     int chunk_len, float log_tau, int* accept_len, int* emit_tokens, int* n_emit, int* row_argmax,
                     float* row_zmax, float* row_zdraft, void* workspace, size_t ws_bytes, void* cuda_stream) {
@@ -838,15 +827,9 @@ int hsd_verify_page(hsd_ctx* c, const hsd_kv* kv, int seq_slot, const int* pendi
   rc = check_ws(c, workspace, ws_bytes, chunk_len + 1, 1);
   if (rc) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const Ws w = carve(c, workspace, chunk_len + 1, 1);
-  int* cu = w.cu_one;
-  {
-    Scope s(c, st, KC_SETUP);
-    page_cu_q_kernel<<<1, 1, 0, st>>>(cu, chunk_len + 1);
-  }
   StepArgs a = {};
   a.n_seqs = 1; a.total_q = chunk_len + 1; a.max_q_len = chunk_len + 1; a.prefill = false;
-  a.cu_q = cu; a.tokens = nullptr; a.pending = pending_token; a.draft = draft_chunk;
+  a.cu_q = nullptr; a.tokens = nullptr; a.pending = pending_token; a.draft = draft_chunk;
   a.seq_slots = nullptr; a.slot_base = seq_slot;
   return verify_common(c, kv, a, log_tau, accept_len, emit_tokens, n_emit, row_argmax, row_zmax, row_zdraft, workspace,
                        ws_bytes, st);

@@ -137,14 +137,14 @@ constexpr int kTileCost = 3, kMinPiece = 2, kLineGain = 8, kPlanThreads = 512;
 __global__ void __launch_bounds__(kPlanThreads) attn_plan_kernel(RowMeta rm, AttnPlan pl, KvView kv, int n_seqs,
                                                                  int tokens_per_tile, int max_shares, int min_chunk,
                                                                  int max_slices, int no_cut, const int* tile_count,
-                                                                 const int* status) {
+                                                                 const int2* verdict, int n_verdicts, int* status) {
   pdl_wait();
   pdl_launch_dependents();
   // one round: creation order of the items; line: cuts (q-tile, block) and how many of them lie inside q-tiles so far
   __shared__ int s_ct[kAttnMaxShares + 1], s_co[kAttnMaxShares + 1], s_rank[kAttnMaxShares + 1];
   __shared__ int s_warp[kPlanThreads / 32], s_longest, s_blocks, s_count, s_slice;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (*status) {
+  if (status_from_verdicts(verdict, n_verdicts, status)) {
     if (tid == 0) *pl.n_shares = 0;
     for (int b = tid; b < pl.grid; b += kPlanThreads) pl.first[3 * b + 2] = make_int4(0, 0, 0, 0);
     return;
@@ -334,9 +334,9 @@ __global__ void __launch_bounds__(kPlanThreads) attn_plan_kernel(RowMeta rm, Att
 
 void launch_attn_plan(cudaStream_t st, const RowMeta& rm, const AttnPlan& pl, const KvView& kv, int n_seqs,
                       int tokens_per_tile, int max_shares, int min_chunk, int max_slices, bool no_cut, const int* tile_count,
-                      const int* status, bool pdl) {
+                      const int2* verdict, int n_verdicts, int* status, bool pdl) {
   launch_kernel(attn_plan_kernel, dim3(1), dim3(kPlanThreads), 0, st, pdl, rm, pl, kv, n_seqs, tokens_per_tile, max_shares,
-                min_chunk, max_slices, no_cut ? 1 : 0, tile_count, status);
+                min_chunk, max_slices, no_cut ? 1 : 0, tile_count, verdict, n_verdicts, status);
 }
 
 // ------------------------------------------------------------------------------------------------

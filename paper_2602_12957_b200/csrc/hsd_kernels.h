@@ -51,9 +51,10 @@ enum KernelClass {
 const char* kernel_class_name(int kc);
 
 // ---- small kernels (hsd_small.cu) ---------------------------------------------------------------
+constexpr int kSetupRows = 16;   // packed rows a set-up CTA takes
 struct SetupArgs {
   int n_seqs, total_q, max_q_len, vocab, tokens_per_tile;
-  const int* cu_q;          // dev [S+1]
+  const int* cu_q;          // dev [S+1], or nullptr: one sequence of total_q rows
   const int* tokens;        // dev [T] or nullptr (page mode)
   const int* pending;       // dev [1] page mode: token of row 0
   const int* draft;         // dev [T-1] page mode: tokens of rows 1..
@@ -62,14 +63,19 @@ struct SetupArgs {
   int slot_base;            // slot of sequence 0 when seq_slots == nullptr
   int allow_embed_rows;     // prefill: token id < 0 means "use the embeds row"
   float rope_base;
-  int head_dim;
+  int head_dim, d;
+  const bf16* table;        // embedding table
+  const bf16* embeds;       // prefill: rows used where the token id is negative
+  float* x;                 // [T, d] residual stream
+  unsigned long long* row_best;   // [T] (trees: [2T]) cleared for the LM head
+  float* zdraft;            // likewise, NaN
+  int2* verdict;            // [setup_ctas(T)] {status code, offending index} of every CTA
 };
 // `pdl` (here and below): launch with programmatic stream serialization; these kernels wait for their
 // predecessor at their first instruction, so the flag only hides launch latency.
-void launch_setup_rows(cudaStream_t st, const SetupArgs& a, const KvView& kv, const RowMeta& rm, int* status,
-                       int* tile_count, bool pdl);
-void launch_embed(cudaStream_t st, const RowMeta& rm, const bf16* table, const bf16* embeds, float* x, int T, int d,
-                  const int* status, bool pdl);
+int setup_ctas(int total_q);
+void launch_setup_rows(cudaStream_t st, const SetupArgs& a, const KvView& kv, const RowMeta& rm, int* tile_count, bool pdl);
+void launch_status(cudaStream_t st, const int2* verdict, int n, int* status, bool pdl);
 // h[r] = bf16(rmsnorm(x[src]) * gain), src = sel_rows ? sel_rows[r] : r.  The gather form (sel_rows != nullptr) writes
 // nothing when *status is set or src is outside [0, src_rows): the index comes from an earlier kernel of the step.
 void launch_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
@@ -177,7 +183,7 @@ struct AttnPlan {
 };
 void launch_attn_plan(cudaStream_t st, const RowMeta& rm, const AttnPlan& pl, const KvView& kv, int n_seqs,
                       int tokens_per_tile, int max_shares, int min_chunk, int max_slices, bool no_cut, const int* tile_count,
-                      const int* status, bool pdl);
+                      const int2* verdict, int n_verdicts, int* status, bool pdl);
 int launch_attn_sm100(cudaStream_t st, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                       const AttnPlan& plan, const KvView& kv, const ModelDims& md, int layer, bf16* out, int n_sms,
                       int device, int* status, float* split_ws, const uint4* anc, bool pdl);

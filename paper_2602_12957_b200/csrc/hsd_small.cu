@@ -12,101 +12,109 @@ const char* kernel_class_name(int kc) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// Row metadata.  One CTA per sequence.  Validates what the host cannot see (device-resident lengths and
-// tables); any violation sets the status words, and every kernel that follows an indirection returns early.
-constexpr int kSetupRows = 64;   // rows of one sequence handled by one CTA
-__global__ void setup_rows_kernel(SetupArgs a, KvView kv, RowMeta rm, int* status, int* tile_count) {
-  pdl_wait();               // everything below reads or writes what earlier kernels of the step produced
+// Row metadata, embedding gather and the LM head's cleared rows: what a step needs before its first layer, in one launch.
+// A CTA takes kSetupRows packed rows whatever the sequences they belong to; one more CTA writes the per-sequence metadata.
+// Validates what the host cannot see (device-resident offsets, lengths and tables).  A CTA leaves its verdict {code, index}
+// in `verdict`, and the kernel that follows (attn_plan_kernel, or status_kernel where the plan is not made) turns the
+// verdicts into the status words: nothing has to be zeroed first.  Every kernel that follows an indirection returns early
+// on a violation.
+// (Separate launches for the status words, the metadata by sequence, the gather and the cleared rows, with the parent
+// walk through global memory, took 16 to 30 us of a step.)
+constexpr int kSetupThreads = 256, kSetupMaxCu = 1024;
+__device__ __forceinline__ int setup_cu(const SetupArgs& a, int s) { return a.cu_q ? a.cu_q[s] : (s ? a.total_q : 0); }
+
+__global__ void __launch_bounds__(kSetupThreads) setup_rows_kernel(SetupArgs a, KvView kv, RowMeta rm, int* tile_count) {
+  pdl_wait();               // everything below reads or writes what earlier kernels of the stream produced
   pdl_launch_dependents();
-  const int i = blockIdx.x;
-  const int tid = threadIdx.x;
-  __shared__ int s_red[32];
-  __shared__ int s_bad;
-  if (tid == 0) s_bad = 0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ int s_cu[kSetupMaxCu + 1];
+  __shared__ int s_code, s_where;
+  __shared__ int s_par[HSD_MAX_TREE_ROWS + kSetupRows];
+  __shared__ int s_tok[kSetupRows], s_depth[kSetupRows], s_len[kSetupRows];
+  __shared__ int s_warp[kSetupThreads / 32];
+  if (tid == 0) s_code = s_where = 0;
   __syncthreads();
-
-  // every CTA scans cu_q once: monotone + total, and the exclusive scan of q-tiles before sequence i
-  int my_tiles = 0, bad = 0;
-  for (int s = tid; s < a.n_seqs; s += blockDim.x) {
-    const int n = a.cu_q[s + 1] - a.cu_q[s];
-    if (n < 0) bad = 1;
-    if (n > a.max_q_len) bad = 2;
-    if (s < i && n > 0) my_tiles += (n + a.tokens_per_tile - 1) / a.tokens_per_tile;
+  auto fail = [&](int code, int where) {
+    if (atomicCAS(&s_code, 0, code) == 0) s_where = where;
+  };
+  // every CTA checks the offsets once, and keeps them where they fit
+  int bad = 0;
+  for (int s = tid; s < a.n_seqs; s += kSetupThreads) {
+    const int lo = setup_cu(a, s), n = setup_cu(a, s + 1) - lo;
+    if (n < 0) bad = DEV_CU_Q;
+    if (n > a.max_q_len && !bad) bad = DEV_TOO_LONG;
+    if (s < kSetupMaxCu) s_cu[s] = lo;
   }
-  if (tid == 0 && (a.cu_q[0] != 0 || a.cu_q[a.n_seqs] != a.total_q)) bad = 1;
-  for (int o = 16; o; o >>= 1) my_tiles += __shfl_xor_sync(0xffffffffu, my_tiles, o);
-  if ((tid & 31) == 0) s_red[tid >> 5] = my_tiles;
-  if (bad) atomicMax(&s_bad, bad);
+  if (tid == 0 && (setup_cu(a, 0) != 0 || setup_cu(a, a.n_seqs) != a.total_q)) bad = DEV_CU_Q;
+  if (bad) atomicMax(&s_code, bad == DEV_TOO_LONG ? 2 : 1);
   __syncthreads();
-  int tile0 = 0;
-  for (int w = 0; w < (blockDim.x >> 5); ++w) tile0 += s_red[w];
-  if (s_bad) {
-    if (tid == 0 && blockIdx.y == 0) dev_fail(status, s_bad == 2 ? DEV_TOO_LONG : DEV_CU_Q, i);
+  if (s_code) {
+    if (tid == 0) a.verdict[blockIdx.x] = make_int2(s_code == 2 ? DEV_TOO_LONG : DEV_CU_Q, 0);
     return;
   }
 
-  const int q0 = a.cu_q[i];
-  const int n = a.cu_q[i + 1] - q0;
-  const int slot = a.seq_slots ? a.seq_slots[i] : a.slot_base + i;
-  if (slot < 0 || slot >= kv.n_slots) {
-    if (tid == 0) dev_fail(status, DEV_KV_CAPACITY, i);
+  if (blockIdx.x == gridDim.x - 1) {        // the sequences, with the exclusive scan of their attention q-tiles
+    int base = 0;
+    for (int s0 = 0; s0 < a.n_seqs; s0 += kSetupThreads) {
+      const int s = s0 + tid;
+      int q0 = 0, n = 0, slot = 0, L = 0;
+      if (s < a.n_seqs) {
+        q0 = setup_cu(a, s);
+        n = setup_cu(a, s + 1) - q0;
+        slot = a.seq_slots ? a.seq_slots[s] : a.slot_base + s;
+        if (slot < 0 || slot >= kv.n_slots) {
+          fail(DEV_KV_CAPACITY, s);
+        } else {
+          L = kv.seq_lens[slot];
+          if (L < 0 || (long long)L + n > (long long)kv.max_blocks * HSD_KV_BLOCK) fail(DEV_KV_CAPACITY, s);
+        }
+      }
+      const int tiles = (n + a.tokens_per_tile - 1) / a.tokens_per_tile;
+      int incl = tiles;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      if (lane == 31) s_warp[warp] = incl;
+      __syncthreads();
+      int before = base, all = 0;
+      for (int w = 0; w < kSetupThreads / 32; ++w) {
+        if (w < warp) before += s_warp[w];
+        all += s_warp[w];
+      }
+      if (s < a.n_seqs) {
+        rm.seq_q0[s] = q0;
+        rm.seq_n[s] = n;
+        rm.seq_len[s] = L;
+        rm.seq_slot[s] = slot;
+        rm.seq_tile0[s] = before + incl - tiles;
+      }
+      base += all;
+      __syncthreads();
+    }
+    for (int r = a.total_q + tid; r < a.n_seqs; r += kSetupThreads) a.row_best[r] = 0ull;   // (LM-head rows of empty sequences)
+    if (tid == 0) {
+      rm.seq_tile0[a.n_seqs] = base;
+      *tile_count = base;
+      a.verdict[blockIdx.x] = make_int2(s_code, s_where);
+    }
     return;
   }
-  const int L = kv.seq_lens[slot];
-  if (L < 0 || (long long)L + n > (long long)kv.max_blocks * HSD_KV_BLOCK) {
-    if (tid == 0) dev_fail(status, DEV_KV_CAPACITY, i);
-    return;
-  }
-  if (tid == 0 && blockIdx.y == 0) {
-    rm.seq_q0[i] = q0;
-    rm.seq_n[i] = n;
-    rm.seq_len[i] = L;
-    rm.seq_slot[i] = slot;
-    rm.seq_tile0[i] = tile0;
-    if (i == a.n_seqs - 1) {
-      const int t = tile0 + (n + a.tokens_per_tile - 1) / a.tokens_per_tile;
-      rm.seq_tile0[a.n_seqs] = t;
-      *tile_count = t;
+
+  const int r0 = blockIdx.x * kSetupRows, n_rows = min(kSetupRows, a.total_q - r0);
+  const int par0 = max(0, r0 - HSD_MAX_TREE_ROWS);      // a row's ancestors lie among the 127 packed rows before it
+  if (a.parent)
+    for (int j = par0 + tid; j < r0 + n_rows; j += kSetupThreads) s_par[j - par0] = a.parent[j];
+  __syncthreads();
+  if (tid < n_rows) {
+    const int r = r0 + tid;
+    int lo = 0, hi = a.n_seqs;                          // the sequence of row r: the last that begins at or before it
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if ((mid < kSetupMaxCu ? s_cu[mid] : setup_cu(a, mid)) <= r) lo = mid; else hi = mid;
     }
-  }
-  const int j_lo = blockIdx.y * kSetupRows;
-  const int j_hi = min(n, j_lo + kSetupRows);
-  const int half = a.head_dim / 2;
-  // Candidate tree: a row's rotary position is its depth below the pending token, not its index in the call
-  // (Sec. 3.2: a node continues the path pi(v), whatever else is packed beside it).
-  __shared__ int s_depth[kSetupRows];
-  if (a.parent) {
-    for (int j = j_lo + tid; j < j_hi; j += blockDim.x) {
-      uint32_t m[4] = {0u, 0u, 0u, 0u};
-      int d = 0, pj = j;
-      bool ok = j < 128;
-      if (ok) m[j >> 5] |= 1u << (j & 31);
-      if (j > 0 && a.parent[q0 + j] == -2) pj = 0;      // padding row: no parent, no children, sees only itself
-      while (ok && pj > 0) {
-        const int pp = a.parent[q0 + pj];
-        if (pp < 0 || pp >= pj) { ok = false; break; }
-        pj = pp;
-        m[pj >> 5] |= 1u << (pj & 31);
-        ++d;
-      }
-      if (j == 0 && a.parent[q0] != -1) ok = false;
-      if (!ok) {
-        dev_fail(status, DEV_TREE, q0 + j);
-        d = 0;
-      }
-      s_depth[j - j_lo] = d;
-      const int r = q0 + j;
-      rm.anc[r] = make_uint4(m[0], m[1], m[2], m[3]);
-      rm.lm_src[r] = r;
-      rm.lm_next[r] = -1;
-      const bool child = ok && j > 0 && a.parent[r] >= 0;
-      rm.lm_src[a.total_q + r] = child ? q0 + a.parent[r] : r;
-      rm.lm_next[a.total_q + r] = child ? a.tokens[r] : -1;
-    }
-    __syncthreads();
-  }
-  for (int j = j_lo + tid; j < j_hi; j += blockDim.x) {
-    const int r = q0 + j;
+    const int i = lo, q0 = lo < kSetupMaxCu ? s_cu[lo] : setup_cu(a, lo);
+    const int j = r - q0, n = setup_cu(a, i + 1) - q0;
     int tok, nxt = -1;
     if (a.tokens) {
       tok = a.tokens[r];
@@ -115,63 +123,106 @@ __global__ void setup_rows_kernel(SetupArgs a, KvView kv, RowMeta rm, int* statu
       tok = (j == 0) ? a.pending[0] : a.draft[j - 1];
       if (j + 1 < n) nxt = a.draft[j];
     }
+    const int slot = a.seq_slots ? a.seq_slots[i] : a.slot_base + i;
+    int L = 0, phys = 0;
+    if (slot < 0 || slot >= kv.n_slots) {
+      fail(DEV_KV_CAPACITY, i);
+    } else {
+      L = kv.seq_lens[slot];
+      if (L < 0 || (long long)L + n > (long long)kv.max_blocks * HSD_KV_BLOCK) {
+        fail(DEV_KV_CAPACITY, i);
+        L = 0;
+      } else {
+        phys = kv.block_table[(size_t)slot * kv.max_blocks + (L + j) / HSD_KV_BLOCK];
+        if (phys < 0 || phys >= kv.n_blocks) {
+          fail(DEV_BLOCK_RANGE, r);
+          phys = 0;
+        }
+      }
+    }
     if (tok >= a.vocab || (tok < 0 && !a.allow_embed_rows)) {
-      dev_fail(status, DEV_TOKEN_RANGE, r);
+      fail(DEV_TOKEN_RANGE, r);
       tok = 0;
     }
     if (tok < 0) tok = -1;
-    const int pos = L + j;
-    int phys = kv.block_table[(size_t)slot * kv.max_blocks + pos / HSD_KV_BLOCK];
-    if (phys < 0 || phys >= kv.n_blocks) {
-      dev_fail(status, DEV_BLOCK_RANGE, r);
-      phys = 0;
+    // Candidate tree: a row's rotary position is its depth below the pending token, not its index in the call
+    // (Sec. 3.2: a node continues the path pi(v), whatever else is packed beside it).
+    int d = 0;
+    if (a.parent) {
+      uint32_t m[4] = {0u, 0u, 0u, 0u};
+      const int own = s_par[r - par0];
+      int pj = j;
+      bool ok = j < HSD_MAX_TREE_ROWS;
+      if (ok) m[j >> 5] |= 1u << (j & 31);
+      if (j > 0 && own == -2) pj = 0;                   // padding row: no parent, no children, sees only itself
+      while (ok && pj > 0) {
+        const int pp = s_par[q0 + pj - par0];
+        if (pp < 0 || pp >= pj) { ok = false; break; }
+        pj = pp;
+        m[pj >> 5] |= 1u << (pj & 31);
+        ++d;
+      }
+      if (j == 0 && own != -1) ok = false;
+      if (!ok) {
+        fail(DEV_TREE, r);
+        d = 0;
+      }
+      rm.anc[r] = make_uint4(m[0], m[1], m[2], m[3]);
+      const bool child = ok && j > 0 && own >= 0;
+      rm.lm_src[r] = r;
+      rm.lm_next[r] = -1;
+      rm.lm_src[a.total_q + r] = child ? q0 + own : r;
+      rm.lm_next[a.total_q + r] = child ? tok : -1;
+      a.row_best[a.total_q + r] = 0ull;
+      a.zdraft[a.total_q + r] = __int_as_float(0x7fc00000);
     }
     rm.row_seq[r] = i;
-    rm.row_pos[r] = a.parent ? L + s_depth[j - j_lo] : pos;
+    rm.row_pos[r] = L + (a.parent ? d : j);
     rm.row_tok[r] = tok;
-    rm.row_kv[r] = phys * HSD_KV_BLOCK + pos % HSD_KV_BLOCK;
+    rm.row_kv[r] = phys * HSD_KV_BLOCK + (L + j) % HSD_KV_BLOCK;
     rm.row_next[r] = (a.allow_embed_rows || a.parent) ? -1 : nxt;
+    a.row_best[r] = 0ull;                               // the LM head's running best and captured logit
+    a.zdraft[r] = __int_as_float(0x7fc00000);
+    s_tok[tid] = tok;
+    s_len[tid] = L + (a.parent ? d : j);
   }
-  // rotary table: (cos, sin) of pos * base^(-2i/D), angle formed in double so long contexts keep accuracy
-  for (int e = j_lo * half + tid; e < j_hi * half; e += blockDim.x) {
-    const int j = e / half, f = e % half;
-    const double inv = exp2(-(double)(2 * f) / (double)a.head_dim * log2((double)a.rope_base));
+  __syncthreads();
+  if (tid == 0) a.verdict[blockIdx.x] = make_int2(s_code, s_where);
+  // embedding gather: x[r] = fp32(table[tok]) or fp32(embeds[r]), a warp per row, 16-byte loads
+  for (int k = warp; k < n_rows; k += kSetupThreads / 32) {
+    const int tok = s_tok[k];
+    const bf16* src = tok >= 0 ? a.table + (size_t)tok * a.d : a.embeds + (size_t)(r0 + k) * a.d;
+    float* dst = a.x + (size_t)(r0 + k) * a.d;
+#pragma unroll 4
+    for (int c = lane * 8; c < a.d; c += 256) {
+      const uint4 v = *reinterpret_cast<const uint4*>(src + c);
+      *reinterpret_cast<float4*>(dst + c) = make_float4(bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y));
+      *reinterpret_cast<float4*>(dst + c + 4) = make_float4(bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w));
+    }
+  }
+  // rotary table: (cos, sin) of pos * base^(-2f/D), angle formed in double so long contexts keep accuracy
+  const int half = a.head_dim / 2, f = tid % half;      // (half divides the CTA: a thread stays with one frequency)
+  const double inv = exp2(-(double)(2 * f) / (double)a.head_dim * log2((double)a.rope_base));
+  for (int k = tid / half; k < n_rows; k += kSetupThreads / half) {
     double sn, cs;
-    sincos((double)(L + (a.parent ? s_depth[j - j_lo] : j)) * inv, &sn, &cs);
-    rm.rope_cs[(size_t)(q0 + j) * half + f] = make_float2((float)cs, (float)sn);
+    sincos((double)s_len[k] * inv, &sn, &cs);
+    rm.rope_cs[(size_t)(r0 + k) * half + f] = make_float2((float)cs, (float)sn);
   }
 }
 
-void launch_setup_rows(cudaStream_t st, const SetupArgs& a, const KvView& kv, const RowMeta& rm, int* status,
-                       int* tile_count, bool pdl) {
-  dim3 grid(a.n_seqs, (a.max_q_len + kSetupRows - 1) / kSetupRows);
-  launch_kernel(setup_rows_kernel, grid, dim3(256), 0, st, pdl, a, kv, rm, status, tile_count);
+int setup_ctas(int total_q) { return (total_q + kSetupRows - 1) / kSetupRows + 1; }
+void launch_setup_rows(cudaStream_t st, const SetupArgs& a, const KvView& kv, const RowMeta& rm, int* tile_count, bool pdl) {
+  launch_kernel(setup_rows_kernel, dim3(setup_ctas(a.total_q)), dim3(kSetupThreads), 0, st, pdl, a, kv, rm, tile_count);
 }
 
-// ------------------------------------------------------------------------------------------------
-// Embedding gather: x[r] = fp32(table[tok]) or fp32(embeds[r]).  One warp per row, 16-byte loads.
-__global__ void embed_kernel(RowMeta rm, const bf16* __restrict__ table, const bf16* __restrict__ embeds,
-                             float* __restrict__ x, int T, int d, const int* status) {
-  pdl_wait();               // everything below reads or writes what earlier kernels of the step produced
+// The status words from the verdicts, where no attention plan is made (the plain attention kernels' contexts).
+__global__ void status_kernel(const int2* verdict, int n, int* status) {
+  pdl_wait();
   pdl_launch_dependents();
-  if (*status) return;
-  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (r >= T) return;
-  const int lane = threadIdx.x & 31;
-  const int tok = rm.row_tok[r];
-  const bf16* src = tok >= 0 ? table + (size_t)tok * d : embeds + (size_t)r * d;
-  float* dst = x + (size_t)r * d;
-  for (int c = lane * 8; c < d; c += 256) {
-    uint4 v = *reinterpret_cast<const uint4*>(src + c);
-    float4 lo = make_float4(bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y));
-    float4 hi = make_float4(bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w));
-    *reinterpret_cast<float4*>(dst + c) = lo;
-    *reinterpret_cast<float4*>(dst + c + 4) = hi;
-  }
+  status_from_verdicts(verdict, n, status);
 }
-void launch_embed(cudaStream_t st, const RowMeta& rm, const bf16* table, const bf16* embeds, float* x, int T, int d,
-                  const int* status, bool pdl) {
-  launch_kernel(embed_kernel, dim3((T + 7) / 8), dim3(256), 0, st, pdl, rm, table, embeds, x, T, d, status);
+void launch_status(cudaStream_t st, const int2* verdict, int n, int* status, bool pdl) {
+  launch_kernel(status_kernel, dim3(1), dim3(256), 0, st, pdl, verdict, n, status);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -384,57 +435,57 @@ void launch_attn_simt(cudaStream_t st, const bf16* q, const RowMeta& rm, const K
 }
 
 // ------------------------------------------------------------------------------------------------
-// Draft compare + longest-prefix accept + emit.  One warp per sequence.
+// Draft compare + longest-prefix accept + emit.  One CTA per sequence: a warp per sequence spent 45 us on a 2,049-row chunk,
+// two dependent reads for every 32 rows.
 // Row j (0-based) of a sequence holds the distribution after [.., pending, d_1..d_j]; its next draft token is
 // d_{j+1}.  a = first j < k whose test fails (or k).  Exact mode: argmax == d_{j+1}.  Threshold mode:
 // z[d_{j+1}] - z_max >= log_tau.
-__global__ void accept_kernel(AcceptArgs a, RowMeta rm, const int* status) {
+constexpr int kAcceptThreads = 256;
+__global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a, RowMeta rm, const int* status) {
   pdl_wait();               // everything below reads or writes what earlier kernels of the step produced
   pdl_launch_dependents();
-  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (i >= a.n_seqs) return;
-  const int lane = threadIdx.x & 31;
+  const int i = blockIdx.x, tid = threadIdx.x;
+  __shared__ int s_acc;
   // (three independent reads in flight together; after a failed check the two row words are unwritten and unused)
   const int failed = *status;
   const int q0 = rm.seq_q0[i], n = rm.seq_n[i];
   if (failed) {             // a failed step decides nothing: -1 makes the commit that follows leave the lengths alone
-    if (lane == 0) { a.accept_len[i] = -1; a.n_emit[i] = 0; }
+    if (tid == 0) { a.accept_len[i] = -1; a.n_emit[i] = 0; }
     return;
   }
   if (n <= 0) {
-    if (lane == 0) { a.accept_len[i] = 0; a.n_emit[i] = 0; }
+    if (tid == 0) { a.accept_len[i] = 0; a.n_emit[i] = 0; }
     return;
   }
   const int k = n - 1;
-  int acc = k;
-  for (int j0 = 0; j0 < k && acc == k; j0 += 32) {
-    const int j = j0 + lane;
-    bool ok = true;
+  if (tid == 0) s_acc = k;
+  __syncthreads();
+  int first = k;
+  for (int j = tid; j < n; j += kAcceptThreads) {
+    const unsigned long long best = a.row_best[q0 + j];
+    const int nxt = rm.row_next[q0 + j];
+    const float zd = a.zdraft[q0 + j];
     if (j < k) {
-      const unsigned long long best = a.row_best[q0 + j];
-      const int nxt = rm.row_next[q0 + j];
-      if (a.log_tau == 0.f) ok = (key_col(best) == nxt);
-      else ok = (a.zdraft[q0 + j] - key_value(best) >= a.log_tau);
+      const bool ok = a.log_tau == 0.f ? key_col(best) == nxt : zd - key_value(best) >= a.log_tau;
+      if (!ok) first = min(first, j);
     }
-    const unsigned fail = __ballot_sync(0xffffffffu, !ok);
-    if (fail) acc = j0 + __ffs(fail) - 1;
+    if (a.row_argmax) a.row_argmax[q0 + j] = key_col(best);
+    if (a.row_zmax) a.row_zmax[q0 + j] = key_value(best);
+    if (a.row_zdraft) a.row_zdraft[q0 + j] = zd;
   }
+  if (first < k) atomicMin(&s_acc, first);
+  __syncthreads();
+  const int acc = s_acc;
   int* emit = a.emit_tokens + (size_t)i * a.max_q_len;
-  for (int j = lane; j < acc; j += 32) emit[j] = rm.row_next[q0 + j];
-  if (lane == 0) {
+  for (int j = tid; j < acc; j += kAcceptThreads) emit[j] = rm.row_next[q0 + j];
+  if (tid == 0) {
     emit[acc] = key_col(a.row_best[q0 + acc]);
     a.accept_len[i] = acc;
     a.n_emit[i] = acc + 1;
   }
-  for (int j = lane; j < n; j += 32) {
-    const unsigned long long best = a.row_best[q0 + j];
-    if (a.row_argmax) a.row_argmax[q0 + j] = key_col(best);
-    if (a.row_zmax) a.row_zmax[q0 + j] = key_value(best);
-    if (a.row_zdraft) a.row_zdraft[q0 + j] = a.zdraft[q0 + j];
-  }
 }
 void launch_accept(cudaStream_t st, const AcceptArgs& a, const RowMeta& rm, const int* status, bool pdl) {
-  launch_kernel(accept_kernel, dim3((a.n_seqs + 3) / 4), dim3(128), 0, st, pdl, a, rm, status);
+  launch_kernel(accept_kernel, dim3(a.n_seqs), dim3(kAcceptThreads), 0, st, pdl, a, rm, status);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -458,11 +509,12 @@ __global__ void tree_accept_kernel(TreeAcceptArgs a, RowMeta rm, const int* stat
   }
   int* emit = a.emit_tokens + (size_t)i * a.max_q_len;
   int* path = a.accept_rows + (size_t)i * a.max_q_len;
-  // every lane keeps four nodes (lane, lane + 32, ..) in registers: the walk itself then only fetches the row it
-  // stands on
+  // every lane keeps four nodes (lane, lane + 32, ..) in registers, their rows' best among them: the walk itself touches
+  // no memory (a read of the row it stands on cost ~0.3 us a step)
   constexpr int kPer = HSD_MAX_TREE_ROWS / 32;
   int npar[kPer], ntok[kPer];
   float nz[kPer];
+  unsigned long long nbest[kPer];
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     const int c = lane + 32 * k;
@@ -470,10 +522,18 @@ __global__ void tree_accept_kernel(TreeAcceptArgs a, RowMeta rm, const int* stat
     npar[k] = in ? a.parent[q0 + c] : -3;
     ntok[k] = in ? rm.row_tok[q0 + c] : -1;
     nz[k] = in ? a.zdraft[T + q0 + c] : 0.f;
+    nbest[k] = c < n ? a.row_best[q0 + c] : 0ull;
   }
+  auto best_of = [&](int row) -> unsigned long long {
+    unsigned long long b = 0ull;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+      if (k == row >> 5) b = nbest[k];
+    return __shfl_sync(0xffffffffu, b, row & 31);
+  };
   int s = 0, acc = 0;
   for (int step = 0; step < n; ++step) {
-    const unsigned long long best = a.row_best[q0 + s];
+    const unsigned long long best = best_of(s);
     const int uhat = key_col(best);
     int pick = -1, pick_tok = -1;
     float pick_z = 0.f;
@@ -526,16 +586,19 @@ __global__ void tree_accept_kernel(TreeAcceptArgs a, RowMeta rm, const int* stat
     ++acc;
     s = pick;
   }
+  const unsigned long long last = best_of(s);
   if (lane == 0) {
-    emit[acc] = key_col(a.row_best[q0 + s]);
+    emit[acc] = key_col(last);
     a.accept_len[i] = acc;
     a.n_emit[i] = acc + 1;
   }
-  for (int j = lane; j < n; j += 32) {
-    const unsigned long long best = a.row_best[q0 + j];
-    if (a.row_argmax) a.row_argmax[q0 + j] = key_col(best);
-    if (a.row_zmax) a.row_zmax[q0 + j] = key_value(best);
-    if (a.row_zchild) a.row_zchild[q0 + j] = j > 0 ? a.zdraft[T + q0 + j] : __int_as_float(0x7fc00000);
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int j = lane + 32 * k;
+    if (j >= n) continue;
+    if (a.row_argmax) a.row_argmax[q0 + j] = key_col(nbest[k]);
+    if (a.row_zmax) a.row_zmax[q0 + j] = key_value(nbest[k]);
+    if (a.row_zchild) a.row_zchild[q0 + j] = j > 0 ? nz[k] : __int_as_float(0x7fc00000);
   }
 }
 void launch_tree_accept(cudaStream_t st, const TreeAcceptArgs& a, const RowMeta& rm, const int* status, bool pdl) {
@@ -544,8 +607,11 @@ void launch_tree_accept(cudaStream_t st, const TreeAcceptArgs& a, const RowMeta&
 
 // KV maintenance after a tree step (Sec. 4.2: rollbacks and cache maintenance are part of the decode loop): the
 // accepted path's rows move from their packed places L + r_d to the places L + d their rotary positions stand for.
-// One CTA per (sequence, layer); a path's rows increase strictly, so moving depth by depth never overwrites a row
-// that is still to be read.
+// One CTA per (sequence, layer), one thread per 16-byte chunk of a token's K and V rows, kCompactBatch depths at a time:
+// a path's rows increase strictly and none lies before its place (r_d >= d), so a store to depth d can only hit the source
+// of a depth below d, which the same thread has read before; the loads of later depths never depend on it.  (Depth by
+// depth with a barrier between them, the launch took 19 us for a path of 22 nodes.)
+constexpr int kCompactBatch = 16;
 __global__ void tree_compact_kernel(KvView kv, int n_kv_heads, int head_dim, int n_seqs, const int* seq_slots,
                                     const int* accept_len, const int* accept_rows, int max_q_len) {
   pdl_wait();               // everything below reads or writes what earlier kernels of the step produced
@@ -560,22 +626,38 @@ __global__ void tree_compact_kernel(KvView kv, int n_kv_heads, int head_dim, int
   const int* bt = kv.block_table + (size_t)slot * kv.max_blocks;
   const int row_chunks = head_dim / 8;                   // 16-byte chunks of one (token, kv head) row
   const int chunks = n_kv_heads * 2 * row_chunks;        // ... of one token's K and V rows in a layer
-  for (int d = 1; d <= a && d < max_q_len; ++d) {
-    const int r = accept_rows[(size_t)i * max_q_len + d - 1];
-    if (r != d && r > 0 && r < max_q_len) {              // a row of this call (L + r is within the table, see above)
-      const int ps = L + r, pd = L + d;
-      const int bs = bt[ps / HSD_KV_BLOCK], bd = bt[pd / HSD_KV_BLOCK];
-      if (bs >= 0 && bs < kv.n_blocks && bd >= 0 && bd < kv.n_blocks) {
-        for (int t = threadIdx.x; t < chunks; t += blockDim.x) {
-          const int c16 = t % row_chunks, pool = (t / row_chunks) & 1, h = t / (2 * row_chunks);
-          bf16* base = pool ? kv.v_pool : kv.k_pool;
-          const size_t src = ((((size_t)layer * kv.n_blocks + bs) * n_kv_heads + h) * 64 + ps % HSD_KV_BLOCK) * head_dim;
-          const size_t dst = ((((size_t)layer * kv.n_blocks + bd) * n_kv_heads + h) * 64 + pd % HSD_KV_BLOCK) * head_dim;
-          reinterpret_cast<uint4*>(base + dst)[c16] = reinterpret_cast<const uint4*>(base + src)[c16];
-        }
+  __shared__ int s_row[HSD_MAX_TREE_ROWS];               // source row of depth d (0: stays where it is)
+  __shared__ int s_blk[HSD_MAX_TREE_ROWS / HSD_KV_BLOCK + 2];   // physical blocks of cache rows L .. L + 127
+  const int n = min(a, max_q_len - 1), blk0 = L / HSD_KV_BLOCK;
+  for (int d = threadIdx.x; d < HSD_MAX_TREE_ROWS; d += blockDim.x) {
+    const int r = d >= 1 && d <= n ? accept_rows[(size_t)i * max_q_len + d - 1] : 0;
+    s_row[d] = r != d && r > 0 && r < max_q_len ? r : 0;    // a row of this call (L + r is within the table, see above)
+  }
+  if (threadIdx.x < HSD_MAX_TREE_ROWS / HSD_KV_BLOCK + 2)
+    s_blk[threadIdx.x] = blk0 + (int)threadIdx.x < kv.max_blocks ? bt[blk0 + threadIdx.x] : -1;
+  __syncthreads();
+  for (int t = threadIdx.x; t < chunks; t += blockDim.x) {
+    const int c16 = t % row_chunks, pool = (t / row_chunks) & 1, h = t / (2 * row_chunks);
+    uint4* base = reinterpret_cast<uint4*>(pool ? kv.v_pool : kv.k_pool) + c16;
+    auto place = [&](int row, size_t& at) -> bool {        // 16-byte index of this thread's chunk of cache row L + row
+      const int p = L + row, b = s_blk[p / HSD_KV_BLOCK - blk0];
+      at = ((((size_t)layer * kv.n_blocks + b) * n_kv_heads + h) * 64 + p % HSD_KV_BLOCK) * row_chunks;
+      return b >= 0 && b < kv.n_blocks;
+    };
+    for (int d0 = 1; d0 <= n; d0 += kCompactBatch) {
+      uint4 v[kCompactBatch];
+      size_t src, dst;
+#pragma unroll
+      for (int k = 0; k < kCompactBatch; ++k) {
+        const int r = d0 + k <= n ? s_row[d0 + k] : 0;
+        if (r && place(r, src)) v[k] = base[src];
+      }
+#pragma unroll
+      for (int k = 0; k < kCompactBatch; ++k) {
+        const int r = d0 + k <= n ? s_row[d0 + k] : 0;
+        if (r && place(r, src) && place(d0 + k, dst)) base[dst] = v[k];
       }
     }
-    __syncthreads();
   }
 }
 void launch_tree_compact(cudaStream_t st, const KvView& kv, int n_layers, int n_kv_heads, int head_dim, int n_seqs,
