@@ -674,19 +674,24 @@ void launch_tree_compact(cudaStream_t st, const KvView& kv, int n_layers, int n_
 //  3. warp 0 grows the prefix tree level by level (Eq. 7): at depth d every live candidate moves to the child
 //     that carries its d-th token, creating it while the node budget lasts; a candidate whose node cannot be
 //     created stops.  Node ids are creation order, so parents precede children and the id is the packed row.
+// A round of 2. tests kDsvPer positions per thread across draft borders; in 3. a lane holds candidates `lane` and
+// `lane + 32`, and a level is one match over (current node, token): the lowest candidate of a group creates its node, in
+// candidate order, as if they went one after another.  (Draft after draft in rounds of 128 positions and candidate after
+// candidate, 16 drafts of 320 tokens took 111 us, 2 drafts 48 us.)
 // Every sequence gets exactly max_rows rows: row 0 = the pending token, then the nodes, then padding rows
 // (parent -2) that no traversal can enter.
 constexpr int kDsvMaxCands = 64;
 constexpr int kDsvMaxWindow = 8;
-__global__ void dsv_build_kernel(DsvArgs a) {
+constexpr int kDsvThreads = 512, kDsvPer = 4, kDsvDrafts = 64;   // drafts taken together
+__global__ void __launch_bounds__(kDsvThreads) dsv_build_kernel(DsvArgs a) {
   pdl_wait();               // everything below reads or writes what earlier kernels of the step produced
   pdl_launch_dependents();
   const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ int s_w[kDsvMaxWindow];
-  __shared__ int s_cstart[kDsvMaxCands], s_clen[kDsvMaxCands], s_ccur[kDsvMaxCands];
+  __shared__ int s_cstart[kDsvMaxCands], s_clen[kDsvMaxCands];
+  __shared__ int s_d0[kDsvDrafts], s_pos[kDsvDrafts + 1], s_cnt[kDsvThreads / 32];   // drafts: first token, first position
   __shared__ int s_ntok[HSD_MAX_TREE_ROWS], s_npar[HSD_MAX_TREE_ROWS];
-  __shared__ int s_ctok[kDsvMaxCands][HSD_MAX_TREE_ROWS];   // the part of every candidate a tree of this size can hold
-  __shared__ unsigned s_ballot[4];
+  __shared__ int s_ctok[kDsvMaxCands][HSD_MAX_TREE_ROWS + 1];   // the part of every candidate a tree of this size can hold
   __shared__ int s_ncand, s_nnodes;
   const int n = a.window_n;
   if (tid == 0) {
@@ -724,37 +729,81 @@ __global__ void dsv_build_kernel(DsvArgs a) {
     const bool owned = a.seq_map ? (owner >= 0 && owner < a.n_owners) : true;
     const int d_lo = owned ? min(max(a.seq_draft_off[owner], 0), a.n_drafts) : 0;
     const int d_hi = owned ? min(max(a.seq_draft_off[owner + 1], 0), a.n_drafts) : 0;
-    for (int d = d_lo; d < d_hi; ++d) {
-      const int d0 = min(max(a.draft_off[d], 0), a.total_draft_tokens);
-      const int len = min(max(a.draft_off[d + 1], d0), a.total_draft_tokens) - d0;
-      for (int j0 = 0; j0 + n < len; j0 += blockDim.x) {      // j + n < len: a non-empty suffix follows the window
-        if (s_ncand >= kDsvMaxCands) break;
-        const int j = j0 + tid;
-        bool hit = j + n < len;
-        for (int i = 0; hit && i < n; ++i) hit = a.draft_tokens[d0 + j + i] == s_w[i];
-        const unsigned b = __ballot_sync(0xffffffffu, hit);
-        if (lane == 0) s_ballot[warp] = b;
+    for (int db = d_lo; db < d_hi && s_ncand < kDsvMaxCands; db += kDsvDrafts) {
+      const int nd = min(kDsvDrafts, d_hi - db);
+      if (warp == 0) {
+        // positions a window can begin at with a non-empty suffix behind it, draft after draft
+        int before = 0;
+        for (int k0 = 0; k0 < nd; k0 += 32) {
+          const int k = k0 + lane;
+          int d0 = 0, cnt = 0;
+          if (k < nd) {
+            d0 = min(max(a.draft_off[db + k], 0), a.total_draft_tokens);
+            cnt = max(0, min(max(a.draft_off[db + k + 1], d0), a.total_draft_tokens) - d0 - n);
+          }
+          int incl = cnt;
+          for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+          }
+          if (k < nd) {
+            s_d0[k] = d0;
+            s_pos[k] = before + incl - cnt;
+          }
+          before += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) s_pos[nd] = before;
+      }
+      __syncthreads();
+      const int n_pos = s_pos[nd];
+      for (int v0 = 0; v0 < n_pos && s_ncand < kDsvMaxCands; v0 += kDsvThreads * kDsvPer) {
+        const int v = v0 + tid * kDsvPer;
+        int lo = 0, hi = nd;                              // the draft of position v: the last that begins at or before it
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (s_pos[mid] <= v) lo = mid; else hi = mid;
+        }
+        int dk[kDsvPer], hits = 0;
+#pragma unroll
+        for (int e = 0; e < kDsvPer; ++e) {
+          while (lo + 1 < nd && s_pos[lo + 1] <= v + e) ++lo;
+          dk[e] = lo;
+          bool hit = v + e < n_pos;
+          const int at = s_d0[lo] + (v + e - s_pos[lo]);
+          for (int i = 0; hit && i < n; ++i) hit = a.draft_tokens[at + i] == s_w[i];
+          hits |= (hit ? 1 : 0) << e;
+        }
+        int incl = __popc(hits);
+        for (int o = 1; o < 32; o <<= 1) {
+          const int x = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += x;
+        }
+        if (lane == 31) s_cnt[warp] = incl;
         __syncthreads();
-        int before = s_ncand;
-        for (int w = 0; w < warp; ++w) before += __popc(s_ballot[w]);
-        const int slot = before + __popc(b & ((1u << lane) - 1u));
-        if (hit && slot < kDsvMaxCands) {
-          s_cstart[slot] = d0 + j + n;
-          s_clen[slot] = len - (j + n);
-          s_ccur[slot] = 0;
+        int slot = s_ncand + incl - __popc(hits), all = 0;
+        for (int w = 0; w < kDsvThreads / 32; ++w) {
+          if (w < warp) slot += s_cnt[w];
+          all += s_cnt[w];
+        }
+#pragma unroll
+        for (int e = 0; e < kDsvPer; ++e) {
+          if (!((hits >> e) & 1)) continue;
+          if (slot < kDsvMaxCands) {
+            const int j = v + e - s_pos[dk[e]];
+            s_cstart[slot] = s_d0[dk[e]] + j + n;
+            s_clen[slot] = s_pos[dk[e] + 1] - s_pos[dk[e]] - j;      // tokens behind the window
+          }
+          ++slot;
         }
         __syncthreads();
-        if (tid == 0) {
-          int tot = s_ncand;
-          for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += __popc(s_ballot[w]);
-          s_ncand = min(tot, kDsvMaxCands);
-        }
+        if (tid == 0) s_ncand = min(kDsvMaxCands, s_ncand + all);
         __syncthreads();
       }
+      __syncthreads();                                    // s_pos is rewritten
     }
   }
   __syncthreads();
-  for (int idx = tid; idx < s_ncand * HSD_MAX_TREE_ROWS; idx += blockDim.x) {
+  for (int idx = tid; idx < s_ncand * HSD_MAX_TREE_ROWS; idx += kDsvThreads) {
     const int c = idx / HSD_MAX_TREE_ROWS, d = idx % HSD_MAX_TREE_ROWS;
     s_ctok[c][d] = d < s_clen[c] ? a.draft_tokens[s_cstart[c] + d] : -1;
   }
@@ -762,30 +811,56 @@ __global__ void dsv_build_kernel(DsvArgs a) {
   // ---- prefix tree, level by level (warp 0; node ids 1.. in creation order, id 0 = root)
   if (warp == 0) {
     const int ncand = s_ncand, budget = a.max_rows - 1;
-    int nn = 0;
-    unsigned long long alive = ncand >= 64 ? ~0ull : ((1ull << ncand) - 1ull);
-    for (int depth = 0; alive && depth < HSD_MAX_TREE_ROWS; ++depth) {
-      const int level0 = nn + 1;       // a node's children are all created while its level is expanded: search only those
-      for (int c = 0; c < ncand; ++c) {
-        if (!((alive >> c) & 1ull)) continue;
-        if (depth >= s_clen[c]) { alive &= ~(1ull << c); continue; }
-        const int u = s_ctok[c][depth];
-        const int cur = s_ccur[c];
-        int found = 0;
-        for (int base = level0; base <= nn && !found; base += 32) {
-          const int id = base + lane;
-          const bool hit = id <= nn && s_npar[id] == cur && s_ntok[id] == u;
-          const unsigned m = __ballot_sync(0xffffffffu, hit);
-          if (m) found = base + __ffs(m) - 1;
+    const unsigned below = (1u << lane) - 1u;
+    int nn = 0, cur[2] = {0, 0};
+    bool alive[2] = {lane < ncand, lane + 32 < ncand};
+    const int len[2] = {lane < ncand ? s_clen[lane] : 0, lane + 32 < ncand ? s_clen[lane + 32] : 0};
+    for (int depth = 0; depth < HSD_MAX_TREE_ROWS; ++depth) {
+      alive[0] = alive[0] && depth < len[0];
+      alive[1] = alive[1] && depth < len[1];
+      const unsigned on0 = __ballot_sync(0xffffffffu, alive[0]), on1 = __ballot_sync(0xffffffffu, alive[1]);
+      if (!(on0 | on1)) break;
+      // two candidates go to the same child iff they stand on the same node and carry the same token
+      const int tok0 = alive[0] ? s_ctok[lane][depth] : 0, tok1 = alive[1] ? s_ctok[lane + 32][depth] : 0;
+      const unsigned long long key0 = ((unsigned long long)cur[0] << 32) | (unsigned)tok0;
+      const unsigned long long key1 = ((unsigned long long)cur[1] << 32) | (unsigned)tok1;
+      unsigned same = 0u;
+      if (alive[0]) same = __match_any_sync(on0, key0);
+      __syncwarp();
+      const bool lead0 = alive[0] && (same & below) == 0u;
+      const unsigned leads0 = __ballot_sync(0xffffffffu, lead0);
+      const int mine0 = nn + 1 + __popc(leads0 & below);
+      const int id0 = __shfl_sync(0xffffffffu, mine0, alive[0] ? __ffs(same) - 1 : lane);
+      if (lead0 && mine0 <= budget) { s_ntok[mine0] = tok0; s_npar[mine0] = cur[0]; }
+      nn = min(budget, nn + __popc(leads0));
+      if (alive[0]) {
+        alive[0] = id0 <= budget;                         // a node that could not be created ends its candidates
+        cur[0] = id0;
+      }
+      if (on1) {
+        int id1 = 0;
+        for (unsigned m = leads0; m; m &= m - 1) {        // children that candidates 0..31 have just reached
+          const int src = __ffs(m) - 1;
+          const unsigned long long k = __shfl_sync(0xffffffffu, key0, src);
+          const int id = __shfl_sync(0xffffffffu, mine0, src);
+          if (alive[1] && k == key1) id1 = id;
         }
-        if (!found) {
-          if (nn >= budget) { alive &= ~(1ull << c); continue; }
-          ++nn;
-          if (lane == 0) { s_ntok[nn] = u; s_npar[nn] = cur; }
-          found = nn;
-        }
-        if (lane == 0) s_ccur[c] = found;
+        const bool rest = alive[1] && id1 == 0;
+        const unsigned onr = __ballot_sync(0xffffffffu, rest);
+        unsigned same1 = 0u;
+        if (rest) same1 = __match_any_sync(onr, key1);
         __syncwarp();
+        const bool lead1 = rest && (same1 & below) == 0u;
+        const unsigned leads1 = __ballot_sync(0xffffffffu, lead1);
+        const int mine1 = nn + 1 + __popc(leads1 & below);
+        const int got = __shfl_sync(0xffffffffu, mine1, rest ? __ffs(same1) - 1 : lane);
+        if (rest) id1 = got;
+        if (lead1 && mine1 <= budget) { s_ntok[mine1] = tok1; s_npar[mine1] = cur[1]; }
+        nn = min(budget, nn + __popc(leads1));
+        if (alive[1]) {
+          alive[1] = id1 <= budget;
+          cur[1] = id1;
+        }
       }
     }
     if (lane == 0) s_nnodes = nn;
@@ -793,7 +868,7 @@ __global__ void dsv_build_kernel(DsvArgs a) {
   __syncthreads();
   // ---- packed rows
   const int nn = s_nnodes, pending = s_w[n - 1];
-  for (int r = tid; r < a.max_rows; r += blockDim.x) {
+  for (int r = tid; r < a.max_rows; r += kDsvThreads) {
     const size_t o = (size_t)s * a.max_rows + r;
     if (r == 0) { a.q_tokens[o] = pending; a.parent[o] = -1; }
     else if (r <= nn) { a.q_tokens[o] = s_ntok[r]; a.parent[o] = s_npar[r]; }
@@ -802,7 +877,7 @@ __global__ void dsv_build_kernel(DsvArgs a) {
   if (tid == 0) a.n_rows[s] = nn + 1;
 }
 void launch_dsv_build(cudaStream_t st, const DsvArgs& a, bool pdl) {
-  launch_kernel(dsv_build_kernel, dim3(a.n_seqs), dim3(128), 0, st, pdl, a);
+  launch_kernel(dsv_build_kernel, dim3(a.n_seqs), dim3(kDsvThreads), 0, st, pdl, a);
 }
 
 // ------------------------------------------------------------------------------------------------
