@@ -489,120 +489,82 @@ void launch_accept(cudaStream_t st, const AcceptArgs& a, const RowMeta& rm, cons
 }
 
 // ------------------------------------------------------------------------------------------------
-// Greedy traversal of a candidate tree (Eq. 9-12), one warp per sequence.  At the current node s: u_hat = the
-// full-vocabulary argmax at s; u* = the child of s with the best score (exact mode: the child that carries u_hat);
-// move to it iff z[u*] - z[u_hat] >= log tau; stop when the test fails or s has no child; emit pi(s) + u_hat.
-__global__ void tree_accept_kernel(TreeAcceptArgs a, RowMeta rm, const int* status) {
+// Greedy traversal of a candidate tree (Eq. 9-12), one CTA per sequence, one thread per node.  At the current node s:
+// u_hat = the full-vocabulary argmax at s; u* = the child of s with the best score (exact mode: the child that carries
+// u_hat); move to it iff z[u*] - z[u_hat] >= log tau; stop when the test fails or s has no child; emit pi(s) + u_hat.
+// Every node finds its own move first, all at once; the walk is then a chase through shared memory (a step that searched
+// the children with warp reductions cost ~0.7 us: 36 us for the longest of 16 paths).
+__global__ void __launch_bounds__(HSD_MAX_TREE_ROWS) tree_accept_kernel(TreeAcceptArgs a, RowMeta rm, const int* status) {
   pdl_wait();               // everything below reads or writes what earlier kernels of the step produced
   pdl_launch_dependents();
-  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (i >= a.n_seqs) return;
-  const int lane = threadIdx.x & 31;
-  if (*status) {            // a failed step decides nothing: the compaction and the commit that follow skip -1
-    if (lane == 0) { a.accept_len[i] = -1; a.n_emit[i] = 0; }
-    return;
-  }
+  const int i = blockIdx.x, c = threadIdx.x;
+  __shared__ unsigned long long s_key[HSD_MAX_TREE_ROWS];     // best (score, then lower token) among a node's children
+  __shared__ unsigned long long s_best[HSD_MAX_TREE_ROWS];    // the node's own argmax word
+  __shared__ int s_child[HSD_MAX_TREE_ROWS], s_tok[HSD_MAX_TREE_ROWS], s_path[HSD_MAX_TREE_ROWS], s_acc;
+  const int failed = *status;
   const int q0 = rm.seq_q0[i], n = rm.seq_n[i], T = a.total_q;
-  if (n <= 0) {
-    if (lane == 0) { a.accept_len[i] = 0; a.n_emit[i] = 0; }
+  if (failed) {             // a failed step decides nothing: the compaction and the commit that follow skip -1
+    if (c == 0) { a.accept_len[i] = -1; a.n_emit[i] = 0; }
     return;
   }
+  if (n <= 0) {
+    if (c == 0) { a.accept_len[i] = 0; a.n_emit[i] = 0; }
+    return;
+  }
+  constexpr int kNone = 0x7fffffff;
+  const bool node = c >= 1 && c < n;
+  const int par = node ? a.parent[q0 + c] : -3, tok = node ? rm.row_tok[q0 + c] : -1;
+  const float z = node ? a.zdraft[T + q0 + c] : 0.f;
+  const unsigned long long best = c < n ? a.row_best[q0 + c] : 0ull;
+  s_best[c] = best;
+  s_key[c] = 0ull;
+  s_child[c] = kNone;
+  s_tok[c] = tok;
+  __syncthreads();
+  const bool child = node && par >= 0 && par < n;
+  if (a.log_tau == 0.f) {
+    // the child that carries u_hat (lowest row if a caller packed the same token twice under one parent)
+    if (child && tok == key_col(s_best[par])) atomicMin(&s_child[par], c);
+  } else {
+    // best child by (score, then lower token id), then lower row among equals
+    const unsigned long long key = argmax_key(z, tok);
+    if (child) atomicMax(&s_key[par], key);
+    __syncthreads();
+    if (child && s_key[par] == key) atomicMin(&s_child[par], c);
+    __syncthreads();
+    const int u = s_child[c];
+    if (u != kNone && !(key_value(s_key[c]) - key_value(best) >= a.log_tau)) s_child[c] = kNone;
+  }
+  __syncthreads();
+  if (c == 0) {
+    int s = 0, acc = 0;
+    while (s_child[s] != kNone && acc < n) {
+      s = s_child[s];
+      s_path[acc++] = s;
+    }
+    s_acc = acc;
+  }
+  __syncthreads();
+  const int acc = s_acc;
   int* emit = a.emit_tokens + (size_t)i * a.max_q_len;
   int* path = a.accept_rows + (size_t)i * a.max_q_len;
-  // every lane keeps four nodes (lane, lane + 32, ..) in registers, their rows' best among them: the walk itself touches
-  // no memory (a read of the row it stands on cost ~0.3 us a step)
-  constexpr int kPer = HSD_MAX_TREE_ROWS / 32;
-  int npar[kPer], ntok[kPer];
-  float nz[kPer];
-  unsigned long long nbest[kPer];
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const int c = lane + 32 * k;
-    const bool in = c >= 1 && c < n;
-    npar[k] = in ? a.parent[q0 + c] : -3;
-    ntok[k] = in ? rm.row_tok[q0 + c] : -1;
-    nz[k] = in ? a.zdraft[T + q0 + c] : 0.f;
-    nbest[k] = c < n ? a.row_best[q0 + c] : 0ull;
+  if (c < acc) {
+    path[c] = s_path[c];
+    emit[c] = s_tok[s_path[c]];
   }
-  auto best_of = [&](int row) -> unsigned long long {
-    unsigned long long b = 0ull;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k)
-      if (k == row >> 5) b = nbest[k];
-    return __shfl_sync(0xffffffffu, b, row & 31);
-  };
-  int s = 0, acc = 0;
-  for (int step = 0; step < n; ++step) {
-    const unsigned long long best = best_of(s);
-    const int uhat = key_col(best);
-    int pick = -1, pick_tok = -1;
-    float pick_z = 0.f;
-    if (a.log_tau == 0.f) {
-      // the child that carries u_hat (lowest row if a caller packed the same token twice under one parent)
-      int mine = 0x7fffffff;
-#pragma unroll
-      for (int k = kPer - 1; k >= 0; --k)
-        if (npar[k] == s && ntok[k] == uhat) mine = lane + 32 * k;
-      for (int o = 16; o; o >>= 1) mine = min(mine, __shfl_xor_sync(0xffffffffu, mine, o));
-      if (mine != 0x7fffffff) pick = mine;
-    } else {
-      // best child by (score, then lower token id), then lower row among equals
-      unsigned long long bk = 0ull;
-      int bc = 0x7fffffff;
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {
-        if (npar[k] != s) continue;
-        const unsigned long long key = argmax_key(nz[k], ntok[k]);
-        if (bc == 0x7fffffff || key > bk) { bk = key; bc = lane + 32 * k; }
-      }
-      unsigned long long wk = bc != 0x7fffffff ? bk : 0ull;
-      const unsigned has = __ballot_sync(0xffffffffu, bc != 0x7fffffff);
-      for (int o = 16; o; o >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xffffffffu, wk, o);
-        wk = other > wk ? other : wk;
-      }
-      if (has) {
-        int lo = (bc != 0x7fffffff && bk == wk) ? bc : 0x7fffffff;
-        for (int o = 16; o; o >>= 1) lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        pick = lo;
-      }
-    }
-    if (pick >= 0) {      // the owner lane broadcasts the node's token and score
-      const int owner = pick & 31, k = pick >> 5;
-      int tk = -1;
-      float zk = 0.f;
-#pragma unroll
-      for (int kk = 0; kk < kPer; ++kk)
-        if (kk == k) { tk = ntok[kk]; zk = nz[kk]; }
-      pick_tok = __shfl_sync(0xffffffffu, tk, owner);
-      pick_z = __shfl_sync(0xffffffffu, zk, owner);
-      if (a.log_tau != 0.f && !(pick_z - key_value(best) >= a.log_tau)) pick = -1;
-    }
-    if (pick < 0) break;
-    if (lane == 0) {
-      path[acc] = pick;
-      emit[acc] = pick_tok;
-    }
-    ++acc;
-    s = pick;
-  }
-  const unsigned long long last = best_of(s);
-  if (lane == 0) {
-    emit[acc] = key_col(last);
+  if (c == 0) {
+    emit[acc] = key_col(s_best[acc ? s_path[acc - 1] : 0]);
     a.accept_len[i] = acc;
     a.n_emit[i] = acc + 1;
   }
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const int j = lane + 32 * k;
-    if (j >= n) continue;
-    if (a.row_argmax) a.row_argmax[q0 + j] = key_col(nbest[k]);
-    if (a.row_zmax) a.row_zmax[q0 + j] = key_value(nbest[k]);
-    if (a.row_zchild) a.row_zchild[q0 + j] = j > 0 ? nz[k] : __int_as_float(0x7fc00000);
+  if (c < n) {
+    if (a.row_argmax) a.row_argmax[q0 + c] = key_col(best);
+    if (a.row_zmax) a.row_zmax[q0 + c] = key_value(best);
+    if (a.row_zchild) a.row_zchild[q0 + c] = c > 0 ? z : __int_as_float(0x7fc00000);
   }
 }
 void launch_tree_accept(cudaStream_t st, const TreeAcceptArgs& a, const RowMeta& rm, const int* status, bool pdl) {
-  launch_kernel(tree_accept_kernel, dim3((a.n_seqs + 3) / 4), dim3(128), 0, st, pdl, a, rm, status);
+  launch_kernel(tree_accept_kernel, dim3(a.n_seqs), dim3(HSD_MAX_TREE_ROWS), 0, st, pdl, a, rm, status);
 }
 
 // KV maintenance after a tree step (Sec. 4.2: rollbacks and cache maintenance are part of the decode loop): the
@@ -815,6 +777,7 @@ __global__ void __launch_bounds__(kDsvThreads) dsv_build_kernel(DsvArgs a) {
     int nn = 0, cur[2] = {0, 0};
     bool alive[2] = {lane < ncand, lane + 32 < ncand};
     const int len[2] = {lane < ncand ? s_clen[lane] : 0, lane + 32 < ncand ? s_clen[lane + 32] : 0};
+    bool apart = false;                                   // no two candidates stand on one node: they never meet again
     for (int depth = 0; depth < HSD_MAX_TREE_ROWS; ++depth) {
       alive[0] = alive[0] && depth < len[0];
       alive[1] = alive[1] && depth < len[1];
@@ -822,6 +785,17 @@ __global__ void __launch_bounds__(kDsvThreads) dsv_build_kernel(DsvArgs a) {
       if (!(on0 | on1)) break;
       // two candidates go to the same child iff they stand on the same node and carry the same token
       const int tok0 = alive[0] ? s_ctok[lane][depth] : 0, tok1 = alive[1] ? s_ctok[lane + 32][depth] : 0;
+      if (apart) {                                        // every live candidate has a child of its own
+        const int id0 = nn + 1 + __popc(on0 & below), id1 = min(budget, nn + __popc(on0)) + 1 + __popc(on1 & below);
+        if (alive[0] && id0 <= budget) { s_ntok[id0] = tok0; s_npar[id0] = cur[0]; }
+        if (alive[1] && id1 <= budget) { s_ntok[id1] = tok1; s_npar[id1] = cur[1]; }
+        alive[0] = alive[0] && id0 <= budget;
+        alive[1] = alive[1] && id1 <= budget;
+        cur[0] = id0;
+        cur[1] = id1;
+        nn = min(budget, nn + __popc(on0) + __popc(on1));
+        continue;
+      }
       const unsigned long long key0 = ((unsigned long long)cur[0] << 32) | (unsigned)tok0;
       const unsigned long long key1 = ((unsigned long long)cur[1] << 32) | (unsigned)tok1;
       unsigned same = 0u;
@@ -833,6 +807,7 @@ __global__ void __launch_bounds__(kDsvThreads) dsv_build_kernel(DsvArgs a) {
       const int id0 = __shfl_sync(0xffffffffu, mine0, alive[0] ? __ffs(same) - 1 : lane);
       if (lead0 && mine0 <= budget) { s_ntok[mine0] = tok0; s_npar[mine0] = cur[0]; }
       nn = min(budget, nn + __popc(leads0));
+      apart = leads0 == on0;
       if (alive[0]) {
         alive[0] = id0 <= budget;                         // a node that could not be created ends its candidates
         cur[0] = id0;
@@ -857,6 +832,7 @@ __global__ void __launch_bounds__(kDsvThreads) dsv_build_kernel(DsvArgs a) {
         if (rest) id1 = got;
         if (lead1 && mine1 <= budget) { s_ntok[mine1] = tok1; s_npar[mine1] = cur[1]; }
         nn = min(budget, nn + __popc(leads1));
+        apart = apart && leads1 == on1;
         if (alive[1]) {
           alive[1] = id1 <= budget;
           cur[1] = id1;
