@@ -411,6 +411,7 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
         g.tmB = &c->tm_gate_up[l];
         g.tmC = tm_act_st;
         g.M = T; g.n_out = 2 * md.ffn; g.K = md.d; g.mode = GS_SWIGLU;
+        g.out.C = w.act; g.out.ldc = md.ffn;
         g.status = w.status; g.n_sms = c->n_sms; g.device = c->device; g.max_splits = 1; g.pdl = c->pdl; g.pair = c->pair;
         if (launch_gemm_sm100(st, g)) return fail_cuda(c);
       }
@@ -1146,6 +1147,7 @@ int hsd_op_linear(hsd_ctx* c, const void* A, const void* W, void* C, int M, int 
   if (mode == 1 ? make_tmap_2d_f32(&g.tmC, C, M, ldc, 32) : make_tmap_2d(&g.tmC, C, M, ldc, 32)) return HSD_ERR_CUDA;
   g.tmB = &wm;
   g.M = M; g.n_out = n_out; g.K = K; g.mode = mode;
+  g.out.C = C; g.out.ldc = ldc;
   g.status = nullptr; g.n_sms = c->n_sms; g.device = c->device; g.max_splits = c->max_splits; g.pdl = false; g.pair = c->pair;
   g.force_bn = c->force_bn; g.force_splits = c->force_splits;
   if (launch_gemm_sm100(st, g)) return fail_cuda(c);

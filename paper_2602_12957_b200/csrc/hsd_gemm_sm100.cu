@@ -400,6 +400,24 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           }
           ++n_stores;
         }
+      } else if (MODE == GS_SWIGLU && OUT_N == 32) {
+        // the narrow tile: a row's 32 outputs are 64 bytes, stored as they are
+        if (slab_ok) {
+          uint32_t g[32], u[32];
+          tmem_ld32(t_acc, g);
+          tmem_ld32(t_acc + OUT_N, u);
+          tmem_ld_wait();
+#pragma unroll
+          for (int e = 0; e < 32; ++e) {
+            const float gv = __uint_as_float(g[e]);
+            g[e] = __float_as_uint(__fdividef(gv, 1.f + __expf(-gv)) * __uint_as_float(u[e]));
+          }
+          if (row_ok) {
+            uint4* dst = reinterpret_cast<uint4*>(static_cast<bf16*>(p.out.C) + (size_t)row * p.out.ldc + n0);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) dst[v] = pack8(g + 8 * v);
+          }
+        }
       } else if (MODE == GS_SWIGLU) {
 #pragma unroll 1
         for (int c = 0; slab_ok && c < OUT_N; c += 64) {
@@ -713,14 +731,14 @@ static void pick_tile(int mode, int n_cols, int M, int K, int n_sms, int max_spl
   const int k_blocks = K / KSUB;
   const int cands[4] = {256, 256, 128, 64};     // first entry: a CTA pair on a 256 x 256 tile
   double best_cost = 1e30;
-  *bn_out = (mode == GS_SWIGLU || mode == GS_QKV_ROPE128) ? 128 : 64;
+  *bn_out = mode == GS_QKV_ROPE128 ? 128 : 64;
   *splits_out = 1;
   *pair_out = false;
   for (int i = allow_pair && M > 64 ? 0 : 1; i < 4; ++i) {       // (a pair's tile needs whole boxes)
     const bool pair = i == 0;
     const int bn = cands[i];
     const int out_n = (mode == GS_SWIGLU) ? bn / 2 : bn;
-    if (n_cols % out_n || out_n % 64) continue;
+    if (n_cols % out_n || out_n % 32) continue;
     if (mode == GS_QKV_ROPE128 && bn < 128) continue;     // a tile holds whole 128-column heads
     const int tile_m = pair ? 2 * BM : BM;
     const int walkers = pair ? n_sms / 2 : n_sms;
@@ -749,7 +767,7 @@ static int launch_mode(cudaStream_t st, const GemmSm100Args& a) {
   if (a.force_bn) {
     const int fbn = a.force_bn == 512 ? 256 : a.force_bn;       // 512 = a CTA pair on 256-column tiles
     const int out_n = (MODE == GS_SWIGLU) ? fbn / 2 : fbn;
-    if ((fbn != 64 && fbn != 128 && fbn != 256) || out_n % 64 || n_cols % out_n) return -1;
+    if ((fbn != 64 && fbn != 128 && fbn != 256) || out_n % 32 || n_cols % out_n) return -1;
     if (MODE == GS_QKV_ROPE128 && fbn < 128) return -1;
     bn = fbn;
     pair = a.force_bn == 512 && a.M > 64;
@@ -764,7 +782,7 @@ static int launch_mode(cudaStream_t st, const GemmSm100Args& a) {
     case 256: return launch_one<256, MODE, false>(st, a, splits);
     case 128: return launch_one<128, MODE, false>(st, a, splits);
     default:
-      if (MODE == GS_SWIGLU || MODE == GS_QKV_ROPE128) return launch_one<128, MODE, false>(st, a, splits);
+      if (MODE == GS_QKV_ROPE128) return launch_one<128, MODE, false>(st, a, splits);
       return launch_one<64, MODE, false>(st, a, splits);
   }
 }
