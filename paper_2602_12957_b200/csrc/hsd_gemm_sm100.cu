@@ -750,7 +750,7 @@ static void pick_tile(int mode, int n_cols, int M, int K, int n_sms, int max_spl
       const long long rounds = (units + walkers - 1) / walkers;
       const double fill = (double)(gemm_a_box_rows(M) + (pair ? bn / 2 : bn)) * (KSUB * 2) / 55.0;
       const double per_kb = pair ? 770.0 : (fill > 250.0 ? fill : 250.0);
-      const double epi = 700.0 + 10.0 * bn;
+      const double epi = 700.0 + (mode == GS_SWIGLU ? 13.0 : 20.0) * bn;     // measured: 3.0 us of reduce-adds for 256 columns
       const double cost = (double)rounds * (kbs * per_kb + 300.0) + epi + (sp > 1 ? 200.0 * sp : 0.0) + (pair ? 1500.0 : 0.0);
       if (cost < best_cost) { best_cost = cost; *bn_out = bn; *splits_out = sp; *pair_out = pair; }
     }
