@@ -67,14 +67,18 @@ struct hsd_ctx {
 
 namespace {
 
+constexpr int kStatusWords = 16;
+
 struct Ws {
-  int* status;        // 16 ints; [4] = attention q-tile count, [5] = attention shares per kv head
+  int* status;        // kStatusWords ints; [4] = attention q-tile count, [5] = attention shares per kv head
   AttnPlan plan;
   RowMeta rm;
   int* sel_rows;
   int2* verdict;      // what every set-up CTA found
-  int *h_tokens, *h_cu, *h_accept, *h_nemit, *h_emit;   // device staging of hsd_verify_regions_host
-  size_t h_emit_ints;
+  // device staging of hsd_verify_regions_host: [cu_q | q_tokens], and behind the status words [accept_len | n_emit |
+  // emit_tokens], so that the inputs and the results are one transfer each
+  int *h_in, *h_out;
+  size_t h_out_ints;
   float* x;
   bf16* h;
   bf16* q;
@@ -116,7 +120,9 @@ Ws carve(const hsd_ctx* c, void* base, int T, int S) {
     off = align_up(off + bytes, 1024);
     return r;
   };
-  w.status = static_cast<int*>(take(64));
+  w.h_out_ints = 2 * (size_t)S + (size_t)S * (T < HSD_MAX_Q_LEN ? T : HSD_MAX_Q_LEN);
+  w.status = static_cast<int*>(take(sizeof(int) * (kStatusWords + w.h_out_ints)));
+  w.h_out = w.status ? w.status + kStatusWords : nullptr;
   w.rm.row_seq = static_cast<int*>(take(sizeof(int) * T));
   w.rm.row_pos = static_cast<int*>(take(sizeof(int) * T));
   w.rm.row_tok = static_cast<int*>(take(sizeof(int) * T));
@@ -133,12 +139,7 @@ Ws carve(const hsd_ctx* c, void* base, int T, int S) {
   w.rm.lm_next = static_cast<int*>(take(sizeof(int) * T));
   w.sel_rows = static_cast<int*>(take(sizeof(int) * S));
   w.verdict = static_cast<int2*>(take(sizeof(int2) * (size_t)setup_ctas(T)));
-  w.h_tokens = static_cast<int*>(take(sizeof(int) * T));
-  w.h_cu = static_cast<int*>(take(sizeof(int) * (S + 1)));
-  w.h_accept = static_cast<int*>(take(sizeof(int) * S));
-  w.h_nemit = static_cast<int*>(take(sizeof(int) * S));
-  w.h_emit_ints = (size_t)S * (T < HSD_MAX_Q_LEN ? T : HSD_MAX_Q_LEN);
-  w.h_emit = static_cast<int*>(take(sizeof(int) * w.h_emit_ints));
+  w.h_in = static_cast<int*>(take(sizeof(int) * ((size_t)S + 1 + T)));
   w.x = static_cast<float*>(take(sizeof(float) * (size_t)T * md.d));
   w.h = static_cast<bf16*>(take(2 * (size_t)T * md.d));
   w.q = static_cast<bf16*>(take(2 * (size_t)T * md.Hq * md.D));
@@ -865,11 +866,13 @@ int hsd_verify_regions_host(hsd_ctx* c, const hsd_kv* kv, int n_seqs, const int*
   if (rc) return rc;
   const Ws w = carve(c, workspace, total_q, n_seqs);
   const size_t emit_ints = (size_t)n_seqs * max_q;
-  if (emit_ints > w.h_emit_ints) return HSD_ERR_WORKSPACE;
+  const size_t out_ints = 2 * (size_t)n_seqs + emit_ints;
+  if (out_ints > w.h_out_ints) return HSD_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
 
-  // pinned staging: [cu_q | q_tokens | accept_len | n_emit | status words | emit_tokens]
-  const size_t need = (size_t)(n_seqs + 1) + total_q + 2 * (size_t)n_seqs + 4 + emit_ints;
+  // pinned staging: [cu_q | q_tokens], from the next 16 bytes on [status words | accept_len | n_emit | emit_tokens]
+  const size_t in_ints = (size_t)n_seqs + 1 + total_q, out_at = align_up(in_ints, 4);
+  const size_t need = out_at + align_up(kStatusWords + out_ints, 4);
   if (need > c->pin_ints) {
     if (c->hg_exec) { cudaGraphExecDestroy(c->hg_exec); c->hg_exec = nullptr; }   // it names the old staging
     c->hg_seen_valid = false;
@@ -882,10 +885,10 @@ int hsd_verify_regions_host(hsd_ctx* c, const hsd_kv* kv, int n_seqs, const int*
   }
   int* p_cu = c->pin;
   int* p_tok = p_cu + n_seqs + 1;
-  int* p_acc = p_tok + total_q;
+  int* p_status = c->pin + out_at;
+  int* p_acc = p_status + kStatusWords;
   int* p_nem = p_acc + n_seqs;
-  int* p_status = p_nem + n_seqs;
-  int* p_emit = p_status + 4;
+  int* p_emit = p_nem + n_seqs;
   memcpy(p_cu, cu_q, sizeof(int) * (n_seqs + 1));
   memcpy(p_tok, q_tokens, sizeof(int) * total_q);
 
@@ -904,22 +907,23 @@ int hsd_verify_regions_host(hsd_ctx* c, const hsd_kv* kv, int n_seqs, const int*
 
   // the whole step on the stream: inputs in, verify (+ commit), results and status words out
   auto enqueue = [&]() -> int {
-    if (cudaMemcpyAsync(w.h_cu, p_cu, sizeof(int) * (n_seqs + 1), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(w.h_tokens, p_tok, sizeof(int) * total_q, cudaMemcpyHostToDevice, st) != cudaSuccess)
-      return fail_cuda(c);
-    int r = hsd_verify_regions(c, kv, n_seqs, w.h_cu, w.h_tokens, seq_slots, max_q, total_q, log_tau, w.h_accept,
-                               w.h_emit, w.h_nemit, nullptr, nullptr, nullptr, workspace, ws_bytes, cuda_stream);
+    {
+      Scope s(c, st, KC_SETUP);
+      launch_copy_words(st, w.h_in, c->pin, in_ints, false);   // (first of the call: nothing to overlap with)
+    }
+    int *accept = w.h_out, *n_em = accept + n_seqs, *emit = n_em + n_seqs;
+    int r = hsd_verify_regions(c, kv, n_seqs, w.h_in, w.h_in + n_seqs + 1, seq_slots, max_q, total_q, log_tau, accept, emit,
+                               n_em, nullptr, nullptr, nullptr, workspace, ws_bytes, cuda_stream);
     if (r) return r;
     if (commit) {
-      r = hsd_kv_commit(c, kv, n_seqs, seq_slots, w.h_accept, nullptr, cuda_stream);
+      r = hsd_kv_commit(c, kv, n_seqs, seq_slots, accept, nullptr, cuda_stream);
       if (r) return r;
     }
-    if (cudaMemcpyAsync(p_acc, w.h_accept, sizeof(int) * n_seqs, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(p_nem, w.h_nemit, sizeof(int) * n_seqs, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(p_emit, w.h_emit, sizeof(int) * emit_ints, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(p_status, workspace, sizeof(int) * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess)
-      return fail_cuda(c);
-    return HSD_OK;
+    {
+      Scope s(c, st, KC_COMMIT);
+      launch_copy_words(st, p_status, w.status, kStatusWords + out_ints, c->pdl);
+    }
+    return check_cuda(c);
   };
 
   const bool graph_stream = c->host_graph_ok && !c->profiling && st != nullptr && st != cudaStreamLegacy &&

@@ -159,6 +159,8 @@ void launch_stage_advance(cudaStream_t st, const StageDev& sd, const KvView& kv,
 void launch_stage_aggregate(cudaStream_t st, const StageDev& sd, int* draft_tokens, int capacity, int* draft_off, bool pdl);
 void launch_first_token(cudaStream_t st, const unsigned long long* row_best, int n_seqs, int* first_token,
                         const RowMeta& rm, const KvView& kv, const int* status, bool pdl);
+// dst and src on 16 bytes, with room for n rounded up to 4 words
+void launch_copy_words(cudaStream_t st, int* dst, const int* src, size_t n, bool pdl);
 void launch_commit(cudaStream_t st, const KvView& kv, int n_seqs, const int* seq_slots, const int* accept_len,
                    int* blocks_in_use, bool pdl);
 void launch_clear_best(cudaStream_t st, unsigned long long* row_best, float* zdraft, int rows, bool pdl);
