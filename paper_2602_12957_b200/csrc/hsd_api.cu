@@ -70,7 +70,7 @@ namespace {
 constexpr int kStatusWords = 16;
 
 struct Ws {
-  int* status;        // kStatusWords ints; [4] = attention q-tile count, [5] = attention shares per kv head
+  int* status;        // kStatusWords ints; [5] = attention shares per kv head
   AttnPlan plan;
   RowMeta rm;
   int* sel_rows;
@@ -93,7 +93,7 @@ struct Ws {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Shortest slice of a q-tile's KV range in 64-key blocks, and slices a q-tile is cut into at most: see attn_plan_kernel.
+// Shortest slice of a q-tile's KV range in 64-key blocks, and slices a q-tile is cut into at most: see make_attn_plan.
 constexpr int kAttnMinChunk = 8, kAttnMaxSlices = 12;
 
 // CTAs of an attention launch: as many as are resident at once
@@ -286,19 +286,17 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
     sa.row_best = w.row_best;
     sa.zdraft = w.zdraft;
     sa.verdict = w.verdict;
-    launch_setup_rows(st, sa, kv, w.rm, w.status + 4, c->pdl);
+    // (a context with a fixed summation order never cuts a KV range: where the cuts fall depends on the batch)
+    sa.make_plan = !c->attn_simt;
+    sa.plan = w.plan;
+    sa.rule.max_shares = max(1, min(attn_max_shares(c), c->attn_target_items / md.Hkv));
+    sa.rule.min_chunk = c->attn_min_chunk;
+    sa.rule.max_slices = kAttnMaxSlices;
+    sa.rule.no_cut = c->max_splits == 1;
+    launch_setup_rows(st, sa, kv, w.rm, c->pdl);
   }
 
   CUtensorMap tm_h, tm_attn, tm_act, tm_q, tm_k, tm_v, tm_x_add, tm_q_st, tm_act_st;
-  if (c->attn_simt) {
-    Scope s(c, st, KC_SETUP);
-    launch_status(st, w.verdict, setup_ctas(T), w.status, c->pdl);
-  } else {
-    Scope s(c, st, KC_SETUP);
-    // (a context with a fixed summation order never cuts a KV range: where the cuts fall depends on the batch)
-    launch_attn_plan(st, w.rm, w.plan, kv, a.n_seqs, tokens_per_tile, max(1, min(attn_max_shares(c), c->attn_target_items / md.Hkv)),
-                     c->attn_min_chunk, kAttnMaxSlices, c->max_splits == 1, w.status + 4, w.verdict, setup_ctas(T), w.status, c->pdl);
-  }
   if (!c->simt) {
     const uint32_t box = gemm_a_box_rows(T);
     if (make_tmap_2d(&tm_h, w.h, T, md.d, box) || make_tmap_2d(&tm_attn, w.attn, T, md.Hq * md.D, box) ||
@@ -322,7 +320,8 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
   for (int l = 0; l < md.n_layers; ++l) {
     {
       Scope s(c, st, KC_RMSNORM);
-      launch_rmsnorm(st, w.x, c->attn_norm[l], w.h, T, md.d, md.eps, nullptr, T, w.status, c->pdl);
+      if (l == 0) launch_first_rmsnorm(st, w.x, c->attn_norm[l], w.h, T, md.d, md.eps, w.verdict, setup_ctas(T), w.status, c->pdl);
+      else launch_rmsnorm(st, w.x, c->attn_norm[l], w.h, T, md.d, md.eps, nullptr, T, w.status, c->pdl);
     }
     if (int rc = tap(l, HSD_TAP_H_ATTN, w.h, 2 * row_d)) return rc;
     const size_t layer_elems = (size_t)kv.n_blocks * md.Hkv * 64 * md.D;

@@ -7,7 +7,7 @@
 // sequence x the `group` query heads that share the kv head (GQA packing, so K/V blocks are read once per
 // group).  A q-tile's KV range is run whole or cut into slices so that a launch has one share of work per CTA slot,
 // whatever the mix of context lengths (one page chunk over a long context, or many short regions); the plan is made
-// once per step on the device (attn_plan_kernel) and reused by every layer.  Slices leave
+// once per step on the device (make_attn_plan) and reused by every layer.  Slices leave
 // (unnormalised O, exponent reference, sum) partials in the workspace and the last slice to finish combines them in
 // slice order, so the result does not depend on which CTA ran what.
 //
@@ -37,6 +37,7 @@
 // exponentials of its rows.  Fetching the next block's scores before the P store is waited for was slower (register
 // moves), and so was a barrier probe without the suspend-time hint.
 // Every wait is a bounded mbarrier wait, so one that gives up takes the whole CTA to the common exit.
+#include "hsd_attn_plan.cuh"
 #include "hsd_kernels.h"
 
 namespace hsd {
@@ -102,242 +103,10 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
   return y;
 }
-// The unit (share, kv head) that CTA `bx` of a grid of `G` starts with (n: none).  A launch with fewer units than CTAs
-// leaves some SMs with one busy CTA (the grid is two CTAs per SM, and CTA b shares its SM with CTA b + G/2 under the usual
-// placement); a CTA that has its SM alone walks its blocks faster, so the longest units go to those SMs and the others
-// pair a long one with a short one (shares of a one-round plan are sorted longest first).
-__device__ __forceinline__ int attn_unit_at(int bx, int n, int G) {
-  const int half = G / 2;
-  if (n <= half || n > G) return bx;
-  const int n_second = n - half;                       // busy CTAs in the second half of the grid
-  if (bx < half) return bx >= n_second ? bx - n_second : (half - n_second) + bx;
-  return bx - half < n_second ? n - 1 - (bx - half) : n;
-}
-
 // Where the partials of a sliced q-tile's slices lie.  One-round plans: every item has a slot of its own, `z` names slice
 // 0's.  Line plans: z = 2 k0 + 1 with k0 the share whose last item is slice 0; slice k > 0 is the first item of share
 // k0 + k, so two slots per share keep all slices apart.  Either way z is unique to the q-tile (its arrival counter).
 __device__ __forceinline__ int slice_slot(int z, int slice, int line) { return !line ? z + slice : slice == 0 ? z : z - 1 + 2 * slice; }
-
-// ------------------------------------------------------------------------------------------------
-// Plan: one CTA.  Work is counted in 64-key blocks.  A kv head has `max_shares` CTA slots; every kv head has the same
-// plan, so a launch runs n_shares x n_kv_heads units, unit u = share u / n_kv_heads of head u % n_kv_heads.
-//
-// One round: a q-tile is cut into equal slices of at least min_chunk blocks, each a share of its own, as fine as leaves no
-// slot with two.  A slice costs a hand-over (~3 us, four blocks' time), so nothing is cut finer than the launch needs.
-// Line: where that leaves the longest slice more than kLineGain blocks above the mean (more q-tiles than slots, or
-// q-tiles a little longer than the mean, which only halves would shorten), the q-tiles' ranges are laid end to end, each
-// with kTileCost blocks added for what an item costs beside its blocks (Q, first product, output), and the line is cut into
-// equal shares; a cut that would leave a piece of fewer than kMinPiece blocks moves to the q-tile's edge.
-// Measured, step times with equal shares of the line always against one round always: 2,048 rows over 16,384 (33
-// q-tiles of 272 blocks on 37 slots) 7.10 / 7.57 ms; 16 regions (25 q-tiles of 4 to 17 blocks) 1.78 / 1.73; 512 rows over
-// 7,936 2.07 / 2.02.
-// no_cut (contexts with a fixed summation order): q-tiles are never cut, cuts of the line move to the nearer edge.
-constexpr int kTileCost = 3, kMinPiece = 2, kLineGain = 8, kPlanThreads = 512;
-__global__ void __launch_bounds__(kPlanThreads) attn_plan_kernel(RowMeta rm, AttnPlan pl, KvView kv, int n_seqs,
-                                                                 int tokens_per_tile, int max_shares, int min_chunk,
-                                                                 int max_slices, int no_cut, const int* tile_count,
-                                                                 const int2* verdict, int n_verdicts, int* status) {
-  pdl_wait();
-  pdl_launch_dependents();
-  // one round: creation order of the items; line: cuts (q-tile, block) and how many of them lie inside q-tiles so far
-  __shared__ int s_ct[kAttnMaxShares + 1], s_co[kAttnMaxShares + 1], s_rank[kAttnMaxShares + 1];
-  __shared__ int s_warp[kPlanThreads / 32], s_longest, s_blocks, s_count, s_slice;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (status_from_verdicts(verdict, n_verdicts, status)) {
-    if (tid == 0) *pl.n_shares = 0;
-    for (int b = tid; b < pl.grid; b += kPlanThreads) pl.first[3 * b + 2] = make_int4(0, 0, 0, 0);
-    return;
-  }
-  if (tid == 0) s_longest = s_blocks = 0;
-  const int n_tiles = *tile_count;
-  for (int s = tid; s < n_seqs; s += kPlanThreads)
-    for (int t = rm.seq_tile0[s]; t < rm.seq_tile0[s + 1]; ++t) pl.tile_seq[t] = s;
-  __syncthreads();
-  auto blocks_of = [&](int t) -> int {                 // 64-key blocks q-tile t can see
-    const int s = pl.tile_seq[t];
-    return (rm.seq_len[s] + min(rm.seq_n[s], (t - rm.seq_tile0[s] + 1) * tokens_per_tile) + 63) >> 6;
-  };
-  auto tile_item = [&](int t, int& tok0) -> int4 {
-    const int s = pl.tile_seq[t];
-    tok0 = (t - rm.seq_tile0[s]) * tokens_per_tile;
-    return make_int4(rm.seq_q0[s] + tok0, rm.seq_len[s] + tok0, min(tokens_per_tile, rm.seq_n[s] - tok0), rm.seq_slot[s]);
-  };
-  // exclusive sum over the CTA, in thread order; `all` = the total (every thread calls it the same number of times)
-  auto scan = [&](int v, int& all) -> int {
-    int incl = v;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += x;
-    }
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    int before = 0;
-    all = 0;
-    for (int w = 0; w < kPlanThreads / 32; ++w) {
-      if (w < warp) before += s_warp[w];
-      all += s_warp[w];
-    }
-    __syncthreads();
-    return before + incl - v;
-  };
-  // lengths, and where every q-tile begins on the line
-  int total = 0;
-  for (int t0 = 0; t0 < n_tiles; t0 += kPlanThreads) {
-    const int t = t0 + tid;
-    const int n = t < n_tiles ? blocks_of(t) : 0;
-    int all;
-    const int pos = scan(t < n_tiles ? n + kTileCost : 0, all);
-    if (t < n_tiles) {
-      pl.tile_pos[t] = total + pos;
-      atomicMax(&s_longest, n);
-      atomicAdd(&s_blocks, n);
-    }
-    total += all;
-  }
-  __syncthreads();
-  const int longest = s_longest, mean = (s_blocks + max_shares - 1) / max_shares;
-  // one round: the slice length is grown until the items fit the slots
-  int chunk = max(max(min_chunk, mean), (longest + max_slices - 1) / max_slices);
-  bool line = n_tiles > max_shares;
-  if (no_cut) {
-    chunk = longest;
-  } else if (!line) {
-    for (;;) {                                            // every thread runs the same iterations
-      if (tid == 0) s_count = s_slice = 0;
-      __syncthreads();
-      for (int t = tid; t < n_tiles; t += kPlanThreads) {
-        const int n = blocks_of(t), ns = max(1, (n + chunk - 1) / chunk);
-        atomicAdd(&s_count, ns);
-        atomicMax(&s_slice, (n + ns - 1) / ns);
-      }
-      __syncthreads();
-      const int count = s_count;
-      __syncthreads();
-      if (count <= max_shares || chunk >= longest) break;
-      chunk += max(1, chunk >> 5);
-    }
-    line = s_slice > max(mean, min_chunk) + kLineGain;
-  }
-  int P;
-  if (!line) {
-    P = 0;
-    for (int t0 = 0; t0 < n_tiles; t0 += kPlanThreads) {
-      const int t = t0 + tid;
-      const int n = t < n_tiles ? blocks_of(t) : 0;
-      const int ns = t < n_tiles ? max(1, (n + chunk - 1) / chunk) : 0;
-      int all;
-      const int at = P + scan(ns, all);
-      for (int k = 0; k < ns; ++k) {                     // q-tile, slice (| slices << 16), length of item at + k
-        s_ct[at + k] = t;
-        s_co[at + k] = k | (ns << 16);
-        s_rank[at + k] = n / ns + (k < n % ns ? 1 : 0);
-      }
-      P += all;
-    }
-    __syncthreads();
-    for (int i = tid; i < P; i += kPlanThreads) {         // longest first (rank sort, ties by creation order)
-      const int len = s_rank[i], t = s_ct[i], k = s_co[i] & 0xffff, ns = s_co[i] >> 16;
-      int rank = 0;
-      for (int j = 0; j < P; ++j) rank += (s_rank[j] > len) || (s_rank[j] == len && j < i);
-      const int n = blocks_of(t), from = k * (n / ns) + min(k, n % ns);
-      int tok0;
-      pl.items[2 * rank] = tile_item(t, tok0);
-      pl.items[2 * rank + 1] = make_int4(from | ((from + len) << 16), k | (ns << 8) | (tok0 << 16), i - k, 0);
-      pl.share_start[rank] = rank;
-    }
-    if (tid == 0) pl.share_start[P] = P;
-  } else {
-    P = max(1, min(max_shares, total / max(min_chunk, (longest + max_slices - 1) / max_slices)));
-    for (int k = tid; k <= P; k += kPlanThreads) {
-      int t = n_tiles, off = 0;
-      if (k < P) {
-        const int b = (int)((long long)k * total / P);
-        int lo = 0, hi = n_tiles;                          // last q-tile that begins at or before b
-        while (hi - lo > 1) {
-          const int mid = (lo + hi) >> 1;
-          if (pl.tile_pos[mid] <= b) lo = mid; else hi = mid;
-        }
-        t = lo;
-        const int n = blocks_of(t);
-        off = b - pl.tile_pos[t] - kTileCost;
-        if (off < kMinPiece || (no_cut && 2 * off < n)) {
-          off = 0;
-        } else if (no_cut || n - off < kMinPiece) {
-          ++t;
-          off = 0;
-        }
-      }
-      s_ct[k] = t;
-      s_co[k] = off;
-    }
-    __syncthreads();
-    if (warp == 0) {
-      int sum = 0;
-      for (int k0 = 0; k0 <= P; k0 += 32) {
-        const int k = k0 + lane;
-        const unsigned in = __ballot_sync(0xffffffffu, k <= P && s_co[min(k, P)] > 0);
-        if (k <= P) s_rank[k] = sum + __popc(in & (0xffffffffu >> (31 - lane)));
-        sum += __popc(in);
-      }
-    }
-    __syncthreads();
-    // a share begins with item (its q-tile + the cuts inside q-tiles up to it); a q-tile's slices follow one another
-    for (int k = tid; k <= P; k += kPlanThreads) pl.share_start[k] = s_ct[k] + s_rank[k];
-    for (int t = tid; t < n_tiles; t += kPlanThreads) {
-      int lo = 0, hi = P;                                  // first cut inside q-tile t or beyond it (cut P lies beyond all)
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (s_ct[mid] > t || (s_ct[mid] == t && s_co[mid] > 0)) hi = mid; else lo = mid + 1;
-      }
-      const int k0 = lo;
-      int ns = 1;
-      while (k0 + ns - 1 <= P && s_ct[k0 + ns - 1] == t) ++ns;
-      int tok0;
-      const int4 ia = tile_item(t, tok0);
-      const int n = blocks_of(t), first = t + s_rank[k0] - (s_co[k0] > 0 ? 1 : 0);
-      int from = 0;
-      for (int k = 0; k < ns; ++k) {
-        const int to = k + 1 < ns ? s_co[k0 + k] : n;
-        pl.items[2 * (first + k)] = ia;
-        pl.items[2 * (first + k) + 1] = make_int4(from | (to << 16), k | (ns << 8) | (tok0 << 16), 2 * (k0 - 1) + 1, 1);
-        from = to;
-      }
-    }
-  }
-  if (tid == 0) *pl.n_shares = P;
-  // slice-arrival counters: zero at the start of a step, reset by the combiner
-  for (int i = tid; i < 2 * P * pl.n_kv_heads * 4; i += kPlanThreads) pl.counters[i] = 0;
-  // what every CTA of the attention grid starts with, in one record: its first item and the physical blocks of that
-  // item's first two KV blocks, so that a CTA's first loads do not wait for a chain of dependent reads (item -> block table)
-  __syncthreads();
-  for (int b = tid; b < pl.grid; b += kPlanThreads) {
-    const int share = attn_unit_at(b, P * pl.n_kv_heads, pl.grid) / pl.n_kv_heads;
-    const int i0 = share < P ? pl.share_start[share] : 0, count = share < P ? pl.share_start[share + 1] - i0 : 0;
-    if (count == 0) {
-      pl.first[3 * b + 2] = make_int4(0, 0, 0, 0);
-      continue;
-    }
-    const int4 ia = pl.items[2 * i0], ib = pl.items[2 * i0 + 1];
-    const int kt_lo = ib.x & 0xffff, kt_hi = ib.x >> 16;
-    int phys0 = 0, phys1 = 0;
-    if (kt_hi > kt_lo && ia.w >= 0 && ia.w < kv.n_slots && kt_hi <= kv.max_blocks) {
-      const int* bt = kv.block_table + (size_t)ia.w * kv.max_blocks;
-      phys0 = bt[kt_lo];
-      phys1 = bt[kt_lo + 1 < kt_hi ? kt_lo + 1 : kt_lo];
-    }
-    pl.first[3 * b] = ia;
-    pl.first[3 * b + 1] = ib;
-    pl.first[3 * b + 2] = make_int4(i0, count, phys0, phys1);
-  }
-}
-
-void launch_attn_plan(cudaStream_t st, const RowMeta& rm, const AttnPlan& pl, const KvView& kv, int n_seqs,
-                      int tokens_per_tile, int max_shares, int min_chunk, int max_slices, bool no_cut, const int* tile_count,
-                      const int2* verdict, int n_verdicts, int* status, bool pdl) {
-  launch_kernel(attn_plan_kernel, dim3(1), dim3(kPlanThreads), 0, st, pdl, rm, pl, kv, n_seqs, tokens_per_tile, max_shares,
-                min_chunk, max_slices, no_cut ? 1 : 0, tile_count, verdict, n_verdicts, status);
-}
 
 // ------------------------------------------------------------------------------------------------
 template <int HD>

@@ -28,9 +28,9 @@ __device__ __forceinline__ void dev_fail(int* status, int code, int where) {
   if (status && atomicCAS(status, 0, code) == 0) status[1] = where;
 }
 
-// The status words (but [4] and [5]) from the verdicts of a step's set-up CTAs: the first violation, or zeros.  Called by
-// every thread of one CTA; returns whether a check failed.
-__device__ __forceinline__ bool status_from_verdicts(const int2* verdict, int n, int* status) {
+// The status words (but [5], the plan's share count) from the verdicts of a step's set-up CTAs: the first violation, or zeros.  Called by
+// every thread of one CTA.
+__device__ __forceinline__ void status_from_verdicts(const int2* verdict, int n, int* status) {
   __shared__ int s_first;
   if (threadIdx.x == 0) s_first = 0x7fffffff;
   __syncthreads();
@@ -38,11 +38,10 @@ __device__ __forceinline__ bool status_from_verdicts(const int2* verdict, int n,
     if (verdict[i].x) atomicMin(&s_first, i);
   __syncthreads();
   const bool failed = s_first != 0x7fffffff;
-  if (threadIdx.x < 16 && threadIdx.x != 4 && threadIdx.x != 5) {
+  if (threadIdx.x < 16 && threadIdx.x != 5) {
     const int2 v = failed ? verdict[s_first] : make_int2(0, 0);
     status[threadIdx.x] = threadIdx.x == 0 ? v.x : threadIdx.x == 1 ? v.y : 0;
   }
-  return failed;
 }
 
 // Per-row and per-sequence metadata of one packed batch, all in the workspace.

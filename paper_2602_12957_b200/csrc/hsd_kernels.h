@@ -50,6 +50,27 @@ enum KernelClass {
 };
 const char* kernel_class_name(int kc);
 
+// ---- attention plan (hsd_attn_plan.cuh): made once per step on the device, read by every layer's launch ----
+constexpr int kAttnMaxShares = 1024;   // most shares the work of a kv head is cut into
+struct AttnPlan {
+  int4* items;      // two int4 per (q-tile, slice) item, share after share: {first packed row, position of the first token,
+                    // tokens, KV slot}, {first | (last + 1) << 16 KV block, slice | slices << 8 | first token of the q-tile
+                    // within its sequence << 16, slot of the q-tile's slice 0, plan form: see slice_slot}
+  int* share_start; // [shares + 1] first item of every share
+  int* n_shares;
+  int* tile_seq;    // [max_tiles] sequence of a q-tile
+  int* tile_pos;    // [max_tiles] where it begins on the line the shares are cut from
+  int* counters;    // [2 shares, n_kv_heads, 4] slices that have delivered their partial of a 32-row quarter
+  int4* first;      // [grid CTAs][3]: the item a CTA of the attention grid starts with, ready to use: the item's two
+                    // words, then {first item of its share, items of its share, first two physical KV blocks}
+  int n_kv_heads;
+  int grid;         // CTAs of the attention launches this plan is made for
+};
+struct AttnPlanRule {
+  int max_shares, min_chunk, max_slices;   // see make_attn_plan
+  bool no_cut;
+};
+
 // ---- small kernels (hsd_small.cu) ---------------------------------------------------------------
 constexpr int kSetupRows = 16;   // packed rows a set-up CTA takes
 struct SetupArgs {
@@ -70,16 +91,22 @@ struct SetupArgs {
   unsigned long long* row_best;   // [T] (trees: [2T]) cleared for the LM head
   float* zdraft;            // likewise, NaN
   int2* verdict;            // [setup_ctas(T)] {status code, offending index} of every CTA
+  bool make_plan;           // the attention plan too (not where the plain attention kernel runs)
+  AttnPlan plan;
+  AttnPlanRule rule;
 };
 // `pdl` (here and below): launch with programmatic stream serialization; these kernels wait for their
 // predecessor at their first instruction, so the flag only hides launch latency.
 int setup_ctas(int total_q);
-void launch_setup_rows(cudaStream_t st, const SetupArgs& a, const KvView& kv, const RowMeta& rm, int* tile_count, bool pdl);
-void launch_status(cudaStream_t st, const int2* verdict, int n, int* status, bool pdl);
+void launch_setup_rows(cudaStream_t st, const SetupArgs& a, const KvView& kv, const RowMeta& rm, bool pdl);
 // h[r] = bf16(rmsnorm(x[src]) * gain), src = sel_rows ? sel_rows[r] : r.  The gather form (sel_rows != nullptr) writes
 // nothing when *status is set or src is outside [0, src_rows): the index comes from an earlier kernel of the step.
 void launch_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
                     const int* sel_rows, int src_rows, const int* status, bool pdl);
+// The first of a step (every row, in place order), which follows launch_setup_rows: it also turns the verdicts into the
+// status words.
+void launch_first_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
+                          const int2* verdict, int n_verdicts, int* status, bool pdl);
 // last row of every sequence (prefill's LM-head rows); -1 for every sequence when *status is set
 void launch_select_last_rows(cudaStream_t st, const RowMeta& rm, int n_seqs, int* sel_rows, const int* status, bool pdl);
 // q_norm / k_norm: per-head RMSNorm gains applied before the rotation, or nullptr
@@ -167,25 +194,7 @@ void launch_clear_best(cudaStream_t st, unsigned long long* row_best, float* zdr
 void launch_unpack_best(cudaStream_t st, const unsigned long long* row_best, int rows, int* argmax, float* zmax,
                         bool pdl);
 
-// ---- attention plan (hsd_attn_sm100.cu): made once per step on the device, read by every layer's launch ----
-constexpr int kAttnMaxShares = 1024;   // most shares the work of a kv head is cut into
-struct AttnPlan {
-  int4* items;      // two int4 per (q-tile, slice) item, share after share: {first packed row, position of the first token,
-                    // tokens, KV slot}, {first | (last + 1) << 16 KV block, slice | slices << 8 | first token of the q-tile
-                    // within its sequence << 16, slot of the q-tile's slice 0, plan form: see slice_slot}
-  int* share_start; // [shares + 1] first item of every share
-  int* n_shares;
-  int* tile_seq;    // [max_tiles] sequence of a q-tile
-  int* tile_pos;    // [max_tiles] where it begins on the line the shares are cut from
-  int* counters;    // [2 shares, n_kv_heads, 4] slices that have delivered their partial of a 32-row quarter
-  int4* first;      // [grid CTAs][3]: the item a CTA of the attention grid starts with, ready to use: the item's two
-                    // words, then {first item of its share, items of its share, first two physical KV blocks}
-  int n_kv_heads;
-  int grid;         // CTAs of the attention launches this plan is made for
-};
-void launch_attn_plan(cudaStream_t st, const RowMeta& rm, const AttnPlan& pl, const KvView& kv, int n_seqs,
-                      int tokens_per_tile, int max_shares, int min_chunk, int max_slices, bool no_cut, const int* tile_count,
-                      const int2* verdict, int n_verdicts, int* status, bool pdl);
+// ---- attention (hsd_attn_sm100.cu) ----
 int launch_attn_sm100(cudaStream_t st, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                       const AttnPlan& plan, const KvView& kv, const ModelDims& md, int layer, bf16* out, int n_sms,
                       int device, int* status, float* split_ws, const uint4* anc, bool pdl);

@@ -1,5 +1,6 @@
 // Memory- and latency-bound kernels of the verify step: row metadata + checks, embedding gather,
 // RMSNorm, RoPE + paged KV write, the plain SIMT attention (debug cross-check), accept/emit, KV commit.
+#include "hsd_attn_plan.cuh"
 #include "hsd_kernels.h"
 
 namespace hsd {
@@ -13,17 +14,22 @@ const char* kernel_class_name(int kc) {
 
 // ------------------------------------------------------------------------------------------------
 // Row metadata, embedding gather and the LM head's cleared rows: what a step needs before its first layer, in one launch.
-// A CTA takes kSetupRows packed rows whatever the sequences they belong to; one more CTA writes the per-sequence metadata.
+// A CTA takes kSetupRows packed rows whatever the sequences they belong to; the first CTA writes the per-sequence metadata
+// and makes the attention plan from it, beside the others' work.
 // Validates what the host cannot see (device-resident offsets, lengths and tables).  A CTA leaves its verdict {code, index}
-// in `verdict`, and the kernel that follows (attn_plan_kernel, or status_kernel where the plan is not made) turns the
-// verdicts into the status words: nothing has to be zeroed first.  Every kernel that follows an indirection returns early
+// in `verdict`, and the kernel that follows (the first RMSNorm) turns the verdicts into the status words: nothing has to be zeroed first.  Every kernel that follows an indirection returns early
 // on a violation.
 // (Separate launches for the status words, the metadata by sequence, the gather and the cleared rows, with the parent
-// walk through global memory, took 16 to 30 us of a step.)
+// walk through global memory, took 16 to 30 us of a step.  The plan in a launch of its own behind this one: one small layer
+// 53 us, now 50; 16 plain rows 0.8925 ms, now 0.8895; one lane's 192-node tree 1.186 ms, now 1.180.)
 constexpr int kSetupThreads = 256, kSetupMaxCu = 1024;
 __device__ __forceinline__ int setup_cu(const SetupArgs& a, int s) { return a.cu_q ? a.cu_q[s] : (s ? a.total_q : 0); }
 
-__global__ void __launch_bounds__(kSetupThreads) setup_rows_kernel(SetupArgs a, KvView kv, RowMeta rm, int* tile_count) {
+__global__ void __launch_bounds__(kSetupThreads) setup_rows_kernel(SetupArgs a, KvView kv, RowMeta rm) {
+  // rotary frequency base^(-2f/D) of this thread (half divides the CTA: a thread stays with one), in double so that the
+  // angles of long contexts keep accuracy
+  const int half = a.head_dim / 2, f = threadIdx.x % half;
+  const double inv = exp2(-(double)(2 * f) / (double)a.head_dim * log2((double)a.rope_base));
   pdl_wait();               // everything below reads or writes what earlier kernels of the stream produced
   pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -32,6 +38,7 @@ __global__ void __launch_bounds__(kSetupThreads) setup_rows_kernel(SetupArgs a, 
   __shared__ int s_par[HSD_MAX_TREE_ROWS + kSetupRows];
   __shared__ int s_tok[kSetupRows], s_depth[kSetupRows], s_len[kSetupRows];
   __shared__ int s_warp[kSetupThreads / 32];
+  int2* verdict = a.verdict + (blockIdx.x ? blockIdx.x - 1 : gridDim.x - 1);     // the rows' ahead of the sequences'
   if (tid == 0) s_code = s_where = 0;
   __syncthreads();
   auto fail = [&](int code, int where) {
@@ -49,11 +56,11 @@ __global__ void __launch_bounds__(kSetupThreads) setup_rows_kernel(SetupArgs a, 
   if (bad) atomicMax(&s_code, bad == DEV_TOO_LONG ? 2 : 1);
   __syncthreads();
   if (s_code) {
-    if (tid == 0) a.verdict[blockIdx.x] = make_int2(s_code == 2 ? DEV_TOO_LONG : DEV_CU_Q, 0);
+    if (tid == 0) *verdict = make_int2(s_code == 2 ? DEV_TOO_LONG : DEV_CU_Q, 0);
     return;
   }
 
-  if (blockIdx.x == gridDim.x - 1) {        // the sequences, with the exclusive scan of their attention q-tiles
+  if (blockIdx.x == 0) {                    // the sequences, with the exclusive scan of their attention q-tiles
     int base = 0;
     for (int s0 = 0; s0 < a.n_seqs; s0 += kSetupThreads) {
       const int s = s0 + tid;
@@ -95,13 +102,14 @@ __global__ void __launch_bounds__(kSetupThreads) setup_rows_kernel(SetupArgs a, 
     for (int r = a.total_q + tid; r < a.n_seqs; r += kSetupThreads) a.row_best[r] = 0ull;   // (LM-head rows of empty sequences)
     if (tid == 0) {
       rm.seq_tile0[a.n_seqs] = base;
-      *tile_count = base;
-      a.verdict[blockIdx.x] = make_int2(s_code, s_where);
+      *verdict = make_int2(s_code, s_where);
     }
+    __syncthreads();
+    if (a.make_plan && !s_code) make_attn_plan<kSetupThreads>(rm, a.plan, kv, a.rule, a.n_seqs, base, a.tokens_per_tile);
     return;
   }
 
-  const int r0 = blockIdx.x * kSetupRows, n_rows = min(kSetupRows, a.total_q - r0);
+  const int r0 = (blockIdx.x - 1) * kSetupRows, n_rows = min(kSetupRows, a.total_q - r0);
   const int par0 = max(0, r0 - HSD_MAX_TREE_ROWS);      // a row's ancestors lie among the 127 packed rows before it
   if (a.parent)
     for (int j = par0 + tid; j < r0 + n_rows; j += kSetupThreads) s_par[j - par0] = a.parent[j];
@@ -187,7 +195,7 @@ __global__ void __launch_bounds__(kSetupThreads) setup_rows_kernel(SetupArgs a, 
     s_len[tid] = L + (a.parent ? d : j);
   }
   __syncthreads();
-  if (tid == 0) a.verdict[blockIdx.x] = make_int2(s_code, s_where);
+  if (tid == 0) *verdict = make_int2(s_code, s_where);
   // embedding gather: x[r] = fp32(table[tok]) or fp32(embeds[r]), a warp per row, 16-byte loads
   for (int k = warp; k < n_rows; k += kSetupThreads / 32) {
     const int tok = s_tok[k];
@@ -200,9 +208,7 @@ __global__ void __launch_bounds__(kSetupThreads) setup_rows_kernel(SetupArgs a, 
       *reinterpret_cast<float4*>(dst + c + 4) = make_float4(bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w));
     }
   }
-  // rotary table: (cos, sin) of pos * base^(-2f/D), angle formed in double so long contexts keep accuracy
-  const int half = a.head_dim / 2, f = tid % half;      // (half divides the CTA: a thread stays with one frequency)
-  const double inv = exp2(-(double)(2 * f) / (double)a.head_dim * log2((double)a.rope_base));
+  // rotary table: (cos, sin) of the position times the frequency
   for (int k = tid / half; k < n_rows; k += kSetupThreads / half) {
     double sn, cs;
     sincos((double)s_len[k] * inv, &sn, &cs);
@@ -211,18 +217,8 @@ __global__ void __launch_bounds__(kSetupThreads) setup_rows_kernel(SetupArgs a, 
 }
 
 int setup_ctas(int total_q) { return (total_q + kSetupRows - 1) / kSetupRows + 1; }
-void launch_setup_rows(cudaStream_t st, const SetupArgs& a, const KvView& kv, const RowMeta& rm, int* tile_count, bool pdl) {
-  launch_kernel(setup_rows_kernel, dim3(setup_ctas(a.total_q)), dim3(kSetupThreads), 0, st, pdl, a, kv, rm, tile_count);
-}
-
-// The status words from the verdicts, where no attention plan is made (the plain attention kernels' contexts).
-__global__ void status_kernel(const int2* verdict, int n, int* status) {
-  pdl_wait();
-  pdl_launch_dependents();
-  status_from_verdicts(verdict, n, status);
-}
-void launch_status(cudaStream_t st, const int2* verdict, int n, int* status, bool pdl) {
-  launch_kernel(status_kernel, dim3(1), dim3(256), 0, st, pdl, verdict, n, status);
+void launch_setup_rows(cudaStream_t st, const SetupArgs& a, const KvView& kv, const RowMeta& rm, bool pdl) {
+  launch_kernel(setup_rows_kernel, dim3(setup_ctas(a.total_q)), dim3(kSetupThreads), 0, st, pdl, a, kv, rm);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -231,9 +227,13 @@ void launch_status(cudaStream_t st, const int2* verdict, int n, int* status, boo
 template <int VEC>   // VEC float4 per lane: d = 128 * VEC
 __global__ void rmsnorm_kernel(const float* __restrict__ x, const bf16* __restrict__ gain, bf16* __restrict__ h,
                                int rows, int d, float eps, const int* __restrict__ sel_rows, int src_rows,
-                               const int* __restrict__ status) {
+                               const int* __restrict__ status, const int2* verdict, int n_verdicts, int* status_out) {
   pdl_wait();               // everything below reads or writes what earlier kernels of the step produced
   pdl_launch_dependents();
+  if (verdict && blockIdx.x == gridDim.x - 1) {        // one CTA more: the status words of the step
+    status_from_verdicts(verdict, n_verdicts, status_out);
+    return;
+  }
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (r >= rows) return;
   const int lane = threadIdx.x & 31;
@@ -265,17 +265,28 @@ __global__ void rmsnorm_kernel(const float* __restrict__ x, const bf16* __restri
     hp[lane + 32 * i] = o;
   }
 }
-void launch_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
-                    const int* sel_rows, int src_rows, const int* status, bool pdl) {
-  if (rows <= 0) return;
-  dim3 grid((rows + 7) / 8), block(256);
-#define HSD_RMS_CASE(V) \
-  case V: launch_kernel(rmsnorm_kernel<V>, grid, block, 0, st, pdl, x, gain, h, rows, d, eps, sel_rows, src_rows, status); break;
+static void launch_rmsnorm_any(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
+                               const int* sel_rows, int src_rows, const int* status, const int2* verdict, int n_verdicts,
+                               int* status_out, bool pdl) {
+  dim3 grid((rows + 7) / 8 + (verdict ? 1 : 0)), block(256);
+#define HSD_RMS_CASE(V)                                                                                                  \
+  case V:                                                                                                                \
+    launch_kernel(rmsnorm_kernel<V>, grid, block, 0, st, pdl, x, gain, h, rows, d, eps, sel_rows, src_rows, status, verdict, \
+                  n_verdicts, status_out);                                                                               \
+    break;
   switch (d / 128) {
     HSD_RMS_CASE(1) HSD_RMS_CASE(2) HSD_RMS_CASE(4) HSD_RMS_CASE(8) HSD_RMS_CASE(16) HSD_RMS_CASE(32)
     default: break;   // hsd_create rejects other widths
   }
 #undef HSD_RMS_CASE
+}
+void launch_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
+                    const int* sel_rows, int src_rows, const int* status, bool pdl) {
+  if (rows > 0) launch_rmsnorm_any(st, x, gain, h, rows, d, eps, sel_rows, src_rows, status, nullptr, 0, nullptr, pdl);
+}
+void launch_first_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
+                          const int2* verdict, int n_verdicts, int* status, bool pdl) {
+  launch_rmsnorm_any(st, x, gain, h, rows, d, eps, nullptr, rows, nullptr, verdict, n_verdicts, status, pdl);
 }
 
 __global__ void select_last_rows_kernel(RowMeta rm, int n_seqs, int* sel_rows, const int* status) {
