@@ -12,7 +12,7 @@
 // TMA and MMA instructions take their operands as they are; a lane chosen by its number paid ~0.25 us for a TMA
 // instruction and ~90 cycles for an MMA, and an election at every stage ~70 cycles for each of a stage's narrow MMAs.
 // Verification steps, election at every stage / once: 16 plain rows 0.910 / 0.893 ms, 136 rows 1.040 / 1.019 ms, 320 rows
-// 1.658 / 1.636 ms, one lane's 192-node tree 1.200 / 1.182 ms.
+// 1.658 / 1.636 ms, one lane's 128-node tree 1.200 / 1.182 ms.
 // Two accumulator buffers in TMEM let the epilogue of unit i overlap the main loop of unit i+1.
 //
 // Epilogues (all fused; results leave the SM through swizzled staging buffers and TMA stores, so global

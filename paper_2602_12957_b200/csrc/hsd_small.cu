@@ -21,7 +21,7 @@ const char* kernel_class_name(int kc) {
 // on a violation.
 // (Separate launches for the status words, the metadata by sequence, the gather and the cleared rows, with the parent
 // walk through global memory, took 16 to 30 us of a step.  The plan in a launch of its own behind this one: one small layer
-// 53 us, now 50; 16 plain rows 0.8925 ms, now 0.8895; one lane's 192-node tree 1.186 ms, now 1.180.)
+// 53 us, now 50; 16 plain rows 0.8925 ms, now 0.8895; one lane's 128-node tree 1.186 ms, now 1.180.)
 constexpr int kSetupThreads = 256, kSetupMaxCu = 1024;
 __device__ __forceinline__ int setup_cu(const SetupArgs& a, int s) { return a.cu_q ? a.cu_q[s] : (s ? a.total_q : 0); }
 
