@@ -21,9 +21,16 @@ __device__ __forceinline__ int attn_unit_at(int bx, int n, int G) {
 // slots; every kv head has the same plan, so a launch runs n_shares x n_kv_heads units, unit u = share u / n_kv_heads of
 // head u % n_kv_heads.
 //
-// One round: a q-tile is cut into equal slices of at least min_chunk blocks, each a share of its own, as fine as leaves no
-// slot with two.  A slice costs a hand-over (~3 us, four blocks' time), so nothing is cut finer than the launch needs.
-// Line: where that leaves the longest slice more than kLineGain blocks above the mean (more q-tiles than slots, or
+// One round: a q-tile is cut into equal slices of about `chunk` blocks, each a share of its own, as fine as leaves no slot
+// with two.  Cutting costs a hand-over (~3 us, five blocks' time), so a q-tile of up to 4/3 min_chunk blocks stays whole, and
+// the last slice to finish adds up the others' results (~0.6 us each, about a block's time): n blocks in slices of c take
+// c + kSliceCost n / c, which is least at c = sqrt(kSliceCost n).  Measured, steps of the 24-layer decoder in slices of
+// 4 / 6 / 8 / 12 / 16 blocks: one q-tile of 32 blocks 0.881 / 0.862 / 0.885 / 0.904 / 0.971 ms; one of 126 blocks 1.272 /
+// 1.153 / 1.112 / 1.061 / 1.067; two of 75 blocks 1.255 / 1.226 / 1.175 / 1.149 / 1.193; 16 of 4 to 17 blocks 0.878 / 0.879 /
+// 0.884 / 0.886 / 0.927; two of 7 blocks cut in half 0.950, whole 0.921.
+// Results are added up three at a time, so a fourth slice costs a round (~1 us): up to kThreeSlices blocks are cut in three
+// where four would save two blocks' time at most (12 regions of ~50 rows and up to 24 blocks: 1.284 ms with four, 1.269 with three).
+// Line: where that leaves the longest slice more than kLineGain blocks above the mean, or above kLineGain (more q-tiles than slots, or
 // q-tiles a little longer than the mean, which only halves would shorten), the q-tiles' ranges are laid end to end, each
 // with kTileCost blocks added for what an item costs beside its blocks (Q, first product, output), and the line is cut into
 // equal shares; a cut that would leave a piece of fewer than kMinPiece blocks moves to the q-tile's edge.
@@ -31,11 +38,12 @@ __device__ __forceinline__ int attn_unit_at(int bx, int n, int G) {
 // q-tiles of 272 blocks on 37 slots) 7.10 / 7.57 ms; 16 regions (25 q-tiles of 4 to 17 blocks) 1.78 / 1.73; 512 rows over
 // 7,936 2.07 / 2.02.
 // no_cut (contexts with a fixed summation order): q-tiles are never cut, cuts of the line move to the nearer edge.
-constexpr int kTileCost = 3, kMinPiece = 2, kLineGain = 8, kPlanTiles = 512;
+constexpr float kSliceCost = 1.4f;
+constexpr int kTileCost = 3, kMinPiece = 2, kLineGain = 8, kPlanTiles = 512, kThreeSlices = 24;
 template <int THREADS>
 __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvView& kv, const AttnPlanRule& rule, int n_seqs,
                                int n_tiles, int tokens_per_tile) {
-  const int max_shares = rule.max_shares, min_chunk = rule.min_chunk, max_slices = rule.max_slices;
+  const int max_shares = rule.max_shares, min_chunk = rule.min_chunk, whole = 4 * min_chunk / 3;
   const bool no_cut = rule.no_cut;
   // one round: creation order of the items; line: cuts (q-tile, block) and how many of them lie inside q-tiles so far
   __shared__ int s_ct[kAttnMaxShares + 1], s_co[kAttnMaxShares + 1], s_rank[kAttnMaxShares + 1];
@@ -91,8 +99,14 @@ __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvVi
   }
   __syncthreads();
   const int longest = s_longest, mean = (s_blocks + max_shares - 1) / max_shares;
+  const int shortest = max(min_chunk, (int)ceilf(sqrtf(kSliceCost * (float)longest)));
   // one round: the slice length is grown until the items fit the slots
-  int chunk = max(max(min_chunk, mean), (longest + max_slices - 1) / max_slices);
+  int chunk = max(shortest, mean);
+  auto slices_of = [&](int n) -> int {
+    if (n <= whole) return 1;
+    const int ns = (n + chunk - 1) / chunk;
+    return ns == 4 && n <= kThreeSlices ? 3 : ns;
+  };
   bool line = n_tiles > max_shares;
   if (no_cut) {
     chunk = longest;
@@ -101,7 +115,7 @@ __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvVi
       if (tid == 0) s_count = s_slice = 0;
       __syncthreads();
       for (int t = tid; t < n_tiles; t += THREADS) {
-        const int n = blocks_of(t), ns = max(1, (n + chunk - 1) / chunk);
+        const int n = blocks_of(t), ns = slices_of(n);
         atomicAdd(&s_count, ns);
         atomicMax(&s_slice, (n + ns - 1) / ns);
       }
@@ -111,7 +125,7 @@ __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvVi
       if (count <= max_shares || chunk >= longest) break;
       chunk += max(1, chunk >> 5);
     }
-    line = s_slice > max(mean, min_chunk) + kLineGain;
+    line = s_slice > max(max(mean, shortest), kLineGain) + kLineGain;
   }
   int P;
   if (!line) {
@@ -119,7 +133,7 @@ __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvVi
     for (int t0 = 0; t0 < n_tiles; t0 += THREADS) {
       const int t = t0 + tid;
       const int n = t < n_tiles ? blocks_of(t) : 0;
-      const int ns = t < n_tiles ? max(1, (n + chunk - 1) / chunk) : 0;
+      const int ns = t < n_tiles ? slices_of(n) : 0;
       int all;
       const int at = P + scan(ns, all);
       for (int k = 0; k < ns; ++k) {                     // q-tile, slice (| slices << 16), length of item at + k
@@ -142,7 +156,7 @@ __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvVi
     }
     if (tid == 0) pl.share_start[P] = P;
   } else {
-    P = max(1, min(max_shares, total / max(min_chunk, (longest + max_slices - 1) / max_slices)));
+    P = max(1, min(max_shares, total / shortest));
     for (int k = tid; k <= P; k += THREADS) {
       int t = n_tiles, off = 0;
       if (k < P) {

@@ -67,7 +67,7 @@ struct AttnPlan {
   int grid;         // CTAs of the attention launches this plan is made for
 };
 struct AttnPlanRule {
-  int max_shares, min_chunk, max_slices;   // see make_attn_plan
+  int max_shares, min_chunk;   // see make_attn_plan
   bool no_cut;
 };
 
