@@ -141,13 +141,15 @@ Ws carve(const hsd_ctx* c, void* base, int T, int S) {
   w.sel_rows = static_cast<int*>(take(sizeof(int) * S));
   w.verdict = static_cast<int2*>(take(sizeof(int2) * (size_t)setup_ctas(T)));
   w.h_in = static_cast<int*>(take(sizeof(int) * ((size_t)S + 1 + T)));
+  // a prefill's LM head runs over one row per sequence, and sequences without rows make those more than T
+  const size_t lm_rows = T > S ? T : S;
   w.x = static_cast<float*>(take(sizeof(float) * (size_t)T * md.d));
-  w.h = static_cast<bf16*>(take(2 * (size_t)T * md.d));
+  w.h = static_cast<bf16*>(take(2 * lm_rows * md.d));
   w.q = static_cast<bf16*>(take(2 * (size_t)T * md.Hq * md.D));
   w.attn = static_cast<bf16*>(take(2 * (size_t)T * md.Hq * md.D));
   w.act = static_cast<bf16*>(take(2 * (size_t)T * md.ffn));
   w.qkv_f32 = c->simt ? static_cast<float*>(take(sizeof(float) * (size_t)T * md.qkv_out)) : nullptr;
-  w.row_best = static_cast<unsigned long long*>(take(sizeof(unsigned long long) * T));
+  w.row_best = static_cast<unsigned long long*>(take(sizeof(unsigned long long) * lm_rows));
   w.zdraft = static_cast<float*>(take(sizeof(float) * T));
   w.split_ws = c->simt ? nullptr : static_cast<float*>(take(sizeof(float) * split_ws_floats(c)));
   {

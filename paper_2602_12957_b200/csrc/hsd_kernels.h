@@ -88,8 +88,8 @@ struct SetupArgs {
   const bf16* table;        // embedding table
   const bf16* embeds;       // prefill: rows used where the token id is negative
   float* x;                 // [T, d] residual stream
-  unsigned long long* row_best;   // [T] (trees: [2T]) cleared for the LM head
-  float* zdraft;            // likewise, NaN
+  unsigned long long* row_best;   // [max(T, S)] (trees: [2T]) cleared for the LM head
+  float* zdraft;            // [T] (trees: [2T]) set to NaN
   int2* verdict;            // [setup_ctas(T)] {status code, offending index} of every CTA
   bool make_plan;           // the attention plan too (not where the plain attention kernel runs)
   AttnPlan plan;
