@@ -106,9 +106,17 @@ inline int attn_max_shares(const hsd_ctx* c) {
   const int n = attn_grid(c) / c->md.Hkv;
   return n < 1 ? 1 : (n > kAttnMaxShares ? kAttnMaxShares : n);
 }
-// Partial results of sliced q-tiles: two slots per share, each 128 rows of an fp32 accumulator row plus (reference, sum).
-inline size_t split_ws_floats(const hsd_ctx* c) {
-  return (size_t)2 * attn_max_shares(c) * c->md.Hkv * (c->md.D + 2) * 128;
+// Partial results of sliced q-tiles.  A slot holds what one slice of a q-tile leaves for every kv head: per 32-row quarter an
+// fp32 accumulator row plus (reference, sum) for each row, of as many quarters as a q-tile of a call of T rows can have.
+// Two slots per share are all a plan can use, 20 MB with 16 / 8 heads of 64; a small call gets the room of eight whole
+// slices of each of its q-tiles (one row 2.2 MB, 64 rows 4.3 MB) and its plan makes do with it.
+inline int attn_quarters(const ModelDims& md, int T) {
+  const int tokens = 128 / md.group;
+  return ((T < tokens ? T : tokens) * md.group + 31) / 32;
+}
+inline int split_quarters(const hsd_ctx* c, int T, int S) {      // all slots together, of one kv head
+  const long long most = 2ll * attn_max_shares(c) * attn_quarters(c->md, T), small = 32ll * attn_max_tiles(c->md, T, S);
+  return (int)(most < small ? most : small);
 }
 
 Ws carve(const hsd_ctx* c, void* base, int T, int S) {
@@ -118,7 +126,7 @@ Ws carve(const hsd_ctx* c, void* base, int T, int S) {
   char* p = static_cast<char*>(base);
   auto take = [&](size_t bytes) {
     void* r = p ? p + off : nullptr;
-    off = align_up(off + bytes, 1024);
+    off = align_up(off + bytes, 256);
     return r;
   };
   w.h_out_ints = 2 * (size_t)S + (size_t)S * (T < HSD_MAX_Q_LEN ? T : HSD_MAX_Q_LEN);
@@ -151,20 +159,25 @@ Ws carve(const hsd_ctx* c, void* base, int T, int S) {
   w.qkv_f32 = c->simt ? static_cast<float*>(take(sizeof(float) * (size_t)T * md.qkv_out)) : nullptr;
   w.row_best = static_cast<unsigned long long*>(take(sizeof(unsigned long long) * lm_rows));
   w.zdraft = static_cast<float*>(take(sizeof(float) * T));
-  w.split_ws = c->simt ? nullptr : static_cast<float*>(take(sizeof(float) * split_ws_floats(c)));
+  w.split_ws = c->simt ? nullptr : static_cast<float*>(take(sizeof(float) * (size_t)split_quarters(c, T, S) * md.Hkv * (md.D + 2) * 32));
   {
-    const int mt = attn_max_tiles(md, T, S), shares = attn_max_shares(c);
+    const int mt = attn_max_tiles(md, T, S), room = split_quarters(c, T, S), most = attn_max_shares(c);
+    w.plan.quarters = attn_quarters(md, T);
+    w.plan.slots = room / w.plan.quarters;
+    w.plan.max_shares = most < 16 * mt ? most : 16 * mt;
+    if (w.plan.max_shares > w.plan.slots) w.plan.max_shares = w.plan.slots;
+    const int shares = most < 16 * mt ? most : 16 * mt;     // (the arrays do not shrink where a q-tile gets more quarters)
     w.plan.items = static_cast<int4*>(take(sizeof(int4) * 2 * (size_t)(mt + shares)));
     w.plan.share_start = static_cast<int*>(take(sizeof(int) * (shares + 1)));
     w.plan.tile_seq = static_cast<int*>(take(sizeof(int) * mt));
     w.plan.tile_pos = static_cast<int*>(take(sizeof(int) * mt));
-    w.plan.counters = static_cast<int*>(take(sizeof(int) * 2 * (size_t)shares * md.Hkv * 4));
+    w.plan.counters = static_cast<int*>(take(sizeof(int) * (size_t)room * md.Hkv));
     w.plan.first = static_cast<int4*>(take(sizeof(int4) * 3 * (size_t)attn_grid(c)));
     w.plan.n_shares = w.status ? w.status + 5 : nullptr;
     w.plan.n_kv_heads = md.Hkv;
     w.plan.grid = attn_grid(c);
   }
-  w.bytes = off;
+  w.bytes = align_up(off, 1024);
   return w;
 }
 
@@ -292,7 +305,7 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
     // (a context with a fixed summation order never cuts a KV range: where the cuts fall depends on the batch)
     sa.make_plan = !c->attn_simt;
     sa.plan = w.plan;
-    sa.rule.max_shares = max(1, min(attn_max_shares(c), c->attn_target_items / md.Hkv));
+    sa.rule.max_shares = max(1, min(w.plan.max_shares, c->attn_target_items / md.Hkv));
     sa.rule.min_chunk = c->attn_min_chunk;
     sa.rule.no_cut = c->max_splits == 1;
     launch_setup_rows(st, sa, kv, w.rm, c->pdl);

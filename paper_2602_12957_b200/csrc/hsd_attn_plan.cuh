@@ -156,7 +156,7 @@ __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvVi
     }
     if (tid == 0) pl.share_start[P] = P;
   } else {
-    P = max(1, min(max_shares, total / shortest));
+    P = max(1, min(min(max_shares, pl.slots / 2), total / shortest));
     for (int k = tid; k <= P; k += THREADS) {
       int t = n_tiles, off = 0;
       if (k < P) {
@@ -215,7 +215,7 @@ __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvVi
   }
   if (tid == 0) *pl.n_shares = P;
   // slice-arrival counters: zero at the start of a step, reset by the combiner
-  for (int i = tid; i < 2 * P * pl.n_kv_heads * 4; i += THREADS) pl.counters[i] = 0;
+  for (int i = tid; i < (line ? 2 : 1) * P * pl.n_kv_heads * pl.quarters; i += THREADS) pl.counters[i] = 0;
   // what every CTA of the attention grid starts with, in one record: its first item and the physical blocks of that
   // item's first two KV blocks, so that a CTA's first loads do not wait for a chain of dependent reads (item -> block table)
   __syncthreads();

@@ -69,7 +69,7 @@ struct AttnParams {
   const int* block_table;
   int max_blocks, n_blocks, Hq, Hkv, group, layer;
   bf16* out;            // [T, Hq*HD]
-  float* split_ws;      // partials of sliced items: [slot][kv head][quarter][2 + HD][32 rows], see slice_slot
+  float* split_ws;      // partials of sliced items: [slot][kv head][quarter][32 (2 + HD)], see slice_slot
   const uint4* anc;     // [T] ancestry masks of candidate-tree rows, or nullptr: plain causal order within the call
   int* status;
 };
@@ -507,7 +507,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // bytes.  A quarter is handed over by itself: the warp whose slice arrives last combines its 32 rows, so the
         // CTA's warps do not wait for one another here.
         constexpr int PART = (2 + HD) * 32;
-        auto slice = [&](int k) -> float* { return p.split_ws + (size_t)((slice_slot(ib.z, k, ib.w) * p.Hkv + kvh) * 4 + quarter) * PART; };
+        auto slice = [&](int k) -> float* { return p.split_ws + (size_t)((slice_slot(ib.z, k, ib.w) * p.Hkv + kvh) * p.plan.quarters + quarter) * PART; };
         float* part = slice(split) + lane;
         part[0] = m_ref;
         part[32] = l;
@@ -527,7 +527,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         __syncwarp();
         int arrived = 0;
         if (lane == 0) {
-          int* ctr = p.plan.counters + (ib.z * p.Hkv + kvh) * 4 + quarter;
+          int* ctr = p.plan.counters + (ib.z * p.Hkv + kvh) * p.plan.quarters + quarter;
           arrived = atomicAdd(ctr, 1);
           if (arrived == n_split - 1) *ctr = 0;          // ready for the next layer
         }

@@ -60,10 +60,13 @@ struct AttnPlan {
   int* n_shares;
   int* tile_seq;    // [max_tiles] sequence of a q-tile
   int* tile_pos;    // [max_tiles] where it begins on the line the shares are cut from
-  int* counters;    // [2 shares, n_kv_heads, 4] slices that have delivered their partial of a 32-row quarter
+  int* counters;    // [slots, n_kv_heads, quarters] slices that have delivered their partial of a 32-row quarter
   int4* first;      // [grid CTAs][3]: the item a CTA of the attention grid starts with, ready to use: the item's two
                     // words, then {first item of its share, items of its share, first two physical KV blocks}
   int n_kv_heads;
+  int quarters;     // 32-row quarters a q-tile of the call can have tokens in
+  int slots;        // partial results there is room for: see slice_slot
+  int max_shares;   // shares there is room for
   int grid;         // CTAs of the attention launches this plan is made for
 };
 struct AttnPlanRule {

@@ -185,3 +185,50 @@ def long_document_oracle():
     _long_job.update(seq=I.SeqInput(emb, ids, 2048, 0, draft, True), draft=draft, weights=weights, pending=pending,
                      results=results)
     return _long_job
+
+
+def attention_float64(cfg, kv, q, lens, rows):
+    """Layer 0's attention output for the queries `q` [T, n_heads * head_dim] as the library formed them, over the cache as
+    it stands, in float64: (out, spread), spread = sqrt(sum w^2 v^2) of every output element."""
+    import torch
+    D, group = cfg.head_dim, cfg.n_heads // cfg.n_kv_heads
+    outs, spreads, r0 = [], [], 0
+    for s, (L, n) in enumerate(zip(lens, rows)):
+        keys = L + n
+        table = kv.block_table[s, :(keys + 63) // 64].long()
+        k, v = (p[0][table].permute(1, 0, 2, 3).reshape(cfg.n_kv_heads, -1, D)[:, :keys].double() for p in (kv.k_pool, kv.v_pool))
+        qs = q[r0:r0 + n].view(n, cfg.n_heads, D).double()
+        out = torch.empty(n, cfg.n_heads, D, dtype=torch.float64, device=q.device)
+        spread = torch.empty_like(out)
+        hidden = torch.arange(keys, device=q.device)[None] > (L + torch.arange(n, device=q.device))[:, None]
+        for h in range(cfg.n_heads):
+            w = torch.softmax((qs[:, h] @ k[h // group].T / D ** 0.5).masked_fill(hidden, -float("inf")), 1)
+            out[:, h] = w @ v[h // group]
+            spread[:, h] = ((w * w) @ (v[h // group] ** 2)).sqrt()
+        outs.append(out.reshape(n, -1))
+        spreads.append(spread.reshape(n, -1))
+        r0 += n
+    return torch.cat(outs), torch.cat(spreads)
+
+
+def attention_tolerance(want, spread):
+    """Bound on |library - float64|.  The output is rounded to bf16 (2^-9 of it); every weight is, before it multiplies its V
+    row: independent errors of at most 2^-9 w v and a root mean square below 2^-9 w v / sqrt(3), so ten standard deviations
+    of their sum are 5.8 * 2^-9 * sqrt(sum w^2 v^2).  Scores, exponentials and sums are fp32 (below 2^-16 of a weight)."""
+    return 2.0 ** -9 * (1.02 * want.abs() + 6.0 * spread) + 1e-6
+
+
+def layer0_attention(eng, tokens, cu, lens, rows):
+    """(q, attention output) of layer 0 for one verify call, tapped in two calls on the same state."""
+    import torch
+    from paper_2602_12957_b200 import binding as B
+    cfg, total = eng.model.cfg, int(sum(rows))
+    got = []
+    for which in (B.HSD_TAP_Q, B.HSD_TAP_ATTN):
+        eng.kv.seq_lens[:len(lens)] = torch.tensor(lens, dtype=torch.int32, device=eng.dev)
+        out = torch.empty(total, cfg.n_heads * cfg.head_dim, dtype=torch.bfloat16, device=eng.dev)
+        B.check(B.hsd_debug_tap(eng.model.ctx, 0, which, out, 2 * out.numel()))
+        eng.verify_regions(tokens, cu, int(max(rows)), total)
+        eng.check_device()
+        got.append(out)
+    return got
