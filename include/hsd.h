@@ -389,7 +389,8 @@ HSD_API int hsd_debug_set_gemm_tile(hsd_ctx *ctx, int tile_n, int k_slices);
 
 /* Test-only: the attention launch cuts the KV ranges of the query tiles into slices so that it has about `target_items`
  * work items (never more than CTA slots in one round), none shorter than `min_kv_tiles` 128-token KV tiles (two paged
- * blocks; 0 = the library's defaults).
+ * blocks; 0 = the library's defaults).  With `min_kv_tiles` > 0 a range is cut that finely wherever there are CTA slots and
+ * workspace for it, also where the library would not think it worth its cost.
  * Results do not depend on the setting beyond fp32 summation order; tests use it to force many or no slices. */
 HSD_API int hsd_debug_set_attn_plan(hsd_ctx *ctx, int target_items, int min_kv_tiles);
 

@@ -41,6 +41,7 @@ struct hsd_ctx {
   int force_bn, force_splits;   // hsd_debug_set_gemm_tile
   int pair;                     // GEMMs may run as CTA pairs
   int attn_target_items, attn_min_chunk;   // attention plan: units (share x kv head) aimed at per launch, shortest slice in KV blocks
+  bool attn_fine;                          // hsd_debug_set_attn_plan has named the shortest slice
   int tap_layer, tap_which;                // hsd_debug_tap: armed for the next forward (tap_layer < 0: none)
   void* tap_dst;
   size_t tap_bytes;
@@ -317,6 +318,7 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
     sa.rule.max_shares = max(1, min(w.plan.max_shares, c->attn_target_items / md.Hkv));
     sa.rule.min_chunk = c->attn_min_chunk;
     sa.rule.no_cut = c->max_splits == 1;
+    sa.rule.fine = c->attn_fine;
     launch_setup_rows(st, sa, kv, w.rm, c->pdl);
   }
 
@@ -604,6 +606,7 @@ int hsd_create(const hsd_model_config* cfg, const hsd_weights* w, hsd_ctx** out)
   c->hg_launches = 0;
   c->attn_target_items = attn_grid(c);
   c->attn_min_chunk = attn_min_chunk(c->md);
+  c->attn_fine = false;
   c->tap_layer = -1; c->tap_which = 0; c->tap_dst = nullptr; c->tap_bytes = 0;
   c->last_cuda_error = 0;
   c->launches = 0;
@@ -1153,6 +1156,7 @@ int hsd_debug_set_attn_plan(hsd_ctx* c, int target_items, int min_kv_tiles) {
   if (!c || target_items < 0 || min_kv_tiles < 0) return HSD_ERR_INVALID_ARG;
   c->attn_target_items = target_items ? target_items : attn_grid(c);
   c->attn_min_chunk = min_kv_tiles ? 2 * min_kv_tiles : attn_min_chunk(c->md);
+  c->attn_fine = min_kv_tiles != 0;
   return HSD_OK;
 }
 

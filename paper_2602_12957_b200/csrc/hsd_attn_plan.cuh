@@ -99,13 +99,13 @@ __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvVi
   }
   __syncthreads();
   const int longest = s_longest, mean = (s_blocks + max_shares - 1) / max_shares;
-  const int shortest = max(min_chunk, (int)ceilf(sqrtf(kSliceCost * (float)longest)));
+  const int shortest = rule.fine ? min_chunk : max(min_chunk, (int)ceilf(sqrtf(kSliceCost * (float)longest)));
   // one round: the slice length is grown until the items fit the slots
   int chunk = max(shortest, mean);
   auto slices_of = [&](int n) -> int {
     if (n <= whole) return 1;
     const int ns = (n + chunk - 1) / chunk;
-    return ns == 4 && n <= kThreeSlices ? 3 : ns;
+    return ns == 4 && n <= kThreeSlices && !rule.fine ? 3 : ns;
   };
   bool line = n_tiles > max_shares;
   if (no_cut) {

@@ -72,6 +72,7 @@ struct AttnPlan {
 struct AttnPlanRule {
   int max_shares, min_chunk;   // see make_attn_plan
   bool no_cut;
+  bool fine;                   // slices as short as min_chunk, whatever cutting costs (hsd_debug_set_attn_plan)
 };
 
 // ---- small kernels (hsd_small.cu) ---------------------------------------------------------------
