@@ -28,8 +28,6 @@ __device__ __forceinline__ int attn_unit_at(int bx, int n, int G) {
 // 4 / 6 / 8 / 12 / 16 blocks: one q-tile of 32 blocks 0.881 / 0.862 / 0.885 / 0.904 / 0.971 ms; one of 126 blocks 1.272 /
 // 1.153 / 1.112 / 1.061 / 1.067; two of 75 blocks 1.255 / 1.226 / 1.175 / 1.149 / 1.193; 16 of 4 to 17 blocks 0.878 / 0.879 /
 // 0.884 / 0.886 / 0.927; two of 7 blocks cut in half 0.950, whole 0.921.
-// Results are added up three at a time, so a fourth slice costs a round (~1 us): up to kThreeSlices blocks are cut in three
-// where four would save two blocks' time at most (12 regions of ~50 rows and up to 24 blocks: 1.284 ms with four, 1.269 with three).
 // Line: where that leaves the longest slice more than kLineGain blocks above the mean, or above kLineGain (more q-tiles than slots, or
 // q-tiles a little longer than the mean, which only halves would shorten), the q-tiles' ranges are laid end to end, each
 // with kTileCost blocks added for what an item costs beside its blocks (Q, first product, output), and the line is cut into
@@ -39,7 +37,7 @@ __device__ __forceinline__ int attn_unit_at(int bx, int n, int G) {
 // 7,936 2.07 / 2.02.
 // no_cut (contexts with a fixed summation order): q-tiles are never cut, cuts of the line move to the nearer edge.
 constexpr float kSliceCost = 1.4f;
-constexpr int kTileCost = 3, kMinPiece = 2, kLineGain = 8, kPlanTiles = 512, kThreeSlices = 24;
+constexpr int kTileCost = 3, kMinPiece = 2, kLineGain = 8, kPlanTiles = 512;
 template <int THREADS>
 __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvView& kv, const AttnPlanRule& rule, int n_seqs,
                                int n_tiles, int tokens_per_tile) {
@@ -102,11 +100,7 @@ __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvVi
   const int shortest = rule.fine ? min_chunk : max(min_chunk, (int)ceilf(sqrtf(kSliceCost * (float)longest)));
   // one round: the slice length is grown until the items fit the slots
   int chunk = max(shortest, mean);
-  auto slices_of = [&](int n) -> int {
-    if (n <= whole) return 1;
-    const int ns = (n + chunk - 1) / chunk;
-    return ns == 4 && n <= kThreeSlices && !rule.fine ? 3 : ns;
-  };
+  auto slices_of = [&](int n) -> int { return n <= whole ? 1 : (n + chunk - 1) / chunk; };
   bool line = n_tiles > max_shares;
   if (no_cut) {
     chunk = longest;
