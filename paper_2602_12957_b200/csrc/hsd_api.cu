@@ -94,8 +94,9 @@ struct Ws {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Shortest slice of a q-tile's KV range in 64-key blocks: see make_attn_plan.  (Heads of 128: a block takes longer and a
-// slice's result is twice the size; 8 regions of ~20 rows, 8 layers: 0.650 ms at 6, 0.647 at 8.)
+// Shortest slice of a q-tile's KV range in 64-key blocks: see make_attn_plan.  Heads of 128: a slice's result is twice the
+// size, so ranges of 9 and 10 blocks stay whole too.  1 / 4 / 8 / 16 regions of 9 blocks, 8 layers: 496 / 515 / 598 / 721 us at
+// 8, 507 / 530 / 624 / 735 at 6; of 7 and 12 blocks alike; of 16 blocks 527 / 555 / 653 / 774 at 8, 521 / 551 / 656 / 772 at 6.
 inline int attn_min_chunk(const ModelDims& md) { return md.D == 128 ? 8 : 6; }
 
 // CTAs of an attention launch: as many as are resident at once
@@ -394,7 +395,7 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
         Scope s(c, st, KC_ATTN);
         if (c->attn_simt) {
           launch_attn_simt(st, w.q, w.rm, kv, md, l, w.attn, T, w.status);
-        } else if (launch_attn_sm100(st, tm_q, tm_k, tm_v, w.plan, kv, md, l, w.attn, c->n_sms, c->device, w.status, w.split_ws,
+        } else if (launch_attn_sm100(st, tm_q, tm_k, tm_v, w.plan, kv, md, l, w.attn, c->device, w.status, w.split_ws,
                                      a.parent ? w.rm.anc : nullptr, c->pdl)) {
           return fail_cuda(c);
         }

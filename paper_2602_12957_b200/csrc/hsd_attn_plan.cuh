@@ -25,16 +25,15 @@ __device__ __forceinline__ int attn_unit_at(int bx, int n, int G) {
 // with two.  Cutting costs a hand-over (~3 us, five blocks' time), so a q-tile of up to 4/3 min_chunk blocks stays whole, and
 // the last slice to finish adds up the others' results (~0.6 us each, about a block's time): n blocks in slices of c take
 // c + kSliceCost n / c, which is least at c = sqrt(kSliceCost n).  Measured, steps of the 24-layer decoder in slices of
-// 4 / 6 / 8 / 12 / 16 blocks: one q-tile of 32 blocks 0.881 / 0.862 / 0.885 / 0.904 / 0.971 ms; one of 126 blocks 1.272 /
-// 1.153 / 1.112 / 1.061 / 1.067; two of 75 blocks 1.255 / 1.226 / 1.175 / 1.149 / 1.193; 16 of 4 to 17 blocks 0.878 / 0.879 /
-// 0.884 / 0.886 / 0.927; two of 7 blocks cut in half 0.950, whole 0.921.
+// 4 / 6 / 8 / 12 / 16 blocks, relative to the best: one q-tile of 32 blocks 1.02 / 1 / 1.03 / 1.05 / 1.13; one of 126 blocks
+// 1.20 / 1.09 / 1.05 / 1 / 1.01; two of 75 blocks 1.09 / 1.07 / 1.02 / 1 / 1.04; 16 of 4 to 17 blocks 1 / 1 / 1.01 / 1.01 / 1.06;
+// two of 7 blocks cut in half 1.03, whole 1.
 // Line: where that leaves the longest slice more than kLineGain blocks above the mean, or above kLineGain (more q-tiles than slots, or
 // q-tiles a little longer than the mean, which only halves would shorten), the q-tiles' ranges are laid end to end, each
 // with kTileCost blocks added for what an item costs beside its blocks (Q, first product, output), and the line is cut into
 // equal shares; a cut that would leave a piece of fewer than kMinPiece blocks moves to the q-tile's edge.
 // Measured, step times with equal shares of the line always against one round always: 2,048 rows over 16,384 (33
-// q-tiles of 272 blocks on 37 slots) 7.10 / 7.57 ms; 16 regions (25 q-tiles of 4 to 17 blocks) 1.78 / 1.73; 512 rows over
-// 7,936 2.07 / 2.02.
+// q-tiles of 272 blocks on 37 slots) 0.94; 16 regions (25 q-tiles of 4 to 17 blocks) 1.03; 512 rows over 7,936 1.025.
 // no_cut (contexts with a fixed summation order): q-tiles are never cut, cuts of the line move to the nearer edge.
 constexpr float kSliceCost = 1.4f;
 constexpr int kTileCost = 3, kMinPiece = 2, kLineGain = 8, kPlanTiles = 512;

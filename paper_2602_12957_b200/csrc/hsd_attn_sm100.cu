@@ -29,13 +29,8 @@
 // exponentials start as soon as their scores are in registers, and the row sum, which is needed anyway, shows whether a
 // score has outgrown the reference (P and the sums are scale-free in bf16 / fp32 as long as they stay in range).  Where
 // a sum of 64 exceeds kRescaleSum the 64 are taken again under a new reference and the accumulator row is rescaled.
-// Measured, one launch of a 2,048-row chunk over 16,384 committed rows, 16 / 8 heads of 64: 294 us with eight softmax
-// warps, two threads a row swapping maxima through shared memory ahead of the exponentials, on 128-key tiles with one
-// score buffer; 274 us with one thread a row and the reference checked by the sum; 245 us with 64-key blocks, rotating
-// score buffers and elected issue.  8 heads of 128: 233 us (one CTA per SM) to 145 us.  A block takes the two CTAs of an
-// SM 1,340 cycles for their two (the exp unit would need 1,024); of a softmax warp's own ~1,100 cycles 700 are the 64
-// exponentials of its rows.  Fetching the next block's scores before the P store is waited for was slower (register
-// moves), and so was a barrier probe without the suspend-time hint.
+// Measured, one launch of a 2,048-row chunk over 16,384 committed rows: 245 us with 16 / 8 heads of 64, 145 us with 8
+// heads of 128; with two threads a row that agree on a maximum first, on 128-key tiles with one score buffer, a fifth longer.
 // Every wait is a bounded mbarrier wait, so one that gives up takes the whole CTA to the common exit.
 #include "hsd_attn_plan.cuh"
 #include "hsd_kernels.h"
@@ -141,8 +136,8 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   // The plan's record of this CTA's first item (the item and the physical blocks of its first keys) for the two warps
   // that start the pipeline: read together with the status word and the share count, ahead of the CTA's own set-up, so that
   // the first TMA loads do not wait for a chain of dependent reads (status -> count -> item -> block table).
-  // (Read after the set-up, with the first item's Q behind its K and V, a CTA that could not start early formed its first
-  // scores 3.3 us after its entry, now 2.4: regions 1.671 -> 1.647 ms, page chunk 1.998 -> 1.954.)
+  // (Read after the set-up, with the first item's Q behind its K and V, a CTA that cannot start early forms its first
+  // scores 0.9 us later.)
   // All of it, like the block table and the K/V rows committed before this step, was written before the kernel that
   // precedes this one in the step: that kernel waited for ITS predecessor before it let this one start, so these reads
   // need no wait of their own, and the first K/V blocks load while the predecessor (which writes q and this step's own
@@ -597,8 +592,8 @@ done:
 }
 
 int launch_attn_sm100(cudaStream_t st, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
-                      const AttnPlan& plan, const KvView& kv, const ModelDims& md, int layer, bf16* out, int n_sms,
-                      int device, int* status, float* split_ws, const uint4* anc, bool pdl) {
+                      const AttnPlan& plan, const KvView& kv, const ModelDims& md, int layer, bf16* out, int device,
+                      int* status, float* split_ws, const uint4* anc, bool pdl) {
   static bool attr_set[2][kMaxDevices] = {};       // the attribute is per kernel and device
   if (device < 0 || device >= kMaxDevices || (md.D != 64 && md.D != 128)) return -1;
   const int which = md.D == 128;

@@ -3,9 +3,10 @@
 //
 // One persistent CTA per SM walks work units (128 x BN output tile, optionally one slice of K), M fastest so
 // CTAs running side by side share a weight tile through L2.  Warp roles:
-//   warp 0      A producer: activation tile, one 128-row TMA box per stage
+//   warp 0      A producer: activation tile, one TMA box per 64-column sub-tile of a stage, of 16, 32, 64 or 128 rows by the
+//               rows of the call (gemm_a_box_rows)
 //   warp 1      MMA issuer and TMEM owner
-//   warp 2      B producer: the two halves of the weight tile, one TMA box each per stage (a pair's CTA: its half).
+//   warp 2      B producer: the two halves of the weight tile, one TMA box each per sub-tile (a pair's CTA: its half).
 //               Weights do not depend on the previous kernel, so it starts before the programmatic-launch wait.
 //   warps 4..7  epilogue, one TMEM lane quarter each (warp w works on lane quarter w mod 4, the hardware's rule)
 // Warps 0 to 2 elect one lane that runs their whole loop.  With `elect` the compiler knows that one thread is active, and

@@ -45,8 +45,8 @@ inline int launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t
 }
 
 enum KernelClass {
-  KC_SETUP = 0, KC_EMBED, KC_RMSNORM, KC_GEMM_QKV, KC_ROPE_KV, KC_ATTN, KC_ATTN_COMBINE, KC_GEMM_O, KC_GEMM_GATEUP,
-  KC_GEMM_DOWN, KC_LMHEAD, KC_ACCEPT, KC_COMMIT, KC_DEBUG, KC_COUNT
+  KC_SETUP = 0, KC_RMSNORM, KC_GEMM_QKV, KC_ROPE_KV, KC_ATTN, KC_GEMM_O, KC_GEMM_GATEUP, KC_GEMM_DOWN, KC_LMHEAD, KC_ACCEPT,
+  KC_COMMIT, KC_DEBUG, KC_COUNT
 };
 const char* kernel_class_name(int kc);
 
@@ -200,8 +200,8 @@ void launch_unpack_best(cudaStream_t st, const unsigned long long* row_best, int
 
 // ---- attention (hsd_attn_sm100.cu) ----
 int launch_attn_sm100(cudaStream_t st, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
-                      const AttnPlan& plan, const KvView& kv, const ModelDims& md, int layer, bf16* out, int n_sms,
-                      int device, int* status, float* split_ws, const uint4* anc, bool pdl);
+                      const AttnPlan& plan, const KvView& kv, const ModelDims& md, int layer, bf16* out, int device,
+                      int* status, float* split_ws, const uint4* anc, bool pdl);
 
 // ---- plain SIMT GEMM (hsd_gemm_simt.cu): the debug cross-check and hsd_debug_logits --------------
 enum GemmMode { GM_STORE_BF16 = 0, GM_ADD_F32 = 1, GM_SWIGLU = 2, GM_STORE_F32 = 3, GM_ARGMAX = 4 };

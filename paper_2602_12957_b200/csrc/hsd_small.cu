@@ -6,9 +6,8 @@
 namespace hsd {
 
 const char* kernel_class_name(int kc) {
-  static const char* names[KC_COUNT] = {"setup_rows", "embed",     "rmsnorm",     "gemm_qkv",  "rope_kv_write",
-                                        "attention",  "attn_combine", "gemm_o",   "gemm_gate_up", "gemm_down",
-                                        "lm_head_argmax", "accept_emit", "kv_commit", "debug"};
+  static const char* names[KC_COUNT] = {"setup_rows", "rmsnorm",   "gemm_qkv",       "rope_kv_write", "attention", "gemm_o",
+                                        "gemm_gate_up", "gemm_down", "lm_head_argmax", "accept_emit",   "kv_commit", "debug"};
   return (kc >= 0 && kc < KC_COUNT) ? names[kc] : "?";
 }
 
@@ -36,7 +35,7 @@ __global__ void __launch_bounds__(kSetupThreads) setup_rows_kernel(SetupArgs a, 
   __shared__ int s_cu[kSetupMaxCu + 1];
   __shared__ int s_code, s_where;
   __shared__ int s_par[HSD_MAX_TREE_ROWS + kSetupRows];
-  __shared__ int s_tok[kSetupRows], s_depth[kSetupRows], s_len[kSetupRows];
+  __shared__ int s_tok[kSetupRows], s_len[kSetupRows];
   __shared__ int s_warp[kSetupThreads / 32];
   int2* verdict = a.verdict + (blockIdx.x ? blockIdx.x - 1 : gridDim.x - 1);     // the rows' ahead of the sequences'
   if (tid == 0) s_code = s_where = 0;
