@@ -28,6 +28,8 @@ __device__ __forceinline__ int attn_unit_at(int bx, int n, int G) {
 // 4 / 6 / 8 / 12 / 16 blocks, relative to the best: one q-tile of 32 blocks 1.02 / 1 / 1.03 / 1.05 / 1.13; one of 126 blocks
 // 1.20 / 1.09 / 1.05 / 1 / 1.01; two of 75 blocks 1.09 / 1.07 / 1.02 / 1 / 1.04; 16 of 4 to 17 blocks 1 / 1 / 1.01 / 1.01 / 1.06;
 // two of 7 blocks cut in half 1.03, whole 1.
+// Results are added up three at a time, so a fourth slice costs a round (~1 us): up to kThreeSlices blocks are cut in three
+// where four would save two blocks' time at most.
 // Line: where that leaves the longest slice more than kLineGain blocks above the mean, or above kLineGain (more q-tiles than slots, or
 // q-tiles a little longer than the mean, which only halves would shorten), the q-tiles' ranges are laid end to end, each
 // with kTileCost blocks added for what an item costs beside its blocks (Q, first product, output), and the line is cut into
@@ -36,7 +38,7 @@ __device__ __forceinline__ int attn_unit_at(int bx, int n, int G) {
 // q-tiles of 272 blocks on 37 slots) 0.94; 16 regions (25 q-tiles of 4 to 17 blocks) 1.03; 512 rows over 7,936 1.025.
 // no_cut (contexts with a fixed summation order): q-tiles are never cut, cuts of the line move to the nearer edge.
 constexpr float kSliceCost = 1.4f;
-constexpr int kTileCost = 3, kMinPiece = 2, kLineGain = 8, kPlanTiles = 512;
+constexpr int kTileCost = 3, kMinPiece = 2, kLineGain = 8, kPlanTiles = 512, kThreeSlices = 24;
 template <int THREADS>
 __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvView& kv, const AttnPlanRule& rule, int n_seqs,
                                int n_tiles, int tokens_per_tile) {
@@ -99,7 +101,11 @@ __device__ void make_attn_plan(const RowMeta& rm, const AttnPlan& pl, const KvVi
   const int shortest = rule.fine ? min_chunk : max(min_chunk, (int)ceilf(sqrtf(kSliceCost * (float)longest)));
   // one round: the slice length is grown until the items fit the slots
   int chunk = max(shortest, mean);
-  auto slices_of = [&](int n) -> int { return n <= whole ? 1 : (n + chunk - 1) / chunk; };
+  auto slices_of = [&](int n) -> int {
+    if (n <= whole) return 1;
+    const int ns = (n + chunk - 1) / chunk;
+    return ns == 4 && n <= kThreeSlices && !rule.fine ? 3 : ns;
+  };
   bool line = n_tiles > max_shares;
   if (no_cut) {
     chunk = longest;
