@@ -1,6 +1,6 @@
 """Attention over every form of plan against a float64 softmax of the same bf16 queries, keys and values: the context lengths
-where the number of slices of a q-tile changes (8 KV blocks stay whole, 9 are cut in two, up to 24 in three, a long context in
-a square root's worth), slices as short as they come (4, 5, 7 and more of a q-tile: the combining pass takes three at a
+where the number of slices of a q-tile changes (8 KV blocks stay whole, heads of 128: 10; 12 are cut in two, 24 in three, 25 in
+five, a long context in a square root's worth), slices as short as they come (4, 5, 7 and more of a q-tile: the combining pass takes three at a
 time), whole ranges, and equal shares of the line with a q-tile cut across several shares.  Keys are spread widely enough that
 a q-tile's slices differ in maximum and sum."""
 import numpy as np
