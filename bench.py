@@ -39,9 +39,9 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # captures summarised under profiles/, per workload; a class is absent (-> null) when its kernel has changed since
 # its counters were taken, or when no capture of that workload exists.
 NCU_TRAFFIC_BYTES = {
-    "region": {"attention": 30_975_744 + 4_352, "gemm_gate_up": 19_522_048, "gemm_qkv": 7_284_992 + 1_280,
-               "gemm_o": 10_249_984, "gemm_down": 24_669_696},
-    "long2048": {"attention": 42_460_928 + 4_530_176},
+    "region": {"attention": 30_976_768 + 512, "gemm_gate_up": 19_521_024, "gemm_qkv": 7_287_296 + 4_608,
+               "gemm_o": 10_247_936, "gemm_down": 24_669_440},
+    "long2048": {"attention": 42_723_584 + 3_332_096},
 }
 
 

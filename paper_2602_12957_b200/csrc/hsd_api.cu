@@ -95,8 +95,8 @@ struct Ws {
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Shortest slice of a q-tile's KV range in 64-key blocks: see make_attn_plan.  Heads of 128: a slice's result is twice the
-// size, so ranges of 9 and 10 blocks stay whole too.  1 / 4 / 8 / 16 regions of 9 blocks, 8 layers: 496 / 515 / 598 / 721 us at
-// 8, 507 / 530 / 624 / 735 at 6; of 7 and 12 blocks alike; of 16 blocks 527 / 555 / 653 / 774 at 8, 521 / 551 / 656 / 772 at 6.
+// size, so ranges of 9 and 10 blocks stay whole too.  1 / 4 / 8 regions of 9 blocks, 8 layers, graph replays: 477 / 499 / 578 us at
+// 8, 486 / 511 / 602 at 6; of 7 and 12 blocks alike; of 16 blocks 507 / 533 / 634 at 8, 504 / 529 / 634 at 6.
 inline int attn_min_chunk(const ModelDims& md) { return md.D == 128 ? 8 : 6; }
 
 // CTAs of an attention launch: as many as are resident at once
