@@ -141,15 +141,16 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   // All of it, like the block table and the K/V rows committed before this step, was written before the kernel that
   // precedes this one in the step: that kernel waited for ITS predecessor before it let this one start, so these reads
   // need no wait of their own, and the first K/V blocks load while the predecessor (which writes q and this step's own
-  // K/V rows) is still running.
+  // K/V rows) is still running.  They go to L2, where completed kernels have left it: a line that an earlier launch put into
+  // this SM's L1 may be a former step's.
   int4 rec_a = make_int4(0, 0, 0, 0), rec_b = rec_a, rec_c = rec_a;
   if (warp < 2) {
     const int4* rec = p.plan.first + 3 * (size_t)blockIdx.x;
-    rec_a = rec[0];
-    rec_b = rec[1];
-    rec_c = rec[2];
+    rec_a = __ldcg(rec);
+    rec_b = __ldcg(rec + 1);
+    rec_c = __ldcg(rec + 2);
   }
-  const int status_now = *p.status, n_shares_now = *p.plan.n_shares;
+  const int status_now = __ldcg(p.status), n_shares_now = __ldcg(p.plan.n_shares);
   if (threadIdx.x == 32) {
     tma_prefetch_desc(&tmK);
     tma_prefetch_desc(&tmV);
@@ -215,7 +216,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       const int4 ia = recorded ? rec_a : p.plan.items[2 * i], ib = recorded ? rec_b : p.plan.items[2 * i + 1];
       const int kt_lo = ib.x & 0xffff, kt_hi = ib.x >> 16;
       const int* bt = p.block_table + (size_t)ia.w * p.max_blocks;
-      auto phys_of = [&](int kt) -> int { return recorded && kt < kt_lo + 2 ? (kt == kt_lo ? rec_c.z : rec_c.w) : bt[kt]; };
+      auto phys_of = [&](int kt) -> int { return recorded && kt < kt_lo + 2 ? (kt == kt_lo ? rec_c.z : rec_c.w) : __ldcg(bt + kt); };
       int early = kt_lo;                                 // K and V of [kt_lo, early) are on their way
       if (recorded) {
         // blocks that hold committed rows only, as many as the rings take, ahead of the grid dependency
