@@ -383,7 +383,8 @@ HSD_API int hsd_op_linear(hsd_ctx *ctx, const void *A, const void *W, void *C, i
 
 /* Test-only: make hsd_op_linear use output tiles of `tile_n` columns (64, 128, 256, or 512 = a pair of CTAs sharing a
  * 256-row x 256-column tile) and, for mode 1, `k_slices`
- * slices of K per tile, instead of what the library would choose for the problem; 0 = choose.  A combination the
+ * slices of K per tile (the 64-wide tile cuts K in steps of 128 columns, into fewer slices where one would be empty),
+ * instead of what the library would choose for the problem; 0 = choose.  A combination the
  * problem does not allow makes hsd_op_linear return HSD_ERR_CUDA.  Lets the parity tests reach every tile shape. */
 HSD_API int hsd_debug_set_gemm_tile(hsd_ctx *ctx, int tile_n, int k_slices);
 

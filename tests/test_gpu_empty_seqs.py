@@ -7,10 +7,10 @@ from paper_2602_12957_b200 import inputs as I
 
 pytestmark = pytest.mark.gpu
 
-S, HAVE = 700, {0: 3, 7: 1, 500: 4, 699: 2}          # sequence -> rows; 700 sequences, 10 rows
+HAVE = {0: 3, 7: 1, 500: 4, 699: 2}                  # sequence -> rows (10 in all)
 
 
-def _engine():
+def _engine(S):
     import torch
     from paper_2602_12957_b200 import binding as B
     from paper_2602_12957_b200 import runtime as R
@@ -26,9 +26,10 @@ def _engine():
 
 
 @pytest.mark.parametrize("prefill", [False, True])
-def test_more_sequences_than_rows(prefill):
+@pytest.mark.parametrize("S", [700, 1500])
+def test_more_sequences_than_rows(S, prefill):
     import torch
-    eng = _engine()
+    eng = _engine(S)
     rows = np.array([HAVE.get(i, 0) for i in range(S)])
     some = sorted(HAVE)
     toks = eng._i32(np.random.default_rng(2).integers(0, I.TINY.vocab, rows.sum()))
