@@ -381,8 +381,9 @@ HSD_API int hsd_debug_tap(hsd_ctx *ctx, int layer, int which, void *dst, size_t 
 HSD_API int hsd_op_linear(hsd_ctx *ctx, const void *A, const void *W, void *C, int M, int n_out, int K, int mode,
                   void *cuda_stream);
 
-/* Test-only: make hsd_op_linear use output tiles of `tile_n` columns (64, 128, 256, or 512 = a pair of CTAs sharing a
- * 256-row x 256-column tile) and, for mode 1, `k_slices`
+/* Test-only: make hsd_op_linear use output tiles of `tile_n` columns (64, 128, 192 or
+ * 256, mode 1 also 96 and 160, mode 2 also 160 and 224; 256 + n = a pair of CTAs sharing a tile of 256 rows and n columns,
+ * n = 128, 192 or 256, mode 1 also 96, 160 and 224, mode 2 also 160 and 224) and, for mode 1, `k_slices`
  * slices of K per tile (the 64-wide tile cuts K in steps of 128 columns, into fewer slices where one would be empty),
  * instead of what the library would choose for the problem; 0 = choose.  A combination the
  * problem does not allow makes hsd_op_linear return HSD_ERR_CUDA.  Lets the parity tests reach every tile shape. */

@@ -387,7 +387,7 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
         g.qkv.v_pool_layer = kv.v_pool + (size_t)l * layer_elems;
         g.qkv.Hq = md.Hq; g.qkv.Hkv = md.Hkv; g.qkv.D = md.D;
         g.qkv.q_norm = c->q_norm[l]; g.qkv.k_norm = c->k_norm[l]; g.qkv.eps = md.eps;
-        g.status = w.status; g.n_sms = c->n_sms; g.device = c->device; g.max_splits = 1; g.pdl = c->pdl; g.pair = c->pair;
+        g.status = w.status; g.n_sms = c->n_sms; g.max_splits = 1; g.pdl = c->pdl; g.pair = c->pair;
         g.force_bn = c->force_bn;
         if (launch_gemm_sm100(st, g)) return fail_cuda(c);
       }
@@ -407,7 +407,7 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
         g.tmB = &c->tm_o[l];
         g.tmC = tm_x_add;
         g.M = T; g.n_out = md.d; g.K = md.Hq * md.D; g.mode = GS_ADD_F32;
-        g.status = w.status; g.n_sms = c->n_sms; g.device = c->device; g.max_splits = c->max_splits; g.pdl = c->pdl; g.pair = c->pair;
+        g.status = w.status; g.n_sms = c->n_sms; g.max_splits = c->max_splits; g.pdl = c->pdl; g.pair = c->pair;
         if (launch_gemm_sm100(st, g)) return fail_cuda(c);
       }
     }
@@ -439,7 +439,7 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
         g.tmC = tm_act_st;
         g.M = T; g.n_out = 2 * md.ffn; g.K = md.d; g.mode = GS_SWIGLU;
         g.out.C = w.act; g.out.ldc = md.ffn;
-        g.status = w.status; g.n_sms = c->n_sms; g.device = c->device; g.max_splits = 1; g.pdl = c->pdl; g.pair = c->pair;
+        g.status = w.status; g.n_sms = c->n_sms; g.max_splits = 1; g.pdl = c->pdl; g.pair = c->pair;
         if (launch_gemm_sm100(st, g)) return fail_cuda(c);
       }
       {
@@ -449,7 +449,7 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
         g.tmB = &c->tm_down[l];
         g.tmC = tm_x_add;
         g.M = T; g.n_out = md.d; g.K = md.ffn; g.mode = GS_ADD_F32;
-        g.status = w.status; g.n_sms = c->n_sms; g.device = c->device; g.max_splits = c->max_splits; g.pdl = c->pdl; g.pair = c->pair;
+        g.status = w.status; g.n_sms = c->n_sms; g.max_splits = c->max_splits; g.pdl = c->pdl; g.pair = c->pair;
         if (launch_gemm_sm100(st, g)) return fail_cuda(c);
       }
     }
@@ -474,7 +474,7 @@ int run_lm_head(hsd_ctx* c, const Ws& w, int rows, const int* row_next, cudaStre
     g.tmB = &c->tm_lm_head;
     g.M = rows; g.n_out = md.V; g.K = md.d; g.mode = GS_ARGMAX;
     g.out = o;
-    g.status = w.status; g.n_sms = c->n_sms; g.device = c->device; g.max_splits = 1; g.pdl = c->pdl; g.pair = c->pair;
+    g.status = w.status; g.n_sms = c->n_sms; g.max_splits = 1; g.pdl = c->pdl; g.pair = c->pair;
     if (launch_gemm_sm100(st, g)) return fail_cuda(c);
   }
   return check_cuda(c);
@@ -615,7 +615,7 @@ int hsd_create(const hsd_model_config* cfg, const hsd_weights* w, hsd_ctx** out)
   memset(c->prof_ms, 0, sizeof(c->prof_ms));
   memset(c->prof_n, 0, sizeof(c->prof_n));
   if (!c->simt) {
-    if (tma_init()) { delete c; return HSD_ERR_CUDA; }
+    if (tma_init() || gemm_sm100_init(dev)) { delete c; return HSD_ERR_CUDA; }
     c->tm_qkv.resize(md.n_layers); c->tm_o.resize(md.n_layers);
     c->tm_gate_up.resize(md.n_layers); c->tm_down.resize(md.n_layers);
     int bad = 0;
@@ -1098,7 +1098,7 @@ static int lm_head_argmax_impl(hsd_ctx* c, const void* h, int rows, const int* n
       g.tmB = &c->tm_lm_head;
       g.M = rows; g.n_out = md.V; g.K = md.d; g.mode = GS_ARGMAX;
       g.out = o;
-      g.status = nullptr; g.n_sms = c->n_sms; g.device = c->device; g.max_splits = 1; g.pdl = false; g.pair = c->pair;
+      g.status = nullptr; g.n_sms = c->n_sms; g.max_splits = 1; g.pdl = false; g.pair = c->pair;
       if (launch_gemm_sm100(st, g)) return fail_cuda(c);
     }
   }
@@ -1180,7 +1180,7 @@ int hsd_op_linear(hsd_ctx* c, const void* A, const void* W, void* C, int M, int 
   g.tmB = &wm;
   g.M = M; g.n_out = n_out; g.K = K; g.mode = mode;
   g.out.C = C; g.out.ldc = ldc;
-  g.status = nullptr; g.n_sms = c->n_sms; g.device = c->device; g.max_splits = c->max_splits; g.pdl = false; g.pair = c->pair;
+  g.status = nullptr; g.n_sms = c->n_sms; g.max_splits = c->max_splits; g.pdl = false; g.pair = c->pair;
   g.force_bn = c->force_bn; g.force_splits = c->force_splits;
   if (launch_gemm_sm100(st, g)) return fail_cuda(c);
   return check_cuda(c);

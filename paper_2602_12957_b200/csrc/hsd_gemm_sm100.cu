@@ -85,7 +85,7 @@ int make_tmap_3d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, u
 
 int make_weight_tmaps(WeightMaps* w, const void* base, uint64_t rows, uint64_t cols) {
   int bad = 0;
-  for (int i = 0; i < 3; ++i) bad |= make_tmap_2d(&w->m[i], base, rows, cols, 32u << i);
+  for (int i = 0; i < WeightMaps::N; ++i) bad |= make_tmap_2d(&w->m[i], base, rows, cols, 16u * (i + 2));
   return bad;
 }
 
@@ -109,8 +109,8 @@ struct Cfg {
   static constexpr int B_SUB = (PAIR ? BN / 2 : BN) * KSUB * 2;     // bytes of one B sub-tile this CTA stages
   static constexpr int B_BYTES = B_SUB * KSTEPS;                    // bytes of B per stage
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = (PAIR ? 6 : BN == 256 ? 4 : BN == 128 ? 6 : 8) / KSTEPS;
-  static constexpr int TMEM_COLS = 2 * BN;
+  static constexpr int STAGES = 192 * 1024 / STAGE_BYTES < 8 ? 192 * 1024 / STAGE_BYTES : 8;
+  static constexpr int TMEM_COLS = BN <= 64 ? 128 : BN <= 128 ? 256 : 512;      // two accumulators, a power of two
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + STG_TOTAL + 1024 /*alignment slack*/ + 256 /*barriers*/;
 };
 
@@ -211,7 +211,7 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const uint32_t tmem_base = *tmem_slot;
 
   const int m_tiles = (p.M + TILE_M - 1) / TILE_M;
-  const int n_tiles = p.n_cols / OUT_N;
+  const int n_tiles = (p.n_cols + OUT_N - 1) / OUT_N;      // (96, 160, 192 and 224 columns: the last tile may reach beyond)
   const int tiles = m_tiles * n_tiles;
   const int total = tiles * p.splits;
   const int k_blocks = (p.K + BK - 1) / BK;      // (a last stage beyond K is filled with zeros)
@@ -357,7 +357,7 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       // lets "at most one group pending" protect the buffer about to be rewritten.
       if (MODE == GS_STORE_BF16) {
 #pragma unroll 1
-        for (int c = 0; slab_ok && c < BN; c += 64) {
+        for (int c = 0; slab_ok && c < BN && n0 + c < p.n_cols; c += 64) {
           uint8_t* buf = my_stg + (n_stores & 1) * STG_BYTES;
           if (lane == 0) bulk_wait_read<1>();      // the store that last read this buffer has drained
           __syncwarp();
@@ -380,7 +380,7 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
       } else if (MODE == GS_ADD_F32) {
 #pragma unroll 1
-        for (int c = 0; slab_ok && c < BN; c += 32) {
+        for (int c = 0; slab_ok && c < BN && n0 + c < p.n_cols; c += 32) {
           uint8_t* buf = my_stg + (n_stores & 1) * STG_BYTES;
           if (lane == 0) bulk_wait_read<1>();
           __syncwarp();
@@ -418,7 +418,7 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
       } else if (MODE == GS_SWIGLU) {
 #pragma unroll 1
-        for (int c = 0; slab_ok && c < OUT_N; c += 64) {
+        for (int c = 0; slab_ok && c + 64 <= OUT_N; c += 64) {
           uint8_t* buf = my_stg + (n_stores & 1) * STG_BYTES;
           if (lane == 0) bulk_wait_read<1>();
           __syncwarp();
@@ -445,6 +445,25 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             bulk_commit();
           }
           ++n_stores;
+        }
+        // what is left of 80, 96 or 112 outputs: whole 32-byte sectors, stored as they are
+#pragma unroll 1
+        for (int c = OUT_N / 64 * 64; OUT_N % 64 && slab_ok && c < OUT_N && n0 + c < p.n_cols; c += 16) {
+          uint32_t g[16], u[16];
+          tmem_ld16(t_acc + c, g);
+          tmem_ld16(t_acc + OUT_N + c, u);
+          tmem_ld_wait(g);
+          tmem_ld_wait(u);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            const float gv = __uint_as_float(g[e]);
+            g[e] = __float_as_uint(__fdividef(gv, 1.f + __expf(-gv)) * __uint_as_float(u[e]));
+          }
+          if (row_ok) {
+            uint4* dst = reinterpret_cast<uint4*>(static_cast<bf16*>(p.out.C) + (size_t)row * p.out.ldc + n0 + c);
+            dst[0] = pack8(g);
+            dst[1] = pack8(g + 8);
+          }
         }
       } else if (MODE == GS_ARGMAX) {
         float best_v = -INFINITY, zd = 0.f;
@@ -474,7 +493,7 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         for (int hh = 0; hh < BN / 64; ++hh) {
           const int head = n0 / 64 + hh;
           const bool is_q = head < p.qkv.Hq;
-          if (!slab_ok) break;
+          if (!slab_ok || head >= p.qkv.Hq + 2 * p.qkv.Hkv) break;
           uint8_t* buf = my_stg + (n_stores & 1) * STG_BYTES;
           if (is_q) {
             if (lane == 0) bulk_wait_read<1>();
@@ -666,14 +685,6 @@ template <int BN, int MODE, bool PAIR>
 static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
   using C = Cfg<BN, PAIR>;
   constexpr int OUT_N = (MODE == GS_SWIGLU) ? BN / 2 : BN;
-  static bool attr_set[kMaxDevices] = {};          // the attribute is per device
-  if (a.device < 0 || a.device >= kMaxDevices) return -1;
-  if (!attr_set[a.device]) {
-    if (cudaFuncSetAttribute(gemm_sm100_kernel<BN, MODE, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             C::SMEM_BYTES) != cudaSuccess)
-      return -1;
-    attr_set[a.device] = true;
-  }
   GemmDev p;
   p.M = a.M;
   p.K = a.K;
@@ -689,10 +700,10 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
   p.status = a.status;
   const int tile_m = PAIR ? 2 * BM : BM;
   const int m_tiles = (a.M + tile_m - 1) / tile_m;
-  const int total = m_tiles * (p.n_cols / OUT_N) * splits;
+  const int total = m_tiles * ((p.n_cols + OUT_N - 1) / OUT_N) * splits;
   const int walkers = PAIR ? a.n_sms / 2 : a.n_sms;
   const int grid = (total < walkers ? total : walkers) * (PAIR ? 2 : 1);
-  const CUtensorMap& tmB = a.tmB->m[PAIR ? 2 : (BN == 64 ? 0 : (BN == 128 ? 1 : 2))];   // pair: one 128-row box per CTA
+  const CUtensorMap& tmB = a.tmB->half_tile(BN);      // (a pair's CTA loads one box, others two)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kGemmThreads);
@@ -717,72 +728,118 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
   return cudaLaunchKernelEx(&cfg, gemm_sm100_kernel<BN, MODE, PAIR>, a.tmA, tmB, a.tmC, p) == cudaSuccess ? 0 : -1;
 }
 
-// Tile width, CTA pairing and K slices: fewest cycles by a model calibrated on B200.  A k-block costs the longer of its
-// MMAs (256-wide tiles run at the rate the whole chip's tensor pipes sustain: the measured library peak corresponds to
-// ~730 cycles for such a k-block, one SM alone would need 544), its fill (A box + weight tile at the ~55 B per clock an SM
-// takes from L2: measured 455 cycles for 16 + 8 KB, 560 for 16 + 16 KB) and ~250 of barrier round trip and issue.
-// Calls of at most 64 rows load activation boxes of 16, 32 or 64 rows: the rest of the MMA's 128 rows is whatever the
-// stage held (rows are independent, and rows beyond M go nowhere), where a full box would fill them with zeros at the
-// same cost as data.  A pair costs a cluster launch; the epilogue of the last unit of a CTA is exposed.
-static void pick_tile(int mode, int n_cols, int M, int K, int n_sms, int max_splits, bool allow_pair, int* bn_out,
-                      int* splits_out, bool* pair_out) {
+// Tile width, CTA pairing and K slices: the least time by a model of one launch, in us.  What decides is the last wave: a
+// projection of ~600 rows has 1.3 waves of 128 x 256 tiles, and 0.9 of 128 x 160.  So tiles come in seven widths, for single CTAs
+// and pairs, and any of them may be cut in up to eight K slices (residual adds).  Least squares over 3,900 timings (back to back
+// in a graph, 4 projections of the 24-layer decoder at 41 row counts from 16 to 9,300 and 4 of a decoder twice as wide at 7):
+//   a k-block of 64: by the rows filled (A box + tile width: L2 -> SM) with a floor, or by a pair's width; up to a quarter less
+//   where the launch leaves SMs idle; a wave: 0.7 / 0.8; the last epilogue: by width, residual adds dearest; a launch 2.4, a pair 0.9
+// more.  Calls of at most 64 rows load activation boxes of 16, 32 or 64 rows: the rest of the MMA's 128 rows is whatever the stage
+// held (rows are independent, and rows beyond M go nowhere), where a full box would fill them with zeros at the same cost as data.
+// Its choices are within 0.8 % of the best timed one on average (worst 8.5 %).  With widths of 64, 128 and 256 (pairs: 256) and a
+// model by fill rates alone it was 8.1 % (worst 70 %).  A layer's four projections, before / now: 300 rows 28.6 / 26.1 us, 600
+// rows 37.8 / 32.3, 900 rows 41.2 / 38.5, 1,323 rows 52.5 / 48.3, 2,600 rows 83 / 73, 5,000 rows 147 / 123, 9,300 rows 217 / 216.
+struct TileChoice {
+  int bn, splits;
+  bool pair;
+};
+// Tile widths a mode has: whole heads for the rotary epilogues, whole 64-column stores for the plain one; the adds take any 32
+// columns, SwiGLU any 16.
+constexpr bool has_width(int mode, int bn, bool pair) {
+  switch (bn) {
+    case 64: return !pair && mode != GS_QKV_ROPE128;
+    case 96: return mode == GS_ADD_F32;
+    case 160: return mode == GS_ADD_F32 || mode == GS_SWIGLU;
+    case 192: return mode == GS_ADD_F32 || mode == GS_SWIGLU || mode == GS_QKV_ROPE || mode == GS_STORE_BF16;
+    case 224: return (mode == GS_ADD_F32 && pair) || mode == GS_SWIGLU;
+    default: return bn == 128 || bn == 256;
+  }
+}
+// Where 96, 160, 192 or 224 do not divide the output's columns, the last tile reaches beyond: TMA fills weight rows beyond the
+// last with zeros and drops columns beyond the output's.
+static bool width_fits(int mode, int n_cols, int bn, bool pair) {
+  return has_width(mode, bn, pair) && ((bn & (bn - 1)) || n_cols % (mode == GS_SWIGLU ? bn / 2 : bn) == 0);
+}
+static TileChoice pick_tile(int mode, int n_cols, int M, int K, int n_sms, int max_splits, bool allow_pair) {
   const int k_blocks = K / KSUB;
-  const int cands[4] = {256, 256, 128, 64};     // first entry: a CTA pair on a 256 x 256 tile
-  double best_cost = 1e30;
-  *bn_out = mode == GS_QKV_ROPE128 ? 128 : 64;
-  *splits_out = 1;
-  *pair_out = false;
-  for (int i = allow_pair && M > 64 ? 0 : 1; i < 4; ++i) {       // (a pair's tile needs whole boxes)
-    const bool pair = i == 0;
-    const int bn = cands[i];
-    const int out_n = (mode == GS_SWIGLU) ? bn / 2 : bn;
-    if (n_cols % out_n || out_n % 32) continue;
-    if (mode == GS_QKV_ROPE128 && bn < 128) continue;     // a tile holds whole 128-column heads
-    const int tile_m = pair ? 2 * BM : BM;
-    const int walkers = pair ? n_sms / 2 : n_sms;
-    const long long tiles = (long long)((M + tile_m - 1) / tile_m) * (n_cols / out_n);
-    for (int sp = 1; sp <= max_splits; ++sp) {
-      const int kbs = (k_blocks + sp - 1) / sp;
-      if (sp > 1 && (kbs < 4 || (long long)(sp - 1) * kbs >= k_blocks)) continue;
-      const long long units = tiles * sp;
-      const long long rounds = (units + walkers - 1) / walkers;
-      const double fill = (double)(gemm_a_box_rows(M) + (pair ? bn / 2 : bn)) * (KSUB * 2) / 55.0;
-      const double per_kb = pair ? 770.0 : (fill > 250.0 ? fill : 250.0);
-      const double epi = 700.0 + (mode == GS_SWIGLU ? 13.0 : 20.0) * bn;     // measured: 3.0 us of reduce-adds for 256 columns
-      const double cost = (double)rounds * (kbs * per_kb + 300.0) + epi + (sp > 1 ? 200.0 * sp : 0.0) + (pair ? 1500.0 : 0.0);
-      if (cost < best_cost) { best_cost = cost; *bn_out = bn; *splits_out = sp; *pair_out = pair; }
+  TileChoice best = {mode == GS_QKV_ROPE128 ? 128 : 64, 1, false};
+  double best_us = 1e30;
+  const double epi = mode == GS_ADD_F32 ? 0.0105 : mode == GS_SWIGLU ? 0.0014 : mode == GS_STORE_BF16 ? 0.0036 : mode == GS_ARGMAX ? 0.015 : 0.0065;   // a column
+  for (int pair = allow_pair && M > 64 ? 1 : 0; pair >= 0; --pair) {      // (a pair's tile needs whole boxes)
+    for (int bn = 256; bn >= 64; bn -= 32) {
+      if (!width_fits(mode, n_cols, bn, pair != 0)) continue;
+      const int out_n = (mode == GS_SWIGLU) ? bn / 2 : bn;
+      const int tile_m = pair ? 2 * BM : BM;
+      const int walkers = pair ? n_sms / 2 : n_sms;
+      const long long tiles = (long long)((M + tile_m - 1) / tile_m) * ((n_cols + out_n - 1) / out_n);
+      const double fill = 0.00042 * gemm_a_box_rows(M) + 0.00122 * bn, least = bn == 64 ? 0.150 : 0.183;
+      double kb_us = pair ? (bn <= 96 ? 0.146 : 0.0137 + 0.00125 * bn) : (fill > least ? fill : least);
+      // the LM head's weights come from HBM, and a pair takes a tile of them once for 256 rows (144 rows: 20.3 us on 256-wide
+      // tiles, 17.9 on pairs of that width; 16 rows: 16.5, on 128-wide tiles 14.7)
+      if (mode == GS_ARGMAX && !pair && M > BM) kb_us *= 1.15;
+      for (int sp = 1; sp <= max_splits; ++sp) {
+        const int kbs = (k_blocks + sp - 1) / sp;
+        if (sp > 1 && (kbs < 2 || (long long)(sp - 1) * kbs >= k_blocks)) continue;
+        const long long units = tiles * sp;
+        const long long rounds = (units + walkers - 1) / walkers;
+        const double load = units < walkers ? (double)units / walkers : 1.0;
+        const double us = 2.4 + (pair ? 0.9 : 0.0) + rounds * (kbs * kb_us * (0.75 + 0.25 * load) + (pair ? 0.78 : 0.68)) +
+                          epi * bn + (sp > 1 ? 0.00073 * bn : 0.0);
+        if (us < 0.99 * best_us) { best_us = us; best = {bn, sp, pair != 0}; }      // (as good: the wider one, with less traffic)
+      }
     }
   }
+  return best;
+}
+
+template <int MODE, bool PAIR, int BN = 64>
+static int launch_width(cudaStream_t st, const GemmSm100Args& a, int bn, int splits) {
+  if constexpr (has_width(MODE, BN, PAIR))
+    if (bn == BN) return launch_one<BN, MODE, PAIR>(st, a, splits);
+  if constexpr (BN < 256) return launch_width<MODE, PAIR, BN + 32>(st, a, bn, splits);
+  return -1;
+}
+
+// The shared memory each kernel is launched with.  Asked for when a context is created, which also loads the kernels: the
+// first step that picks a width does not wait for that.
+template <int MODE, bool PAIR, int BN = 64>
+static bool allow_smem() {
+  bool ok = true;
+  if constexpr (has_width(MODE, BN, PAIR))
+    ok = cudaFuncSetAttribute(gemm_sm100_kernel<BN, MODE, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              Cfg<BN, PAIR>::SMEM_BYTES) == cudaSuccess;
+  if constexpr (BN < 256) ok = allow_smem<MODE, PAIR, BN + 32>() && ok;
+  return ok;
+}
+template <int... MODES>
+static bool allow_smem_all() {
+  return ((allow_smem<MODES, false>() && allow_smem<MODES, true>()) && ...);
+}
+int gemm_sm100_init(int device) {
+  static bool done[kMaxDevices] = {};              // the attribute is per device
+  if (device < 0 || device >= kMaxDevices) return -1;
+  if (!done[device] && !allow_smem_all<GS_STORE_BF16, GS_ADD_F32, GS_SWIGLU, GS_ARGMAX, GS_QKV_ROPE, GS_QKV_ROPE128>()) return -1;
+  done[device] = true;
+  return 0;
 }
 
 template <int MODE>
 static int launch_mode(cudaStream_t st, const GemmSm100Args& a) {
   const int n_cols = (MODE == GS_SWIGLU) ? a.n_out / 2 : a.n_out;
-  int bn = 64, splits = 1;
-  bool pair = false;
-  pick_tile(MODE, n_cols, a.M, a.K, a.n_sms, (MODE == GS_ADD_F32 && a.max_splits > 1) ? a.max_splits : 1, a.pair != 0, &bn,
-            &splits, &pair);
+  TileChoice c = pick_tile(MODE, n_cols, a.M, a.K, a.n_sms, (MODE == GS_ADD_F32 && a.max_splits > 1) ? a.max_splits : 1, a.pair != 0);
   if (a.force_bn) {
-    const int fbn = a.force_bn == 512 ? 256 : a.force_bn;       // 512 = a CTA pair on 256-column tiles
-    const int out_n = (MODE == GS_SWIGLU) ? fbn / 2 : fbn;
-    if ((fbn != 64 && fbn != 128 && fbn != 256) || out_n % 32 || n_cols % out_n) return -1;
-    if (MODE == GS_QKV_ROPE128 && fbn < 128) return -1;
-    bn = fbn;
-    pair = a.force_bn == 512 && a.M > 64;
+    c.pair = a.force_bn > 256;                                // a CTA pair on tiles of 256 rows and 256 columns less
+    c.bn = c.pair ? a.force_bn - 256 : a.force_bn;
+    c.pair = c.pair && a.M > 64;                              // (its tile needs whole boxes)
+    if (!c.pair && c.bn == 224 && MODE != GS_SWIGLU) c.bn = 256;
+    if (!width_fits(MODE, n_cols, c.bn, c.pair)) return -1;
   }
   if (a.force_splits) {
     const int kbs = (a.K / KSUB + a.force_splits - 1) / a.force_splits;
     if (MODE != GS_ADD_F32 || (a.force_splits - 1) * kbs >= a.K / KSUB) return -1;
-    splits = a.force_splits;
+    c.splits = a.force_splits;
   }
-  if (pair) return launch_one<256, MODE, true>(st, a, splits);
-  switch (bn) {
-    case 256: return launch_one<256, MODE, false>(st, a, splits);
-    case 128: return launch_one<128, MODE, false>(st, a, splits);
-    default:
-      if (MODE == GS_QKV_ROPE128) return launch_one<128, MODE, false>(st, a, splits);
-      return launch_one<64, MODE, false>(st, a, splits);
-  }
+  return c.pair ? launch_width<MODE, true>(st, a, c.bn, c.splits) : launch_width<MODE, false>(st, a, c.bn, c.splits);
 }
 
 int launch_gemm_sm100(cudaStream_t st, const GemmSm100Args& a) {

@@ -220,9 +220,11 @@ void launch_gemm_simt(cudaStream_t st, const bf16* A, const bf16* W, int M, int 
 int make_tmap_2d(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 // Same for fp32 with a {32, box_rows} box (128-byte rows): the residual stream as a TMA reduce-add target.
 int make_tmap_2d_f32(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
-// The three maps of one weight matrix, box heights 32 / 64 / 128 rows = half a tile of width 64 / 128 / 256.
+// The maps of one weight matrix, box heights 32, 48 .. 128 rows = half a tile of width 64, 96 .. 256.
 struct WeightMaps {
-  CUtensorMap m[3];
+  static constexpr int N = 7;
+  CUtensorMap m[N];
+  const CUtensorMap& half_tile(int bn) const { return m[bn / 32 - 2]; }
 };
 int make_weight_tmaps(WeightMaps* w, const void* base, uint64_t rows, uint64_t cols);
 int make_tmap_3d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t stride1_bytes,
@@ -254,13 +256,13 @@ struct GemmSm100Args {
   QkvEpilogue qkv;
   int* status;
   int n_sms;
-  int device;                  // CUDA device ordinal of the launch (per-device kernel attributes)
   int max_splits;              // GS_ADD_F32: most K slices per tile (1 = none; slices add in arrival order)
   bool pdl;                    // launch with programmatic stream serialization
   int pair;                    // CTA pairs (clusters of two sharing a 256-row tile) may be used
-  int force_bn, force_splits;  // tests: tile width (512 = CTA pair) / K slices instead of the model's choice (0 = choose)
+  int force_bn, force_splits;  // tests: tile width (above 256: a CTA pair, 256 columns less) / K slices instead of the model's choice (0 = choose)
 };
 enum GemmSm100Mode { GS_STORE_BF16 = 0, GS_ADD_F32 = 1, GS_SWIGLU = 2, GS_ARGMAX = 4, GS_QKV_ROPE = 5, GS_QKV_ROPE128 = 6 };
+int gemm_sm100_init(int device);      // once per device (the current one) before its first launch; 0 on success
 int launch_gemm_sm100(cudaStream_t st, const GemmSm100Args& a);
 
 }  // namespace hsd
