@@ -92,7 +92,6 @@ int make_weight_tmaps(WeightMaps* w, const void* base, uint64_t rows, uint64_t c
 // ------------------------------------------------------------------------------------------------
 constexpr int BM = 128;
 constexpr int KSUB = 64;                         // one 128-byte-swizzled sub-tile spans 64 bf16 of K
-constexpr int A_SUB = BM * KSUB * 2;             // bytes of one A sub-tile
 constexpr int kGemmThreads = 256;
 constexpr int STG_BYTES = 4096;                  // one epilogue staging buffer: 32 rows x 128 bytes
 constexpr int STG_TOTAL = 4 * 2 * STG_BYTES;     // four epilogue warps, two buffers each
@@ -101,15 +100,20 @@ constexpr int STG_TOTAL = 4 * 2 * STG_BYTES;     // four epilogue warps, two buf
 // KSTEPS: sub-tiles of a stage.  A stage is one barrier round trip of ~250 cycles.  The MMAs or the fill of the 128- and
 // 256-wide tiles' stages cover it (two sub-tiles: 256 wide the same, 128 wide 1 % slower steps, fewer stages being in
 // flight), those of the 64-wide tile do not: plain decode 0.965 -> 0.947 ms, short drafts 1.059 -> 1.046 with two.
-template <int BN, bool PAIR = false>
+// ROWS: rows of A a stage has room for.  A call of at most 16 or 64 rows has its own kernels for the 64-wide tile: the MMA
+// takes 128 rows all the same, and reads beyond a sub-tile's ROWS whatever lies behind it in the stage (rows are independent,
+// and those go nowhere), but 18 or 12 k-blocks are under way in place of 8.  Steps of 16 plain rows 868 -> 861 us (gate/up 6.8 ->
+// 6.5 us a launch, QKV 5.8 -> 5.55); what is left of the loop is the MMAs, whose 128 rows of A cost 32 cycles of shared memory each.
+template <int BN, bool PAIR, int ROWS>
 struct Cfg {
+  static constexpr int A_SUB = ROWS * KSUB * 2;                     // bytes of one A sub-tile
   static constexpr int KSTEPS = BN == 64 ? 2 : 1;
   static constexpr int BK = KSUB * KSTEPS;                          // K extent of one stage
   static constexpr int A_BYTES = A_SUB * KSTEPS;
   static constexpr int B_SUB = (PAIR ? BN / 2 : BN) * KSUB * 2;     // bytes of one B sub-tile this CTA stages
   static constexpr int B_BYTES = B_SUB * KSTEPS;                    // bytes of B per stage
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = 192 * 1024 / STAGE_BYTES < 8 ? 192 * 1024 / STAGE_BYTES : 8;
+  static constexpr int STAGES = 192 * 1024 / STAGE_BYTES < 9 ? 192 * 1024 / STAGE_BYTES : BN == 64 ? 9 : 8;
   static constexpr int TMEM_COLS = BN <= 64 ? 128 : BN <= 128 ? 256 : 512;      // two accumulators, a power of two
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + STG_TOTAL + 1024 /*alignment slack*/ + 256 /*barriers*/;
 };
@@ -155,12 +159,13 @@ __device__ __forceinline__ uint4 pack8(const uint32_t* r) {
   return o;
 }
 
-template <int BN, int MODE, bool PAIR>
+template <int BN, int MODE, bool PAIR, int ROWS>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const __grid_constant__ CUtensorMap tmC, GemmDev p) {
-  using C = Cfg<BN, PAIR>;
-  constexpr int KSTEPS = C::KSTEPS, BK = C::BK, A_BYTES = C::A_BYTES;
+  using C = Cfg<BN, PAIR, ROWS>;
+  static_assert((C::KSTEPS - 1) * C::A_SUB + BM * KSUB * 2 <= C::STAGE_BYTES, "an MMA reads 128 rows from every sub-tile on");
+  constexpr int KSTEPS = C::KSTEPS, BK = C::BK, A_BYTES = C::A_BYTES, A_SUB = C::A_SUB;
   constexpr int OUT_N = (MODE == GS_SWIGLU) ? BN / 2 : BN;   // output columns per tile
   constexpr int HALF_B = BN / 2 * KSUB * 2;                  // bytes of one weight half-tile of one sub-tile
   constexpr int TILE_M = PAIR ? 2 * BM : BM;                 // rows of one work unit (both CTAs of a pair)
@@ -681,9 +686,9 @@ done:
 }
 
 // ------------------------------------------------------------------------------------------------
-template <int BN, int MODE, bool PAIR>
+template <int BN, int MODE, bool PAIR, int ROWS = BM>
 static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
-  using C = Cfg<BN, PAIR>;
+  using C = Cfg<BN, PAIR, ROWS>;
   constexpr int OUT_N = (MODE == GS_SWIGLU) ? BN / 2 : BN;
   GemmDev p;
   p.M = a.M;
@@ -725,7 +730,7 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
   }
   cfg.attrs = attr;
   cfg.numAttrs = n_attr;
-  return cudaLaunchKernelEx(&cfg, gemm_sm100_kernel<BN, MODE, PAIR>, a.tmA, tmB, a.tmC, p) == cudaSuccess ? 0 : -1;
+  return cudaLaunchKernelEx(&cfg, gemm_sm100_kernel<BN, MODE, PAIR, ROWS>, a.tmA, tmB, a.tmC, p) == cudaSuccess ? 0 : -1;
 }
 
 // Tile width, CTA pairing and K slices: the least time by a model of one launch, in us.  What decides is the last wave: a
@@ -794,20 +799,31 @@ static TileChoice pick_tile(int mode, int n_cols, int M, int K, int n_sms, int m
 
 template <int MODE, bool PAIR, int BN = 64>
 static int launch_width(cudaStream_t st, const GemmSm100Args& a, int bn, int splits) {
-  if constexpr (has_width(MODE, BN, PAIR))
-    if (bn == BN) return launch_one<BN, MODE, PAIR>(st, a, splits);
+  if constexpr (has_width(MODE, BN, PAIR)) {
+    if (bn == BN) {
+      if constexpr (BN == 64) {
+        if (a.M <= 16) return launch_one<BN, MODE, PAIR, 16>(st, a, splits);
+        if (a.M <= 64) return launch_one<BN, MODE, PAIR, 64>(st, a, splits);
+      }
+      return launch_one<BN, MODE, PAIR>(st, a, splits);
+    }
+  }
   if constexpr (BN < 256) return launch_width<MODE, PAIR, BN + 32>(st, a, bn, splits);
   return -1;
 }
 
 // The shared memory each kernel is launched with.  Asked for when a context is created, which also loads the kernels: the
 // first step that picks a width does not wait for that.
+template <int BN, int MODE, bool PAIR, int ROWS = BM>
+static bool allow_smem_one() {
+  return cudaFuncSetAttribute(gemm_sm100_kernel<BN, MODE, PAIR, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              Cfg<BN, PAIR, ROWS>::SMEM_BYTES) == cudaSuccess;
+}
 template <int MODE, bool PAIR, int BN = 64>
 static bool allow_smem() {
   bool ok = true;
-  if constexpr (has_width(MODE, BN, PAIR))
-    ok = cudaFuncSetAttribute(gemm_sm100_kernel<BN, MODE, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              Cfg<BN, PAIR>::SMEM_BYTES) == cudaSuccess;
+  if constexpr (has_width(MODE, BN, PAIR)) ok = allow_smem_one<BN, MODE, PAIR>();
+  if constexpr (has_width(MODE, BN, PAIR) && BN == 64) ok = allow_smem_one<BN, MODE, PAIR, 16>() && allow_smem_one<BN, MODE, PAIR, 64>() && ok;
   if constexpr (BN < 256) ok = allow_smem<MODE, PAIR, BN + 32>() && ok;
   return ok;
 }
