@@ -202,8 +202,7 @@ HSD_API int hsd_verify_page(hsd_ctx *ctx, const hsd_kv *kv, int seq_slot, const 
  *   row_zchild      dev fp32 [total_q] out or NULL: the logit of the row's own token under its parent's
  *                   distribution (NaN on row 0)
  * The K/V rows of ALL nodes are written at cache rows committed length + row index; hsd_kv_commit_tree keeps the
- * accepted ones.  The workspace must be sized for 2 * total_q rows (the LM head evaluates every node once for its
- * argmax and once more, through its parent, for its own token).  A parent pointer that does not name an earlier row
+ * accepted ones.  The workspace must be sized for 2 * total_q rows.  A parent pointer that does not name an earlier row
  * sets device status 7 and turns the step into a no-op.  Errors otherwise as hsd_verify_regions; contexts created
  * with a SIMT debug flag return HSD_ERR_INVALID_ARG. */
 HSD_API int hsd_verify_tree(hsd_ctx *ctx, const hsd_kv *kv, int n_seqs, const int *cu_q, const int *q_tokens,

@@ -151,8 +151,8 @@ Ws carve(const hsd_ctx* c, void* base, int T, int S) {
   w.rm.seq_slot = static_cast<int*>(take(sizeof(int) * S));
   w.rm.seq_tile0 = static_cast<int*>(take(sizeof(int) * (S + 1)));
   w.rm.anc = static_cast<uint4*>(take(sizeof(uint4) * T));
-  w.rm.lm_src = static_cast<int*>(take(sizeof(int) * T));        // a tree call carves for 2 x its rows
-  w.rm.lm_next = static_cast<int*>(take(sizeof(int) * T));
+  w.rm.child_src = static_cast<int*>(take(sizeof(int) * T));
+  w.rm.child_tok = static_cast<int*>(take(sizeof(int) * T));
   w.sel_rows = static_cast<int*>(take(sizeof(int) * S));
   w.verdict = static_cast<int2*>(take(sizeof(int2) * (size_t)setup_ctas(T)));
   w.h_in = static_cast<int*>(take(sizeof(int) * ((size_t)S + 1 + T)));
@@ -713,7 +713,7 @@ int hsd_verify_tree(hsd_ctx* c, const hsd_kv* kv, int n_seqs, const int* cu_q, c
   int rc = check_kv(kv);
   if (rc) return rc;
   if ((long long)max_q_len > (long long)kv->max_blocks_per_seq * HSD_KV_BLOCK) return HSD_ERR_KV_CAPACITY;
-  // the LM head runs over 2 x total_q rows (every node, and every node's parent for the node's own token)
+  // (sized for 2 x total_q rows, as its contract has it)
   rc = check_ws(c, workspace, ws_bytes, 2 * total_q, n_seqs);
   if (rc) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
@@ -725,17 +725,18 @@ int hsd_verify_tree(hsd_ctx* c, const hsd_kv* kv, int n_seqs, const int* cu_q, c
   if (rc) return rc;
   {
     Scope s(c, st, KC_RMSNORM);
-    launch_rmsnorm(st, w.x, c->final_norm, w.h, 2 * total_q, c->md.d, c->md.eps, w.rm.lm_src, total_q, w.status, c->pdl);
+    launch_tree_final_norm(st, w.x, c->final_norm, w.h, total_q, c->md.d, c->md.eps, w.rm, c->lm_head, c->md.V, w.zdraft, w.status,
+                           c->pdl);
   }
-  rc = run_lm_head(c, w, 2 * total_q, w.rm.lm_next, st);
+  rc = run_lm_head(c, w, total_q, nullptr, st);
   if (rc) return rc;
   {
     Scope s(c, st, KC_ACCEPT);
     TreeAcceptArgs ta;
-    ta.n_seqs = n_seqs; ta.max_q_len = max_q_len; ta.total_q = total_q; ta.log_tau = log_tau;
+    ta.n_seqs = n_seqs; ta.max_q_len = max_q_len; ta.log_tau = log_tau;
     ta.parent = parent;
     ta.row_best = w.row_best;
-    ta.zdraft = w.zdraft;
+    ta.zchild = w.zdraft;
     ta.accept_len = accept_len; ta.emit_tokens = emit_tokens; ta.n_emit = n_emit; ta.accept_rows = accept_rows;
     ta.row_argmax = row_argmax; ta.row_zmax = row_zmax; ta.row_zchild = row_zchild;
     launch_tree_accept(st, ta, w.rm, w.status, c->pdl);

@@ -59,8 +59,8 @@ struct RowMeta {
   int* seq_tile0;   // [S+1] first attention q-tile of the sequence (exclusive scan)
   // candidate trees (Sec. 3.2, Eq. 7): written only by calls that pass parent pointers
   uint4* anc;       // [T] ancestry bit mask: bit i set iff row i of the sequence is the row itself or an ancestor
-  int* lm_src;      // [2T] source row of every LM-head row: [0, T) the rows themselves, [T, 2T) each row's parent
-  int* lm_next;     // [2T] token whose logit the LM-head row captures: -1, and in [T, 2T) the row's own token
+  int* child_src;   // [T] packed row of a node's parent
+  int* child_tok;   // [T] the node's token, -1 for rows that are no one's child
 };
 
 // ------------------------------------------------------------------------------------------------

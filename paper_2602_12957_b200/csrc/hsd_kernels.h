@@ -92,8 +92,8 @@ struct SetupArgs {
   const bf16* table;        // embedding table
   const bf16* embeds;       // prefill: rows used where the token id is negative
   float* x;                 // [T, d] residual stream
-  unsigned long long* row_best;   // [max(T, S)] (trees: [2T]) cleared for the LM head
-  float* zdraft;            // [T] (trees: [2T]) set to NaN
+  unsigned long long* row_best;   // [max(T, S)] cleared for the LM head
+  float* zdraft;            // [T] set to NaN
   int2* verdict;            // [setup_ctas(T)] {status code, offending index} of every CTA
   bool make_plan;           // the attention plan too (not where the plain attention kernel runs)
   AttnPlan plan;
@@ -131,14 +131,16 @@ struct AcceptArgs {
   float* row_zdraft;
 };
 void launch_accept(cudaStream_t st, const AcceptArgs& a, const RowMeta& rm, const int* status, bool pdl);
-// Greedy traversal of candidate trees (Eq. 9-12).  LM-head row r < T holds the argmax at node r, row T + r the
-// logit of node r's own token under its parent's distribution.
+// The final norm of a tree step: h as launch_rmsnorm's, zchild[r] = the logit of node r's token under its parent's distribution.
+void launch_tree_final_norm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
+                            const RowMeta& rm, const bf16* lm_head, int vocab, float* zchild, const int* status, bool pdl);
+// Greedy traversal of candidate trees (Eq. 9-12).
 struct TreeAcceptArgs {
-  int n_seqs, max_q_len, total_q;
+  int n_seqs, max_q_len;
   float log_tau;
   const int* parent;
-  const unsigned long long* row_best;   // [2T]
-  const float* zdraft;                  // [2T]
+  const unsigned long long* row_best;   // [T] argmax at every node
+  const float* zchild;                  // [T] see launch_tree_final_norm
   int* accept_len;
   int* emit_tokens;
   int* n_emit;

@@ -176,12 +176,8 @@ __global__ void __launch_bounds__(kSetupThreads) setup_rows_kernel(SetupArgs a, 
       }
       rm.anc[r] = make_uint4(m[0], m[1], m[2], m[3]);
       const bool child = ok && j > 0 && own >= 0;
-      rm.lm_src[r] = r;
-      rm.lm_next[r] = -1;
-      rm.lm_src[a.total_q + r] = child ? q0 + own : r;
-      rm.lm_next[a.total_q + r] = child ? tok : -1;
-      a.row_best[a.total_q + r] = 0ull;
-      a.zdraft[a.total_q + r] = __int_as_float(0x7fc00000);
+      rm.child_src[r] = child ? q0 + own : r;
+      rm.child_tok[r] = child ? tok : -1;
     }
     rm.row_seq[r] = i;
     rm.row_pos[r] = L + (a.parent ? d : j);
@@ -286,6 +282,77 @@ void launch_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, 
 void launch_first_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
                           const int2* verdict, int n_verdicts, int* status, bool pdl) {
   launch_rmsnorm_any(st, x, gain, h, rows, d, eps, nullptr, rows, nullptr, verdict, n_verdicts, status, pdl);
+}
+
+// The final norm of a tree step: h as above, and for every node the logit of its own token under its PARENT's distribution,
+// which the traversal compares (Eq. 10): the parent's normed row, made again from x and rounded as it is in h, times the
+// token's row of the LM head.  A warp per row; bound by the latency of the token's row (2 KB at d = 1024, scattered in HBM).
+// (As rows T .. 2T of the LM head's own GEMM, each against the whole vocabulary for one captured column, 2,048 nodes took
+// 162 us there and 4.5 us in the norm; now 78 and 6.  128 nodes: 18 and 2, now 14 and 4.7.)
+template <int VEC>
+__global__ void tree_final_norm_kernel(const float* __restrict__ x, const bf16* __restrict__ gain, bf16* __restrict__ h, int rows, int d,
+                                       float eps, const int* __restrict__ child_src, const int* __restrict__ child_tok,
+                                       const bf16* __restrict__ lm_head, int vocab, float* __restrict__ zchild,
+                                       const int* __restrict__ status) {
+  // The indices come from the step's set-up, which the kernel before this one waited for before it let this one start: they and
+  // the token's row are under way while that kernel still runs.
+  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const bool dead = r >= rows || __ldcg(status);         // (after a failed device-side check the indices were never written)
+  const int src = dead ? -1 : __ldcg(child_src + r), tok = dead ? -1 : __ldcg(child_tok + r);
+  const bool child = tok >= 0 && tok < vocab && src >= 0 && src < rows;
+  const uint2* gp = reinterpret_cast<const uint2*>(gain);
+  uint2 w[VEC], o[VEC];
+  if (child) {
+    const uint2* wp = reinterpret_cast<const uint2*>(lm_head + (size_t)tok * d);
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) w[i] = __ldg(wp + lane + 32 * i);
+  }
+  pdl_wait();               // x is what the kernel before wrote
+  pdl_launch_dependents();
+  if (dead) return;
+  auto normed = [&](int row) {
+    const float4* xp = reinterpret_cast<const float4*>(x + (size_t)row * d);
+    float4 v[VEC];
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) v[i] = xp[lane + 32 * i];
+    float ss = 0.f;
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+    for (int s = 16; s; s >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, s);
+    const float rs = rsqrtf(ss / (float)d + eps);
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) {
+      const uint2 g = __ldg(gp + lane + 32 * i);
+      o[i] = make_uint2(pack_bf16(v[i].x * rs * bf16_lo(g.x), v[i].y * rs * bf16_hi(g.x)),
+                        pack_bf16(v[i].z * rs * bf16_lo(g.y), v[i].w * rs * bf16_hi(g.y)));
+    }
+  };
+  normed(r);
+  uint2* hp = reinterpret_cast<uint2*>(h + (size_t)r * d);
+#pragma unroll
+  for (int i = 0; i < VEC; ++i) hp[lane + 32 * i] = o[i];
+  if (!child) return;
+  normed(src);
+  float z = 0.f;
+#pragma unroll
+  for (int i = 0; i < VEC; ++i)
+    z += (bf16_lo(o[i].x) * bf16_lo(w[i].x) + bf16_hi(o[i].x) * bf16_hi(w[i].x)) +
+         (bf16_lo(o[i].y) * bf16_lo(w[i].y) + bf16_hi(o[i].y) * bf16_hi(w[i].y));
+  for (int s = 16; s; s >>= 1) z += __shfl_xor_sync(0xffffffffu, z, s);
+  if (lane == 0) zchild[r] = z;
+}
+void launch_tree_final_norm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
+                            const RowMeta& rm, const bf16* lm_head, int vocab, float* zchild, const int* status, bool pdl) {
+#define HSD_TREE_NORM_CASE(V)                                                                                                   \
+  case V:                                                                                                                      \
+    launch_kernel(tree_final_norm_kernel<V>, dim3((rows + 7) / 8), dim3(256), 0, st, pdl, x, gain, h, rows, d, eps, rm.child_src, \
+                  rm.child_tok, lm_head, vocab, zchild, status);                                                               \
+    break;
+  switch (d / 128) {
+    HSD_TREE_NORM_CASE(1) HSD_TREE_NORM_CASE(2) HSD_TREE_NORM_CASE(4) HSD_TREE_NORM_CASE(8) HSD_TREE_NORM_CASE(16) HSD_TREE_NORM_CASE(32)
+    default: break;   // hsd_create rejects other widths
+  }
+#undef HSD_TREE_NORM_CASE
 }
 
 __global__ void select_last_rows_kernel(RowMeta rm, int n_seqs, int* sel_rows, const int* status) {
@@ -512,7 +579,7 @@ __global__ void __launch_bounds__(HSD_MAX_TREE_ROWS) tree_accept_kernel(TreeAcce
   __shared__ unsigned long long s_best[HSD_MAX_TREE_ROWS];    // the node's own argmax word
   __shared__ int s_child[HSD_MAX_TREE_ROWS], s_tok[HSD_MAX_TREE_ROWS], s_path[HSD_MAX_TREE_ROWS], s_acc;
   const int failed = *status;
-  const int q0 = rm.seq_q0[i], n = rm.seq_n[i], T = a.total_q;
+  const int q0 = rm.seq_q0[i], n = rm.seq_n[i];
   if (failed) {             // a failed step decides nothing: the compaction and the commit that follow skip -1
     if (c == 0) { a.accept_len[i] = -1; a.n_emit[i] = 0; }
     return;
@@ -524,7 +591,7 @@ __global__ void __launch_bounds__(HSD_MAX_TREE_ROWS) tree_accept_kernel(TreeAcce
   constexpr int kNone = 0x7fffffff;
   const bool node = c >= 1 && c < n;
   const int par = node ? a.parent[q0 + c] : -3, tok = node ? rm.row_tok[q0 + c] : -1;
-  const float z = node ? a.zdraft[T + q0 + c] : 0.f;
+  float z = node ? a.zchild[q0 + c] : 0.f;
   const unsigned long long best = c < n ? a.row_best[q0 + c] : 0ull;
   s_best[c] = best;
   s_key[c] = 0ull;
@@ -532,6 +599,8 @@ __global__ void __launch_bounds__(HSD_MAX_TREE_ROWS) tree_accept_kernel(TreeAcce
   s_tok[c] = tok;
   __syncthreads();
   const bool child = node && par >= 0 && par < n;
+  // the parent's argmax has the logit that the LM head found for it (the two sums differ in order)
+  if (child && tok == key_col(s_best[par])) z = key_value(s_best[par]);
   if (a.log_tau == 0.f) {
     // the child that carries u_hat (lowest row if a caller packed the same token twice under one parent)
     if (child && tok == key_col(s_best[par])) atomicMin(&s_child[par], c);
