@@ -39,8 +39,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # captures summarised under profiles/, per workload; a class is absent (-> null) when its kernel has changed since
 # its counters were taken, or when no capture of that workload exists.
 NCU_TRAFFIC_BYTES = {
-    "region": {"attention": 30_976_768 + 512, "gemm_gate_up": 19_521_024, "gemm_qkv": 7_287_296 + 4_608,
-               "gemm_o": 10_247_936, "gemm_down": 24_669_440},
+    "region": {"attention": 30_976_768 + 512},
     "long2048": {"attention": 42_723_584 + 3_332_096},
 }
 
@@ -317,7 +316,7 @@ def build_gpu_state(name, model, rank, world=1, sharded=False, mixed_k=0, random
                 plant_rounds=plant_rounds, accept_det=accept_det)
 
 
-def kernel_work_table(cfg, work: RF.StepWork, T: int, lm_rows: int):
+def kernel_work_table(cfg, work: RF.StepWork, T: int):
     """Algorithmic (flops, bytes) per launch of each kernel class."""
     d, f, V = cfg.d_model, cfg.d_ffn, cfg.vocab
     L = cfg.n_layers
@@ -326,7 +325,7 @@ def kernel_work_table(cfg, work: RF.StepWork, T: int, lm_rows: int):
     t["gemm_o"] = RF.gemm_work(T, d, cfg.n_heads * cfg.head_dim, 8.0)          # fp32 read-modify-write
     t["gemm_gate_up"] = (2.0 * T * 2 * f * d, 2.0 * (T * d + 2 * f * d) + 2.0 * T * f)
     t["gemm_down"] = RF.gemm_work(T, d, f, 8.0)
-    t["lm_head_argmax"] = (2.0 * lm_rows * V * d, 2.0 * (lm_rows * d + V * d) + 12.0 * lm_rows)
+    t["lm_head_argmax"] = (2.0 * T * V * d, 2.0 * (T * d + V * d) + 12.0 * T)
     t["attention"] = (work.attn_flops / L, work.kv_read_bytes / L + 4.0 * T * cfg.n_heads * cfg.head_dim)
     t["rmsnorm"] = (0.0, 6.0 * T * d)
     return t
@@ -539,10 +538,9 @@ def choose_peak(peaks, clocks):
 def roofline_report(st, prof, prof_steps, ms_step, clocks, peaks, peak_src, traffic_table=None):
     cfg = st["cfg"]
     T = st["total_q"]
-    tree = st["dsv"] is not None
     ctx_lens = [int(x) for x in st["prefix_lens"].cpu().numpy().tolist()]
     work = RF.step_work(cfg, ctx_lens, [k + 1 for k in st["ks"]])
-    table = kernel_work_table(cfg, work, T, 2 * T if tree else T)
+    table = kernel_work_table(cfg, work, T)
     tot_ms = sum(v[0] for v in prof.values()) or 1.0
     kernels = {k: {"ms_per_step": v[0] / prof_steps, "launches_per_step": v[1] / prof_steps,
                    "share": v[0] / tot_ms} for k, v in prof.items()}
