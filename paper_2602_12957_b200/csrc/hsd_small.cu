@@ -263,7 +263,10 @@ __global__ void rmsnorm_kernel(const float* __restrict__ x, const bf16* __restri
 static void launch_rmsnorm_any(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
                                const int* sel_rows, int src_rows, const int* status, const int2* verdict, int n_verdicts,
                                int* status_out, bool pdl) {
-  dim3 grid((rows + 7) / 8 + (verdict ? 1 : 0)), block(256);
+  // Four rows a CTA while that leaves no SM with two of them, eight otherwise: 16 rows 1.95 us a launch with eight and 1.81 with
+  // four, 513 rows 2.55 and 2.37, ~1,090 rows 3.19 and 3.74 (two rows a CTA as four, sixteen 2.57 / 2.78 / 3.25).
+  const int per = rows <= 4 * 148 ? 4 : 8;
+  dim3 grid((rows + per - 1) / per + (verdict ? 1 : 0)), block(32 * per);
 #define HSD_RMS_CASE(V)                                                                                                  \
   case V:                                                                                                                \
     launch_kernel(rmsnorm_kernel<V>, grid, block, 0, st, pdl, x, gain, h, rows, d, eps, sel_rows, src_rows, status, verdict, \
