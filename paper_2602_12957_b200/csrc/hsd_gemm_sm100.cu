@@ -735,7 +735,7 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
 
 // Tile width, CTA pairing and K slices: the least time by a model of one launch, in us.  What decides is the last wave: a
 // projection of ~600 rows has 1.3 waves of 128 x 256 tiles, and 0.9 of 128 x 160.  So tiles come in seven widths, for single CTAs
-// and pairs, and any of them may be cut in up to eight K slices (residual adds).  Least squares over 3,900 timings (back to back
+// and pairs, and any of them may be cut in up to eight K slices (residual adds).  Least squares over 8,000 timings (back to back
 // in a graph, 4 projections of the 24-layer decoder at 41 row counts from 16 to 9,300 and 4 of a decoder twice as wide at 7):
 //   a k-block of 64: by the rows filled (A box + tile width: L2 -> SM) with a floor, or by a pair's width; up to a quarter less
 //   where the launch leaves SMs idle; a wave: 0.7 / 0.8; the last epilogue: by width, residual adds dearest; a launch 2.4, a pair 0.9
