@@ -200,7 +200,7 @@ HSD_API int hsd_verify_page(hsd_ctx *ctx, const hsd_kv *kv, int seq_slot, const 
  *   accept_rows     dev int32 [n_seqs, max_q_len] out: rows of the accepted path after the root
  *   row_argmax, row_zmax   dev [total_q] out or NULL, as in hsd_verify_regions
  *   row_zchild      dev fp32 [total_q] out or NULL: the logit of the row's own token under its parent's
- *                   distribution (NaN on row 0)
+ *                   distribution (NaN on row 0); never above the parent's row_zmax, and equal to it where the token is its argmax
  * The K/V rows of ALL nodes are written at cache rows committed length + row index; hsd_kv_commit_tree keeps the
  * accepted ones.  The workspace must be sized for 2 * total_q rows.  A parent pointer that does not name an earlier row
  * sets device status 7 and turns the step into a no-op.  Errors otherwise as hsd_verify_regions; contexts created

@@ -602,8 +602,15 @@ __global__ void __launch_bounds__(HSD_MAX_TREE_ROWS) tree_accept_kernel(TreeAcce
   s_tok[c] = tok;
   __syncthreads();
   const bool child = node && par >= 0 && par < n;
-  // the parent's argmax has the logit that the LM head found for it (the two sums differ in order)
-  if (child && tok == key_col(s_best[par])) z = key_value(s_best[par]);
+  // A child's logit and its parent's maximum are summed in different orders.  The child that carries the argmax has the LM head's
+  // logit for it.  Of any other the LM head has found that it is no larger than the maximum, and smaller if its id is lower: where
+  // the other sum says otherwise (equal or nearly equal logits) it is held to that, so that no sibling passes the argmax.  NaN stays.
+  if (child) {
+    const int hat = key_col(s_best[par]);
+    const float zmax = key_value(s_best[par]), most = tok < hat ? nextafterf(zmax, -INFINITY) : zmax;
+    if (tok == hat) z = zmax;
+    else if (z > most) z = most;
+  }
   if (a.log_tau == 0.f) {
     // the child that carries u_hat (lowest row if a caller packed the same token twice under one parent)
     if (child && tok == key_col(s_best[par])) atomicMin(&s_child[par], c);
