@@ -388,6 +388,10 @@ HSD_API int hsd_op_linear(hsd_ctx *ctx, const void *A, const void *W, void *C, i
  * problem does not allow makes hsd_op_linear return HSD_ERR_CUDA.  Lets the parity tests reach every tile shape. */
 HSD_API int hsd_debug_set_gemm_tile(hsd_ctx *ctx, int tile_n, int k_slices);
 
+/* Test-only: host work of this context so far: `tile_choices` = how often it has chosen a GEMM tile (once per projection of a
+ * call, whatever its layers). */
+HSD_API int hsd_debug_host_work(const hsd_ctx *ctx, long long *tile_choices);
+
 /* Test-only: the attention launch cuts the KV ranges of the query tiles into slices so that it has about `target_items`
  * work items (never more than CTA slots in one round), none shorter than `min_kv_tiles` 128-token KV tiles (two paged
  * blocks; 0 = the library's defaults).  With `min_kv_tiles` > 0 a range is cut that finely wherever there are CTA slots and

@@ -33,7 +33,7 @@ EXPORTS = [
     "hsd_status_string", "hsd_create", "hsd_destroy", "hsd_workspace_bytes", "hsd_prefill", "hsd_verify_regions",
     "hsd_verify_page", "hsd_kv_commit", "hsd_verify_regions_host", "hsd_device_status", "hsd_last_cuda_error", "hsd_launch_count",
     "hsd_profile_enable", "hsd_profile_read", "hsd_debug_logits", "hsd_debug_buffer", "hsd_op_linear",
-    "hsd_op_lm_head_argmax", "hsd_op_lm_head_argmax_noalloc", "hsd_debug_set_gemm_tile", "hsd_debug_set_attn_plan",
+    "hsd_op_lm_head_argmax", "hsd_op_lm_head_argmax_noalloc", "hsd_debug_set_gemm_tile", "hsd_debug_set_attn_plan", "hsd_debug_host_work",
     "hsd_verify_tree", "hsd_kv_commit_tree", "hsd_dsv_build", "hsd_debug_tap", "hsd_stage_begin", "hsd_stage_advance",
     "hsd_stage_aggregate",
 ]
@@ -110,6 +110,7 @@ def _load():
     lib.hsd_debug_tap.argtypes = [vp, i, i, vp, sz]
     lib.hsd_debug_set_gemm_tile.argtypes = [vp, i, i]
     lib.hsd_debug_set_attn_plan.argtypes = [vp, i, i]
+    lib.hsd_debug_host_work.argtypes = [vp, C.POINTER(C.c_longlong)]
     lib.hsd_op_linear.argtypes = [vp, vp, vp, vp, i, i, i, i, vp]
     lib.hsd_op_lm_head_argmax.argtypes = [vp, vp, i, vp, vp, sz, vp, vp, vp, vp]
     lib.hsd_op_lm_head_argmax_noalloc.argtypes = [vp, vp, i, vp, vp, vp, vp, vp]
@@ -322,6 +323,12 @@ def hsd_debug_tap(ctx, layer: int, which: int, dst, dst_bytes: int) -> int:
 
 def hsd_debug_set_gemm_tile(ctx, tile_n: int, k_slices: int) -> int:
     return _lib.hsd_debug_set_gemm_tile(ctx, tile_n, k_slices)
+
+
+def hsd_debug_host_work(ctx):
+    n = C.c_longlong(0)
+    st = _lib.hsd_debug_host_work(ctx, C.byref(n))
+    return st, {"tile_choices": n.value}
 
 
 def hsd_debug_set_attn_plan(ctx, target_items: int, min_kv_tiles: int) -> int:

@@ -51,6 +51,7 @@ struct hsd_ctx {
   bool attn_simt;     // attention through the plain kernel (debug)
   int last_cuda_error;
   long long launches;
+  long long tile_choices;       // hsd_debug_host_work
   bool profiling;
   // hsd_verify_regions_host: pinned staging and the cached graph of the last repeated call shape
   bool host_graph_ok;
@@ -259,6 +260,11 @@ int check_kv(const hsd_kv* kv) {
   return HSD_OK;
 }
 
+TileChoice choose_tile(hsd_ctx* c, const GemmSm100Args& g, int force_bn, int force_splits) {
+  ++c->tile_choices;
+  return gemm_choose_tile(g, force_bn, force_splits);
+}
+
 struct StepArgs {
   int n_seqs, total_q, max_q_len;
   bool prefill;
@@ -344,6 +350,31 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
       return HSD_ERR_CUDA;
   }
 
+  // what the projections of every layer have in common, the tiles among it
+  GemmSm100Args g_qkv, g_o, g_gate_up, g_down;
+  if (!c->simt) {
+    auto projection = [&](GemmSm100Args& g, const CUtensorMap& tmA, const CUtensorMap& tmC, int n_out, int K, int mode, int max_splits,
+                          int force_bn) {
+      g = {};
+      g.tmA = tmA;
+      g.tmC = tmC;
+      g.M = T; g.n_out = n_out; g.K = K; g.mode = mode;
+      g.status = w.status; g.n_sms = c->n_sms; g.max_splits = max_splits; g.pdl = c->pdl; g.pair = c->pair;
+      g.tile = choose_tile(c, g, force_bn, 0);
+    };
+    projection(g_qkv, tm_h, tm_q_st, md.qkv_out, md.d, md.D == 128 ? GS_QKV_ROPE128 : GS_QKV_ROPE, 1, c->force_bn);
+    g_qkv.qkv.row_kv = w.rm.row_kv;
+    g_qkv.qkv.kv_rows = kv.n_blocks * HSD_KV_BLOCK;
+    g_qkv.qkv.rope_cs = w.rm.rope_cs;
+    g_qkv.qkv.q_out = w.q;
+    g_qkv.qkv.Hq = md.Hq; g_qkv.qkv.Hkv = md.Hkv; g_qkv.qkv.D = md.D;
+    g_qkv.qkv.eps = md.eps;
+    projection(g_o, tm_attn, tm_x_add, md.d, md.Hq * md.D, GS_ADD_F32, c->max_splits, 0);
+    projection(g_gate_up, tm_h, tm_act_st, 2 * md.ffn, md.d, GS_SWIGLU, 1, 0);
+    g_gate_up.out.C = w.act; g_gate_up.out.ldc = md.ffn;
+    projection(g_down, tm_act, tm_x_add, md.d, md.ffn, GS_ADD_F32, c->max_splits, 0);
+  }
+
   for (int l = 0; l < md.n_layers; ++l) {
     {
       Scope s(c, st, KC_RMSNORM);
@@ -374,22 +405,11 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
     } else {
       {
         Scope s(c, st, KC_GEMM_QKV);
-        GemmSm100Args g = {};
-        g.tmA = tm_h;
-        g.tmB = &c->tm_qkv[l];
-        g.tmC = tm_q_st;
-        g.M = T; g.n_out = md.qkv_out; g.K = md.d; g.mode = md.D == 128 ? GS_QKV_ROPE128 : GS_QKV_ROPE;
-        g.qkv.row_kv = w.rm.row_kv;
-        g.qkv.kv_rows = kv.n_blocks * HSD_KV_BLOCK;
-        g.qkv.rope_cs = w.rm.rope_cs;
-        g.qkv.q_out = w.q;
-        g.qkv.k_pool_layer = kv.k_pool + (size_t)l * layer_elems;
-        g.qkv.v_pool_layer = kv.v_pool + (size_t)l * layer_elems;
-        g.qkv.Hq = md.Hq; g.qkv.Hkv = md.Hkv; g.qkv.D = md.D;
-        g.qkv.q_norm = c->q_norm[l]; g.qkv.k_norm = c->k_norm[l]; g.qkv.eps = md.eps;
-        g.status = w.status; g.n_sms = c->n_sms; g.max_splits = 1; g.pdl = c->pdl; g.pair = c->pair;
-        g.force_bn = c->force_bn;
-        if (launch_gemm_sm100(st, g)) return fail_cuda(c);
+        g_qkv.tmB = &c->tm_qkv[l];
+        g_qkv.qkv.k_pool_layer = kv.k_pool + (size_t)l * layer_elems;
+        g_qkv.qkv.v_pool_layer = kv.v_pool + (size_t)l * layer_elems;
+        g_qkv.qkv.q_norm = c->q_norm[l]; g_qkv.qkv.k_norm = c->k_norm[l];
+        if (launch_gemm_sm100(st, g_qkv)) return fail_cuda(c);
       }
       {
         Scope s(c, st, KC_ATTN);
@@ -402,13 +422,8 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
       }
       {
         Scope s(c, st, KC_GEMM_O);
-        GemmSm100Args g = {};
-        g.tmA = tm_attn;
-        g.tmB = &c->tm_o[l];
-        g.tmC = tm_x_add;
-        g.M = T; g.n_out = md.d; g.K = md.Hq * md.D; g.mode = GS_ADD_F32;
-        g.status = w.status; g.n_sms = c->n_sms; g.max_splits = c->max_splits; g.pdl = c->pdl; g.pair = c->pair;
-        if (launch_gemm_sm100(st, g)) return fail_cuda(c);
+        g_o.tmB = &c->tm_o[l];
+        if (launch_gemm_sm100(st, g_o)) return fail_cuda(c);
       }
     }
     if (int rc = tap(l, HSD_TAP_Q, w.q, 2 * row_q)) return rc;
@@ -433,24 +448,13 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
     } else {
       {
         Scope s(c, st, KC_GEMM_GATEUP);
-        GemmSm100Args g = {};
-        g.tmA = tm_h;
-        g.tmB = &c->tm_gate_up[l];
-        g.tmC = tm_act_st;
-        g.M = T; g.n_out = 2 * md.ffn; g.K = md.d; g.mode = GS_SWIGLU;
-        g.out.C = w.act; g.out.ldc = md.ffn;
-        g.status = w.status; g.n_sms = c->n_sms; g.max_splits = 1; g.pdl = c->pdl; g.pair = c->pair;
-        if (launch_gemm_sm100(st, g)) return fail_cuda(c);
+        g_gate_up.tmB = &c->tm_gate_up[l];
+        if (launch_gemm_sm100(st, g_gate_up)) return fail_cuda(c);
       }
       {
         Scope s(c, st, KC_GEMM_DOWN);
-        GemmSm100Args g = {};
-        g.tmA = tm_act;
-        g.tmB = &c->tm_down[l];
-        g.tmC = tm_x_add;
-        g.M = T; g.n_out = md.d; g.K = md.ffn; g.mode = GS_ADD_F32;
-        g.status = w.status; g.n_sms = c->n_sms; g.max_splits = c->max_splits; g.pdl = c->pdl; g.pair = c->pair;
-        if (launch_gemm_sm100(st, g)) return fail_cuda(c);
+        g_down.tmB = &c->tm_down[l];
+        if (launch_gemm_sm100(st, g_down)) return fail_cuda(c);
       }
     }
     if (int rc = tap(l, HSD_TAP_ACT, w.act, 2 * (size_t)T * md.ffn)) return rc;
@@ -475,6 +479,7 @@ int run_lm_head(hsd_ctx* c, const Ws& w, int rows, const int* row_next, cudaStre
     g.M = rows; g.n_out = md.V; g.K = md.d; g.mode = GS_ARGMAX;
     g.out = o;
     g.status = w.status; g.n_sms = c->n_sms; g.max_splits = 1; g.pdl = c->pdl; g.pair = c->pair;
+    g.tile = choose_tile(c, g, 0, 0);
     if (launch_gemm_sm100(st, g)) return fail_cuda(c);
   }
   return check_cuda(c);
@@ -611,6 +616,7 @@ int hsd_create(const hsd_model_config* cfg, const hsd_weights* w, hsd_ctx** out)
   c->tap_layer = -1; c->tap_which = 0; c->tap_dst = nullptr; c->tap_bytes = 0;
   c->last_cuda_error = 0;
   c->launches = 0;
+  c->tile_choices = 0;
   c->profiling = false;
   memset(c->prof_ms, 0, sizeof(c->prof_ms));
   memset(c->prof_n, 0, sizeof(c->prof_n));
@@ -1100,6 +1106,7 @@ static int lm_head_argmax_impl(hsd_ctx* c, const void* h, int rows, const int* n
       g.M = rows; g.n_out = md.V; g.K = md.d; g.mode = GS_ARGMAX;
       g.out = o;
       g.status = nullptr; g.n_sms = c->n_sms; g.max_splits = 1; g.pdl = false; g.pair = c->pair;
+      g.tile = choose_tile(c, g, 0, 0);
       if (launch_gemm_sm100(st, g)) return fail_cuda(c);
     }
   }
@@ -1154,6 +1161,12 @@ int hsd_debug_set_gemm_tile(hsd_ctx* c, int tile_n, int k_slices) {
   return HSD_OK;
 }
 
+int hsd_debug_host_work(const hsd_ctx* c, long long* tile_choices) {
+  if (!c || !tile_choices) return HSD_ERR_INVALID_ARG;
+  *tile_choices = c->tile_choices;
+  return HSD_OK;
+}
+
 int hsd_debug_set_attn_plan(hsd_ctx* c, int target_items, int min_kv_tiles) {
   if (!c || target_items < 0 || min_kv_tiles < 0) return HSD_ERR_INVALID_ARG;
   c->attn_target_items = target_items ? target_items : attn_grid(c);
@@ -1182,7 +1195,7 @@ int hsd_op_linear(hsd_ctx* c, const void* A, const void* W, void* C, int M, int 
   g.M = M; g.n_out = n_out; g.K = K; g.mode = mode;
   g.out.C = C; g.out.ldc = ldc;
   g.status = nullptr; g.n_sms = c->n_sms; g.max_splits = c->max_splits; g.pdl = false; g.pair = c->pair;
-  g.force_bn = c->force_bn; g.force_splits = c->force_splits;
+  g.tile = choose_tile(c, g, c->force_bn, c->force_splits);
   if (launch_gemm_sm100(st, g)) return fail_cuda(c);
   return check_cuda(c);
 }

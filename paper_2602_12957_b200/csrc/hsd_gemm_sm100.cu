@@ -744,10 +744,8 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
 // Its choices are within 0.8 % of the best timed one on average (worst 8.5 %).  With widths of 64, 128 and 256 (pairs: 256) and a
 // model by fill rates alone it was 8.1 % (worst 70 %).  A layer's four projections, before / now: 300 rows 28.6 / 26.1 us, 600
 // rows 37.8 / 32.3, 900 rows 41.2 / 38.5, 1,323 rows 52.5 / 48.3, 2,600 rows 83 / 73, 5,000 rows 147 / 123, 9,300 rows 217 / 216.
-struct TileChoice {
-  int bn, splits;
-  bool pair;
-};
+// A choice takes ~0.25 us of the host: it is made once a call and projection, not for every layer (enqueueing a 24-layer step of
+// 144 rows 455 -> 427 us, of 1,058 rows 447 -> 430).
 // Tile widths a mode has: whole heads for the rotary epilogues, whole 64-column stores for the plain one; the adds take any 32
 // columns, SwiGLU any 16.
 constexpr bool has_width(int mode, int bn, bool pair) {
@@ -839,23 +837,28 @@ int gemm_sm100_init(int device) {
   return 0;
 }
 
+TileChoice gemm_choose_tile(const GemmSm100Args& a, int force_bn, int force_splits) {
+  const int n_cols = (a.mode == GS_SWIGLU) ? a.n_out / 2 : a.n_out;
+  const TileChoice none = {0, 0, false};
+  TileChoice c = pick_tile(a.mode, n_cols, a.M, a.K, a.n_sms, (a.mode == GS_ADD_F32 && a.max_splits > 1) ? a.max_splits : 1, a.pair != 0);
+  if (force_bn) {
+    c.pair = force_bn > 256;                                // a CTA pair on tiles of 256 rows and 256 columns less
+    c.bn = c.pair ? force_bn - 256 : force_bn;
+    c.pair = c.pair && a.M > 64;                            // (its tile needs whole boxes)
+    if (!c.pair && c.bn == 224 && a.mode != GS_SWIGLU) c.bn = 256;
+    if (!width_fits(a.mode, n_cols, c.bn, c.pair)) return none;
+  }
+  if (force_splits) {
+    const int kbs = (a.K / KSUB + force_splits - 1) / force_splits;
+    if (a.mode != GS_ADD_F32 || (force_splits - 1) * kbs >= a.K / KSUB) return none;
+    c.splits = force_splits;
+  }
+  return c;
+}
+
 template <int MODE>
 static int launch_mode(cudaStream_t st, const GemmSm100Args& a) {
-  const int n_cols = (MODE == GS_SWIGLU) ? a.n_out / 2 : a.n_out;
-  TileChoice c = pick_tile(MODE, n_cols, a.M, a.K, a.n_sms, (MODE == GS_ADD_F32 && a.max_splits > 1) ? a.max_splits : 1, a.pair != 0);
-  if (a.force_bn) {
-    c.pair = a.force_bn > 256;                                // a CTA pair on tiles of 256 rows and 256 columns less
-    c.bn = c.pair ? a.force_bn - 256 : a.force_bn;
-    c.pair = c.pair && a.M > 64;                              // (its tile needs whole boxes)
-    if (!c.pair && c.bn == 224 && MODE != GS_SWIGLU) c.bn = 256;
-    if (!width_fits(MODE, n_cols, c.bn, c.pair)) return -1;
-  }
-  if (a.force_splits) {
-    const int kbs = (a.K / KSUB + a.force_splits - 1) / a.force_splits;
-    if (MODE != GS_ADD_F32 || (a.force_splits - 1) * kbs >= a.K / KSUB) return -1;
-    c.splits = a.force_splits;
-  }
-  return c.pair ? launch_width<MODE, true>(st, a, c.bn, c.splits) : launch_width<MODE, false>(st, a, c.bn, c.splits);
+  return a.tile.pair ? launch_width<MODE, true>(st, a, a.tile.bn, a.tile.splits) : launch_width<MODE, false>(st, a, a.tile.bn, a.tile.splits);
 }
 
 int launch_gemm_sm100(cudaStream_t st, const GemmSm100Args& a) {

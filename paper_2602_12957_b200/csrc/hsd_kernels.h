@@ -248,6 +248,10 @@ struct QkvEpilogue {      // fused RoPE + paged KV write (QKV projection)
 // Rows of the activation boxes a GEMM over M rows loads (the box height of GemmSm100Args::tmA): a call of few rows does
 // not fill the rest of its 128-row tile (see hsd_gemm_sm100.cu).
 inline uint32_t gemm_a_box_rows(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : 128; }
+struct TileChoice {
+  int bn, splits;              // tile width (0: the problem does not allow what a test asked for), K slices
+  bool pair;
+};
 struct GemmSm100Args {
   CUtensorMap tmA;             // activations, box {64, gemm_a_box_rows(M)}
   const WeightMaps* tmB;       // weights
@@ -261,10 +265,14 @@ struct GemmSm100Args {
   int max_splits;              // GS_ADD_F32: most K slices per tile (1 = none; slices add in arrival order)
   bool pdl;                    // launch with programmatic stream serialization
   int pair;                    // CTA pairs (clusters of two sharing a 256-row tile) may be used
-  int force_bn, force_splits;  // tests: tile width (above 256: a CTA pair, 256 columns less) / K slices instead of the model's choice (0 = choose)
+  TileChoice tile;             // gemm_choose_tile's
 };
 enum GemmSm100Mode { GS_STORE_BF16 = 0, GS_ADD_F32 = 1, GS_SWIGLU = 2, GS_ARGMAX = 4, GS_QKV_ROPE = 5, GS_QKV_ROPE128 = 6 };
 int gemm_sm100_init(int device);      // once per device (the current one) before its first launch; 0 on success
+// The tile of a problem, by its M, n_out, K, mode, n_sms, max_splits and pair alone: one choice serves every layer of a call.
+// Tests: `force_bn` = tile width (above 256: a CTA pair, 256 columns less), `force_splits` = K slices instead of the model's
+// choice (0 = choose).
+TileChoice gemm_choose_tile(const GemmSm100Args& a, int force_bn, int force_splits);
 int launch_gemm_sm100(cudaStream_t st, const GemmSm100Args& a);
 
 }  // namespace hsd
