@@ -389,8 +389,9 @@ HSD_API int hsd_op_linear(hsd_ctx *ctx, const void *A, const void *W, void *C, i
 HSD_API int hsd_debug_set_gemm_tile(hsd_ctx *ctx, int tile_n, int k_slices);
 
 /* Test-only: host work of this context so far: `tile_choices` = how often it has chosen a GEMM tile (once per projection of a
- * call, whatever its layers). */
-HSD_API int hsd_debug_host_work(const hsd_ctx *ctx, long long *tile_choices);
+ * call, whatever its layers), `weight_maps` and `gemm_kernels` = tensor maps encoded and GEMM kernels loaded (or found loaded) by
+ * its creation: of the tile widths that its model's projections can be given. */
+HSD_API int hsd_debug_host_work(const hsd_ctx *ctx, long long *tile_choices, int *weight_maps, int *gemm_kernels);
 
 /* Test-only: the attention launch cuts the KV ranges of the query tiles into slices so that it has about `target_items`
  * work items (never more than CTA slots in one round), none shorter than `min_kv_tiles` 128-token KV tiles (two paged

@@ -110,7 +110,7 @@ def _load():
     lib.hsd_debug_tap.argtypes = [vp, i, i, vp, sz]
     lib.hsd_debug_set_gemm_tile.argtypes = [vp, i, i]
     lib.hsd_debug_set_attn_plan.argtypes = [vp, i, i]
-    lib.hsd_debug_host_work.argtypes = [vp, C.POINTER(C.c_longlong)]
+    lib.hsd_debug_host_work.argtypes = [vp, C.POINTER(C.c_longlong), C.POINTER(i), C.POINTER(i)]
     lib.hsd_op_linear.argtypes = [vp, vp, vp, vp, i, i, i, i, vp]
     lib.hsd_op_lm_head_argmax.argtypes = [vp, vp, i, vp, vp, sz, vp, vp, vp, vp]
     lib.hsd_op_lm_head_argmax_noalloc.argtypes = [vp, vp, i, vp, vp, vp, vp, vp]
@@ -326,9 +326,9 @@ def hsd_debug_set_gemm_tile(ctx, tile_n: int, k_slices: int) -> int:
 
 
 def hsd_debug_host_work(ctx):
-    n = C.c_longlong(0)
-    st = _lib.hsd_debug_host_work(ctx, C.byref(n))
-    return st, {"tile_choices": n.value}
+    n, maps, kernels = C.c_longlong(0), C.c_int(0), C.c_int(0)
+    st = _lib.hsd_debug_host_work(ctx, C.byref(n), C.byref(maps), C.byref(kernels))
+    return st, {"tile_choices": n.value, "weight_maps": maps.value, "gemm_kernels": kernels.value}
 
 
 def hsd_debug_set_attn_plan(ctx, target_items: int, min_kv_tiles: int) -> int:

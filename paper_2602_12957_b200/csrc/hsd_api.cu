@@ -51,7 +51,8 @@ struct hsd_ctx {
   bool attn_simt;     // attention through the plain kernel (debug)
   int last_cuda_error;
   long long launches;
-  long long tile_choices;       // hsd_debug_host_work
+  long long tile_choices;       // hsd_debug_host_work: tiles chosen, weight maps encoded, GEMM kernels of its modes
+  int n_weight_maps, n_gemm_kernels;
   bool profiling;
   // hsd_verify_regions_host: pinned staging and the cached graph of the last repeated call shape
   bool host_graph_ok;
@@ -572,9 +573,11 @@ int hsd_create(const hsd_model_config* cfg, const hsd_weights* w, hsd_ctx** out)
   }
 
   int dev = 0;
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return HSD_ERR_NO_DEVICE;
-  if (prop.major != 10) return HSD_ERR_NO_DEVICE;
+  int major = 0, n_sms = 0;      // (the two attributes alone: cudaGetDeviceProperties took 2.3 of a context's 2.5 ms)
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return HSD_ERR_NO_DEVICE;
+  if (major != 10) return HSD_ERR_NO_DEVICE;
 
   hsd_ctx* c = new (std::nothrow) hsd_ctx();
   if (!c) return HSD_ERR_INVALID_ARG;
@@ -596,7 +599,7 @@ int hsd_create(const hsd_model_config* cfg, const hsd_weights* w, hsd_ctx** out)
     c->q_norm.push_back(cfg->qk_norm ? static_cast<const bf16*>(w->q_norm[l]) : nullptr);
     c->k_norm.push_back(cfg->qk_norm ? static_cast<const bf16*>(w->k_norm[l]) : nullptr);
   }
-  c->n_sms = prop.multiProcessorCount;
+  c->n_sms = n_sms;
   c->device = dev;
   c->simt = (cfg->flags & HSD_FLAG_SIMT_DEBUG) != 0;
   c->attn_simt = c->simt || (cfg->flags & HSD_FLAG_SIMT_ATTENTION) != 0;
@@ -617,21 +620,25 @@ int hsd_create(const hsd_model_config* cfg, const hsd_weights* w, hsd_ctx** out)
   c->last_cuda_error = 0;
   c->launches = 0;
   c->tile_choices = 0;
+  c->n_weight_maps = c->n_gemm_kernels = 0;
   c->profiling = false;
   memset(c->prof_ms, 0, sizeof(c->prof_ms));
   memset(c->prof_n, 0, sizeof(c->prof_n));
   if (!c->simt) {
-    if (tma_init() || gemm_sm100_init(dev)) { delete c; return HSD_ERR_CUDA; }
+    const int qkv_mode = md.D == 128 ? GS_QKV_ROPE128 : GS_QKV_ROPE;
+    int bad = tma_init();
+    for (int mode : {qkv_mode, (int)GS_ADD_F32, (int)GS_SWIGLU, (int)GS_ARGMAX}) bad = bad || gemm_sm100_prepare(dev, mode, &c->n_gemm_kernels);
+    if (bad) { delete c; return HSD_ERR_CUDA; }
     c->tm_qkv.resize(md.n_layers); c->tm_o.resize(md.n_layers);
     c->tm_gate_up.resize(md.n_layers); c->tm_down.resize(md.n_layers);
-    int bad = 0;
+    int* n = &c->n_weight_maps;
     for (int l = 0; l < md.n_layers; ++l) {
-      bad |= make_weight_tmaps(&c->tm_qkv[l], c->w_qkv[l], md.qkv_out, md.d);
-      bad |= make_weight_tmaps(&c->tm_o[l], c->w_o[l], md.d, md.Hq * md.D);
-      bad |= make_weight_tmaps(&c->tm_gate_up[l], c->w_gate_up[l], 2 * md.ffn, md.d);
-      bad |= make_weight_tmaps(&c->tm_down[l], c->w_down[l], md.d, md.ffn);
+      bad |= make_weight_tmaps(&c->tm_qkv[l], c->w_qkv[l], md.qkv_out, md.d, qkv_mode, n);
+      bad |= make_weight_tmaps(&c->tm_o[l], c->w_o[l], md.d, md.Hq * md.D, GS_ADD_F32, n);
+      bad |= make_weight_tmaps(&c->tm_gate_up[l], c->w_gate_up[l], 2 * md.ffn, md.d, GS_SWIGLU, n);
+      bad |= make_weight_tmaps(&c->tm_down[l], c->w_down[l], md.d, md.ffn, GS_ADD_F32, n);
     }
-    bad |= make_weight_tmaps(&c->tm_lm_head, c->lm_head, md.V, md.d);
+    bad |= make_weight_tmaps(&c->tm_lm_head, c->lm_head, md.V, md.d, GS_ARGMAX, n);
     if (bad) { delete c; return HSD_ERR_CUDA; }
   }
   *out = c;
@@ -1161,9 +1168,11 @@ int hsd_debug_set_gemm_tile(hsd_ctx* c, int tile_n, int k_slices) {
   return HSD_OK;
 }
 
-int hsd_debug_host_work(const hsd_ctx* c, long long* tile_choices) {
-  if (!c || !tile_choices) return HSD_ERR_INVALID_ARG;
+int hsd_debug_host_work(const hsd_ctx* c, long long* tile_choices, int* weight_maps, int* gemm_kernels) {
+  if (!c || !tile_choices || !weight_maps || !gemm_kernels) return HSD_ERR_INVALID_ARG;
   *tile_choices = c->tile_choices;
+  *weight_maps = c->n_weight_maps;
+  *gemm_kernels = c->n_gemm_kernels;
   return HSD_OK;
 }
 
@@ -1189,13 +1198,16 @@ int hsd_op_linear(hsd_ctx* c, const void* A, const void* W, void* C, int M, int 
   }
   GemmSm100Args g = {};
   WeightMaps wm;
-  if (make_tmap_2d(&g.tmA, A, M, K, gemm_a_box_rows(M)) || make_weight_tmaps(&wm, W, n_out, K)) return HSD_ERR_CUDA;
+  if (make_tmap_2d(&g.tmA, A, M, K, gemm_a_box_rows(M))) return HSD_ERR_CUDA;
   if (mode == 1 ? make_tmap_2d_f32(&g.tmC, C, M, ldc, 32) : make_tmap_2d(&g.tmC, C, M, ldc, 32)) return HSD_ERR_CUDA;
   g.tmB = &wm;
   g.M = M; g.n_out = n_out; g.K = K; g.mode = mode;
   g.out.C = C; g.out.ldc = ldc;
   g.status = nullptr; g.n_sms = c->n_sms; g.max_splits = c->max_splits; g.pdl = false; g.pair = c->pair;
   g.tile = choose_tile(c, g, c->force_bn, c->force_splits);
+  int kernels = 0;
+  if (gemm_sm100_prepare(c->device, mode, &kernels)) return fail_cuda(c);
+  if (g.tile.bn && make_tmap_2d(&wm.half_tile(g.tile.bn), W, n_out, K, g.tile.bn / 2)) return HSD_ERR_CUDA;
   if (launch_gemm_sm100(st, g)) return fail_cuda(c);
   return check_cuda(c);
 }

@@ -25,6 +25,8 @@
 //                  leave the SM (Eq. 10 of the paper fused into the LM head)
 //   GS_QKV_ROPE    rotary embedding on q and k heads, q -> packed bf16, k/v -> paged KV pool (head_dim 64;
 //                  GS_QKV_ROPE128: the same for head_dim 128)
+#include <atomic>
+
 #include "hsd_kernels.h"
 
 namespace hsd {
@@ -81,12 +83,6 @@ int make_tmap_3d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, u
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? 0 : -1;
-}
-
-int make_weight_tmaps(WeightMaps* w, const void* base, uint64_t rows, uint64_t cols) {
-  int bad = 0;
-  for (int i = 0; i < WeightMaps::N; ++i) bad |= make_tmap_2d(&w->m[i], base, rows, cols, 16u * (i + 2));
-  return bad;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -763,6 +759,16 @@ constexpr bool has_width(int mode, int bn, bool pair) {
 static bool width_fits(int mode, int n_cols, int bn, bool pair) {
   return has_width(mode, bn, pair) && ((bn & (bn - 1)) || n_cols % (mode == GS_SWIGLU ? bn / 2 : bn) == 0);
 }
+int make_weight_tmaps(WeightMaps* w, const void* base, int rows, int cols, int mode, int* n_made) {
+  const int n_cols = mode == GS_SWIGLU ? rows / 2 : rows;
+  int bad = 0;
+  for (int bn = 64; bn <= 256; bn += 32) {
+    if (!width_fits(mode, n_cols, bn, false) && !width_fits(mode, n_cols, bn, true)) continue;
+    bad |= make_tmap_2d(&w->half_tile(bn), base, rows, cols, bn / 2);
+    ++*n_made;
+  }
+  return bad;
+}
 static TileChoice pick_tile(int mode, int n_cols, int M, int K, int n_sms, int max_splits, bool allow_pair) {
   const int k_blocks = K / KSUB;
   TileChoice best = {mode == GS_QKV_ROPE128 ? 128 : 64, 1, false};
@@ -810,8 +816,9 @@ static int launch_width(cudaStream_t st, const GemmSm100Args& a, int bn, int spl
   return -1;
 }
 
-// The shared memory each kernel is launched with.  Asked for when a context is created, which also loads the kernels: the
-// first step that picks a width does not wait for that.
+// The shared memory each kernel is launched with.  Asked for when a context is created, which also loads the kernels, ~50 us each:
+// the first step that picks a width does not wait for that.  A context loads the modes that its model's steps have, 43 kernels
+// with heads of 64 and 38 with heads of 128, of 56; the plain store is hsd_op_linear's alone.
 template <int BN, int MODE, bool PAIR, int ROWS = BM>
 static bool allow_smem_one() {
   return cudaFuncSetAttribute(gemm_sm100_kernel<BN, MODE, PAIR, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -825,16 +832,28 @@ static bool allow_smem() {
   if constexpr (BN < 256) ok = allow_smem<MODE, PAIR, BN + 32>() && ok;
   return ok;
 }
-template <int... MODES>
-static bool allow_smem_all() {
-  return ((allow_smem<MODES, false>() && allow_smem<MODES, true>()) && ...);
-}
-int gemm_sm100_init(int device) {
-  static bool done[kMaxDevices] = {};              // the attribute is per device
-  if (device < 0 || device >= kMaxDevices) return -1;
-  if (!done[device] && !allow_smem_all<GS_STORE_BF16, GS_ADD_F32, GS_SWIGLU, GS_ARGMAX, GS_QKV_ROPE, GS_QKV_ROPE128>()) return -1;
-  done[device] = true;
+template <int MODE>
+static int prepare_mode(int device, int* n_kernels) {
+  static std::atomic<bool> done[kMaxDevices];      // the attribute is per device; contexts may be created by several threads
+  for (int bn = 64; bn <= 256; bn += 32)
+    *n_kernels += has_width(MODE, bn, false) * (bn == 64 ? 3 : 1) + has_width(MODE, bn, true);
+  if (!done[device]) {
+    if (!allow_smem<MODE, false>() || !allow_smem<MODE, true>()) return -1;
+    done[device] = true;
+  }
   return 0;
+}
+int gemm_sm100_prepare(int device, int mode, int* n_kernels) {
+  if (device < 0 || device >= kMaxDevices) return -1;
+  switch (mode) {
+    case GS_STORE_BF16: return prepare_mode<GS_STORE_BF16>(device, n_kernels);
+    case GS_ADD_F32: return prepare_mode<GS_ADD_F32>(device, n_kernels);
+    case GS_SWIGLU: return prepare_mode<GS_SWIGLU>(device, n_kernels);
+    case GS_ARGMAX: return prepare_mode<GS_ARGMAX>(device, n_kernels);
+    case GS_QKV_ROPE: return prepare_mode<GS_QKV_ROPE>(device, n_kernels);
+    case GS_QKV_ROPE128: return prepare_mode<GS_QKV_ROPE128>(device, n_kernels);
+    default: return -1;
+  }
 }
 
 TileChoice gemm_choose_tile(const GemmSm100Args& a, int force_bn, int force_splits) {

@@ -222,13 +222,15 @@ void launch_gemm_simt(cudaStream_t st, const bf16* A, const bf16* W, int M, int 
 int make_tmap_2d(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 // Same for fp32 with a {32, box_rows} box (128-byte rows): the residual stream as a TMA reduce-add target.
 int make_tmap_2d_f32(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
-// The maps of one weight matrix, box heights 32, 48 .. 128 rows = half a tile of width 64, 96 .. 256.
+// The maps of one weight matrix, box heights 32, 48 .. 128 rows = half a tile of width 64, 96 .. 256: of the widths that its
+// projection can be given.
 struct WeightMaps {
   static constexpr int N = 7;
   CUtensorMap m[N];
+  CUtensorMap& half_tile(int bn) { return m[bn / 32 - 2]; }
   const CUtensorMap& half_tile(int bn) const { return m[bn / 32 - 2]; }
 };
-int make_weight_tmaps(WeightMaps* w, const void* base, uint64_t rows, uint64_t cols);
+int make_weight_tmaps(WeightMaps* w, const void* base, int rows, int cols, int mode, int* n_made);   // (mode: GemmSm100Mode)
 int make_tmap_3d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t stride1_bytes,
                  uint64_t stride2_bytes, uint32_t b0, uint32_t b1, uint32_t b2);
 int tma_init();   // resolves cuTensorMapEncodeTiled; 0 on success
@@ -268,7 +270,8 @@ struct GemmSm100Args {
   TileChoice tile;             // gemm_choose_tile's
 };
 enum GemmSm100Mode { GS_STORE_BF16 = 0, GS_ADD_F32 = 1, GS_SWIGLU = 2, GS_ARGMAX = 4, GS_QKV_ROPE = 5, GS_QKV_ROPE128 = 6 };
-int gemm_sm100_init(int device);      // once per device (the current one) before its first launch; 0 on success
+// Loads the kernels of a mode on the current device (ordinal `device`), before their first launch there; 0 on success.
+int gemm_sm100_prepare(int device, int mode, int* n_kernels);
 // The tile of a problem, by its M, n_out, K, mode, n_sms, max_splits and pair alone: one choice serves every layer of a call.
 // Tests: `force_bn` = tile width (above 256: a CTA pair, 256 columns less), `force_splits` = K slices instead of the model's
 // choice (0 = choose).

@@ -1,5 +1,6 @@
 """The host's work around a call's launches does not grow with the decoder's depth: GEMM tiles are chosen once per projection
-of a call and once for its LM head."""
+of a call and once for its LM head.  A context's creation loads the kernels and encodes the maps of the tile widths that its
+projections can be given, and no others."""
 import numpy as np
 import pytest
 
@@ -32,3 +33,19 @@ def test_one_tile_choice_per_projection_and_call(layers):
     x = torch.zeros(64, 64, dtype=torch.bfloat16, device=model.device)
     st = torch.cuda.current_stream().cuda_stream
     assert choices(lambda: B.check(B.hsd_op_linear(model.ctx, x, x, x.clone(), 64, 64, 64, 0, st))) == 1
+
+
+# widths of a projection's tiles, pairs' among them: heads of 64 keep whole heads, heads of 128 too; kernels: three for a width of 64
+# (at most 16, at most 64 and more rows), and one more for each width that pairs have too
+@pytest.mark.parametrize("head_dim,qkv_maps,qkv_kernels", [(64, 4, 6 + 3), (128, 2, 2 + 2)])
+def test_a_context_prepares_its_models_widths_only(head_dim, qkv_maps, qkv_kernels):
+    from paper_2602_12957_b200 import binding as B
+    from paper_2602_12957_b200 import runtime as R
+    cfg = I.ModelConfig(n_layers=3, d_model=512, n_heads=4, n_kv_heads=2, head_dim=head_dim, d_ffn=1024, vocab=1024)
+    model = R.DeviceModel(cfg, I.make_weights(cfg, 1))
+    for m in (model, model.sibling(B.HSD_FLAG_DETERMINISTIC)):
+        work = B.hsd_debug_host_work(m.ctx)[1]
+        # residual adds 64, 96 .. 256, SwiGLU the same without 96, LM head 64, 128, 256
+        assert work["weight_maps"] == 3 * (qkv_maps + 7 + 6 + 7) + 3
+        assert work["gemm_kernels"] == qkv_kernels + (8 + 6) + (8 + 5) + (5 + 2)
+        assert work["tile_choices"] == 0
