@@ -384,8 +384,10 @@ HSD_API int hsd_op_linear(hsd_ctx *ctx, const void *A, const void *W, void *C, i
  * 256, mode 1 also 96 and 160, mode 2 also 160 and 224; 256 + n = a pair of CTAs sharing a tile of 256 rows and n columns,
  * n = 128, 192 or 256, mode 1 also 96, 160 and 224, mode 2 also 160 and 224) and, for mode 1, `k_slices`
  * slices of K per tile (the 64-wide tile cuts K in steps of 128 columns, into fewer slices where one would be empty),
- * instead of what the library would choose for the problem; 0 = choose.  A combination the
- * problem does not allow makes hsd_op_linear return HSD_ERR_CUDA.  Lets the parity tests reach every tile shape. */
+ * instead of what the library would choose for the problem; 0 = choose.  With at most 64 rows a pair's tile is one CTA's of as
+ * many columns (mode 1, 480: of 256).  The width reaches the QKV projection of steps as well, whose tiles are 64 (heads of 64), 128,
+ * 192 (heads of 64) or 256 columns wide, pairs' 128, 192 (heads of 64) or 256.  A combination the problem does not allow makes
+ * hsd_op_linear, or the step, return HSD_ERR_CUDA.  Lets the parity tests reach every tile shape. */
 HSD_API int hsd_debug_set_gemm_tile(hsd_ctx *ctx, int tile_n, int k_slices);
 
 /* Test-only: host work of this context so far: `tile_choices` = how often it has chosen a GEMM tile (once per projection of a

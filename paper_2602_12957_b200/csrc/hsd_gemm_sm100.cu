@@ -863,9 +863,12 @@ TileChoice gemm_choose_tile(const GemmSm100Args& a, int force_bn, int force_spli
   if (force_bn) {
     c.pair = force_bn > 256;                                // a CTA pair on tiles of 256 rows and 256 columns less
     c.bn = c.pair ? force_bn - 256 : force_bn;
-    c.pair = c.pair && a.M > 64;                            // (its tile needs whole boxes)
-    if (!c.pair && c.bn == 224 && a.mode != GS_SWIGLU) c.bn = 256;
     if (!width_fits(a.mode, n_cols, c.bn, c.pair)) return none;
+    if (c.pair && a.M <= 64) {                              // a pair's tile needs whole boxes: one CTA in its place,
+      c.pair = false;                                       // of 256 columns where only pairs have the width
+      if (!has_width(a.mode, c.bn, false)) c.bn = 256;
+      if (!width_fits(a.mode, n_cols, c.bn, false)) return none;
+    }
   }
   if (force_splits) {
     const int kbs = (a.K / KSUB + force_splits - 1) / force_splits;

@@ -49,3 +49,24 @@ def test_widths(model, tile, M, N, K):
                 assert np.abs(got - want).max() <= tol, (mode, slices, np.abs(got - want).max(), tol)
     finally:
         B.hsd_debug_set_gemm_tile(model.ctx, 0, 0)
+
+
+# tile, mode, rows: widths that a mode does not have, and those that only its pairs have (whose place one CTA takes up to 64 rows)
+@pytest.mark.parametrize("tile,mode,M,allowed", [
+    (224, 0, 129, False), (224, 1, 129, False), (224, 1, 16, False), (224, 2, 129, True), (480, 0, 64, False), (480, 0, 129, False),
+    (480, 1, 64, True), (480, 1, 129, True), (480, 2, 64, True), (320, 0, 64, False), (320, 1, 64, False), (320, 1, 129, False),
+    (96, 0, 64, False), (96, 1, 64, True), (352, 0, 64, False), (100, 1, 64, False)])
+def test_forced_widths_are_taken_or_refused(model, tile, mode, M, allowed):
+    import torch
+    from paper_2602_12957_b200 import binding as B
+    N, K = 512, 128
+    A, W = (torch.ones(n, K, dtype=torch.bfloat16, device=model.device) for n in (M, N))
+    C = torch.zeros(M, N // 2 if mode == 2 else N, dtype=torch.float32 if mode == 1 else torch.bfloat16, device=model.device)
+    try:
+        B.check(B.hsd_debug_set_gemm_tile(model.ctx, tile, 0))
+        st = B.hsd_op_linear(model.ctx, A, W, C, M, N, K, mode, torch.cuda.current_stream().cuda_stream)
+    finally:
+        B.hsd_debug_set_gemm_tile(model.ctx, 0, 0)
+    assert st == (B.HSD_OK if allowed else B.HSD_ERR_CUDA)
+    # refused: nothing was launched; sums of K ones are exact (SwiGLU of 128: 128 * 128)
+    assert bool((C == ((K * K if mode == 2 else K) if allowed else 0)).all())
