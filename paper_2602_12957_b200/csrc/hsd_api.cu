@@ -379,8 +379,8 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
   for (int l = 0; l < md.n_layers; ++l) {
     {
       Scope s(c, st, KC_RMSNORM);
-      if (l == 0) launch_first_rmsnorm(st, w.x, c->attn_norm[l], w.h, T, md.d, md.eps, w.verdict, setup_ctas(T), w.status, c->pdl);
-      else launch_rmsnorm(st, w.x, c->attn_norm[l], w.h, T, md.d, md.eps, nullptr, T, w.status, c->pdl);
+      if (l == 0) launch_first_rmsnorm(st, w.x, c->attn_norm[l], w.h, T, md.d, md.eps, w.verdict, setup_ctas(T), w.status, c->n_sms, c->pdl);
+      else launch_rmsnorm(st, w.x, c->attn_norm[l], w.h, T, md.d, md.eps, nullptr, T, w.status, c->n_sms, c->pdl);
     }
     if (int rc = tap(l, HSD_TAP_H_ATTN, w.h, 2 * row_d)) return rc;
     const size_t layer_elems = (size_t)kv.n_blocks * md.Hkv * 64 * md.D;
@@ -432,7 +432,7 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
     if (int rc = tap(l, HSD_TAP_X_MID, w.x, 4 * row_d)) return rc;
     {
       Scope s(c, st, KC_RMSNORM);
-      launch_rmsnorm(st, w.x, c->ffn_norm[l], w.h, T, md.d, md.eps, nullptr, T, w.status, c->pdl);
+      launch_rmsnorm(st, w.x, c->ffn_norm[l], w.h, T, md.d, md.eps, nullptr, T, w.status, c->n_sms, c->pdl);
     }
     if (int rc = tap(l, HSD_TAP_H_FFN, w.h, 2 * row_d)) return rc;
     if (c->simt) {
@@ -502,7 +502,7 @@ int verify_common(hsd_ctx* c, const hsd_kv* kv, const StepArgs& a, float log_tau
   if (rc) return rc;
   {
     Scope s(c, st, KC_RMSNORM);
-    launch_rmsnorm(st, w.x, c->final_norm, w.h, a.total_q, c->md.d, c->md.eps, nullptr, a.total_q, w.status, c->pdl);
+    launch_rmsnorm(st, w.x, c->final_norm, w.h, a.total_q, c->md.d, c->md.eps, nullptr, a.total_q, w.status, c->n_sms, c->pdl);
   }
   rc = run_lm_head(c, w, a.total_q, w.rm.row_next, st);
   if (rc) return rc;
@@ -684,7 +684,7 @@ int hsd_prefill(hsd_ctx* c, const hsd_kv* kv, int n_seqs, const int* cu_len, con
   }
   {
     Scope s(c, st, KC_RMSNORM);
-    launch_rmsnorm(st, w.x, c->final_norm, w.h, n_seqs, c->md.d, c->md.eps, w.sel_rows, total_rows, w.status, c->pdl);
+    launch_rmsnorm(st, w.x, c->final_norm, w.h, n_seqs, c->md.d, c->md.eps, w.sel_rows, total_rows, w.status, c->n_sms, c->pdl);
   }
   rc = run_lm_head(c, w, n_seqs, nullptr, st);
   if (rc) return rc;

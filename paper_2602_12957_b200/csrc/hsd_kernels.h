@@ -106,11 +106,11 @@ void launch_setup_rows(cudaStream_t st, const SetupArgs& a, const KvView& kv, co
 // h[r] = bf16(rmsnorm(x[src]) * gain), src = sel_rows ? sel_rows[r] : r.  The gather form (sel_rows != nullptr) writes
 // nothing when *status is set or src is outside [0, src_rows): the index comes from an earlier kernel of the step.
 void launch_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
-                    const int* sel_rows, int src_rows, const int* status, bool pdl);
+                    const int* sel_rows, int src_rows, const int* status, int n_sms, bool pdl);
 // The first of a step (every row, in place order), which follows launch_setup_rows: it also turns the verdicts into the
 // status words.
 void launch_first_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
-                          const int2* verdict, int n_verdicts, int* status, bool pdl);
+                          const int2* verdict, int n_verdicts, int* status, int n_sms, bool pdl);
 // last row of every sequence (prefill's LM-head rows); -1 for every sequence when *status is set
 void launch_select_last_rows(cudaStream_t st, const RowMeta& rm, int n_seqs, int* sel_rows, const int* status, bool pdl);
 // q_norm / k_norm: per-head RMSNorm gains applied before the rotation, or nullptr

@@ -262,10 +262,10 @@ __global__ void rmsnorm_kernel(const float* __restrict__ x, const bf16* __restri
 }
 static void launch_rmsnorm_any(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
                                const int* sel_rows, int src_rows, const int* status, const int2* verdict, int n_verdicts,
-                               int* status_out, bool pdl) {
-  // Four rows a CTA while that leaves no SM with two of them, eight otherwise: 16 rows 1.95 us a launch with eight and 1.81 with
-  // four, 513 rows 2.55 and 2.37, ~1,090 rows 3.19 and 3.74 (two rows a CTA as four, sixteen 2.57 / 2.78 / 3.25).
-  const int per = rows <= 4 * 148 ? 4 : 8;
+                               int* status_out, int n_sms, bool pdl) {
+  // Four rows a CTA while no SM gets two of the launch's CTAs by that, eight otherwise: 16 rows 1.95 us a launch with eight and 1.81
+  // with four, 513 rows 2.55 and 2.37, ~1,090 rows 3.19 and 3.74 (two rows a CTA as four, sixteen 2.57 / 2.78 / 3.25).
+  const int per = (rows + 3) / 4 + (verdict ? 1 : 0) <= n_sms ? 4 : 8;
   dim3 grid((rows + per - 1) / per + (verdict ? 1 : 0)), block(32 * per);
 #define HSD_RMS_CASE(V)                                                                                                  \
   case V:                                                                                                                \
@@ -279,12 +279,12 @@ static void launch_rmsnorm_any(cudaStream_t st, const float* x, const bf16* gain
 #undef HSD_RMS_CASE
 }
 void launch_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
-                    const int* sel_rows, int src_rows, const int* status, bool pdl) {
-  if (rows > 0) launch_rmsnorm_any(st, x, gain, h, rows, d, eps, sel_rows, src_rows, status, nullptr, 0, nullptr, pdl);
+                    const int* sel_rows, int src_rows, const int* status, int n_sms, bool pdl) {
+  if (rows > 0) launch_rmsnorm_any(st, x, gain, h, rows, d, eps, sel_rows, src_rows, status, nullptr, 0, nullptr, n_sms, pdl);
 }
 void launch_first_rmsnorm(cudaStream_t st, const float* x, const bf16* gain, bf16* h, int rows, int d, float eps,
-                          const int2* verdict, int n_verdicts, int* status, bool pdl) {
-  launch_rmsnorm_any(st, x, gain, h, rows, d, eps, nullptr, rows, nullptr, verdict, n_verdicts, status, pdl);
+                          const int2* verdict, int n_verdicts, int* status, int n_sms, bool pdl) {
+  launch_rmsnorm_any(st, x, gain, h, rows, d, eps, nullptr, rows, nullptr, verdict, n_verdicts, status, n_sms, pdl);
 }
 
 // The final norm of a tree step: h as above, and for every node the logit of its own token under its PARENT's distribution,
