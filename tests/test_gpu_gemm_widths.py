@@ -37,7 +37,8 @@ def test_widths(model, tile, M, N, K):
                 g, u = ref[:, :N // 2], ref[:, N // 2:]
                 want = g / (1.0 + np.exp(-g)) * u
             for slices in ((1, 2, 3, 4) if mode == 1 and K > 320 else (0,)):
-                # rows and columns around the output: must stay as they were
+                # rows behind the output: must stay as they were (a store beyond the last column of a row lands in the next one,
+                # that of the last row in these)
                 C = torch.full((M + 8, want.shape[1]), 3.0, dtype=torch.float32 if mode == 1 else torch.bfloat16, device=dev)
                 B.check(B.hsd_debug_set_gemm_tile(model.ctx, tile, slices))
                 B.check(B.hsd_op_linear(model.ctx, tA, tW, C, M, N, K, mode, st))

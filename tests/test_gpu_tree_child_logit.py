@@ -9,7 +9,7 @@ from paper_2602_12957_b200 import inputs as I
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("d", [128, 256, 1024, 2048, 4096])
+@pytest.mark.parametrize("d", [128, 256, 512, 1024, 2048, 4096])
 @pytest.mark.parametrize("rows", [[1], [9, 1, 128]])
 def test_child_logits(d, rows):
     import torch
