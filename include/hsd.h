@@ -390,8 +390,8 @@ HSD_API int hsd_op_linear(hsd_ctx *ctx, const void *A, const void *W, void *C, i
  * hsd_op_linear, or the step, return HSD_ERR_CUDA.  Lets the parity tests reach every tile shape. */
 HSD_API int hsd_debug_set_gemm_tile(hsd_ctx *ctx, int tile_n, int k_slices);
 
-/* Test-only: host work of this context so far: `tile_choices` = how often it has chosen a GEMM tile (once per projection of a
- * call, whatever its layers), `weight_maps` and `gemm_kernels` = tensor maps encoded and GEMM kernels loaded (or found loaded) by
+/* Test-only: host work of this context so far: `tile_choices` = how often it has chosen a GEMM tile (at its creation, for calls of
+ * up to 8,192 rows; once per projection of a larger call, whatever its layers; by every hsd_op_linear), `weight_maps` and `gemm_kernels` = tensor maps encoded and GEMM kernels loaded (or found loaded) by
  * its creation: of the tile widths that its model's projections can be given. */
 HSD_API int hsd_debug_host_work(const hsd_ctx *ctx, long long *tile_choices, int *weight_maps, int *gemm_kernels);
 

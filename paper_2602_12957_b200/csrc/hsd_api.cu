@@ -28,6 +28,12 @@ struct HostCallKey {
   int pad;
 };
 
+// The tiles of one projection for calls of up to 8,192 rows, by row class; larger calls, which take milliseconds, choose theirs.
+struct TilePlan {
+  static constexpr int kRows = 8192;
+  TileChoice of[3 + kRows / 128];
+};
+
 struct hsd_ctx {
   hsd_model_config cfg;
   ModelDims md;
@@ -36,6 +42,7 @@ struct hsd_ctx {
   std::vector<const bf16*> q_norm, k_norm;    // per layer, nullptr when the model has no per-head q/k norm
   std::vector<WeightMaps> tm_qkv, tm_o, tm_gate_up, tm_down;
   WeightMaps tm_lm_head;
+  TilePlan tiles_qkv, tiles_o, tiles_gate_up, tiles_down, tiles_lm_head;
   int max_splits;     // K slices the residual-add projections may use (1 with HSD_FLAG_DETERMINISTIC)
   bool pdl;           // kernels are launched with programmatic stream serialization
   int force_bn, force_splits;   // hsd_debug_set_gemm_tile
@@ -265,6 +272,18 @@ TileChoice choose_tile(hsd_ctx* c, const GemmSm100Args& g, int force_bn, int for
   ++c->tile_choices;
   return gemm_choose_tile(g, force_bn, force_splits);
 }
+TileChoice planned_tile(hsd_ctx* c, const GemmSm100Args& g, const TilePlan& plan) {
+  return g.M <= TilePlan::kRows ? plan.of[gemm_row_class(g.M)] : choose_tile(c, g, 0, 0);
+}
+void make_tile_plan(hsd_ctx* c, TilePlan* plan, int n_out, int K, int mode) {
+  GemmSm100Args g = {};
+  g.n_out = n_out; g.K = K; g.mode = mode; g.n_sms = c->n_sms; g.pair = c->pair;
+  g.max_splits = mode == GS_ADD_F32 ? c->max_splits : 1;
+  for (int k = 0; k < 3 + TilePlan::kRows / 128; ++k) {
+    g.M = gemm_class_rows(k);
+    plan->of[k] = choose_tile(c, g, 0, 0);
+  }
+}
 
 struct StepArgs {
   int n_seqs, total_q, max_q_len;
@@ -279,8 +298,9 @@ struct StepArgs {
   const int* parent;   // candidate trees: parent row within the sequence, or nullptr (chains)
 };
 
-// The decoder forward over one packed batch: rows -> residual stream x after the last layer.
-int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cudaStream_t st) {
+// The decoder forward over one packed batch: rows -> residual stream x after the last layer.  `tm_h`: where the map of the
+// batch's normed rows goes.
+int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, CUtensorMap& tm_h, cudaStream_t st) {
   const ModelDims& md = c->md;
   const KvView kv = kv_view(kvp);
   const int T = a.total_q;
@@ -330,7 +350,7 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
     launch_setup_rows(st, sa, kv, w.rm, c->pdl);
   }
 
-  CUtensorMap tm_h, tm_attn, tm_act, tm_q, tm_k, tm_v, tm_x_add, tm_q_st, tm_act_st;
+  CUtensorMap tm_attn, tm_act, tm_q, tm_k, tm_v, tm_x_add, tm_q_st, tm_act_st;
   if (!c->simt) {
     const uint32_t box = gemm_a_box_rows(T);
     if (make_tmap_2d(&tm_h, w.h, T, md.d, box) || make_tmap_2d(&tm_attn, w.attn, T, md.Hq * md.D, box) ||
@@ -352,28 +372,28 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
   }
 
   // what the projections of every layer have in common, the tiles among it
-  GemmSm100Args g_qkv, g_o, g_gate_up, g_down;
+  GemmSm100Args g_qkv = {}, g_o = {}, g_gate_up = {}, g_down = {};
   if (!c->simt) {
     auto projection = [&](GemmSm100Args& g, const CUtensorMap& tmA, const CUtensorMap& tmC, int n_out, int K, int mode, int max_splits,
-                          int force_bn) {
-      g = {};
+                          const TilePlan& plan) {
       g.tmA = tmA;
       g.tmC = tmC;
       g.M = T; g.n_out = n_out; g.K = K; g.mode = mode;
       g.status = w.status; g.n_sms = c->n_sms; g.max_splits = max_splits; g.pdl = c->pdl; g.pair = c->pair;
-      g.tile = choose_tile(c, g, force_bn, 0);
+      g.tile = planned_tile(c, g, plan);
     };
-    projection(g_qkv, tm_h, tm_q_st, md.qkv_out, md.d, md.D == 128 ? GS_QKV_ROPE128 : GS_QKV_ROPE, 1, c->force_bn);
+    projection(g_qkv, tm_h, tm_q_st, md.qkv_out, md.d, md.D == 128 ? GS_QKV_ROPE128 : GS_QKV_ROPE, 1, c->tiles_qkv);
+    if (c->force_bn) g_qkv.tile = choose_tile(c, g_qkv, c->force_bn, 0);
     g_qkv.qkv.row_kv = w.rm.row_kv;
     g_qkv.qkv.kv_rows = kv.n_blocks * HSD_KV_BLOCK;
     g_qkv.qkv.rope_cs = w.rm.rope_cs;
     g_qkv.qkv.q_out = w.q;
     g_qkv.qkv.Hq = md.Hq; g_qkv.qkv.Hkv = md.Hkv; g_qkv.qkv.D = md.D;
     g_qkv.qkv.eps = md.eps;
-    projection(g_o, tm_attn, tm_x_add, md.d, md.Hq * md.D, GS_ADD_F32, c->max_splits, 0);
-    projection(g_gate_up, tm_h, tm_act_st, 2 * md.ffn, md.d, GS_SWIGLU, 1, 0);
+    projection(g_o, tm_attn, tm_x_add, md.d, md.Hq * md.D, GS_ADD_F32, c->max_splits, c->tiles_o);
+    projection(g_gate_up, tm_h, tm_act_st, 2 * md.ffn, md.d, GS_SWIGLU, 1, c->tiles_gate_up);
     g_gate_up.out.C = w.act; g_gate_up.out.ldc = md.ffn;
-    projection(g_down, tm_act, tm_x_add, md.d, md.ffn, GS_ADD_F32, c->max_splits, 0);
+    projection(g_down, tm_act, tm_x_add, md.d, md.ffn, GS_ADD_F32, c->max_splits, c->tiles_down);
   }
 
   for (int l = 0; l < md.n_layers; ++l) {
@@ -465,22 +485,22 @@ int run_layers(hsd_ctx* c, const hsd_kv* kvp, const StepArgs& a, const Ws& w, cu
 }
 
 // LM head + running argmax over `rows` rows of h (already selected / normalised into w.h); the set-up kernel cleared them.
-int run_lm_head(hsd_ctx* c, const Ws& w, int rows, const int* row_next, cudaStream_t st) {
+// `tm_h`: run_layers' map of h, where the rows are the batch's, or nullptr.
+int run_lm_head(hsd_ctx* c, const Ws& w, int rows, const CUtensorMap* tm_h, const int* row_next, cudaStream_t st) {
   const ModelDims& md = c->md;
   Scope s(c, st, KC_LMHEAD);
   GemmOut o = {nullptr, 0, w.row_best, w.zdraft, row_next};
   if (c->simt) {
     launch_gemm_simt(st, w.h, c->lm_head, rows, md.V, md.d, GM_ARGMAX, o);
   } else {
-    CUtensorMap tm_h;
-    if (make_tmap_2d(&tm_h, w.h, rows, md.d, gemm_a_box_rows(rows))) return HSD_ERR_CUDA;
     GemmSm100Args g = {};
-    g.tmA = tm_h;
+    if (tm_h) g.tmA = *tm_h;
+    else if (make_tmap_2d(&g.tmA, w.h, rows, md.d, gemm_a_box_rows(rows))) return HSD_ERR_CUDA;
     g.tmB = &c->tm_lm_head;
     g.M = rows; g.n_out = md.V; g.K = md.d; g.mode = GS_ARGMAX;
     g.out = o;
     g.status = w.status; g.n_sms = c->n_sms; g.max_splits = 1; g.pdl = c->pdl; g.pair = c->pair;
-    g.tile = choose_tile(c, g, 0, 0);
+    g.tile = planned_tile(c, g, c->tiles_lm_head);
     if (launch_gemm_sm100(st, g)) return fail_cuda(c);
   }
   return check_cuda(c);
@@ -498,13 +518,14 @@ int verify_common(hsd_ctx* c, const hsd_kv* kv, const StepArgs& a, float log_tau
   int rc = check_ws(c, workspace, ws_bytes, a.total_q, a.n_seqs);
   if (rc) return rc;
   const Ws w = carve(c, workspace, a.total_q, a.n_seqs);
-  rc = run_layers(c, kv, a, w, st);
+  CUtensorMap tm_h;
+  rc = run_layers(c, kv, a, w, tm_h, st);
   if (rc) return rc;
   {
     Scope s(c, st, KC_RMSNORM);
     launch_rmsnorm(st, w.x, c->final_norm, w.h, a.total_q, c->md.d, c->md.eps, nullptr, a.total_q, w.status, c->n_sms, c->pdl);
   }
-  rc = run_lm_head(c, w, a.total_q, w.rm.row_next, st);
+  rc = run_lm_head(c, w, a.total_q, &tm_h, w.rm.row_next, st);
   if (rc) return rc;
   {
     Scope s(c, st, KC_ACCEPT);
@@ -640,6 +661,11 @@ int hsd_create(const hsd_model_config* cfg, const hsd_weights* w, hsd_ctx** out)
     }
     bad |= make_weight_tmaps(&c->tm_lm_head, c->lm_head, md.V, md.d, GS_ARGMAX, n);
     if (bad) { delete c; return HSD_ERR_CUDA; }
+    make_tile_plan(c, &c->tiles_qkv, md.qkv_out, md.d, qkv_mode);
+    make_tile_plan(c, &c->tiles_o, md.d, md.Hq * md.D, GS_ADD_F32);
+    make_tile_plan(c, &c->tiles_gate_up, 2 * md.ffn, md.d, GS_SWIGLU);
+    make_tile_plan(c, &c->tiles_down, md.d, md.ffn, GS_ADD_F32);
+    make_tile_plan(c, &c->tiles_lm_head, md.V, md.d, GS_ARGMAX);
   }
   *out = c;
   return HSD_OK;
@@ -676,7 +702,8 @@ int hsd_prefill(hsd_ctx* c, const hsd_kv* kv, int n_seqs, const int* cu_len, con
   StepArgs a = {};
   a.n_seqs = n_seqs; a.total_q = total_rows; a.max_q_len = max_len; a.prefill = true;
   a.cu_q = cu_len; a.tokens = token_ids; a.embeds = embeds; a.seq_slots = seq_slots; a.slot_base = 0;
-  rc = run_layers(c, kv, a, w, st);
+  CUtensorMap tm_h;
+  rc = run_layers(c, kv, a, w, tm_h, st);
   if (rc) return rc;
   {
     Scope s(c, st, KC_RMSNORM);
@@ -686,7 +713,7 @@ int hsd_prefill(hsd_ctx* c, const hsd_kv* kv, int n_seqs, const int* cu_len, con
     Scope s(c, st, KC_RMSNORM);
     launch_rmsnorm(st, w.x, c->final_norm, w.h, n_seqs, c->md.d, c->md.eps, w.sel_rows, total_rows, w.status, c->n_sms, c->pdl);
   }
-  rc = run_lm_head(c, w, n_seqs, nullptr, st);
+  rc = run_lm_head(c, w, n_seqs, nullptr, nullptr, st);
   if (rc) return rc;
   {
     Scope s(c, st, KC_ACCEPT);
@@ -734,14 +761,15 @@ int hsd_verify_tree(hsd_ctx* c, const hsd_kv* kv, int n_seqs, const int* cu_q, c
   StepArgs a = {};
   a.n_seqs = n_seqs; a.total_q = total_q; a.max_q_len = max_q_len; a.prefill = false;
   a.cu_q = cu_q; a.tokens = q_tokens; a.seq_slots = seq_slots; a.slot_base = 0; a.parent = parent;
-  rc = run_layers(c, kv, a, w, st);
+  CUtensorMap tm_h;
+  rc = run_layers(c, kv, a, w, tm_h, st);
   if (rc) return rc;
   {
     Scope s(c, st, KC_RMSNORM);
     launch_tree_final_norm(st, w.x, c->final_norm, w.h, total_q, c->md.d, c->md.eps, w.rm, c->lm_head, c->md.V, w.zdraft, w.status,
                            c->pdl);
   }
-  rc = run_lm_head(c, w, total_q, nullptr, st);
+  rc = run_lm_head(c, w, total_q, &tm_h, nullptr, st);
   if (rc) return rc;
   {
     Scope s(c, st, KC_ACCEPT);
@@ -1113,7 +1141,7 @@ static int lm_head_argmax_impl(hsd_ctx* c, const void* h, int rows, const int* n
       g.M = rows; g.n_out = md.V; g.K = md.d; g.mode = GS_ARGMAX;
       g.out = o;
       g.status = nullptr; g.n_sms = c->n_sms; g.max_splits = 1; g.pdl = false; g.pair = c->pair;
-      g.tile = choose_tile(c, g, 0, 0);
+      g.tile = planned_tile(c, g, c->tiles_lm_head);
       if (launch_gemm_sm100(st, g)) return fail_cuda(c);
     }
   }

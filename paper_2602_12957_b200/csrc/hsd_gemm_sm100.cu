@@ -740,8 +740,9 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
 // Its choices are within 0.8 % of the best timed one on average (worst 8.5 %).  With widths of 64, 128 and 256 (pairs: 256) and a
 // model by fill rates alone it was 8.1 % (worst 70 %).  A layer's four projections, before / now: 300 rows 28.6 / 26.1 us, 600
 // rows 37.8 / 32.3, 900 rows 41.2 / 38.5, 1,323 rows 52.5 / 48.3, 2,600 rows 83 / 73, 5,000 rows 147 / 123, 9,300 rows 217 / 216.
-// A choice takes ~0.25 us of the host: it is made once a call and projection, not for every layer (enqueueing a 24-layer step of
-// 144 rows 455 -> 427 us, of 1,058 rows 447 -> 430).
+// A choice takes ~0.2 us of the host (residual adds 0.5).  It depends on the rows through gemm_row_class alone: a context makes the
+// choices of every class when it is created and a call looks its five up.  (Made for every layer of a call they were 1 us of a
+// one-layer step's 29 us of enqueueing and 25 us of 24 layers' 430.)
 // Tile widths a mode has: whole heads for the rotary epilogues, whole 64-column stores for the plain one; the adds take any 32
 // columns, SwiGLU any 16.
 constexpr bool has_width(int mode, int bn, bool pair) {
@@ -859,7 +860,7 @@ int gemm_sm100_prepare(int device, int mode, int* n_kernels) {
 TileChoice gemm_choose_tile(const GemmSm100Args& a, int force_bn, int force_splits) {
   const int n_cols = (a.mode == GS_SWIGLU) ? a.n_out / 2 : a.n_out;
   const TileChoice none = {0, 0, false};
-  TileChoice c = pick_tile(a.mode, n_cols, a.M, a.K, a.n_sms, (a.mode == GS_ADD_F32 && a.max_splits > 1) ? a.max_splits : 1, a.pair != 0);
+  TileChoice c = pick_tile(a.mode, n_cols, gemm_class_rows(gemm_row_class(a.M)), a.K, a.n_sms, (a.mode == GS_ADD_F32 && a.max_splits > 1) ? a.max_splits : 1, a.pair != 0);
   if (force_bn) {
     c.pair = force_bn > 256;                                // a CTA pair on tiles of 256 rows and 256 columns less
     c.bn = c.pair ? force_bn - 256 : force_bn;

@@ -250,6 +250,9 @@ struct QkvEpilogue {      // fused RoPE + paged KV write (QKV projection)
 // Rows of the activation boxes a GEMM over M rows loads (the box height of GemmSm100Args::tmA): a call of few rows does
 // not fill the rest of its 128-row tile (see hsd_gemm_sm100.cu).
 inline uint32_t gemm_a_box_rows(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : 128; }
+// What of a call's rows a tile choice depends on: their box, and beyond 64 rows how many 128-row tiles they are.
+inline int gemm_row_class(int M) { return M <= 16 ? 0 : M <= 32 ? 1 : M <= 64 ? 2 : 2 + (M + 127) / 128; }
+inline int gemm_class_rows(int row_class) { return row_class < 3 ? 16 << row_class : (row_class - 2) * 128; }
 struct TileChoice {
   int bn, splits;              // tile width (0: the problem does not allow what a test asked for), K slices
   bool pair;
@@ -267,12 +270,12 @@ struct GemmSm100Args {
   int max_splits;              // GS_ADD_F32: most K slices per tile (1 = none; slices add in arrival order)
   bool pdl;                    // launch with programmatic stream serialization
   int pair;                    // CTA pairs (clusters of two sharing a 256-row tile) may be used
-  TileChoice tile;             // gemm_choose_tile's
+  TileChoice tile;             // gemm_choose_tile's, or a plan's
 };
 enum GemmSm100Mode { GS_STORE_BF16 = 0, GS_ADD_F32 = 1, GS_SWIGLU = 2, GS_ARGMAX = 4, GS_QKV_ROPE = 5, GS_QKV_ROPE128 = 6 };
 // Loads the kernels of a mode on the current device (ordinal `device`), before their first launch there; 0 on success.
 int gemm_sm100_prepare(int device, int mode, int* n_kernels);
-// The tile of a problem, by its M, n_out, K, mode, n_sms, max_splits and pair alone: one choice serves every layer of a call.
+// The tile of a problem, by the row class of its M, n_out, K, mode, n_sms, max_splits and pair alone.
 // Tests: `force_bn` = tile width (above 256: a CTA pair, 256 columns less), `force_splits` = K slices instead of the model's
 // choice (0 = choose).
 TileChoice gemm_choose_tile(const GemmSm100Args& a, int force_bn, int force_splits);

@@ -1,5 +1,5 @@
-"""The host's work around a call's launches does not grow with the decoder's depth: GEMM tiles are chosen once per projection
-of a call and once for its LM head.  A context's creation loads the kernels and encodes the maps of the tile widths that its
+"""The host's work around a call's launches does not grow with the decoder's depth: GEMM tiles are chosen when a context is
+created, for calls of up to 8,192 rows, and once per projection of a larger call.  A context's creation loads the kernels and encodes the maps of the tile widths that its
 projections can be given, and no others."""
 import numpy as np
 import pytest
@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("layers", [1, 7])
-def test_one_tile_choice_per_projection_and_call(layers):
+def test_tile_choices(layers):
     import torch
     from paper_2602_12957_b200 import binding as B
     from paper_2602_12957_b200 import runtime as R
@@ -27,12 +27,16 @@ def test_one_tile_choice_per_projection_and_call(layers):
         eng.check_device()
         return B.hsd_debug_host_work(model.ctx)[1]["tile_choices"] - before
 
-    assert choices(lambda: eng.prefill([None, None], [np.arange(13), np.arange(7)])) == 5
-    assert choices(lambda: eng.verify_regions(toks, cu, 13, 20)) == 5
-    assert choices(lambda: eng.verify_tree(toks, cu, parent, 13, 20)) == 5
+    assert choices(lambda: eng.prefill([None, None], [np.arange(13), np.arange(7)])) == 0
+    assert choices(lambda: eng.verify_regions(toks, cu, 13, 20)) == 0
+    assert choices(lambda: eng.verify_tree(toks, cu, parent, 13, 20)) == 0
     x = torch.zeros(64, 64, dtype=torch.bfloat16, device=model.device)
     st = torch.cuda.current_stream().cuda_stream
     assert choices(lambda: B.check(B.hsd_op_linear(model.ctx, x, x, x.clone(), 64, 64, 64, 0, st))) == 1
+    for rows, n in ((8192, 0), (8193, 4)):                # (the LM head of a prefill has a row a sequence)
+        kv = R.KvCache(model, [rows])
+        eng = R.Engine(model, kv, rows, 1)
+        assert choices(lambda: eng.prefill([None], [np.arange(rows) % cfg.vocab])) == n
 
 
 # widths of a projection's tiles, pairs' among them: heads of 64 keep whole heads, heads of 128 too; kernels: three for a width of 64
@@ -48,4 +52,4 @@ def test_a_context_prepares_its_models_widths_only(head_dim, qkv_maps, qkv_kerne
         # residual adds 64, 96 .. 256, SwiGLU the same without 96, LM head 64, 128, 256
         assert work["weight_maps"] == 3 * (qkv_maps + 7 + 6 + 7) + 3
         assert work["gemm_kernels"] == qkv_kernels + (8 + 6) + (8 + 5) + (5 + 2)
-        assert work["tile_choices"] == 0
+        assert work["tile_choices"] == 5 * (3 + 64)
