@@ -39,7 +39,8 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # captures summarised under profiles/, per workload; a class is absent (-> null) when its kernel has changed since
 # its counters were taken, or when no capture of that workload exists.
 NCU_TRAFFIC_BYTES = {
-    "region": {"attention": 30_976_768 + 512},
+    "region": {"attention": 30_976_768 + 512, "gemm_gate_up": 19_523_840, "gemm_qkv": 7_280_896, "gemm_o": 10_247_936,
+               "gemm_down": 24_668_160},
     "long2048": {"attention": 42_723_584 + 3_332_096},
 }
 

@@ -339,7 +339,8 @@ HSD_API int hsd_profile_enable(hsd_ctx *ctx, int enable);
 HSD_API int hsd_profile_read(hsd_ctx *ctx, int cap, const char **names, double *total_ms, long long *launches);
 
 /* Test-only: full logits of the query rows of the LAST verify call that used `workspace`
- * (fp32 [total_q, vocab], row-major); total_q and n_seqs must be that call's.  Slow plain kernel. */
+ * (fp32 [total_q, vocab], row-major); total_q and n_seqs must be that call's (hsd_verify_tree: 2 * total_q, of whose rows the
+ * first total_q are the nodes').  Slow plain kernel. */
 HSD_API int hsd_debug_logits(hsd_ctx *ctx, const void *workspace, int total_q, int n_seqs, float *logits,
                      void *cuda_stream);
 

@@ -729,22 +729,26 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
   return cudaLaunchKernelEx(&cfg, gemm_sm100_kernel<BN, MODE, PAIR, ROWS>, a.tmA, tmB, a.tmC, p) == cudaSuccess ? 0 : -1;
 }
 
-// Tile width, CTA pairing and K slices: the least time by a model of one launch, in us.  What decides is the last wave: a
-// projection of ~600 rows has 1.3 waves of 128 x 256 tiles, and 0.9 of 128 x 160.  So tiles come in seven widths, for single CTAs
-// and pairs, and any of them may be cut in up to eight K slices (residual adds).  Least squares over 8,000 timings (back to back
-// in a graph, 4 projections of the 24-layer decoder at 41 row counts from 16 to 9,300 and 4 of a decoder twice as wide at 7):
+// Tile width, CTA pairing and K slices: the least time by a model of one launch, in us.  What decides is how full the last wave is
+// and how wide the tiles that it is paid in: 1,323 rows of gate/up are 192 pair tiles of 256 columns, 2.6 waves of 74 pairs paid
+// as three, or 222 of 224 columns, three whole waves; 600 rows are 160 tiles of 256 columns, 1.08 waves paid as two, or 260 of 160,
+// the same two waves with five eighths of the columns each (15.5 -> 11.6 us).  So tiles come in the widths of has_width, and residual adds may cut them in up to eight K slices.
+// Least squares over 8,000 timings (back to back in a graph, 4 projections of the 24-layer decoder at 41 row counts from 16 to
+// 9,300 and 4 of a decoder twice as wide at 7):
 //   a k-block of 64: by the rows filled (A box + tile width: L2 -> SM) with a floor, or by a pair's width; up to a quarter less
 //   where the launch leaves SMs idle; a wave: 0.7 / 0.8; the last epilogue: by width, residual adds dearest; a launch 2.4, a pair 0.9
 // more.  Calls of at most 64 rows load activation boxes of 16, 32 or 64 rows: the rest of the MMA's 128 rows is whatever the stage
 // held (rows are independent, and rows beyond M go nowhere), where a full box would fill them with zeros at the same cost as data.
-// Its choices are within 0.8 % of the best timed one on average (worst 8.5 %).  With widths of 64, 128 and 256 (pairs: 256) and a
+// On these timings, to which it is fitted, its choices are within 0.8 % of the best on average (worst 8.5 %).  With widths of 64, 128 and 256 (pairs: 256) and a
 // model by fill rates alone it was 8.1 % (worst 70 %).  A layer's four projections, before / now: 300 rows 28.6 / 26.1 us, 600
 // rows 37.8 / 32.3, 900 rows 41.2 / 38.5, 1,323 rows 52.5 / 48.3, 2,600 rows 83 / 73, 5,000 rows 147 / 123, 9,300 rows 217 / 216.
 // A choice takes ~0.2 us of the host (residual adds 0.5).  It depends on the rows through gemm_row_class alone: a context makes the
 // choices of every class when it is created and a call looks its five up.  (Made for every layer of a call they were 1 us of a
 // one-layer step's 29 us of enqueueing and 25 us of 24 layers' 430.)
-// Tile widths a mode has: whole heads for the rotary epilogues, whole 64-column stores for the plain one; the adds take any 32
-// columns, SwiGLU any 16.
+// Tile widths a mode has: whole heads for the rotary epilogues, whole 64-column stores for the plain one; the adds could take any 32
+// columns, SwiGLU any 16.  Single CTAs / pairs: adds 64 to 256 without 224 / 96 to 256 (the model would give single CTAs 224 in
+// 0.5 % of the problems), SwiGLU 64, 128 to 256 / 128 to 256, plain stores and heads of 64 64, 128, 192, 256 / 128, 192, 256, heads of
+// 128 128, 256 / 128, 256, LM head 64, 128, 256 / 128, 256.
 constexpr bool has_width(int mode, int bn, bool pair) {
   switch (bn) {
     case 64: return !pair && mode != GS_QKV_ROPE128;
@@ -756,7 +760,7 @@ constexpr bool has_width(int mode, int bn, bool pair) {
   }
 }
 // Where 96, 160, 192 or 224 do not divide the output's columns, the last tile reaches beyond: TMA fills weight rows beyond the
-// last with zeros and drops columns beyond the output's.
+// last with zeros (for SwiGLU's gate half they are the first `up` rows instead) and drops columns beyond the output's.
 static bool width_fits(int mode, int n_cols, int bn, bool pair) {
   return has_width(mode, bn, pair) && ((bn & (bn - 1)) || n_cols % (mode == GS_SWIGLU ? bn / 2 : bn) == 0);
 }
