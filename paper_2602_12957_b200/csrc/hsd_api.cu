@@ -648,7 +648,7 @@ int hsd_create(const hsd_model_config* cfg, const hsd_weights* w, hsd_ctx** out)
   if (!c->simt) {
     const int qkv_mode = md.D == 128 ? GS_QKV_ROPE128 : GS_QKV_ROPE;
     int bad = tma_init();
-    for (int mode : {qkv_mode, (int)GS_ADD_F32, (int)GS_SWIGLU, (int)GS_ARGMAX}) bad = bad || gemm_sm100_prepare(dev, mode, &c->n_gemm_kernels);
+    for (int mode : {qkv_mode, (int)GS_ADD_F32, (int)GS_SWIGLU, (int)GS_ARGMAX}) bad = bad || gemm_sm100_prepare(mode, &c->n_gemm_kernels);
     if (bad) { delete c; return HSD_ERR_CUDA; }
     c->tm_qkv.resize(md.n_layers); c->tm_o.resize(md.n_layers);
     c->tm_gate_up.resize(md.n_layers); c->tm_down.resize(md.n_layers);
@@ -1234,7 +1234,7 @@ int hsd_op_linear(hsd_ctx* c, const void* A, const void* W, void* C, int M, int 
   g.status = nullptr; g.n_sms = c->n_sms; g.max_splits = c->max_splits; g.pdl = false; g.pair = c->pair;
   g.tile = choose_tile(c, g, c->force_bn, c->force_splits);
   int kernels = 0;
-  if (gemm_sm100_prepare(c->device, mode, &kernels)) return fail_cuda(c);
+  if (gemm_sm100_prepare(mode, &kernels)) return fail_cuda(c);
   if (g.tile.bn && make_tmap_2d(&wm.half_tile(g.tile.bn), W, n_out, K, g.tile.bn / 2)) return HSD_ERR_CUDA;
   if (launch_gemm_sm100(st, g)) return fail_cuda(c);
   return check_cuda(c);

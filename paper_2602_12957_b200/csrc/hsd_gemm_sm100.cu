@@ -848,8 +848,9 @@ static int prepare_mode(int device, int* n_kernels) {
   }
   return 0;
 }
-int gemm_sm100_prepare(int device, int mode, int* n_kernels) {
-  if (device < 0 || device >= kMaxDevices) return -1;
+int gemm_sm100_prepare(int mode, int* n_kernels) {
+  int device = -1;
+  if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= kMaxDevices) return -1;
   switch (mode) {
     case GS_STORE_BF16: return prepare_mode<GS_STORE_BF16>(device, n_kernels);
     case GS_ADD_F32: return prepare_mode<GS_ADD_F32>(device, n_kernels);

@@ -273,8 +273,8 @@ struct GemmSm100Args {
   TileChoice tile;             // gemm_choose_tile's, or a plan's
 };
 enum GemmSm100Mode { GS_STORE_BF16 = 0, GS_ADD_F32 = 1, GS_SWIGLU = 2, GS_ARGMAX = 4, GS_QKV_ROPE = 5, GS_QKV_ROPE128 = 6 };
-// Loads the kernels of a mode on the current device (ordinal `device`), before their first launch there; 0 on success.
-int gemm_sm100_prepare(int device, int mode, int* n_kernels);
+// Loads the kernels of a mode on the current device, before their first launch there; 0 on success.
+int gemm_sm100_prepare(int mode, int* n_kernels);
 // The tile of a problem, by the row class of its M, n_out, K, mode, n_sms, max_splits and pair alone.
 // Tests: `force_bn` = tile width (above 256: a CTA pair, 256 columns less), `force_splits` = K slices instead of the model's
 // choice (0 = choose).
