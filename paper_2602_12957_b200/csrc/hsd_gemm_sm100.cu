@@ -788,9 +788,13 @@ static TileChoice pick_tile(int mode, int n_cols, int M, int K, int n_sms, int m
       const long long tiles = (long long)((M + tile_m - 1) / tile_m) * ((n_cols + out_n - 1) / out_n);
       const double fill = 0.00042 * gemm_a_box_rows(M) + 0.00122 * bn, least = bn == 64 ? 0.150 : 0.183;
       double kb_us = pair ? (bn <= 96 ? 0.146 : 0.0137 + 0.00125 * bn) : (fill > least ? fill : least);
-      // the LM head's weights come from HBM, and a pair takes a tile of them once for 256 rows (144 rows: 20.3 us on 256-wide
-      // tiles, 17.9 on pairs of that width; 16 rows: 16.5, on 128-wide tiles 14.7)
-      if (mode == GS_ARGMAX && !pair && M > BM) kb_us *= 1.15;
+      // The LM head's weights come from HBM.  One row tile of it waits for them, and has more of them under way on narrower tiles:
+      // at 1 to 128 rows 128 columns take 0.91 to 1.00 of 256 columns' time (vocabularies of 32,768 to 131,072, K of 512 to 4,096,
+      // L2 flushed; 16 rows, 131,072 x 2,048: 107 and 114 us with the call's two small kernels).  Beyond, a pair takes a tile of
+      // weights once for 256 rows (144 rows: 20.3 us on 256-wide tiles, 17.9 on pairs of that width): 1.11 fits 360 timings at 1 to
+      // 2,049 rows, with choices 2.0 % off the best on average; 1.15 put 640 rows of large vocabularies on pairs, up to 14 % slower.
+      if (mode == GS_ARGMAX && !pair && M <= BM && bn == 256) continue;
+      if (mode == GS_ARGMAX && !pair && M > BM) kb_us *= 1.11;
       for (int sp = 1; sp <= max_splits; ++sp) {
         const int kbs = (k_blocks + sp - 1) / sp;
         if (sp > 1 && (kbs < 2 || (long long)(sp - 1) * kbs >= k_blocks)) continue;
