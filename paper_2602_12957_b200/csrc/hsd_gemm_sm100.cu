@@ -732,16 +732,19 @@ static int launch_one(cudaStream_t st, const GemmSm100Args& a, int splits) {
 // Tile width, CTA pairing and K slices: the least time by a model of one launch, in us.  What decides is how full the last wave is
 // and how wide the tiles that it is paid in: 1,323 rows of gate/up are 192 pair tiles of 256 columns, 2.6 waves of 74 pairs paid
 // as three, or 222 of 224 columns, three whole waves; 600 rows are 160 tiles of 256 columns, 1.08 waves paid as two, or 260 of 160,
-// the same two waves with five eighths of the columns each (15.5 -> 11.6 us).  So tiles come in the widths of has_width, and residual adds may cut them in up to eight K slices.
-// Least squares over 8,000 timings (back to back in a graph, 4 projections of the 24-layer decoder at 41 row counts from 16 to
-// 9,300 and 4 of a decoder twice as wide at 7):
-//   a k-block of 64: by the rows filled (A box + tile width: L2 -> SM) with a floor, or by a pair's width; up to a quarter less
-//   where the launch leaves SMs idle; a wave: 0.7 / 0.8; the last epilogue: by width, residual adds dearest; a launch 2.4, a pair 0.9
-// more.  Calls of at most 64 rows load activation boxes of 16, 32 or 64 rows: the rest of the MMA's 128 rows is whatever the stage
-// held (rows are independent, and rows beyond M go nowhere), where a full box would fill them with zeros at the same cost as data.
-// On these timings, to which it is fitted, its choices are within 0.8 % of the best on average (worst 8.5 %).  With widths of 64, 128 and 256 (pairs: 256) and a
-// model by fill rates alone it was 8.1 % (worst 70 %).  A layer's four projections, before / now: 300 rows 28.6 / 26.1 us, 600
-// rows 37.8 / 32.3, 900 rows 41.2 / 38.5, 1,323 rows 52.5 / 48.3, 2,600 rows 83 / 73, 5,000 rows 147 / 123, 9,300 rows 217 / 216.
+// the same two waves with five eighths of the columns each (15.5 -> 11.6 us).  So tiles come in the widths of has_width, and
+// residual adds may cut them in up to eight K slices.  The model's terms:
+//   a k-block of 64: by the rows filled (A box + tile width: L2 -> SM) with a floor, or by a pair's width; up to a sixth less
+//   where the launch leaves SMs idle; a wave: 1.08 / 0.77; the last epilogue: by width, the rotary one of 128-column heads dearest;
+//   a launch 2.4, a pair 1.25 more.
+// Calls of at most 64 rows load activation boxes of 16, 32 or 64 rows: the rest of the MMA's 128 rows is whatever the stage held
+// (rows are independent, and rows beyond M go nowhere), where a full box would fill them with zeros at the same cost as data.
+// Fitted to 25,000 timings of whole steps in which one projection is given another tile (weights from HBM, the real epilogues:
+// decoders 256 to 4,096 wide, heads of 64 and 128, 16 to 8,019 rows): all of a layer's choices together cost 0.5 to 0.7 % of it over the
+// best ones (before: 1.4 to 1.8 %; with widths of 64, 128 and 256 and a model by fill rates alone 4 to 5 %).  A fit to launches of
+// the plain-store epilogue back to back, their weights in L2, had rated the rotary epilogue of 128-column heads at a fifth (256-wide
+// QKV tiles for 128-wide ones, 121 -> 112 us a layer of 2,048 columns at 612 rows) and single tiles against pairs too well
+// (gate/up of the same layer 121 -> 117).  Fitted to half of the row counts, the model lost 0.75 % on the others.
 // A choice takes ~0.2 us of the host (residual adds 0.5).  It depends on the rows through gemm_row_class alone: a context makes the
 // choices of every class when it is created and a call looks its five up.  (Made for every layer of a call they were 1 us of a
 // one-layer step's 29 us of enqueueing and 25 us of 24 layers' 430.)
@@ -774,11 +777,21 @@ int make_weight_tmaps(WeightMaps* w, const void* base, int rows, int cols, int m
   }
   return bad;
 }
+struct TileModel {
+  double row, col, least64, least;      // a k-block of a single CTA: a row of the A box, a column, the floor (64 columns wide, wider)
+  double pair96, pair0, pair_col;       // of a pair: 96 columns wide, wider
+  double alone;                         // what a k-block takes where a launch has one tile
+  double wave, wave_pair, pair, cut_col;
+};
+constexpr TileModel kProjectionModel = {0.00034, 0.00068, 0.117, 0.120, 0.0883, 0.0240, 0.00060, 0.84, 1.08, 0.766, 1.25, 0.00094};
+constexpr TileModel kLmHeadModel = {0.00042, 0.00122, 0.150, 0.183, 0.146, 0.0137, 0.00125, 0.75, 0.68, 0.78, 0.9, 0.0};
 static TileChoice pick_tile(int mode, int n_cols, int M, int K, int n_sms, int max_splits, bool allow_pair) {
   const int k_blocks = K / KSUB;
   TileChoice best = {mode == GS_QKV_ROPE128 ? 128 : 64, 1, false};
   double best_us = 1e30;
-  const double epi = mode == GS_ADD_F32 ? 0.0105 : mode == GS_SWIGLU ? 0.0014 : mode == GS_STORE_BF16 ? 0.0036 : mode == GS_ARGMAX ? 0.015 : 0.0065;   // a column
+  const TileModel& m = mode == GS_ARGMAX ? kLmHeadModel : kProjectionModel;
+  const double epi = mode == GS_ADD_F32 ? 0.00746 : mode == GS_SWIGLU ? 0.0137 : mode == GS_STORE_BF16 ? 0.0036 : mode == GS_ARGMAX ? 0.015 :
+                     mode == GS_QKV_ROPE128 ? 0.0314 : 0.0082;   // a column
   for (int pair = allow_pair && M > 64 ? 1 : 0; pair >= 0; --pair) {      // (a pair's tile needs whole boxes)
     for (int bn = 256; bn >= 64; bn -= 32) {
       if (!width_fits(mode, n_cols, bn, pair != 0)) continue;
@@ -786,8 +799,8 @@ static TileChoice pick_tile(int mode, int n_cols, int M, int K, int n_sms, int m
       const int tile_m = pair ? 2 * BM : BM;
       const int walkers = pair ? n_sms / 2 : n_sms;
       const long long tiles = (long long)((M + tile_m - 1) / tile_m) * ((n_cols + out_n - 1) / out_n);
-      const double fill = 0.00042 * gemm_a_box_rows(M) + 0.00122 * bn, least = bn == 64 ? 0.150 : 0.183;
-      double kb_us = pair ? (bn <= 96 ? 0.146 : 0.0137 + 0.00125 * bn) : (fill > least ? fill : least);
+      const double fill = m.row * gemm_a_box_rows(M) + m.col * bn, least = bn == 64 ? m.least64 : m.least;
+      double kb_us = pair ? (bn <= 96 ? m.pair96 : m.pair0 + m.pair_col * bn) : (fill > least ? fill : least);
       // The LM head's weights come from HBM.  One row tile of it waits for them, and has more of them under way on narrower tiles:
       // at 1 to 128 rows 128 columns take 0.91 to 1.00 of 256 columns' time (vocabularies of 32,768 to 131,072, K of 512 to 4,096,
       // L2 flushed; 16 rows, 131,072 x 2,048: 107 and 114 us with the call's two small kernels).  Beyond, a pair takes a tile of
@@ -801,8 +814,8 @@ static TileChoice pick_tile(int mode, int n_cols, int M, int K, int n_sms, int m
         const long long units = tiles * sp;
         const long long rounds = (units + walkers - 1) / walkers;
         const double load = units < walkers ? (double)units / walkers : 1.0;
-        const double us = 2.4 + (pair ? 0.9 : 0.0) + rounds * (kbs * kb_us * (0.75 + 0.25 * load) + (pair ? 0.78 : 0.68)) +
-                          epi * bn + (sp > 1 ? 0.00073 * bn : 0.0);
+        const double us = 2.4 + (pair ? m.pair : 0.0) + rounds * (kbs * kb_us * (m.alone + (1.0 - m.alone) * load) + (pair ? m.wave_pair : m.wave)) +
+                          epi * bn + (sp > 1 ? m.cut_col * bn : 0.0);
         if (us < 0.99 * best_us) { best_us = us; best = {bn, sp, pair != 0}; }      // (as good: the wider one, with less traffic)
       }
     }
