@@ -396,6 +396,10 @@ HSD_API int hsd_debug_set_gemm_tile(hsd_ctx *ctx, int tile_n, int k_slices);
  * its creation: of the tile widths that its model's projections can be given. */
 HSD_API int hsd_debug_host_work(const hsd_ctx *ctx, long long *tile_choices, int *weight_maps, int *gemm_kernels);
 
+/* Test-only: the GEMM tile that a call gives one projection for `rows` (1 .. 8192) packed rows: projection 0 = QKV, 1 = O,
+ * 2 = gate/up, 3 = down, 4 = LM head; out[0] = columns, out[1] = K slices, out[2] = 1 for a pair of CTAs. */
+HSD_API int hsd_debug_tile(const hsd_ctx *ctx, int projection, int rows, int *out);
+
 /* Test-only: the attention launch cuts the KV ranges of the query tiles into slices so that it has about `target_items`
  * work items (never more than CTA slots in one round), none shorter than `min_kv_tiles` 128-token KV tiles (two paged
  * blocks; 0 = the library's defaults).  With `min_kv_tiles` > 0 a range is cut that finely wherever there are CTA slots and

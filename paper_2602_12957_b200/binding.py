@@ -34,6 +34,7 @@ EXPORTS = [
     "hsd_verify_page", "hsd_kv_commit", "hsd_verify_regions_host", "hsd_device_status", "hsd_last_cuda_error", "hsd_launch_count",
     "hsd_profile_enable", "hsd_profile_read", "hsd_debug_logits", "hsd_debug_buffer", "hsd_op_linear",
     "hsd_op_lm_head_argmax", "hsd_op_lm_head_argmax_noalloc", "hsd_debug_set_gemm_tile", "hsd_debug_set_attn_plan", "hsd_debug_host_work",
+    "hsd_debug_tile",
     "hsd_verify_tree", "hsd_kv_commit_tree", "hsd_dsv_build", "hsd_debug_tap", "hsd_stage_begin", "hsd_stage_advance",
     "hsd_stage_aggregate",
 ]
@@ -111,6 +112,7 @@ def _load():
     lib.hsd_debug_set_gemm_tile.argtypes = [vp, i, i]
     lib.hsd_debug_set_attn_plan.argtypes = [vp, i, i]
     lib.hsd_debug_host_work.argtypes = [vp, C.POINTER(C.c_longlong), C.POINTER(i), C.POINTER(i)]
+    lib.hsd_debug_tile.argtypes = [vp, i, i, C.POINTER(i)]
     lib.hsd_op_linear.argtypes = [vp, vp, vp, vp, i, i, i, i, vp]
     lib.hsd_op_lm_head_argmax.argtypes = [vp, vp, i, vp, vp, sz, vp, vp, vp, vp]
     lib.hsd_op_lm_head_argmax_noalloc.argtypes = [vp, vp, i, vp, vp, vp, vp, vp]
@@ -329,6 +331,12 @@ def hsd_debug_host_work(ctx):
     n, maps, kernels = C.c_longlong(0), C.c_int(0), C.c_int(0)
     st = _lib.hsd_debug_host_work(ctx, C.byref(n), C.byref(maps), C.byref(kernels))
     return st, {"tile_choices": n.value, "weight_maps": maps.value, "gemm_kernels": kernels.value}
+
+
+def hsd_debug_tile(ctx, projection: int, rows: int):
+    out = (C.c_int * 3)()
+    st = _lib.hsd_debug_tile(ctx, projection, rows, out)
+    return st, tuple(out)
 
 
 def hsd_debug_set_attn_plan(ctx, target_items: int, min_kv_tiles: int) -> int:

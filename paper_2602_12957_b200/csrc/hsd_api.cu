@@ -1204,6 +1204,14 @@ int hsd_debug_host_work(const hsd_ctx* c, long long* tile_choices, int* weight_m
   return HSD_OK;
 }
 
+int hsd_debug_tile(const hsd_ctx* c, int projection, int rows, int* out) {
+  if (!c || c->simt || !out || projection < 0 || projection > 4 || rows < 1 || rows > TilePlan::kRows) return HSD_ERR_INVALID_ARG;
+  const TilePlan* plans[5] = {&c->tiles_qkv, &c->tiles_o, &c->tiles_gate_up, &c->tiles_down, &c->tiles_lm_head};
+  const TileChoice& t = plans[projection]->of[gemm_row_class(rows)];
+  out[0] = t.bn; out[1] = t.splits; out[2] = t.pair;
+  return HSD_OK;
+}
+
 int hsd_debug_set_attn_plan(hsd_ctx* c, int target_items, int min_kv_tiles) {
   if (!c || target_items < 0 || min_kv_tiles < 0) return HSD_ERR_INVALID_ARG;
   c->attn_target_items = target_items ? target_items : attn_grid(c);

@@ -1,8 +1,6 @@
 """The QKV projection with its rotary epilogue and K/V stores on every tile width (192 columns are three heads, and the last tile
 of 32 heads has one too many; pairs too): queries and K/V rows equal the narrowest tile's bit by bit, as K is summed in one order.
 And the width that a step of wide heads takes, whose epilogue is dear."""
-import re
-
 import numpy as np
 import pytest
 
@@ -45,18 +43,13 @@ def test_widths_agree(rows, qk_norm, head_dim):
 
 
 def test_wide_heads_take_narrow_tiles():
-    import torch
-    from torch.profiler import ProfilerActivity, profile
+    from paper_2602_12957_b200 import binding as B
     from paper_2602_12957_b200 import runtime as R
     cfg = I.ModelConfig(n_layers=1, d_model=2048, n_heads=16, n_kv_heads=8, head_dim=128, d_ffn=8192, vocab=4096, qk_norm=True)
     model = R.DeviceModel(cfg, I.make_weights(cfg, 2))
-    rows = 612
-    eng = R.Engine(model, R.KvCache(model, [rows]), rows, 1)
-    toks, cu = eng._i32(np.arange(rows)), eng._i32([0, rows])
-    eng.verify_regions(toks, cu, rows, rows)
-    torch.cuda.synchronize()
-    with profile(activities=[ProfilerActivity.CUDA]) as p:
-        eng.verify_regions(toks, cu, rows, rows)
-        torch.cuda.synchronize()
-    tiles = {int(m[2]): int(m[1]) for m in (re.search(r"gemm_sm100_kernel<(\d+), (\d+), ", e.key) for e in p.key_averages()) if m}
-    assert tiles[6] == 128, tiles          # the rotary epilogue of 128-column heads: 121 us a layer on 256-wide tiles, 112 on these
+    for rows in (513, 612, 640, 700, 768):
+        # the rotary epilogue of 128-column heads: 121 us a layer of 612 rows on 256-wide tiles, 112 on these
+        assert B.hsd_debug_tile(model.ctx, 0, rows) == (B.HSD_OK, (128, 1, 1)), rows
+    for rows in (305, 612):      # gate/up: 88.8 us a layer of 305 rows on single tiles, 85.9 on pairs; 121 and 117 of 612 rows
+        assert B.hsd_debug_tile(model.ctx, 2, rows) == (B.HSD_OK, (224, 1, 1)), rows
+    assert B.hsd_debug_tile(model.ctx, 5, 1)[0] == B.hsd_debug_tile(model.ctx, 0, 8193)[0] == B.HSD_ERR_INVALID_ARG
